@@ -29,8 +29,8 @@
  *     summaries; T_a = ceil(seq_kv / block) chunks exist; W = ceil(T_a / 32) mask words per row.
  *   - Query head h uses KV head h / (h_q / h_kv) (Section 3.2).
  *   - Which kernels run: bf16 tensors take the TMA / tcgen05 kernels (head_dim 64 or 128, every chunk size; prefill
- *     needs g_q = h_q / h_kv >= 2, decode takes every group size); fp32 tensors, g_q = 1 in prefill and the
- *     non-causal mode take CUDA-core kernels that compute the same thing (the correctness path).
+ *     and decode take every group size g_q = h_q / h_kv); fp32 tensors and the non-causal mode take CUDA-core
+ *     kernels that compute the same thing.
  *     The choice is made from the parameters alone, never from the data, and is the same on every call.
  *   - causal = 1 is the paper's setting and the one the tensor-core kernels serve.  causal = 0 (prefill only;
  *     the paper does not define it) is read as: every complete chunk is a candidate of every row; the

@@ -297,10 +297,10 @@ int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void
                                                        (cudaStream_t)stream));
 }
 
-// Layout of the backward scratch: status region, then lse2 and delta [batch][KV head][query tile][128 rows], then the
+// Layout of the backward scratch: status region, then (log-sum-exp, delta) [batch][KV head][query tile][128 rows], then the
 // routed-chunk prefix counts [batch * h_kv * seq_q][W].
 struct BwdLayout {
-  size_t status, lse2, delta, prefix, total;
+  size_t status, stats, prefix, total;
 };
 static BwdLayout bwd_layout(const Dims& dm) {
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -309,8 +309,7 @@ static BwdLayout bwd_layout(const Dims& dm) {
   size_t at = up(STATUS_REGION_BYTES);
   const int tq = std::max(1, std::min(128 / std::max(dm.g_q, 1), dm.B));
   const size_t rows = (size_t)dm.batch * dm.h_kv * (size_t)((dm.seq_q + tq - 1) / tq) * 128;
-  l.lse2 = at; at = up(at + rows * sizeof(float));
-  l.delta = at; at = up(at + rows * sizeof(float));
+  l.stats = at; at = up(at + rows * sizeof(float2));
   // prefix counts [batch * h_kv * seq_q][W], then the tiles' mask unions [batch * h_kv][query tile][W]
   l.prefix = at; at = up(at + ((size_t)dm.batch * dm.h_kv * dm.seq_q + (size_t)dm.batch * dm.h_kv * ((dm.seq_q + tq - 1) / tq)) *
                                   (size_t)dm.W * sizeof(int));
@@ -347,8 +346,8 @@ int dash_attn_bwd_attend_prefill_tc(const dash_params* p, const void* Q, const v
   if (list_bytes > 0) {
     if ((rc = cuda_status(cudaMemsetAsync(dbias, 0, list_bytes, st))) != DASH_OK) return rc;
   }
-  return cuda_status(launch_attend_prefill_bwd_sm100(dm, Q, K, V, dO, mask, blk_bias, at<float>(bwd_workspace, l.lse2),
-                                                     at<float>(bwd_workspace, l.delta), at<int>(bwd_workspace, l.prefix),
+  return cuda_status(launch_attend_prefill_bwd_sm100(dm, Q, K, V, dO, mask, blk_bias, at<float2>(bwd_workspace, l.stats),
+                                                     at<int>(bwd_workspace, l.prefix),
                                                      dQ, dK, dV, dbias, at<StatusBlock>(bwd_workspace, l.status), st));
 }
 

@@ -46,6 +46,16 @@ __device__ inline void kv_locate(const Dims& dm, int b, int t, int* first, int* 
   }
 }
 
+// Where the statistics (log-sum-exp, delta) of a query row live between the kernels of the backward pass: a float2 at byte
+// strides of (batch, KV head, token, head of the group).
+struct RowStats {
+  char* base = nullptr;
+  long long sb = 0, sr = 0, si = 0, sh = 0;
+  __device__ float2* at(int b, int r, int i, int hh) const {
+    return reinterpret_cast<float2*>(base + b * sb + r * sr + i * si + hh * sh);
+  }
+};
+
 // Start of row i's list region inside its (batch, KV head) slab.
 __host__ __device__ inline long long list_row_offset(const Dims& dm, int i) {
   if (dm.decode) return 0;
@@ -261,14 +271,14 @@ bool prefill_sm100_supported(const Dims& dm);
 // inputs_stable: Q, K, V were not written by the kernel launched just before on the stream
 cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const void* K, const void* V,
                                         const uint32_t* mask, const float* blk_bias, void* O, StatusBlock* sb,
-                                        bool inputs_stable, cudaStream_t st, float* lse2 = nullptr,
-                                        float* delta = nullptr, const void* dO = nullptr);
-// Stage 2 backward on tensor cores (bf16, head_dim 128, chunks of 64 or 128 tokens, g_q >= 2); scratch: lse2 and delta
-// [batch][KV head][query tile][128] floats, prefix [batch * h_kv * seq_q][W] ints.
+                                        bool inputs_stable, cudaStream_t st, const RowStats& stats = RowStats(),
+                                        const void* dO = nullptr);
+// Stage 2 backward on tensor cores (bf16, head_dim 128, chunks of 64 or 128 tokens, g_q >= 2); scratch: stats
+// [batch][KV head][query tile][128] pairs (log-sum-exp, delta), prefix [batch * h_kv * seq_q][W] ints.
 bool prefill_bwd_sm100_supported(const Dims& dm);
 cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* dO,
-                                            const uint32_t* mask, const float* blk_bias, float* lse2, float* delta,
-                                            int* prefix, void* dQ, float* dK, float* dV, float* dbias, StatusBlock* sb,
+                                            const uint32_t* mask, const float* blk_bias, float2* stats, int* prefix, void* dQ,
+                                            float* dK, float* dV, float* dbias, StatusBlock* sb,
                                             cudaStream_t st);
 
 }  // namespace dash

@@ -44,8 +44,7 @@ struct BwdArgs {
   long long wait_limit;
   const uint32_t* mask;
   const float* blk_bias;
-  const float* lse2;
-  const float* delta;
+  const float2* stats;          // (log-sum-exp, delta) of every row, [batch][KV head][query tile][128 rows]
   const int* prefix;
   const uint32_t* tile_union;   // [batch * h_kv][query tile][W]: OR of the tile's rows' mask words
   __nv_bfloat16* dQ;
@@ -376,8 +375,8 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float c1 = dm.sm_scale * LOG2E;
     const long long srow = (((long long)b * dm.h_kv + r) * a.n_tiles + tile) * 128 + m;
-    const float lse2 = row_ok ? a.lse2[srow] : 0.f;
-    const float delta = row_ok ? a.delta[srow] : 0.f;
+    const float2 stat = row_ok ? a.stats[srow] : make_float2(0.f, 0.f);
+    const float lse2 = stat.x, delta = stat.y;
     bool ok = true;
     int n_steps = 0x7fffffff;              // known from step 1 on; step 0 (the own chunk) always exists
     for (int j = 0; j < n_steps && ok; ++j) {
@@ -494,8 +493,7 @@ struct Misc {
   int total;                            // number of steps, written with the end marker
   int tile[2];                          // query tile of the stage's step (-1: no more steps)
   float bias[2][MAX_TQ];                // per token of the tile: the chunk's bias (-inf: the token does not attend it)
-  alignas(16) float lse2[2][128];       // the tile's row statistics (bulk copies)
-  alignas(16) float delta[2][128];
+  alignas(16) float2 stats[2][128];     // the tile's row statistics (a bulk copy)
 };
 constexpr uint32_t OFF_K = 0, OFF_V = OFF_K + KV_TILE_BYTES, OFF_Q = OFF_V + KV_TILE_BYTES,   // Q stage s at OFF_Q + s * 2 * Q_BYTES,
                    OFF_P = OFF_Q + 4 * Q_BYTES, OFF_DS = OFF_P + PS_BYTES,                   //   its dO tile Q_BYTES behind
@@ -590,13 +588,12 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (tile_idx >= 0) {
           const int i0 = tile_idx * TQ;
           const uint32_t dst = sbase + OFF_Q + st * 2 * Q_BYTES;
-          ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), 2 * Q_BYTES + 2 * 512);
+          ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), 2 * Q_BYTES + 1024);
           ptx::tma_load_4d(dst, &tmQ, bar(QD_FULL + st), 0, r * g_q, i0, b);
           ptx::tma_load_4d(dst + Q_BYTES / 2, &tmQ, bar(QD_FULL + st), 64, r * g_q, i0, b);
           ptx::tma_load_4d(dst + Q_BYTES, &tmDO, bar(QD_FULL + st), 0, r * g_q, i0, b);
           ptx::tma_load_4d(dst + Q_BYTES + Q_BYTES / 2, &tmDO, bar(QD_FULL + st), 64, r * g_q, i0, b);
-          ptx::bulk_load(ptx::smem_u32(&misc->lse2[st][0]), a.lse2 + stat0 + (long long)tile_idx * 128, 512, bar(QD_FULL + st));
-          ptx::bulk_load(ptx::smem_u32(&misc->delta[st][0]), a.delta + stat0 + (long long)tile_idx * 128, 512, bar(QD_FULL + st));
+          ptx::bulk_load(ptx::smem_u32(&misc->stats[st][0]), a.stats + stat0 + (long long)tile_idx * 128, 1024, bar(QD_FULL + st));
         } else {
           ptx::mbar_arrive(bar(QD_FULL + st));
         }
@@ -789,8 +786,8 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       if (tile_idx < 0) break;
       const int i_row = tile_idx * TQ + t;
       const bool row_ok = i_row < dm.seq_q;
-      const float lse2 = row_ok ? misc->lse2[buf][m] : 0.f;
-      const float delta = row_ok ? misc->delta[buf][m] : 0.f;
+      const float2 stat = row_ok ? misc->stats[buf][m] : make_float2(0.f, 0.f);
+      const float lse2 = stat.x, delta = stat.y;
       const float bias = row_ok ? misc->bias[buf][t] : -INFINITY;
       const float off = bias * LOG2E - lse2;
       const int n_vis = i_row - k0 + 1 - wg * 32;            // visible columns of this warpgroup's half
@@ -887,18 +884,25 @@ bool make_map(CUtensorMap* out, const void* base, long long tokens, int heads, i
 }  // namespace
 
 bool prefill_bwd_sm100_supported(const Dims& dm) {
-  if (!prefill_sm100_supported(dm)) return false;
+  if (!prefill_sm100_supported(dm) || dm.g_q < 2) return false;
   if (dm.d != 128 || (dm.B != 64 && dm.B != 128)) return false;
   if (dm.qs[2] % 8 != 0 || dm.qs[1] % 8 != 0) return false;     // 16-byte stores of dQ rows
   return true;
 }
 
 cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* dO,
-                                            const uint32_t* mask, const float* blk_bias, float* lse2, float* delta,
-                                            int* prefix, void* dQ, float* dK, float* dV, float* dbias, StatusBlock* sb,
+                                            const uint32_t* mask, const float* blk_bias, float2* stats, int* prefix,
+                                             void* dQ, float* dK, float* dV, float* dbias, StatusBlock* sb,
                                             cudaStream_t st) {
-  // 1. forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written)
-  cudaError_t e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, lse2, delta, dO);
+  // 1. forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written), tile-major
+  const long long tile_rows = (long long)((dm.seq_q + 128 / dm.g_q - 1) / (128 / dm.g_q)) * 128;
+  RowStats rs;
+  rs.base = reinterpret_cast<char*>(stats);
+  rs.sh = sizeof(float2);
+  rs.si = rs.sh * dm.g_q;
+  rs.sr = rs.sh * tile_rows;
+  rs.sb = rs.sr * dm.h_kv;
+  cudaError_t e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, rs, dO);
   if (e != cudaSuccess) return e;
   // 2. routed-chunk counts before every mask word
   const long long rows = (long long)dm.batch * dm.h_kv * dm.seq_q;
@@ -912,7 +916,7 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, const void* Q, const
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
   a.n_slices = (dm.seq_kv + NKV - 1) / NKV;
   a.wait_limit = test_hooks().wait_limit_cycles;
-  a.mask = mask; a.blk_bias = blk_bias; a.lse2 = lse2; a.delta = delta; a.prefix = prefix;
+  a.mask = mask; a.blk_bias = blk_bias; a.stats = stats; a.prefix = prefix;
   // the tile unions sit behind the prefix counts in the same scratch region
   uint32_t* tile_union = reinterpret_cast<uint32_t*>(prefix + rows * dm.W);
   a.tile_union = tile_union;

@@ -1,11 +1,11 @@
 // Stage 2, prefill, tensor-core path for sm_100a (Eq. 7 in the form of Proposition 1; Algorithm 3).
 //
-// Tile: one (batch, KV head) and TQ = min(128/g_q, chunk size) consecutive query tokens; the rows of the MMA tile
-// are (token, head-of-group) pairs, token-major (with chunks shorter than 128/g_q tokens the tile holds fewer than
-// 128 live rows; the rest are zero queries whose results are dropped).  A tile never straddles a chunk, so its rows share the own
-// chunk; it takes the own chunk first (its tiles can be fetched before the mask has been read), then walks
-// the UNION of its rows' routed chunks in ascending order, 64 KV tokens per step.  A row that did not route
-// a chunk gets bias -inf for that step (probability exactly 0), so every row still attends to its own
+// Tile: one (batch, KV head) and TQ = 128/g_q consecutive query tokens; the rows of the MMA tile are (token,
+// head-of-group) pairs, token-major.  Tiles start at multiples of TQ.  Where a chunk holds at least TQ tokens the tile's
+// rows share their own chunk; where chunks are shorter (WIDE) the tile spans several, and every row has its own.  The own
+// chunks go first (their tiles can be fetched before the mask has been read; each row sees its own one only, causally),
+// then the tile walks the UNION of its rows' routed chunks in ascending order, 64 KV tokens per step.  A row that did
+// not route a chunk gets bias -inf for that step (probability exactly 0), so every row still attends to its own
 // selection only.
 //
 // Warp roles (256 threads = two warpgroups, two blocks per SM so one block's softmax overlaps the other's MMAs; after
@@ -29,6 +29,7 @@
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
+#include "tile_walk.cuh"
 
 namespace dash {
 
@@ -40,15 +41,15 @@ constexpr int KST = 2, VST = 2;   // ring depths: stage = step parity, like the 
 constexpr int PF_THREADS = 256;   // 4 softmax warps, K producer, MMA issuer, V/bias producer and an idle warp: two whole
                                   // warpgroups, because a warpgroup changes its register budget only when all four of
                                   // its warps ask (a block of seven warps waits for the eighth for ever)
-// Registers per thread after the re-division (two blocks per SM start with 128 each): 128 * (200 - 128) taken by the
-// softmax warpgroup = 128 * (128 - 56) given up by the other one; the block's own pool is all that it can draw from.
-constexpr int PF_REGS_SERVICE = 56, PF_REGS_SOFTMAX = 200;
-static_assert(PF_THREADS == 256 && 128 * (PF_REGS_SOFTMAX - 128) <= 128 * (128 - PF_REGS_SERVICE),
-              "the softmax warpgroup can only take what the service warpgroup released: a larger request never completes");
+// Registers per thread after the re-division (two blocks per SM start with 128 each): what the
+// softmax warpgroup takes is given up by the other one; the block's own pool is all that it can draw from.
+// (A producer lane of a wide tile keeps every token's own chunk, and looks after four tokens where the tile has 128.)
+__host__ __device__ constexpr int regs_service(int wt, int cps) { return wt > 2 ? (cps > 2 ? 96 : 88) : wt > 0 || cps > 2 ? 72 : 56; }
+__host__ __device__ constexpr int regs_softmax(int wt, int cps) { return 256 - regs_service(wt, cps); }
+static_assert(PF_THREADS == 256, "two warpgroups of equal size: one can take exactly what the other released");
 constexpr uint32_t TMEM_COLS = 256;  // S0 [0,64), S1 [64,128), O [128,256)
 constexpr float RESCALE_LOG2 = 8.f;  // the running maximum is moved only when it grew by more than this
 
-constexpr int MAX_TQ = 64;
 // S_FULL[j&1]: QK of step j complete (S readable; K stage j&1 reusable).  PV_DONE[j&1]: PV of step j complete (O stable;
 // S/P buffer and V stage j&1 reusable).  Every tcgen05.commit and every barrier test costs the issuing thread as
 // much as an MMA, so each product signals exactly one barrier and the producers listen to the same ones.
@@ -56,18 +57,19 @@ enum Bar { Q_FULL = 0, META, S_FULL = 2, PV_DONE = 4, P_FULL = 6, V_FULL = 8, K_
 static_assert(KST == 2 && VST == 2, "stage = step parity");
 // CPS = chunks per 64-token step: 1 for chunks of 64 or 128 tokens, 2 / 4 for chunks of 32 / 16 (a step then
 // packs that many chunks of the union list, each with its own per-token bias).
-template <int CPS>
+// MTQ = most tokens a tile can hold.
+template <int CPS, int MTQ>
 struct MiscT {
   unsigned long long bar[N_BARS];
   uint32_t tmem_base;
   int n_steps;
   int abort_flag;
   int kvbase[VST][CPS];
-  float bias[VST][CPS][MAX_TQ];
+  float bias[VST][CPS][MTQ];
 };
 // Shared-memory layout for head_dim HD (64 or 128): tiles are K-major regions of 64 elements (128 bytes, the
 // swizzle span) per row, one region per 64 of head_dim.
-template <int HD, int CPS>
+template <int HD, int CPS, int MTQ>
 struct PfLayout {
   static constexpr uint32_t Q_BYTES = 128 * HD * 2;           // HD = 128: 32 KiB, two 128x64 regions
   static constexpr uint32_t KV_TILE_BYTES = NKV * HD * 2;     // HD = 128: 16 KiB, two 64x64 regions
@@ -75,7 +77,7 @@ struct PfLayout {
   static constexpr uint32_t OFF_K = OFF_Q + Q_BYTES;
   static constexpr uint32_t OFF_V = OFF_K + KST * KV_TILE_BYTES;
   static constexpr uint32_t OFF_MISC = OFF_V + VST * KV_TILE_BYTES;
-  static constexpr uint32_t SMEM = OFF_MISC + sizeof(MiscT<CPS>);
+  static constexpr uint32_t SMEM = OFF_MISC + sizeof(MiscT<CPS, MTQ>);
   static_assert(SMEM <= 115712, "two blocks per SM need <= 113 KiB each");
 };
 
@@ -97,27 +99,28 @@ struct PrefillArgs {
   const uint32_t* mask;
   const float* blk_bias;
   __nv_bfloat16* O;          // may be null when only the row statistics are wanted
-  // Row statistics for the backward pass, [batch][KV head][tile][row of the tile (128)] (null: not wanted): the
-  // log-sum-exp of the row's logits in the log2 domain, and delta = <O_row, dO_row> (dO: strides of O), both from the
-  // fp32 accumulator.
-  float* lse2;
-  float* delta;
+  // Row statistics for the backward pass (base null: not wanted): the log-sum-exp of the row's logits in the log2 domain
+  // and delta = <O_row, dO_row> (dO: strides of O), both from the fp32 accumulator.
+  RowStats stats;
   const __nv_bfloat16* dO;
   StatusBlock* sb;
 };
 
-// SHORT: the tile has fewer than 128 live rows (chunks shorter than 128 / g_q tokens); full tiles compile without
-// any of the padding-row handling.
-// STATS: the kernel also leaves the row statistics the backward pass starts from (a.lse2, a.delta).  delta = <O, dO> feeds
-// the gradient of the routing, which amplifies its error, so in this mode P enters the P V product as two bf16 terms
-// (P = hi + lo, the remainder in the second half of the step's S columns): O, and with it delta, is then accurate to
-// fp32 class instead of bf16 class.
-template <int HD, int CPS, bool SHORT, bool STATS = false>
+// WT > 0: a wide tile, which may span several chunks (chunks shorter than 128 / g_q tokens, or g_q = 1), of at most
+// 32 * WT tokens; tiles inside one chunk (WT = 0, at most 64 tokens) compile without the per-row own chunks.
+// P2: P enters the P V product as two bf16 terms (P = hi + lo, the remainder in the second half of the step's S columns),
+// so O is accurate to fp32 class instead of bf16 class.  Taken for g_q = 1 and, whatever the group size, when the row
+// statistics for the backward pass are wanted (delta = <O, dO> feeds the gradient of the routing, which amplifies its
+// error).
+template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(PF_THREADS, 2)
 attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                             const __grid_constant__ CUtensorMap tmV, PrefillArgs a) {
-  using LY = PfLayout<HD, CPS>;
-  using Misc = MiscT<CPS>;
+  constexpr bool WIDE = WT > 0;
+  constexpr int TPL = WIDE ? WT : 2, MTQ = 32 * TPL;   // tokens a producer lane looks after: lane, lane + 32, ...
+  constexpr int W = NKV / CPS;                         // KV tokens of one chunk slot of a step
+  using LY = PfLayout<HD, CPS, MTQ>;
+  using Misc = MiscT<CPS, MTQ>;
   constexpr uint32_t Q_BYTES = LY::Q_BYTES, KV_TILE_BYTES = LY::KV_TILE_BYTES, OFF_Q = LY::OFF_Q, OFF_K = LY::OFF_K,
                      OFF_V = LY::OFF_V, OFF_MISC = LY::OFF_MISC;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -136,9 +139,10 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   const int b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int TQ = a.TQ, g_q = dm.g_q;
   const int i0 = tile * TQ;
-  const int c_own = i0 / dm.B;
+  const int c_own = i0 / dm.B;                        // own chunk of the tile's first token (WIDE: of that one only)
   const int sub_per_blk = dm.B / NKV;                 // 64-token steps per chunk (1 or 2)
-  const int own_steps = (i0 % dm.B) / NKV + 1;        // steps of the own chunk the tile can see
+  const int own_steps = WIDE ? (TQ + NKV - 1) / NKV   // steps over the tile's own tokens
+                             : (i0 % dm.B) / NKV + 1; // steps of the own chunk the tile can see
 
   if (tid == 0) {
     if ((sbase & 1023u) != 0u) {
@@ -169,15 +173,6 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = misc->tmem_base;
-  // Rows of the Q tile beyond the tile's TQ * g_q live rows (chunks shorter than 128 / g_q tokens) are never written by
-  // the TMA box: they are zeroed once, so that their scores are finite; their probabilities are forced to 0 below.
-  if constexpr (SHORT) {
-    const int first = TQ * g_q * 8;                 // 16-byte pieces before the first dead row (a row is 128 bytes)
-    for (int regn = 0; regn < HD / 64; ++regn)
-      for (int k = first + tid; k < 128 * 8; k += PF_THREADS)
-        *reinterpret_cast<uint4*>(smem + OFF_Q + regn * (Q_BYTES / (HD / 64)) + k * 16) = make_uint4(0u, 0u, 0u, 0u);
-    ptx::fence_proxy_async_smem();
-  }
   // A step's K or V tile for chunks smaller than the step: CPS boxes of NKV / CPS tokens, one per packed chunk.
   [[maybe_unused]] auto load_packed = [&](const CUtensorMap* tm, uint32_t dst, uint32_t barrier, const int* kvs) {
     ptx::mbar_arrive_expect_tx(barrier, KV_TILE_BYTES);
@@ -190,55 +185,35 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   };
   // Q and the own chunk's K / V tiles: they need nothing from the routing kernels (and go first anyway).
   auto own_loads = [&](bool do_k, bool do_v) {
-    const int TR = SHORT ? 128 / g_q : TQ;
     if (lane == 0 && do_k) {
       ptx::prefetch_tensormap(&tmQ);
       ptx::prefetch_tensormap(&tmK);
       ptx::prefetch_tensormap(&tmV);
-      ptx::mbar_arrive_expect_tx(bar(Q_FULL), SHORT ? (uint32_t)(TQ * g_q * HD * 2) : Q_BYTES);   // the box holds the live rows
+      ptx::mbar_arrive_expect_tx(bar(Q_FULL), Q_BYTES);
       ptx::tma_load_4d(sbase + OFF_Q, &tmQ, bar(Q_FULL), 0, r * g_q, i0, b);
       if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_Q + Q_BYTES / 2, &tmQ, bar(Q_FULL), 64, r * g_q, i0, b);
     }
     // The own chunk goes first: its tiles need nothing from the mask, so they are in flight (and the first
     // S = Q K^T can run) while the union of the routed chunks is still being formed.  Stages 0/1 are free.
     for (int sub = 0; sub < own_steps; ++sub) {
-      const int kv0 = c_own * dm.B + sub * NKV;
-      if constexpr (CPS > 1) {
-        // the own chunk fills the first slot of step 0; the other slots repeat it with bias -inf (probability 0)
-        int kvs[CPS];
+      // narrow tile: the own chunk fills the first slot, the other slots repeat it; wide tile: its own chunks in order
+      // (slots behind its last token repeat the first chunk).  bias 0 where the slot is the token's own chunk, -inf elsewhere
+      int kvs[CPS];
+      const int kv0 = WIDE ? i0 + sub * NKV : c_own * dm.B + sub * NKV;
 #pragma unroll
-        for (int s = 0; s < CPS; ++s) kvs[s] = kv0;
-        if (do_k) {
-          if (lane == 0 && !a.inject) load_packed(&tmK, sbase + OFF_K, bar(K_FULL), kvs);
-        } else {
-          for (int t = lane; t < TR; t += 32) {
-            misc->bias[0][0][t] = t < TQ ? 0.f : -INFINITY;     // token slots beyond TQ: padding rows of a short tile
-#pragma unroll
-            for (int s = 1; s < CPS; ++s) misc->bias[0][s][t] = -INFINITY;
-          }
-          if (lane < CPS) misc->kvbase[0][lane] = kv0;
-          __syncwarp();
-          if (lane == 0) load_packed(&tmV, sbase + OFF_V, bar(V_FULL), kvs);
-        }
-        continue;
-      }
+      for (int s = 0; s < CPS; ++s) kvs[s] = WIDE && kv0 + s * W < i0 + TQ ? kv0 + s * W : kv0;
       if (do_k) {
-        if (lane == 0 && !a.inject) {
-          const uint32_t dst = sbase + OFF_K + sub * KV_TILE_BYTES;
-          ptx::mbar_arrive_expect_tx(bar(K_FULL + sub), KV_TILE_BYTES);
-          ptx::tma_load_4d(dst, &tmK, bar(K_FULL + sub), 0, r, kv0, b);
-          if constexpr (HD == 128) ptx::tma_load_4d(dst + KV_TILE_BYTES / 2, &tmK, bar(K_FULL + sub), 64, r, kv0, b);
-        }
+        if (lane == 0 && !a.inject) load_packed(&tmK, sbase + OFF_K + sub * KV_TILE_BYTES, bar(K_FULL + sub), kvs);
       } else {
-        for (int t = lane; t < TR; t += 32) misc->bias[sub][0][t] = t < TQ ? 0.f : -INFINITY;   // beyond TQ: padding rows
-        if (lane == 0) misc->kvbase[sub][0] = kv0;
+        for (int t = lane; t < TQ; t += 32)
+#pragma unroll
+          for (int s = 0; s < CPS; ++s)
+            misc->bias[sub][s][t] = (WIDE ? (kv0 + s * W) / dm.B == (i0 + t) / dm.B : s == 0) ? 0.f : -INFINITY;
+#pragma unroll
+        for (int s = 0; s < CPS; ++s)
+          if (lane == s) misc->kvbase[sub][s] = kvs[s];
         __syncwarp();
-        if (lane == 0) {
-          const uint32_t dst = sbase + OFF_V + sub * KV_TILE_BYTES;
-          ptx::mbar_arrive_expect_tx(bar(V_FULL + sub), KV_TILE_BYTES);
-          ptx::tma_load_4d(dst, &tmV, bar(V_FULL + sub), 0, r, kv0, b);
-          if constexpr (HD == 128) ptx::tma_load_4d(dst + KV_TILE_BYTES / 2, &tmV, bar(V_FULL + sub), 64, r, kv0, b);
-        }
+        if (lane == 0) load_packed(&tmV, sbase + OFF_V + sub * KV_TILE_BYTES, bar(V_FULL + sub), kvs);
       }
     }
   };
@@ -256,148 +231,68 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   if (warp >= 4) {
   // the register file of the block is re-divided between its two warpgroups: this one gives up what the softmax
   // warpgroup takes (each side opens with its own instruction, so the allocator knows the budget of each)
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PF_REGS_SERVICE));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(WT, CPS)));
   if (warp == 4 || warp == 6) {
     // =========================== producers ===========================
     // Two warps walk the same union list: warp 4 feeds the K ring (and loads Q), warp 6 feeds the V ring and
     // the per-token bias of each step.  Split like this, a full V ring never holds back the next K tile.
     const bool do_k = (warp == 4), do_v = (warp == 6);
-    const int TR = SHORT ? 128 / g_q : TQ;   // token slots of the 128 tile rows; slots TQ .. TR-1 are padding (bias -inf)
     if (!a.early_loads) own_loads(do_k, do_v);
-    // union of the tile's mask words (lane t owns tokens t, t+32)
-    const int n_words = (c_own >> 5) + 1;
-    const long long row0 = ((long long)b * dm.h_kv + r) * dm.seq_q;
-    const uint32_t own_word_keep = (c_own & 31) == 31 ? 0xffffffffu : ((2u << (c_own & 31)) - 1u);
-    // four mask words per sweep: a lane's eight loads are in flight together (one L2 round trip per four words
-    // instead of one per word; the step count below is what the MMA thread waits for before its second product)
-    int total = 0;
-    for (int w0 = 0; w0 < n_words; w0 += 4) {
-      uint32_t uu[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int t = lane + 32 * q;
-        if (t < TQ && i0 + t < dm.seq_q) {
-          const uint32_t* mp = a.mask + (row0 + i0 + t) * dm.W + w0;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (w0 + k < n_words) uu[k] |= mp[k];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (w0 + k < n_words) {
-          uint32_t u = __reduce_or_sync(0xffffffffu, uu[k]);
-          if (w0 + k == n_words - 1) u = (u & own_word_keep) | (1u << (c_own & 31));  // own chunk: always, and last
-          total += __popc(u);
-        }
-      }
-    }
-    // the own chunk is always in the union (its bit is set in every row); it contributes own_steps steps
-    const int n_steps = CPS > 1 ? (total - 1 + CPS - 1) / CPS + own_steps : (total - 1) * sub_per_blk + own_steps;
+    TileWalk<CPS, WIDE, TPL> walk(dm, a.mask, ((long long)b * dm.h_kv + r) * dm.seq_q, i0, TQ, lane);
+    const int total = walk.count();
+    const int n_steps = (CPS > 1 ? (total + CPS - 1) / CPS : total * sub_per_blk) + own_steps;
     if (lane == 0 && do_k) {
       misc->n_steps = n_steps;
       ptx::mbar_arrive(bar(META));
     }
-    // start of the compact bias lists of this lane's tokens (lane t owns tokens t and t+32)
-    long long loff[2];
-    for (int q = 0; q < 2; ++q) {
-      const int t = lane + 32 * q;
-      const int i = min(i0 + t, dm.seq_q - 1);
-      loff[q] = ((long long)b * dm.h_kv + r) * dm.list_rows + list_row_offset(dm, i);
-    }
-    auto load_rows = [&](int w, uint32_t* rw) {
-      for (int q = 0; q < 2; ++q) {
-        const int t = lane + 32 * q;
-        rw[q] = (t < TQ && i0 + t < dm.seq_q) ? a.mask[(row0 + i0 + t) * dm.W + w] : 0u;
-      }
-    };
-    auto union_of = [&](int w, const uint32_t* rw) -> uint32_t {
-      uint32_t u = __reduce_or_sync(0xffffffffu, rw[0] | rw[1]);
-      if (w == n_words - 1) u = (u & own_word_keep) | (1u << (c_own & 31));
-      return u;
-    };
-    // The walk pops the chunks of the union in ascending order; mask words are read one word ahead.
-    int w = 0;
-    uint32_t rw[2], rw_n[2] = {0u, 0u};
-    load_rows(0, rw);
-    uint32_t u = union_of(0, rw);
-    if (n_words > 1) load_rows(1, rw_n);
-    int j = own_steps;                 // the own chunk's steps are already under way
+    // the compact bias lists of this lane's tokens
+    const float* list[TPL];
+#pragma unroll
+    for (int q = 0; q < TPL; ++q)
+      list[q] = a.blk_bias + ((long long)b * dm.h_kv + r) * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
+    walk.start();
     bool ok = true;
     // last step loaded into each stage (-1: none): what a block that gives up has to let land before it retires
     int last_j[2] = {-1, -1};
-    for (int sub = 0; sub < (CPS > 1 ? 1 : own_steps); ++sub) last_j[sub] = (do_k && a.inject) ? -1 : sub;
-    {
-      // A step takes the next CPS chunks of the union (CPS > 1: chunks of 32 / 16 tokens packed into the 64-token
-      // step; a short last step repeats its last chunk with bias -inf).  A row's bias for a chunk is read straight
-      // from its list: the entry number is the count of the row's routed bits below the chunk (previous words'
-      // totals kept in `seen`), so the loads of a whole step are issued together, before the wait for the stage,
-      // and nothing walks the lists entry by entry.
-      int seen[2] = {0, 0};
-      auto routed_bits = [&](uint32_t word) -> uint32_t {    // a row's routed chunks in word w: the own chunk and later ones cleared
-        return w == n_words - 1 ? word & own_word_keep & ~(1u << (c_own & 31)) : word;
-      };
-      bool walking = true;
-      while (walking && ok) {
-        int cs[CPS];
-        float bvs[CPS][2];
-        int m = 0;
-        while (m < CPS) {
-          while (u == 0u && walking) {
-            seen[0] += __popc(routed_bits(rw[0]));
-            seen[1] += __popc(routed_bits(rw[1]));
-            if (++w >= n_words) { walking = false; break; }
-            rw[0] = rw_n[0]; rw[1] = rw_n[1];
-            u = union_of(w, rw);
-            if (w + 1 < n_words) load_rows(w + 1, rw_n);
-          }
-          if (!walking) break;
-          const int bit = __ffs(u) - 1;
-          u &= u - 1;
-          const int c = w * 32 + bit;
-          if (c == c_own) { walking = false; break; }        // last of the walk, done first
-          cs[m] = c;
+    for (int sub = 0; sub < own_steps; ++sub) last_j[sub] = (do_k && a.inject) ? -1 : sub;
+    for (int j = own_steps; j < n_steps && ok;) {      // (the own chunks' steps are already under way)
+      // a step takes the next CPS chunks of the union (CPS > 1: chunks of 32 / 16 tokens packed into the 64-token step);
+      // the bias loads of a whole step are issued together, before the wait for the stage
+      int cs[CPS], pos[CPS][TPL];
+      float bvs[CPS][TPL];
+      walk.next(cs, pos);
+      if (do_v) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const uint32_t rb = routed_bits(rw[q]);
-            const bool member = do_v && ((rb >> bit) & 1u);
-            const int e = seen[q] + __popc(rb & ((1u << bit) - 1u));
-            bvs[m][q] = member ? __ldg(a.blk_bias + loff[q] + e) : -INFINITY;
+        for (int s = 0; s < CPS; ++s)
+#pragma unroll
+          for (int q = 0; q < TPL; ++q) bvs[s][q] = pos[s][q] >= 0 ? __ldg(list[q] + pos[s][q]) : -INFINITY;
+      }
+      // chunks of 128 tokens take two 64-token steps with the same bias
+      for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk) && ok; ++sub, ++j) {
+        int kvs[CPS];
+#pragma unroll
+        for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
+        const int st = j & 1, prev_ph = ((j >> 1) - 1) & 1;   // stage, and the phase of step j-2 on the completion barriers
+        if (do_k) {
+          if (j >= 2) ok = wait_on(bar(S_FULL + st), prev_ph);     // QK of step j-2 has read the stage
+          if (!ok) break;
+          if (lane == 0) load_packed(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kvs);
+        } else {
+          if (j >= 2) ok = wait_on(bar(PV_DONE + st), prev_ph);    // PV of step j-2 has read the stage
+          if (!ok) break;
+#pragma unroll
+          for (int s = 0; s < CPS; ++s) {
+#pragma unroll
+            for (int q = 0; q < TPL; ++q) {
+              const int t = lane + 32 * q;
+              if (t < TQ) misc->bias[st][s][t] = bvs[s][q];
+            }
+            if (lane == s) misc->kvbase[st][s] = kvs[s];
           }
-          ++m;
+          __syncwarp();
+          if (lane == 0) load_packed(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kvs);
         }
-        if (m == 0) break;
-#pragma unroll
-        for (int s = 1; s < CPS; ++s)
-          if (s >= m) { cs[s] = cs[m - 1]; bvs[s][0] = bvs[s][1] = -INFINITY; }
-        // chunks of 128 tokens take two 64-token steps with the same bias
-        for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk) && ok; ++sub, ++j) {
-          int kvs[CPS];
-#pragma unroll
-          for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
-          const int st = j & 1, prev_ph = ((j >> 1) - 1) & 1;   // stage, and the phase of step j-2 on the completion barriers
-          if (do_k) {
-            if (j >= 2) ok = wait_on(bar(S_FULL + st), prev_ph);     // QK of step j-2 has read the stage
-            if (!ok) break;
-            if (lane == 0) load_packed(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kvs);
-            last_j[st] = j;
-          } else {
-            if (j >= 2) ok = wait_on(bar(PV_DONE + st), prev_ph);    // PV of step j-2 has read the stage
-            if (!ok) break;
-#pragma unroll
-            for (int s = 0; s < CPS; ++s)
-              for (int q = 0; q < 2; ++q) {
-                const int t = lane + 32 * q;
-                if (t < TR) misc->bias[st][s][t] = t < TQ ? bvs[s][q] : -INFINITY;
-              }
-#pragma unroll
-            for (int s = 0; s < CPS; ++s)
-              if (lane == s) misc->kvbase[st][s] = kvs[s];
-            __syncwarp();
-            if (lane == 0) load_packed(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kvs);
-            last_j[st] = j;
-          }
-        }
+        last_j[st] = j;
       }
     }
     if (!ok && lane == 0) {
@@ -459,7 +354,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
           // A = P from tensor memory: 16 bf16 per K step = 8 packed columns
           ptx::mma_bf16_ts(tmem + 2 * NKV, p_tmem + k * 8, bd, IDESC_PV, (j > 0 || k > 0) ? 1u : 0u);
         }
-        if constexpr (STATS) {
+        if constexpr (P2) {
 #pragma unroll
           for (int k = 0; k < NKV / 16; ++k) {
             const uint64_t bd = vd + (uint64_t)((k * 16 * 128) >> 4);
@@ -473,11 +368,10 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   }
   } else {
     // =========================== softmax / epilogue ===========================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(PF_REGS_SOFTMAX));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_softmax(WT, CPS)));
     const int m = tid;                       // tile row = TMEM lane
     const int t = m / g_q, hh = m % g_q;     // token in tile, head in group
     const int i_row = i0 + t;
-    const bool row_live = t < TQ;            // false for the padding rows of a tile shorter than 128 rows
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
     const float c1 = dm.sm_scale * 1.4426950408889634f;
     bool ok = true;
@@ -497,7 +391,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
       if (!ok) break;
       float b2s[CPS];                                // per packed chunk: bias in the log2 domain (-inf: not routed)
 #pragma unroll
-      for (int s = 0; s < CPS; ++s) b2s[s] = misc->bias[buf][s][t] * 1.4426950408889634f;   // -inf on padding rows
+      for (int s = 0; s < CPS; ++s) b2s[s] = misc->bias[buf][s][t] * 1.4426950408889634f;
       const int kv0 = misc->kvbase[buf][0];
       ok = wait_on(bar(S_FULL + buf), (j >> 1) & 1);
       if (!ok) break;
@@ -516,17 +410,17 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
       bool selected;
       float mloc;
       if constexpr (CPS > 1) {
-        // packed chunks: each slot of W columns has its own bias; only the own chunk (slot 0 of step 0) can be cut
-        // by the causal mask (routed chunks lie wholly before the row)
-        constexpr int W = NKV / CPS;
+        // packed chunks: each slot of W columns has its own bias; only a slot of an own chunk can be cut by the causal
+        // mask (routed chunks lie wholly before the row): slot 0 of step 0, in a wide tile every slot of the first steps
         mloc = -INFINITY;
 #pragma unroll
         for (int s = 0; s < CPS; ++s) {
           if (b2s[s] > -INFINITY) {
-            if (s == 0 && n_vis < W) {
+            const int vis = s == 0 ? n_vis : WIDE && j < own_steps ? i_row - misc->kvbase[buf][s] + 1 : W;
+            if (vis < W) {
 #pragma unroll
               for (int c = 0; c < W; ++c)
-                if (c >= n_vis) sreg[c] = 0xff800000u;   // -inf
+                if (c >= vis) sreg[s * W + c] = 0xff800000u;   // -inf
             }
             float ch[4];
 #pragma unroll
@@ -570,13 +464,12 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
         moved = true;
       }
       l *= corr;
-      [[maybe_unused]] uint32_t packed[STATS ? 1 : 32];
-      if constexpr (STATS) {
+      [[maybe_unused]] uint32_t packed[P2 ? 1 : 32];
+      if constexpr (P2) {
         // P = hi + lo as two bf16 terms, 32 scores at a time, stored as they are formed (the scores are all in registers
         // already): hi into the first 32 columns of the step's S buffer, lo into the second 32
         float2 lsum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         const float2 c1v = make_float2(c1, c1);
-        const float2 offv = make_float2(b2s[0] - m_used, b2s[0] - m_used);
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
           uint32_t hi16[16], lo16[16];
@@ -584,6 +477,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
               const int cc = half * 32 + c;
+              const float2 offv = make_float2(b2s[cc / W] - m_used, b2s[cc / W] - m_used);
               const float2 t = __ffma2_rn(make_float2(__uint_as_float(sreg[cc]), __uint_as_float(sreg[cc + 1])), c1v, offv);
               const float2 pp = make_float2(exp2f(t.x), exp2f(t.y));
               lsum[(c >> 1) & 1] = __fadd2_rn(lsum[(c >> 1) & 1], pp);
@@ -612,7 +506,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
         float2 lsum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
         for (int c = 0; c < NKV; c += 2) {
-          const float2 offv = offs[c / (NKV / CPS)];
+          const float2 offv = offs[c / W];
           const float2 t = __ffma2_rn(make_float2(__uint_as_float(sreg[c]), __uint_as_float(sreg[c + 1])), c1v, offv);
           const float2 pp = make_float2(exp2f(t.x), exp2f(t.y));
           lsum[(c >> 1) & 3] = __fadd2_rn(lsum[(c >> 1) & 3], pp);
@@ -644,7 +538,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
         }
       }
       // P row -> the first 32 columns of this step's S buffer (two bf16 per column)
-      if constexpr (!STATS) DASH_TMEM_ST32(lane_addr + buf * NKV, packed);
+      if constexpr (!P2) DASH_TMEM_ST32(lane_addr + buf * NKV, packed);
       ptx::tmem_wait_st();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(P_FULL + (j & 1)));
@@ -657,14 +551,14 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
       const float inv = l > 0.f ? 1.f / l : 0.f;
       const long long o_off = (long long)b * dm.os[0] + (long long)i_row * dm.os[1] + (long long)(r * g_q + hh) * dm.os[2];
       __nv_bfloat16* op = a.O + o_off;
-      const bool row_out = i_row < dm.seq_q && (!SHORT || row_live);
+      const bool row_out = i_row < dm.seq_q;
       float dot = 0.f;
 #pragma unroll 1
       for (int q = 0; q < HD / 32; ++q) {
         uint32_t o[32];
         DASH_TMEM_LD32(o, lane_addr + 2 * NKV + q * 32);
         ptx::tmem_wait_ld();
-        if (STATS && row_out) {
+        if (P2 && a.stats.base && row_out) {
           const __nv_bfloat16* gp = a.dO + o_off + q * 32;
 #pragma unroll
           for (int c = 0; c < 32; c += 8) {
@@ -692,11 +586,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
           }
         }
       }
-      if (STATS && row_out) {
-        const long long row = (((long long)b * dm.h_kv + r) * a.n_tiles + tile) * 128 + m;
-        a.lse2[row] = m_used + log2f(l);
-        a.delta[row] = dot * inv;
-      }
+      if (P2 && a.stats.base && row_out) *a.stats.at(b, r, i_row, hh) = make_float2(m_used + log2f(l), dot * inv);
     }
     ptx::tc_fence_before();
   }
@@ -727,20 +617,55 @@ bool make_map(CUtensorMap* out, const void* base, int hd, long long tokens, int 
 bool prefill_sm100_supported(const Dims& dm) {
   if (dm.decode || !dm.causal || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128)) return false;
   if (dm.B != 16 && dm.B != 32 && dm.B != 64 && dm.B != 128) return false;
-  if (dm.g_q < 2 || 128 / dm.g_q > MAX_TQ) return false;
   if (dm.os[2] % 8 != 0 || dm.os[1] % 8 != 0) return false;
   return tensor_map_encoder() != nullptr;
 }
 
+template <int HD, int CPS, int WT, bool P2>
+static cudaError_t launch_one(const PrefillArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                              cudaStream_t st) {
+  auto kern = attend_prefill_sm100_kernel<HD, CPS, WT, P2>;
+  constexpr uint32_t smem = PfLayout<HD, CPS, 32 * (WT > 0 ? WT : 2)>::SMEM;
+  static std::atomic<unsigned long long> configured{0};
+  if (cudaError_t e = allow_dynamic_smem(kern, smem, configured); e != cudaSuccess) return e;
+  const unsigned blocks = (unsigned)((long long)a.n_tiles * a.dm.batch * a.dm.h_kv);
+  cudaError_t e = launch_chained(kern, dim3(blocks), dim3(PF_THREADS), smem, st, tq, tk, tv, a);
+  count_launch();
+  return e;
+}
+
+// Tiles of 128 / g_q tokens: g_q = 1 takes the 128-token wide form with two-term probabilities (the precision it had on
+// CUDA cores), chunks shorter than the tile the 64-token wide form.  A tile that keeps all 128 rows live over several
+// chunks walks a larger union than one cut at the chunk's end, but there are fewer tiles and no dead rows: 8192 tokens,
+// 32/8 heads, chunks of 16: 1.43 -> 0.58 ms; 3 x 1999 tokens, 12/12 heads, d 64, chunks of 32: 1.54 ms on CUDA cores
+// (one warp per row) -> 0.07 ms.
+template <int HD, int CPS>
+static cudaError_t launch_cps(const PrefillArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                              cudaStream_t st) {
+  const bool stats = a.stats.base != nullptr;
+  if (a.dm.g_q == 1) return launch_one<HD, CPS, 4, true>(a, tq, tk, tv, st);
+  if constexpr (CPS > 1) {
+    if (a.TQ > a.dm.B)
+      return stats ? launch_one<HD, CPS, 2, true>(a, tq, tk, tv, st) : launch_one<HD, CPS, 2, false>(a, tq, tk, tv, st);
+  }
+  return stats ? launch_one<HD, CPS, 0, true>(a, tq, tk, tv, st) : launch_one<HD, CPS, 0, false>(a, tq, tk, tv, st);
+}
+
+template <int HD>
+static cudaError_t launch_hd(const PrefillArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                             cudaStream_t st) {
+  if (a.dm.B >= NKV) return launch_cps<HD, 1>(a, tq, tk, tv, st);
+  return a.dm.B == 32 ? launch_cps<HD, 2>(a, tq, tk, tv, st) : launch_cps<HD, 4>(a, tq, tk, tv, st);
+}
+
 cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const void* K, const void* V,
                                         const uint32_t* mask, const float* blk_bias, void* O, StatusBlock* sb,
-                                        bool inputs_stable, cudaStream_t st, float* lse2, float* delta, const void* dO) {
+                                        bool inputs_stable, cudaStream_t st, const RowStats& stats, const void* dO) {
   PrefillArgs a;
-  a.lse2 = lse2;
-  a.delta = delta;
+  a.stats = stats;
   a.dO = (const __nv_bfloat16*)dO;
   a.dm = dm;
-  a.TQ = 128 / dm.g_q < dm.B ? 128 / dm.g_q : dm.B;     // a tile stays inside one chunk
+  a.TQ = 128 / dm.g_q;
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
   a.early_loads = inputs_stable ? 1 : 0;
   a.inject = test_hooks().skip_own_k_load;
@@ -754,41 +679,7 @@ cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const voi
   if (!make_map(&tq, Q, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
   if (!make_map(&tk, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, box_kv)) return cudaErrorInvalidValue;
   if (!make_map(&tv, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, box_kv)) return cudaErrorInvalidValue;
-  const long long blocks = (long long)a.n_tiles * dm.batch * dm.h_kv;
-  cudaError_t le = cudaSuccess;
-#define DASH_PF(HDV, CPSV, SHORTV)                                                                                  \
-  {                                                                                                                 \
-    static std::atomic<unsigned long long> configured{0};                                                           \
-    if (cudaError_t e = allow_dynamic_smem(attend_prefill_sm100_kernel<HDV, CPSV, SHORTV>,                          \
-                                           PfLayout<HDV, CPSV>::SMEM, configured);                                  \
-        e != cudaSuccess)                                                                                           \
-      return e;                                                                                                     \
-    le = launch_chained(attend_prefill_sm100_kernel<HDV, CPSV, SHORTV>, dim3((unsigned)blocks), dim3(PF_THREADS),   \
-                        PfLayout<HDV, CPSV>::SMEM, st, tq, tk, tv, a);                                              \
-  }
-#define DASH_PF_HD(HDV)                                                                    \
-  if (cps == 1) DASH_PF(HDV, 1, false)                                                     \
-  else if (cps == 2) { if (short_tile) DASH_PF(HDV, 2, true) else DASH_PF(HDV, 2, false) } \
-  else { if (short_tile) DASH_PF(HDV, 4, true) else DASH_PF(HDV, 4, false) }
-  const int cps = NKV / box_kv;
-  const bool short_tile = a.TQ * dm.g_q < 128;      // only with chunks below 64 tokens
-  if (lse2) {
-    // statistics mode: the shapes the tensor-core backward takes (head_dim 128, chunks of 64 / 128, full tiles)
-    if (dm.d != 128 || cps != 1 || short_tile || !delta || !dO) return cudaErrorInvalidValue;
-    static std::atomic<unsigned long long> configured{0};
-    if (cudaError_t e = allow_dynamic_smem(attend_prefill_sm100_kernel<128, 1, false, true>, PfLayout<128, 1>::SMEM, configured);
-        e != cudaSuccess)
-      return e;
-    le = launch_chained(attend_prefill_sm100_kernel<128, 1, false, true>, dim3((unsigned)blocks), dim3(PF_THREADS),
-                        PfLayout<128, 1>::SMEM, st, tq, tk, tv, a);
-    count_launch();
-    return le;
-  }
-  if (dm.d == 128) { DASH_PF_HD(128) } else { DASH_PF_HD(64) }
-#undef DASH_PF_HD
-#undef DASH_PF
-  count_launch();
-  return le;
+  return dm.d == 128 ? launch_hd<128>(a, tq, tk, tv, st) : launch_hd<64>(a, tq, tk, tv, st);
 }
 
 }  // namespace dash

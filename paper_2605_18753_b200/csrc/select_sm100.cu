@@ -1,8 +1,8 @@
 // Stage 1 on tensor cores for sm_100a (Eq. 2, Eq. 4, Algorithm 2, Proposition 1), bf16 queries, head_dim 128 or 64.
 //
-// Tile = the (token, head-of-group) rows of TQ = min(128/g_q, chunk size) consecutive tokens of one (batch, KV head):
-// 128 rows, or fewer live rows followed by zero-query padding when chunks are shorter than 128/g_q tokens;
-// they share their candidate chunks.  The whole score tile X[128 rows][<= 512 chunks per block] is produced by
+// Tile = the 128 (token, head-of-group) rows of TQ = 128/g_q consecutive tokens of one (batch, KV head).  Where a chunk
+// holds at least TQ tokens they share their candidate chunks; where chunks are shorter (WIDE) the tile spans several
+// chunks, its columns are the candidates of its last row and every row cuts them at its own chunk.  The whole score tile X[128 rows][<= 512 chunks per block] is produced by
 // tcgen05.mma into tensor memory and never leaves the SM (Algorithm 2 writes it to HBM).  The fp32
 // summaries are split beforehand into three bf16 planes (hi + mid + lo = the fp32 value exactly), so that
 // Q (exact in bf16) times the three planes, accumulated in fp32, carries fp32-class accuracy: the support
@@ -100,9 +100,9 @@ __global__ void kbar_split_kernel(const float* __restrict__ kbar, __nv_bfloat16*
   planes[2 * n + i] = __float2bfloat16_rn(r2);
 }
 
-// SHORT: the tile has fewer than 128 live rows (chunks shorter than 128 / g_q tokens); full tiles compile without
-// any of the padding-row handling.
-template <int NST, int G, int CS, int HD, bool SHORT>
+// WIDE: the tile spans several chunks (chunks shorter than 128 / g_q tokens); tiles inside one chunk compile with one
+// candidate count for all rows.
+template <int NST, int G, int CS, int HD, bool WIDE>
 __global__ void __launch_bounds__(sel_threads(NST), NST == 1 ? 2 : 1)
 select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKB, SelectTcArgs a) {
   using SP = SmemPlan<NST>;
@@ -128,8 +128,8 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const int TQ = a.TQ;
   constexpr int g_q = G;
   const int i0 = tile * TQ;
-  const int c_own = i0 / dm.B;
-  // candidates of the tile's rows; with a local window its chunks are not scored (window_rows_kernel lists them)
+  const int c_own = (WIDE ? min(i0 + TQ, dm.seq_q) - 1 : i0) / dm.B;    // own chunk of the tile's rows (WIDE: of its last row)
+  // candidates of the tile's rows (WIDE: the most that any of them has); with a local window its chunks are not scored (window_rows_kernel lists them)
   const int n_cand = min(max(c_own - dm.local_blocks, 0), dm.T_s);   // (c_own <= T_s in a prefill)
   constexpr int CCOLS = CLUSTER_COLS;
   const int c_lo = cr * CCOLS;                                 // first candidate this block holds
@@ -157,15 +157,6 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     ptx::tmem_relinquish();
     ptx::tc_fence_before();
   }
-  // Rows of the Q tile beyond its TQ * g_q live rows (chunks shorter than 128 / g_q tokens) are never written by the
-  // TMA box: zero queries give zero logits, and nothing those rows compute is stored.
-  if constexpr (SHORT) {
-    const int first = TQ * g_q * 8;                 // 16-byte pieces before the first dead row (a row is 128 bytes)
-    for (int regn = 0; regn < HD / 64; ++regn)
-      for (int k = first + tid; k < 128 * 8; k += SEL_TC_THREADS)
-        *reinterpret_cast<uint4*>(smem + SP::OFF_Q + regn * (Q_BYTES / 2) + k * 16) = make_uint4(0u, 0u, 0u, 0u);
-    ptx::fence_proxy_async_smem();
-  }
   __syncthreads();
   if (CS > 1) ptx::cluster_sync_all();     // every block's barriers exist before anybody arrives on them remotely
   ptx::tc_fence_after();
@@ -183,7 +174,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     if (lane == 0 && n_loc > 0) {
       ptx::prefetch_tensormap(&tmQ);
       ptx::prefetch_tensormap(&tmKB);
-      ptx::mbar_arrive_expect_tx(bar(Q_FULL), SHORT ? (uint32_t)(TQ * g_q * HD * 2) : 128 * HD * 2);   // the box holds the live rows
+      ptx::mbar_arrive_expect_tx(bar(Q_FULL), 128 * HD * 2);
       ptx::tma_load_4d(sbase + SP::OFF_Q, &tmQ, bar(Q_FULL), 0, r * g_q, i0, b);
       if constexpr (HD == 128) ptx::tma_load_4d(sbase + SP::OFF_Q + Q_BYTES / 2, &tmQ, bar(Q_FULL), 64, r * g_q, i0, b);
       const long long row0 = ((long long)b * dm.h_kv + r) * dm.T_s + c_lo;
@@ -245,7 +236,11 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int m = q4 * 32 + lane;
     const int t = m / g_q, hh = m % g_q;
     const int i = i0 + t;
-    const bool row_valid = SHORT ? (i < dm.seq_q && t < TQ) : i < dm.seq_q;   // (a short tile ends with zero-query rows)
+    const bool row_valid = i < dm.seq_q;
+    // the row's own chunk, its candidates, and those of them that this block holds
+    const int c_row = WIDE ? min(i / dm.B, c_own) : c_own;
+    const int n_row = WIDE ? min(max(c_row - dm.local_blocks, 0), n_cand) : n_cand;
+    const int l_row = WIDE ? (CS > 1 ? max(0, min(CCOLS, n_row - c_lo)) : n_row) : n_loc;
     const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
     const int e_int = dm.e_int;
     const float e = dm.e, xs = dm.x_scale;
@@ -322,7 +317,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int ei = EI_STATIC >= 0 ? EI_STATIC : e_int;
     const int max_it = ei ? MAX_NEWTON : MAX_NEWTON_GENERIC;
     auto start_tau = [&](float mx, float s1, float s2) -> float {   // s1, s2: sums of (x - mx), (x - mx)^2
-      const float n = (float)n_cand;
+      const float n = (float)n_row;
       float t = -1.f;
       if (ei == 1) {
         t = (s1 - 1.f) / n;
@@ -335,7 +330,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         // It lands near the root where the all-active guess, a lower bound, sits far below it (sparse supports);
         // the larger of the two is taken.  Either side of the root is a valid start (see above), so a row that is
         // far from normal costs a pass at worst.
-        if (n_cand >= 8 && ss > 0.f) {
+        if (n_row >= 8 && ss > 0.f) {
           const float L = -__logf(fminf(fmaxf(ss, 0.3334f), 1e7f));
           const float z = fmaf(fmaf(fmaf(fmaf(-8.93074e-05f, L, -0.0037117f), L, -0.0612527f), L, -0.717421f), L, -0.499476f);
           t = fmaxf(t, fmaf(z, sqrtf(ss / n), mean));
@@ -359,7 +354,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           uint32_t v[32];
           DASH_TMEM_LD32(v, lane_addr + k * 32);
           ptx::tmem_wait_ld();
-          const int lim = n_cand - k * 32;
+          const int lim = n_row - k * 32;
 #pragma unroll
           for (int c = 0; c < 32; ++c) xr[k][c] = c < lim ? __uint_as_float(v[c]) * xs : -INFINITY;
         } else {
@@ -390,6 +385,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const float s2 = (s2v[0].x + s2v[0].y) + (s2v[1].x + s2v[1].y);
       tau = start_tau(mx, s1, s2);
       bool done = false;
+      if (WIDE && n_row == 0) { tau = 0.f; done = true; }
       for (int it = 0; it < max_it; ++it) {
         float f[4] = {0.f, 0.f, 0.f, 0.f}, g[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (EI_STATIC == 2) {
@@ -451,7 +447,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       };
       // columns past the row's last candidate (only in the last chunk) hold scores of later chunks: -inf them
       auto cut_tail = [&](uint32_t (&v)[32], int k) {
-        const int lim = n_loc - k * 32;
+        const int lim = l_row - k * 32;
         if (lim < 32) {
 #pragma unroll
           for (int c = 0; c < 32; ++c) v[c] = c < lim ? v[c] : 0xff800000u;
@@ -469,7 +465,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         uint32_t v[32];
         DASH_TMEM_LD32(v, lane_addr + k * 32);
         ptx::tmem_wait_ld();
-        const int lim = n_loc - k * 32;
+        const int lim = l_row - k * 32;
 #pragma unroll
         for (int c = 0; c < 32; ++c) {
           if (c < lim) {
@@ -490,10 +486,11 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       mx = x_max_a;
       {
         // sum (x - mx) = S1 - n mx,  sum (x - mx)^2 = S2 - 2 mx S1 + n mx^2  (only the start value depends on them)
-        const float n = (float)n_cand, S1 = x_sum_b, S2 = x_sum_c;
+        const float n = (float)n_row, S1 = x_sum_b, S2 = x_sum_c;
         tau = start_tau(mx, S1 - n * mx, fmaxf(fmaf(n * mx, mx, fmaf(-2.f * mx, S1, S2)), 0.f));
       }
       bool done = false;
+      if (WIDE && n_row == 0) { tau = 0.f; done = true; }
       for (int it = 0; it < max_it && ok; ++it) {
         float f[4] = {0.f, 0.f, 0.f, 0.f}, g[4] = {0.f, 0.f, 0.f, 0.f};
         if constexpr (EI_STATIC == 2) {
@@ -600,7 +597,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         ptx::tmem_st_n<OWN>(lane_addr + k * 32, lwv);            // slot q of this lane = chunk own0 + q of step k
         if (row_valid && hh == 0) {
           const int wj = cr * (CCOLS / 32) + k;                // mask word of this step
-          mrow[wj] = bits | (((c_own >> 5) == wj) ? (1u << (c_own & 31)) : 0u);
+          mrow[wj] = bits | (((c_row >> 5) == wj) ? (1u << (c_row & 31)) : 0u);
         }
         nsel += __popc(bits);
       };
@@ -622,7 +619,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           uint32_t v[32];
           DASH_TMEM_LD32(v, lane_addr + k * 32);
           ptx::tmem_wait_ld();
-          const int lim = n_loc - k * 32;
+          const int lim = l_row - k * 32;
 #pragma unroll
           for (int c = 0; c < 32; ++c) {
             const float mm = fmaxf(fmaf(__uint_as_float(v[c]), xs, -tau), 0.f);
@@ -641,7 +638,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       int base = (int)x_below_a;
       const float slog_all = x_sum_b;
       if (row_valid && hh == 0 && my_rank == 0) {
-        for (int j = (n_cand + 31) / 32; j < dm.W; ++j) mrow[j] = ((c_own >> 5) == j) ? (1u << (c_own & 31)) : 0u;
+        for (int j = (n_cand + 31) / 32; j < dm.W; ++j) mrow[j] = ((c_row >> 5) == j) ? (1u << (c_row & 31)) : 0u;
         a.count[row_id] = nsel_all;
       }
       const float mu = nsel_all > 0 ? slog_all / (float)nsel_all : 0.f;
@@ -689,9 +686,10 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 // holds 512 candidates per row in tensor memory; clusters of 2 or 4 blocks extend that to 1024 / 2048.
 int select_sm100_token_limit(const Dims& dm) {
   if (dm.decode || !dm.causal || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128) || dm.T_s < 1) return 0;
-  if (dm.g_q < 2) return 0;
   if (tensor_map_encoder() == nullptr) return 0;
-  const long long lim = (long long)(4 * CLUSTER_COLS + 1) * dm.B;   // own chunk index <= 2048
+  // own chunk index <= 2048, in whole tiles
+  const int tq = 128 / dm.g_q;
+  const long long lim = (long long)(MAX_CS * CLUSTER_COLS + 1) * dm.B / tq * tq;
   return (int)(lim < dm.seq_q ? lim : dm.seq_q);
 }
 
@@ -699,10 +697,10 @@ size_t select_sm100_scratch_bytes(const Dims& dm) {
   return (size_t)3 * dm.batch * dm.h_kv * (size_t)(dm.T_s > 0 ? dm.T_s : 1) * dm.d * sizeof(__nv_bfloat16);
 }
 
-template <int NST, int G, int CS, int HD, bool SHORT = false>
+template <int NST, int G, int CS, int HD, bool WIDE>
 static cudaError_t launch_band(const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a, long long clusters,
                                cudaStream_t st) {
-  auto kern = select_sm100_kernel<NST, G, CS, HD, SHORT>;
+  auto kern = select_sm100_kernel<NST, G, CS, HD, WIDE>;
   static std::atomic<unsigned long long> configured{0};
   if (cudaError_t e = allow_dynamic_smem(kern, SmemPlan<NST>::TOTAL, configured); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -724,35 +722,25 @@ static cudaError_t launch_band(const CUtensorMap& tq, const CUtensorMap& tkb, co
   return e;
 }
 
+template <int NST, int CS, int HD>
+static cudaError_t launch_band_hd(const Dims& dm, const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a,
+                                  long long clusters, cudaStream_t st) {
+  const bool wide = a.TQ > dm.B;      // g_q = 1 with chunks below 128 tokens, 2 with 16 or 32, 4 with 16
+  switch (dm.g_q) {
+    case 1: return wide ? launch_band<NST, 1, CS, HD, true>(tq, tkb, a, clusters, st) : launch_band<NST, 1, CS, HD, false>(tq, tkb, a, clusters, st);
+    case 2: return wide ? launch_band<NST, 2, CS, HD, true>(tq, tkb, a, clusters, st) : launch_band<NST, 2, CS, HD, false>(tq, tkb, a, clusters, st);
+    case 4: return wide ? launch_band<NST, 4, CS, HD, true>(tq, tkb, a, clusters, st) : launch_band<NST, 4, CS, HD, false>(tq, tkb, a, clusters, st);
+    case 8: return launch_band<NST, 8, CS, HD, false>(tq, tkb, a, clusters, st);
+    case 16: return launch_band<NST, 16, CS, HD, false>(tq, tkb, a, clusters, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <int NST, int CS>
 static cudaError_t launch_band_g(const Dims& dm, const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a,
                                  long long clusters, cudaStream_t st) {
-  if (a.TQ * dm.g_q < 128) {      // short tiles: only g_q = 2 (chunks of 16 or 32) and g_q = 4 (chunks of 16)
-    if (dm.d == 64) {
-      if (dm.g_q == 2) return launch_band<NST, 2, CS, 64, true>(tq, tkb, a, clusters, st);
-      if (dm.g_q == 4) return launch_band<NST, 4, CS, 64, true>(tq, tkb, a, clusters, st);
-    } else {
-      if (dm.g_q == 2) return launch_band<NST, 2, CS, 128, true>(tq, tkb, a, clusters, st);
-      if (dm.g_q == 4) return launch_band<NST, 4, CS, 128, true>(tq, tkb, a, clusters, st);
-    }
-    return cudaErrorInvalidValue;
-  }
-  if (dm.d == 64) {
-    switch (dm.g_q) {
-      case 2: return launch_band<NST, 2, CS, 64>(tq, tkb, a, clusters, st);
-      case 4: return launch_band<NST, 4, CS, 64>(tq, tkb, a, clusters, st);
-      case 8: return launch_band<NST, 8, CS, 64>(tq, tkb, a, clusters, st);
-      case 16: return launch_band<NST, 16, CS, 64>(tq, tkb, a, clusters, st);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (dm.g_q) {
-    case 2: return launch_band<NST, 2, CS, 128>(tq, tkb, a, clusters, st);
-    case 4: return launch_band<NST, 4, CS, 128>(tq, tkb, a, clusters, st);
-    case 8: return launch_band<NST, 8, CS, 128>(tq, tkb, a, clusters, st);
-    case 16: return launch_band<NST, 16, CS, 128>(tq, tkb, a, clusters, st);
-    default: return cudaErrorInvalidValue;
-  }
+  return dm.d == 64 ? launch_band_hd<NST, CS, 64>(dm, tq, tkb, a, clusters, st)
+                    : launch_band_hd<NST, CS, 128>(dm, tq, tkb, a, clusters, st);
 }
 
 // Local window: the chunks [c_own - L, c_own) of every row are attended with bias 0 without being scored.  The
@@ -798,7 +786,7 @@ cudaError_t launch_select_sm100(const Dims& dm, int token_limit, const void* Q, 
 
   SelectTcArgs a;
   a.dm = dm;
-  a.TQ = 128 / dm.g_q < dm.B ? 128 / dm.g_q : dm.B;     // a tile stays inside one chunk
+  a.TQ = 128 / dm.g_q;
   a.plane_rows = plane_rows;
   a.mask = mask; a.count = count; a.blk_idx = blk_idx; a.blk_bias = blk_bias; a.tau = tau; a.sb = sb;
 
@@ -818,12 +806,12 @@ cudaError_t launch_select_sm100(const Dims& dm, int token_limit, const void* Q, 
     if (!encode_bf16_sw128_4d(&tkb, planes, dims, strides, box)) return cudaErrorInvalidValue;
   }
   // Bands of tiles by candidate count: <= 512 one block per tile, <= 1024 clusters of 2, <= 2048 clusters of 4.
-  // Tiles are TQ tokens; a tile's candidate count is its own chunk index i0 / B.
+  // Tiles are TQ tokens; a tile's candidate count is the own chunk index of its last token.
   const int groups = dm.batch * dm.h_kv;
   const int total_tiles = (token_limit + a.TQ - 1) / a.TQ;
-  auto tiles_up_to = [&](long long max_cand) -> int {      // tiles whose own chunk index is <= max_cand
+  auto tiles_up_to = [&](long long max_cand) -> int {      // tiles whose own chunk indexes are all <= max_cand
     const long long tokens = (max_cand + 1) * dm.B;
-    const long long t = (tokens + a.TQ - 1) / a.TQ;
+    const long long t = tokens / a.TQ;
     return (int)(t < total_tiles ? t : total_tiles);
   };
   const int t1 = tiles_up_to(CLUSTER_COLS), t2 = tiles_up_to(2 * CLUSTER_COLS), t3 = total_tiles;

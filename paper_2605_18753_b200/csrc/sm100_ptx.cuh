@@ -225,10 +225,11 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool a_mn_ma
                  "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])        \
                : "memory")
 
-// Narrow forms (x2 .. x16 columns of the warp's 32 lanes), for per-lane records shorter than 32 columns.
+// x2 .. x32 columns of the warp's 32 lanes, for per-lane records of a compile-time length.
 template <int N>
 __device__ __forceinline__ void tmem_ld_n(uint32_t* r, uint32_t addr) {
-  static_assert(N == 2 || N == 4 || N == 8 || N == 16, "supported widths");
+  static_assert(N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "supported widths");
+  if constexpr (N == 32) DASH_TMEM_LD32(r, addr);
   if constexpr (N == 2)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];"
                  : "=r"(r[0]), "=r"(r[1])
@@ -252,7 +253,8 @@ __device__ __forceinline__ void tmem_ld_n(uint32_t* r, uint32_t addr) {
 }
 template <int N>
 __device__ __forceinline__ void tmem_st_n(uint32_t addr, const uint32_t* r) {
-  static_assert(N == 2 || N == 4 || N == 8 || N == 16, "supported widths");
+  static_assert(N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "supported widths");
+  if constexpr (N == 32) DASH_TMEM_ST32(addr, r);
   if constexpr (N == 2)
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};"
                  ::"r"(addr), "r"(r[0]), "r"(r[1])
