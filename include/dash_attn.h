@@ -196,22 +196,23 @@ int dash_attn_attend_decode_static(const dash_params* p, const void* Q, const vo
  *   dbias  gradient w.r.t. every entry of blk_bias, fp32, in the layout of blk_bias (entries outside a row's count
  *          stay zero): the quantity a backward of Stage 1 continues from.
  *   dO     incoming gradient of O, dtype p->dtype, strides p->o_stride.
- * mask / blk_bias as written by dash_attn_select for the same parameters.  This is a correctness path on CUDA cores
- * (one warp per row and head, fp32 atomics for dK / dV / dbias, so their last bits vary from run to run); it needs
- * no workspace.  dash_attn_bwd_select_prefill and dash_attn_bwd_block_summaries carry dbias on through the routing. */
+ * mask / blk_bias as written by dash_attn_select for the same parameters.  bf16 tensors (causal) run on tensor cores with
+ * P and dS carried as two bf16 terms each, fp32 and the non-causal mode on CUDA cores (one warp per row and head); either
+ * way some sums are formed by fp32 atomics, so last bits vary from run to run.  No workspace: what the kernels hand to each
+ * other sits in dQ and dbias until those get their values.  dash_attn_bwd_select_prefill and dash_attn_bwd_block_summaries carry dbias on through the routing. */
 int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void* K, const void* V, const void* dO,
                                  const uint32_t* mask, const float* blk_bias, void* dQ, float* dK, float* dV,
                                  float* dbias, void* stream);
 
 /* The same gradients on tensor cores (bf16, head_dim 128, chunks of 64 or 128 tokens, at least two query heads per KV
  * head, causal; anything else returns DASH_ERR_UNSUPPORTED and nothing is enqueued: call dash_attn_bwd_attend_prefill).
- * Five launches: the forward Stage-2 kernel run for its row statistics (log-sum-exp and delta = <O, dO>; O itself is
+ * Four launches: the forward Stage-2 kernel run for its row statistics (log-sum-exp and delta = <O, dO>; O itself is
  * not written, and P enters its P V product as two bf16 terms, so that delta, which the routing's backward amplifies,
- * is accurate to fp32 class), two small kernels over the mask (routed-chunk counts before every mask word; the union
- * of every query tile's mask words), a query-tile-stationary kernel for dQ and dbias, and a key-slice-stationary
- * kernel for dK and dV (no atomics on dQ, dK, dV: every element has one owner and is written whether or not any
- * row attends it; dbias is zeroed and then receives a few atomic adds per entry, whose order cannot change the
- * sum beyond the last bit).  P and dS enter the dQ / dK / dV products rounded to bf16.
+ * is accurate to fp32 class), a small kernel over the mask (routed-chunk counts before every mask word; the union
+ * of every query tile's mask words), a key-slice-stationary kernel for dK and dV (no atomics: every element has one
+ * owner and is written whether or not any row attends it) and a query-tile-stationary kernel for dQ and dbias (dbias is
+ * zeroed and then receives a few atomic adds per entry, whose order cannot change the sum beyond the last bit).
+ * P and dS enter the dQ / dK / dV products rounded to bf16.
  *   bwd_workspace   device scratch of at least dash_attn_bwd_workspace_bytes(p) bytes, 256-byte aligned, owned by the
  *                   caller; it opens with a status word like the forward workspace's (dash_attn_last_status and
  *                   dash_attn_reset_status accept it): a bounded wait that runs out leaves DASH_ERR_TIMEOUT there.

@@ -76,6 +76,7 @@ static int make_dims(const dash_params* p, Dims* dm) {
   dm->T_s = p->seq_kv / p->block;
   dm->T_a = (p->seq_kv + p->block - 1) / p->block;
   dm->W = (dm->T_a + 31) / 32;
+  for (dm->log_b = 4; (1 << dm->log_b) < p->block; ++dm->log_b) {}
   dm->decode = (p->seq_q == 1 && p->seq_kv != 1) ? 1 : 0;
   dm->e = 1.f / (p->alpha - 1.f);
   dm->e_int = p->alpha == 2.f ? 1 : p->alpha == 1.5f ? 2 : p->alpha == 1.25f ? 4 : 0;
@@ -293,34 +294,17 @@ int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void
     return DASH_ERR_INVALID_ARG;
   if ((rc = check_device()) != DASH_OK) return rc;
   StageRange nv("dash_attn: stage 2 prefill attention, backward");
+  if (prefill_bwd_sm100_supported(dm))
+    return cuda_status(launch_attend_prefill_bwd_sm100(dm, true, current_sm_count(), Q, K, V, dO, mask, blk_bias, dQ, dK, dV, dbias,
+                                                       nullptr, (cudaStream_t)stream));
   return cuda_status(launch_attend_prefill_bwd_generic(dm, Q, K, V, dO, mask, blk_bias, dQ, dK, dV, dbias,
                                                        (cudaStream_t)stream));
-}
-
-// Layout of the backward scratch: status region, then (log-sum-exp, delta) [batch][KV head][query tile][128 rows], then the
-// routed-chunk prefix counts [batch * h_kv * seq_q][W].
-struct BwdLayout {
-  size_t status, stats, prefix, total;
-};
-static BwdLayout bwd_layout(const Dims& dm) {
-  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  BwdLayout l;
-  l.status = 0;
-  size_t at = up(STATUS_REGION_BYTES);
-  const int tq = std::max(1, std::min(128 / std::max(dm.g_q, 1), dm.B));
-  const size_t rows = (size_t)dm.batch * dm.h_kv * (size_t)((dm.seq_q + tq - 1) / tq) * 128;
-  l.stats = at; at = up(at + rows * sizeof(float2));
-  // prefix counts [batch * h_kv * seq_q][W], then the tiles' mask unions [batch * h_kv][query tile][W]
-  l.prefix = at; at = up(at + ((size_t)dm.batch * dm.h_kv * dm.seq_q + (size_t)dm.batch * dm.h_kv * ((dm.seq_q + tq - 1) / tq)) *
-                                  (size_t)dm.W * sizeof(int));
-  l.total = at;
-  return l;
 }
 
 size_t dash_attn_bwd_workspace_bytes(const dash_params* p) {
   Dims dm;
   if (make_dims(p, &dm) != DASH_OK || dm.decode) return 0;
-  return bwd_layout(dm).total;
+  return align256(STATUS_REGION_BYTES);      // the status word: what passes between the kernels sits in the gradient buffers
 }
 
 int dash_attn_bwd_attend_prefill_tc(const dash_params* p, const void* Q, const void* K, const void* V, const void* dO,
@@ -335,20 +319,13 @@ int dash_attn_bwd_attend_prefill_tc(const dash_params* p, const void* Q, const v
   if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(dO) || !aligned16(dQ) || !aligned16(dK) ||
       !aligned16(dV))
     return DASH_ERR_INVALID_ARG;
-  const BwdLayout l = bwd_layout(dm);
   if (!bwd_workspace || (reinterpret_cast<uintptr_t>(bwd_workspace) & 255) != 0) return DASH_ERR_WORKSPACE;
-  if (bwd_workspace_bytes < l.total) return DASH_ERR_WORKSPACE;
+  if (bwd_workspace_bytes < align256(STATUS_REGION_BYTES)) return DASH_ERR_WORKSPACE;
   if ((rc = check_device()) != DASH_OK) return rc;
-  if (!prefill_bwd_sm100_supported(dm)) return DASH_ERR_UNSUPPORTED;
-  cudaStream_t st = (cudaStream_t)stream;
-  StageRange nv("dash_attn: stage 2 prefill attention, backward (tensor cores)");
-  const size_t list_bytes = (size_t)dm.batch * dm.h_kv * (size_t)dm.list_rows * sizeof(float);
-  if (list_bytes > 0) {
-    if ((rc = cuda_status(cudaMemsetAsync(dbias, 0, list_bytes, st))) != DASH_OK) return rc;
-  }
-  return cuda_status(launch_attend_prefill_bwd_sm100(dm, Q, K, V, dO, mask, blk_bias, at<float2>(bwd_workspace, l.stats),
-                                                     at<int>(bwd_workspace, l.prefix),
-                                                     dQ, dK, dV, dbias, at<StatusBlock>(bwd_workspace, l.status), st));
+  if (!prefill_bwd_sm100_supported(dm) || dm.d != 128 || dm.B < 64 || dm.g_q < 2) return DASH_ERR_UNSUPPORTED;
+  StageRange nv("dash_attn: stage 2 prefill attention, backward (one-term probabilities)");
+  return cuda_status(launch_attend_prefill_bwd_sm100(dm, false, current_sm_count(), Q, K, V, dO, mask, blk_bias, dQ, dK, dV, dbias,
+                                                     at<StatusBlock>(bwd_workspace, 0), (cudaStream_t)stream));
 }
 
 int dash_attn_bwd_select_prefill(const dash_params* p, const void* Q, const float* Kbar, const int32_t* count,

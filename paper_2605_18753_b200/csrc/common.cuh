@@ -17,6 +17,7 @@ struct Dims {
   int T_s;      // complete chunks (those with summaries): seq_kv / B
   int T_a;      // all chunks: ceil(seq_kv / B)
   int W;        // mask words per row: ceil(T_a / 32)
+  int log_b;    // log2(B)
   int decode;   // 1: one query row per sequence at kv_len[b]-1
   int causal;        // 1: the paper's setting; 0: every row sees every complete chunk (prefill only)
   int local_blocks;  // window chunks before the own chunk: attended with bias 0, not scored
@@ -60,8 +61,8 @@ struct RowStats {
 __host__ __device__ inline long long list_row_offset(const Dims& dm, int i) {
   if (dm.decode) return 0;
   if (!dm.causal) return (long long)i * dm.T_s;
-  long long c = i / dm.B;
-  return (long long)dm.B * c * (c - 1) / 2 + (long long)(i % dm.B) * c;
+  const long long c = i >> dm.log_b;
+  return ((c * (c - 1)) >> 1 << dm.log_b) + (long long)(i & (dm.B - 1)) * c;
 }
 
 // Workspace: 256-byte header (status word first), then regions carved by the host.
@@ -254,6 +255,7 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
                              const float* tau, const float* dbias, float* dQr, float* dKbar, cudaStream_t st);
 cudaError_t launch_summaries_bwd(const Dims& dm, const void* K, const float* qbar, long long qbar_chunk_stride,
                                  const float* dKbar, float* dK, float* dqbar, size_t dqbar_bytes, cudaStream_t st);
+int current_sm_count();      // SMs of the current device, cached per device
 int decode_num_splits(const Dims& dm);
 size_t decode_partial_bytes(const Dims& dm);
 cudaError_t launch_attend_decode(const Dims& dm, const void* Q, const void* K, const void* V, const int* kv_len,
@@ -273,12 +275,11 @@ cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const voi
                                         const uint32_t* mask, const float* blk_bias, void* O, StatusBlock* sb,
                                         bool inputs_stable, cudaStream_t st, const RowStats& stats = RowStats(),
                                         const void* dO = nullptr);
-// Stage 2 backward on tensor cores (bf16, head_dim 128, chunks of 64 or 128 tokens, g_q >= 2); scratch: stats
-// [batch][KV head][query tile][128] pairs (log-sum-exp, delta), prefix [batch * h_kv * seq_q][W] ints.
+// Stage 2 backward on tensor cores (bf16, causal).  two_term: every shape, P and dS as two bf16 terms; else head_dim 128,
+// chunks of 64 or 128 tokens, g_q >= 2, one term.  The gradient buffers double as its scratch.
 bool prefill_bwd_sm100_supported(const Dims& dm);
-cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* dO,
-                                            const uint32_t* mask, const float* blk_bias, float2* stats, int* prefix, void* dQ,
-                                            float* dK, float* dV, float* dbias, StatusBlock* sb,
-                                            cudaStream_t st);
+cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n_sm, const void* Q, const void* K, const void* V,
+                                            const void* dO, const uint32_t* mask, const float* blk_bias, void* dQ, float* dK,
+                                            float* dV, float* dbias, StatusBlock* sb, cudaStream_t st);
 
 }  // namespace dash

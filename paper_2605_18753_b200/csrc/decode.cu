@@ -26,7 +26,7 @@ static bool decode_use_sm100(const Dims& dm) {
 // block, about 2 % of a long group's work: list staging, first loads, partial write).  At 128 groups on 148 SMs
 // s = 5 leaves a fifth wave a third full, s = 8 fills seven waves almost exactly (measured: 0.155 vs 0.150 ms).
 // SM count of the current device, cached per device (a process may drive several GPUs).
-static int current_sm_count() {
+int current_sm_count() {
   static std::atomic<int> cached[64];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 148;

@@ -4,36 +4,42 @@
 // With P = softmax of the row's logits l_j = <q,k_j>/sqrt(d) + bias_c(j) over its selected tokens, dP = dO V^T,
 // delta = <O, dO> per row and dS = P o (dP - delta):
 //     dQ = dS K / sqrt(d),   dK = dS^T Q / sqrt(d),   dV = P^T dO,   dbias_c = sum of dS over the chunk's tokens.
-// Four launches behind the forward kernel run in "statistics" mode (it leaves the log-sum-exp and delta of every row):
-//   mask_prefix_kernel      per row, the number of routed chunks in the mask words before each word (so that a row's
-//                           list entry for a chunk can be found from one word of its mask);
-//   tile_union_kernel       per query tile, the OR of its rows' mask words (which chunks any of its rows attends);
+// Three launches behind the forward kernel run in "statistics" mode (it leaves the log-sum-exp and delta of every row):
+//   list_marks_kernel       per row, the number of routed chunks in the mask words before each word (so that a row's
+//                           list entry for a chunk can be found from one word of its mask), and per query tile the OR of
+//                           its rows' mask words (which chunks any of its rows routed);
+//   attend_bwd_dkv_kernel   key-slice stationary (64 keys of one KV head): walks the query tiles that attend the slice
+//                           (the tiles of its own chunks, causally masked, then every later tile whose union holds one of
+//                           its chunks), computes S and dP, and accumulates dV^T += dO^T P and dK^T += Q^T dS in tensor
+//                           memory (P and dS pass through shared memory as bf16 MN-major operands);
 //   attend_bwd_dq_kernel    query-tile stationary, the forward kernel's walk over the union of the tile's routed
 //                           chunks: S = Q K^T and dP = dO V^T into tensor memory, dS (bf16) back into tensor memory,
-//                           dQ += dS K accumulated in tensor memory; dbias from the row sums of dS;
-//   attend_bwd_dkv_kernel   key-slice stationary (64 keys of one KV head): walks the query tiles that attend the slice
-//                           (the tiles of its own chunk, causally masked, then every later tile whose mask holds the
-//                           chunk), recomputes S and dP, and accumulates dV^T += dO^T P and dK^T += Q^T dS in tensor
-//                           memory (P and dS pass through shared memory as bf16 MN-major operands), so dK and dV need
-//                           no atomics and no zeroing.
-// bf16 operands, fp32 accumulation; head_dim 128; chunks of 64 or 128 tokens; g_q >= 2.  Every wait is bounded.
+//                           dQ += dS K accumulated in tensor memory; dbias from the row sums of dS.
+// What passes between them needs no scratch of its own: a row's statistics sit in the first eight bytes of its dQ row until
+// the dQ kernel, which owns the row, overwrites them; the counts and unions sit in the rows' regions of dbias (a row with
+// own chunk c has c entries there, and c >= 2 floor(c / 32) + 1), which is zeroed behind the dK / dV kernel.
+//
+// bf16 operands, fp32 accumulation.  P2 instantiations (the entry point that takes every shape, which computed P and dS in
+// fp32 when it ran on CUDA cores) carry P and dS as two bf16 terms (hi + lo, 16 bits of mantissa) through every product;
+// the others round them to bf16.  Tiles as in the forward kernel (prefill_sm100.cu).  Every wait is bounded.
+//
+// Bound by the chain of a step (tile landed -> S, dP -> P, dS -> accumulating products), one block per SM.  2 x 1500 tokens,
+// 8/2 heads, d 64, chunks of 32: 2.02 ms on CUDA cores (one warp per row and head, two vector reductions per token and
+// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: 2.0 ms (statistics 0.40, dK / dV 1.04, dQ 0.55).
 #include <cuda.h>
 
-#include <type_traits>
+#include <algorithm>
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
+#include "tile_walk.cuh"
 
 namespace dash {
 
 namespace {
 
 constexpr int NKV = 64;                 // keys per step / per slice
-constexpr int HD = 128;
-constexpr uint32_t Q_BYTES = 128 * HD * 2;          // 32 KiB: a 128-row tile, two 128x64 regions
-constexpr uint32_t KV_TILE_BYTES = NKV * HD * 2;    // 16 KiB
-constexpr int MAX_TQ = 64;
 constexpr float LOG2E = 1.4426950408889634f;
 
 struct BwdArgs {
@@ -41,12 +47,12 @@ struct BwdArgs {
   int TQ;             // tokens per query tile
   int n_tiles;        // query tiles per (batch, KV head)
   int n_slices;       // 64-key slices per (batch, KV head)
+  int n_split;        // blocks that share a slice's query tiles (1: they write dK / dV, more: they add to them)
   long long wait_limit;
   const uint32_t* mask;
   const float* blk_bias;
-  const float2* stats;          // (log-sum-exp, delta) of every row, [batch][KV head][query tile][128 rows]
-  const int* prefix;
-  const uint32_t* tile_union;   // [batch * h_kv][query tile][W]: OR of the tile's rows' mask words
+  RowStats stats;
+  int* marks;         // counts and unions, in the layout of the lists
   __nv_bfloat16* dQ;
   float* dK;
   float* dV;
@@ -54,46 +60,70 @@ struct BwdArgs {
   StatusBlock* sb;
 };
 
-// prefix[row][w] = routed chunks of the row in mask words 0 .. w-1 (the own chunk's bit, which sits behind every routed
-// one, is left out)
-__global__ void __launch_bounds__(256)
-mask_prefix_kernel(Dims dm, const uint32_t* __restrict__ mask, int* __restrict__ prefix) {
-  chain_wait();
-  chain_release();
-  const long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long rows = (long long)dm.batch * dm.h_kv * dm.seq_q;
-  if (row >= rows) return;
-  const int i = (int)(row % dm.seq_q);
-  const int c_own = i / dm.B;
-  int acc = 0;
-  for (int w = 0; w < dm.W; ++w) {
-    prefix[row * dm.W + w] = acc;
-    uint32_t word = mask[row * dm.W + w];
-    if (w == (c_own >> 5)) word &= (1u << (c_own & 31)) - 1u;
-    else if (w > (c_own >> 5)) word = 0u;
-    acc += __popc(word);
-  }
+// Where a row's counts start (entry w - 1: routed chunks in mask words 0 .. w - 1), and the unions of the tile whose last
+// row it is (behind the counts, one per mask word).
+__device__ __forceinline__ long long marks_of(const Dims& dm, long long grp, int i) {
+  return grp * dm.list_rows + list_row_offset(dm, i);
 }
 
-// tile_union[group][tile][w] = OR over the tile's rows of mask word w: which chunks any row of the tile attends
 __global__ void __launch_bounds__(256)
-tile_union_kernel(Dims dm, int TQ, int n_tiles, const uint32_t* __restrict__ mask, uint32_t* __restrict__ tile_union) {
+list_marks_kernel(Dims dm, int TQ, int n_tiles, const uint32_t* __restrict__ mask, int* __restrict__ marks) {
   chain_wait();
   chain_release();
   const long long warp_id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const long long total = (long long)dm.batch * dm.h_kv * n_tiles;
-  if (warp_id >= total) return;
+  if (warp_id >= (long long)dm.batch * dm.h_kv * n_tiles) return;
   const long long grp = warp_id / n_tiles;
-  const int tile = (int)(warp_id % n_tiles);
-  for (int w = 0; w < dm.W; ++w) {
-    uint32_t u = 0u;
-    for (int t = lane; t < TQ; t += 32) {
-      const int i = tile * TQ + t;
-      if (i < dm.seq_q) u |= mask[(grp * dm.seq_q + i) * dm.W + w];
+  const int i0 = (int)(warp_id % n_tiles) * TQ;
+  const int n_live = min(TQ, dm.seq_q - i0), i_last = i0 + n_live - 1, c_last = i_last / dm.B;
+  if (c_last == 0) return;                      // nothing routed, and no room in the rows' regions
+  const long long last = marks_of(dm, grp, i_last) + (c_last >> 5);
+  int acc[4] = {0, 0, 0, 0}, own[4];
+  long long at[4];
+  uint32_t next[4] = {0u, 0u, 0u, 0u};
+  const uint32_t* row[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = min(i0 + lane + 32 * q, i_last);
+    own[q] = lane + 32 * q < n_live ? i >> dm.log_b : -1;      // -1: no such token
+    at[q] = marks_of(dm, grp, i);
+    row[q] = mask + (grp * dm.seq_q + i) * dm.W;
+    if (own[q] >= 0) next[q] = row[q][0];
+  }
+  const int last_w = c_last >> 5;
+  for (int w = 0; w <= last_w; ++w) {
+    uint32_t u = 0u, word[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      word[q] = next[q];
+      if (w < last_w && own[q] >= 0) next[q] = row[q][w + 1];      // one word ahead
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (own[q] >= 0) {
+        const uint32_t bits = routed_bits(word[q], w, own[q]);
+        if (w > 0 && w <= (own[q] >> 5)) marks[at[q] + w - 1] = acc[q];
+        acc[q] += __popc(bits);
+        u |= bits;
+      }
     }
     u = __reduce_or_sync(0xffffffffu, u);
-    if (lane == 0) tile_union[warp_id * dm.W + w] = u;
+    if (lane == 0) marks[last + w] = (int)u;
+  }
+}
+
+// P or dS of 32 columns as packed bf16 pairs; with P2 also the remainders (x = hi + lo)
+template <bool P2>
+__device__ __forceinline__ void pack_terms(const float (&x)[32], uint32_t (&hi)[16], uint32_t (&lo)[16]) {
+#pragma unroll
+  for (int c = 0; c < 32; c += 2) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x[c], x[c + 1]);
+    hi[c >> 1] = *reinterpret_cast<const uint32_t*>(&h);
+    if constexpr (P2) {
+      const float2 hf = __bfloat1622float2(h);
+      const __nv_bfloat162 l = __floats2bfloat162_rn(x[c] - hf.x, x[c + 1] - hf.y);
+      lo[c >> 1] = *reinterpret_cast<const uint32_t*>(&l);
+    }
   }
 }
 
@@ -107,31 +137,44 @@ namespace dq {
 // 60-80 clocks whatever its size, and 20 per step through one thread would be the kernel's pace.
 constexpr int W_KPROD = 8, W_S = 9, W_VPROD = 10, W_DP = 11, W_DQ = 12;
 constexpr int THREADS = 512;              // 8 dS warps, 5 service warps, 3 idle: whole warpgroups, so that the registers can be re-divided
-constexpr int REGS_SERVICE = 56, REGS_SOFTMAX = 200;   // per thread after the re-division (128 each at launch)
-static_assert(THREADS == 512 && 256 * (REGS_SOFTMAX - 128) <= 256 * (128 - REGS_SERVICE),
-              "the dS warpgroups can only take what the service warpgroups released: a larger request never completes");
+// registers per thread after the re-division (128 each at launch); wide tiles keep more per producer lane
+__host__ __device__ constexpr int regs_service(int wt, int cps) { return wt > 2 || (wt > 0 && cps > 2) ? 96 : wt > 0 || cps > 1 ? 80 : 56; }
+static_assert(THREADS == 512, "two pairs of warpgroups: one pair can take exactly what the other released");
 constexpr int KST = 3;                  // K / V ring and S / dP ring: stage = step mod 3, held until the step's dQ product is done
 constexpr uint32_t TMEM_COLS = 512;     // S [0,192) dP [192,384) dQ [384,512)
 constexpr uint32_t COL_DP = 192, COL_DQ = 384;
 enum Bar { QD_FULL = 0, META, S_FULL = 2, DP_FULL = 5, DS_FULL = 8, V_FULL = 11, K_FULL = 14, KV_FREE = 17, N_BARS = 20 };
-struct Misc {
+template <int CPS, int MTQ>
+struct MiscT {
   unsigned long long bar[N_BARS];
   uint32_t tmem_base;
   int n_steps;
   int abort_flag;
-  int kvbase[KST];
-  float bias[KST][MAX_TQ];
-  long long entry[KST][MAX_TQ];         // list entry of the token for the step's chunk (-1: none: own chunk or not routed)
+  int kvbase[KST][CPS];
+  float bias[KST][CPS][MTQ];
+  int pos[KST][CPS][MTQ];               // the chunk's position in the token's list (-1: none: own chunk or not routed)
 };
-constexpr uint32_t OFF_Q = 0, OFF_DO = OFF_Q + Q_BYTES, OFF_K = OFF_DO + Q_BYTES, OFF_V = OFF_K + KST * KV_TILE_BYTES,
-                   OFF_MISC = OFF_V + KST * KV_TILE_BYTES, SMEM = OFF_MISC + sizeof(Misc);
-static_assert(SMEM <= 232448, "one block per SM");
+template <int HD, int CPS, int MTQ>
+struct Layout {
+  static constexpr uint32_t Q_BYTES = 128 * HD * 2;          // HD = 128: 32 KiB, two 128x64 regions
+  static constexpr uint32_t KV_TILE_BYTES = NKV * HD * 2;
+  static constexpr uint32_t OFF_Q = 0, OFF_DO = OFF_Q + Q_BYTES, OFF_K = OFF_DO + Q_BYTES, OFF_V = OFF_K + KST * KV_TILE_BYTES,
+                            OFF_MISC = OFF_V + KST * KV_TILE_BYTES, SMEM = OFF_MISC + sizeof(MiscT<CPS, MTQ>);
+  static_assert(SMEM <= 232448, "one block per SM");
+};
 
+template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(THREADS, 1)
 attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
+  constexpr bool WIDE = WT > 0;
+  constexpr int TPL = WIDE ? WT : 2, MTQ = 32 * TPL, W = NKV / CPS;
+  using LY = Layout<HD, CPS, MTQ>;
+  using Misc = MiscT<CPS, MTQ>;
+  constexpr uint32_t Q_BYTES = LY::Q_BYTES, KV_TILE_BYTES = LY::KV_TILE_BYTES, OFF_Q = LY::OFF_Q, OFF_DO = LY::OFF_DO,
+                     OFF_K = LY::OFF_K, OFF_V = LY::OFF_V;
   extern __shared__ __align__(1024) uint8_t smem[];
-  Misc* misc = reinterpret_cast<Misc*>(smem + OFF_MISC);
+  Misc* misc = reinterpret_cast<Misc*>(smem + LY::OFF_MISC);
   const Dims& dm = a.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sbase = ptx::smem_u32(smem);
@@ -146,9 +189,9 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const int b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int TQ = a.TQ, g_q = dm.g_q;
   const int i0 = tile * TQ;
-  const int c_own = i0 / dm.B;
+  const int c_own = i0 >> dm.log_b;
   const int sub_per_blk = dm.B / NKV;
-  const int own_steps = (i0 % dm.B) / NKV + 1;
+  const int own_steps = WIDE ? (TQ + NKV - 1) / NKV : (i0 % dm.B) / NKV + 1;
 
   if (tid == 0) {
     misc->abort_flag = ((sbase & 1023u) != 0u) ? 1 : 0;
@@ -178,14 +221,18 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
 
-  auto load_kv = [&](const CUtensorMap* tm, uint32_t dst, uint32_t barrier, int kv0) {
+  auto load_packed = [&](const CUtensorMap* tm, uint32_t dst, uint32_t barrier, const int* kvs) {
     ptx::mbar_arrive_expect_tx(barrier, KV_TILE_BYTES);
-    ptx::tma_load_4d(dst, tm, barrier, 0, r, kv0, b);
-    ptx::tma_load_4d(dst + KV_TILE_BYTES / 2, tm, barrier, 64, r, kv0, b);
+#pragma unroll
+    for (int s = 0; s < CPS; ++s) {
+      const uint32_t d = dst + s * W * 128;
+      ptx::tma_load_4d(d, tm, barrier, 0, r, kvs[s], b);
+      if constexpr (HD == 128) ptx::tma_load_4d(d + KV_TILE_BYTES / 2, tm, barrier, 64, r, kvs[s], b);
+    }
   };
 
   if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(WT, CPS)));
   if (warp == W_KPROD || warp == W_VPROD) {
     // =========================== producers: the forward kernel's walk ===========================
     const bool do_k = (warp == W_KPROD), do_v = (warp == W_VPROD);
@@ -196,101 +243,84 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       ptx::prefetch_tensormap(&tmV);
       ptx::mbar_arrive_expect_tx(bar(QD_FULL), 2 * Q_BYTES);
       ptx::tma_load_4d(sbase + OFF_Q, &tmQ, bar(QD_FULL), 0, r * g_q, i0, b);
-      ptx::tma_load_4d(sbase + OFF_Q + Q_BYTES / 2, &tmQ, bar(QD_FULL), 64, r * g_q, i0, b);
+      if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_Q + Q_BYTES / 2, &tmQ, bar(QD_FULL), 64, r * g_q, i0, b);
       ptx::tma_load_4d(sbase + OFF_DO, &tmDO, bar(QD_FULL), 0, r * g_q, i0, b);
-      ptx::tma_load_4d(sbase + OFF_DO + Q_BYTES / 2, &tmDO, bar(QD_FULL), 64, r * g_q, i0, b);
+      if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_DO + Q_BYTES / 2, &tmDO, bar(QD_FULL), 64, r * g_q, i0, b);
     }
-    // own chunk first (steps 0 .. own_steps-1 <= 2 go to stages 0 / 1, which are free)
+    // own chunks first (steps 0 .. own_steps-1 <= 2 go to stages 0 / 1, which are free), as in the forward kernel
     for (int sub = 0; sub < own_steps; ++sub) {
-      const int kv0 = c_own * dm.B + sub * NKV;
+      int kvs[CPS];
+      const int kv0 = WIDE ? i0 + sub * NKV : c_own * dm.B + sub * NKV;
+#pragma unroll
+      for (int s = 0; s < CPS; ++s) kvs[s] = WIDE && kv0 + s * W < i0 + TQ ? kv0 + s * W : kv0;
       if (do_k) {
-        if (lane == 0) load_kv(&tmK, sbase + OFF_K + sub * KV_TILE_BYTES, bar(K_FULL + sub), kv0);
+        if (lane == 0) load_packed(&tmK, sbase + OFF_K + sub * KV_TILE_BYTES, bar(K_FULL + sub), kvs);
       } else {
-        for (int t = lane; t < TQ; t += 32) { misc->bias[sub][t] = 0.f; misc->entry[sub][t] = -1; }
-        if (lane == 0) misc->kvbase[sub] = kv0;
+        for (int t = lane; t < TQ; t += 32)
+#pragma unroll
+          for (int s = 0; s < CPS; ++s) {
+            misc->bias[sub][s][t] = (WIDE ? (kv0 + s * W) >> dm.log_b == (i0 + t) >> dm.log_b : s == 0) ? 0.f : -INFINITY;
+            misc->pos[sub][s][t] = -1;
+          }
+#pragma unroll
+        for (int s = 0; s < CPS; ++s)
+          if (lane == s) misc->kvbase[sub][s] = kvs[s];
         __syncwarp();
-        if (lane == 0) load_kv(&tmV, sbase + OFF_V + sub * KV_TILE_BYTES, bar(V_FULL + sub), kv0);
+        if (lane == 0) load_packed(&tmV, sbase + OFF_V + sub * KV_TILE_BYTES, bar(V_FULL + sub), kvs);
       }
     }
-    const int n_words = (c_own >> 5) + 1;
-    const long long row0 = ((long long)b * dm.h_kv + r) * dm.seq_q;
-    const uint32_t own_word_keep = (c_own & 31) == 31 ? 0xffffffffu : ((2u << (c_own & 31)) - 1u);
-    auto load_rows = [&](int w, uint32_t* rw) {
-      for (int q = 0; q < 2; ++q) {
-        const int t = lane + 32 * q;
-        rw[q] = (t < TQ && i0 + t < dm.seq_q) ? a.mask[(row0 + i0 + t) * dm.W + w] : 0u;
-      }
-    };
-    auto union_of = [&](int w, const uint32_t* rw) -> uint32_t {
-      uint32_t u = __reduce_or_sync(0xffffffffu, rw[0] | rw[1]);
-      if (w == n_words - 1) u = (u & own_word_keep) | (1u << (c_own & 31));
-      return u;
-    };
-    int total = 0;
-    for (int w = 0; w < n_words; ++w) {
-      uint32_t rw[2];
-      load_rows(w, rw);
-      total += __popc(union_of(w, rw));
-    }
-    const int n_steps = (total - 1) * sub_per_blk + own_steps;
+    TileWalk<CPS, WIDE, TPL> walk(dm, a.mask, (long long)grp * dm.seq_q, i0, TQ, lane);
+    const int total = walk.count();
+    const int n_steps = (CPS > 1 ? (total + CPS - 1) / CPS : total * sub_per_blk) + own_steps;
     if (lane == 0 && do_k) {
       misc->n_steps = n_steps;
       ptx::mbar_arrive(bar(META));
     }
-    long long loff[2];
-    for (int q = 0; q < 2; ++q) {
-      const int t = lane + 32 * q;
-      const int i = min(i0 + t, dm.seq_q - 1);
-      loff[q] = ((long long)b * dm.h_kv + r) * dm.list_rows + list_row_offset(dm, i);
-    }
-    int j = own_steps;
+    const float* list[TPL];
+#pragma unroll
+    for (int q = 0; q < TPL; ++q)
+      list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
+    walk.start();
     bool ok = true;
     int last_j[KST];
+#pragma unroll
     for (int s = 0; s < KST; ++s) last_j[s] = s < own_steps ? s : -1;
-    int seen[2] = {0, 0};
-    uint32_t rw[2], rw_n[2] = {0u, 0u};
-    load_rows(0, rw);
-    if (n_words > 1) load_rows(1, rw_n);
-    for (int w = 0; w < n_words && ok; ++w) {
-      uint32_t u = union_of(w, rw);
-      uint32_t rb[2];
-      for (int q = 0; q < 2; ++q) rb[q] = w == n_words - 1 ? rw[q] & own_word_keep & ~(1u << (c_own & 31)) : rw[q];
-      while (u != 0u && ok) {
-        const int bit = __ffs(u) - 1;
-        u &= u - 1;
-        const int c = w * 32 + bit;
-        if (c == c_own) break;                   // last of the walk, done first
-        float bv[2];
-        long long en[2];
-        for (int q = 0; q < 2; ++q) {
-          const bool member = do_v && ((rb[q] >> bit) & 1u);
-          const long long e = loff[q] + seen[q] + __popc(rb[q] & ((1u << bit) - 1u));
-          bv[q] = member ? __ldg(a.blk_bias + e) : -INFINITY;
-          en[q] = member ? e : -1;
-        }
-        for (int sub = 0; sub < sub_per_blk && ok; ++sub, ++j) {
-          const int kv0 = c * dm.B + sub * NKV;
-          const int st = j % KST;
-          if (j >= KST) ok = wait_on(bar(KV_FREE + st), (uint32_t)(j / KST - 1) & 1u);   // every product of step j-3 has read the stage
-          if (!ok) break;
-          if (do_k) {
-            if (lane == 0) load_kv(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kv0);
-          } else {
-            for (int q = 0; q < 2; ++q) {
-              const int t = lane + 32 * q;
-              if (t < TQ) { misc->bias[st][t] = bv[q]; misc->entry[st][t] = en[q]; }
-            }
-            if (lane == 0) misc->kvbase[st] = kv0;
-            __syncwarp();
-            if (lane == 0) load_kv(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kv0);
-          }
-          last_j[st] = j;
-        }
+    for (int j = own_steps; j < n_steps && ok;) {
+      int cs[CPS], pos[CPS][TPL];
+      float bvs[CPS][TPL];
+      walk.next(cs, pos);
+      if (do_v) {
+#pragma unroll
+        for (int s = 0; s < CPS; ++s)
+#pragma unroll
+          for (int q = 0; q < TPL; ++q) bvs[s][q] = pos[s][q] >= 0 ? __ldg(list[q] + pos[s][q]) : -INFINITY;
       }
-      seen[0] += __popc(rb[0]);
-      seen[1] += __popc(rb[1]);
-      rw[0] = rw_n[0]; rw[1] = rw_n[1];
-      if (w + 2 < n_words) load_rows(w + 2, rw_n);
+      for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk) && ok; ++sub, ++j) {
+        int kvs[CPS];
+#pragma unroll
+        for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
+        const int st = j % KST;
+        if (j >= KST) ok = wait_on(bar(KV_FREE + st), (uint32_t)(j / KST - 1) & 1u);   // every product of step j-3 has read the stage
+        if (!ok) break;
+        if (do_k) {
+          if (lane == 0) load_packed(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kvs);
+        } else {
+#pragma unroll
+          for (int s = 0; s < CPS; ++s) {
+#pragma unroll
+            for (int q = 0; q < TPL; ++q) {
+              const int t = lane + 32 * q;
+              if (t < TQ) { misc->bias[st][s][t] = bvs[s][q]; misc->pos[st][s][t] = pos[s][q]; }
+            }
+            if (lane == s) misc->kvbase[st][s] = kvs[s];
+          }
+          __syncwarp();
+          if (lane == 0) load_packed(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kvs);
+        }
+#pragma unroll
+        for (int s = 0; s < KST; ++s)
+          if (s == st) last_j[s] = j;
+      }
     }
     if (!ok && lane == 0) {
       for (int s = 0; s < KST; ++s) {
@@ -354,11 +384,14 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         if (!ok) break;
         ptx::tc_fence_after();
         const uint64_t kmn = kmn0 + (uint64_t)((st * KV_TILE_BYTES) >> 4);
+        // dS of keys 16k .. 16k+15: eight packed columns, keys 0-31 at columns 0-15 and keys 32-63 at columns 32-47 of the
+        // step's S slot; the remainders, with two-term dS, 16 columns behind
 #pragma unroll
-        for (int k = 0; k < NKV / 16; ++k)
-          // dS of keys 16k .. 16k+15: eight packed columns, keys 0-31 at columns 0-15 and keys 32-63 at columns 32-47
-          ptx::mma_bf16_ts(tmem + COL_DQ, tmem + st * NKV + (k >> 1) * 32 + (k & 1) * 8, kmn + (uint64_t)((k * 16 * 128) >> 4),
-                           IDESC_DQ, (j > 0 || k > 0) ? 1u : 0u);
+        for (int term = 0; term < (P2 ? 2 : 1); ++term)
+#pragma unroll
+          for (int k = 0; k < NKV / 16; ++k)
+            ptx::mma_bf16_ts(tmem + COL_DQ, tmem + st * NKV + (k >> 1) * 32 + term * 16 + (k & 1) * 8,
+                             kmn + (uint64_t)((k * 16 * 128) >> 4), IDESC_DQ, (j > 0 || k > 0 || term > 0) ? 1u : 0u);
         ptx::mma_commit(bar(KV_FREE + st));
       }
     }
@@ -366,7 +399,8 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   }
   } else {
     // =========================== dS / epilogue: thread = tile row, warpgroup = column half ===========================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(256 - regs_service(WT, CPS)));
+    constexpr int SPH = CPS == 4 ? 2 : 1;                  // chunk slots in a half of the columns
     const int wg = warp >> 2;
     const int m = (warp & 3) * 32 + lane;
     const int t = m / g_q, hh = m % g_q;
@@ -374,9 +408,9 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const bool row_ok = i_row < dm.seq_q;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float c1 = dm.sm_scale * LOG2E;
-    const long long srow = (((long long)b * dm.h_kv + r) * a.n_tiles + tile) * 128 + m;
-    const float2 stat = row_ok ? a.stats[srow] : make_float2(0.f, 0.f);
+    const float2 stat = row_ok ? *a.stats.at(b, r, i_row, hh) : make_float2(0.f, 0.f);
     const float lse2 = stat.x, delta = stat.y;
+    float* drow = a.dbias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i_row, dm.seq_q - 1));
     bool ok = true;
     int n_steps = 0x7fffffff;              // known from step 1 on; step 0 (the own chunk) always exists
     for (int j = 0; j < n_steps && ok; ++j) {
@@ -388,47 +422,53 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       }
       const int st = j % KST;
       const uint32_t ph = (uint32_t)(j / KST) & 1u;
-      ok = wait_on(bar(V_FULL + st), ph);                  // bias / entry / kvbase of the step visible
+      ok = wait_on(bar(V_FULL + st), ph);                  // bias / pos / kvbase of the step visible
       if (!ok) break;
-      const float bias = row_ok ? misc->bias[st][t] : -INFINITY;
-      const long long entry = misc->entry[st][t];
-      const int kv0 = misc->kvbase[st];
+      float off[SPH];                                      // -inf: the row did not route the chunk
+      int pos[SPH], n_vis[SPH];                            // causal: column c of the half visible iff c < n_vis
+#pragma unroll
+      for (int s = 0; s < SPH; ++s) {
+        const int slot = CPS == 1 ? 0 : wg * SPH + s;
+        off[s] = row_ok ? misc->bias[st][slot][t] * LOG2E - lse2 : -INFINITY;
+        pos[s] = misc->pos[st][slot][t];
+        n_vis[s] = i_row - misc->kvbase[st][slot] + 1 + (CPS == 1 ? -wg * 32 : s * W);
+      }
       ok = wait_on(bar(S_FULL + st), ph) && wait_on(bar(DP_FULL + st), ph);
       if (!ok) break;
       ptx::tc_fence_after();
-      const int n_vis = i_row - kv0 + 1;                   // causal: column c visible iff c < n_vis
-      const float off = bias * LOG2E - lse2;               // -inf: the row did not route the chunk
-      float rowsum = 0.f;
+      float rowsum[SPH];
       {
-        const int half = wg;
         uint32_t sv[32], gv[32];
-        DASH_TMEM_LD32(sv, lane_addr + st * NKV + half * 32);
-        DASH_TMEM_LD32(gv, lane_addr + COL_DP + st * NKV + half * 32);
+        DASH_TMEM_LD32(sv, lane_addr + st * NKV + wg * 32);
+        DASH_TMEM_LD32(gv, lane_addr + COL_DP + st * NKV + wg * 32);
         ptx::tmem_wait_ld();
-        uint32_t packed[16];
+        float ds[32];
 #pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-          float ds[2];
+        for (int s = 0; s < SPH; ++s) {
+          rowsum[s] = 0.f;
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const bool vis = half * 32 + c + u < n_vis;
-            const float p = vis ? exp2f(fmaf(__uint_as_float(sv[c + u]), c1, off)) : 0.f;
-            ds[u] = p * (__uint_as_float(gv[c + u]) - delta);
-            rowsum += ds[u];
+          for (int c = s * (32 / SPH); c < (s + 1) * (32 / SPH); ++c) {
+            const float p = c < n_vis[s] ? exp2f(fmaf(__uint_as_float(sv[c]), c1, off[s])) : 0.f;
+            ds[c] = p * (__uint_as_float(gv[c]) - delta);
+            rowsum[s] += ds[c];
           }
-          __nv_bfloat162 h = __floats2bfloat162_rn(ds[0], ds[1]);
-          packed[c >> 1] = *reinterpret_cast<uint32_t*>(&h);
         }
-        // dS row -> the first 16 columns of this warpgroup's own half of the step's S buffer (two bf16 per column):
-        // the other warpgroup's scores, in the other 32 columns, are never touched
-        ptx::tmem_st_n<16>(lane_addr + st * NKV + half * 32, packed);
+        // dS row -> the first 16 columns of this warpgroup's own half of the step's S buffer (two bf16 per column), the
+        // remainders behind them: the other warpgroup's scores, in the other 32 columns, are never touched
+        uint32_t hi[16], lo[16];
+        pack_terms<P2>(ds, hi, lo);
+        ptx::tmem_st_n<16>(lane_addr + st * NKV + wg * 32, hi);
+        if constexpr (P2) ptx::tmem_st_n<16>(lane_addr + st * NKV + wg * 32 + 16, lo);
       }
       ptx::tmem_wait_st();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(DS_FULL + st));
       // dbias of the (token, chunk): the row sums of the group's heads (adjacent lanes) added up
-      for (int o = 1; o < g_q; o <<= 1) rowsum += __shfl_xor_sync(0xffffffffu, rowsum, o);
-      if (hh == 0 && entry >= 0 && row_ok) atomicAdd(a.dbias + entry, rowsum);
+#pragma unroll
+      for (int s = 0; s < SPH; ++s) {
+        for (int o = 1; o < g_q; o <<= 1) rowsum[s] += __shfl_xor_sync(0xffffffffu, rowsum[s], o);
+        if (hh == 0 && pos[s] >= 0 && row_ok) atomicAdd(drow + pos[s], rowsum[s]);
+      }
     }
     // epilogue: dQ / sqrt(d) -> global; each warpgroup takes half of the row's columns
     if (ok && n_steps > 0) ok = wait_on(bar(KV_FREE + ((n_steps - 1) % KST)), (uint32_t)((n_steps - 1) / KST) & 1u);
@@ -437,7 +477,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       __nv_bfloat16* op = a.dQ + (long long)b * dm.qs[0] + (long long)i_row * dm.qs[1] + (long long)(r * g_q + hh) * dm.qs[2];
       const float sc = dm.sm_scale;
 #pragma unroll 1
-      for (int q = wg * 2; q < wg * 2 + 2; ++q) {
+      for (int q = wg * (HD / 64); q < (wg + 1) * (HD / 64); ++q) {
         uint32_t o[32];
         DASH_TMEM_LD32(o, lane_addr + COL_DQ + q * 32);
         ptx::tmem_wait_ld();
@@ -476,35 +516,68 @@ namespace dkv {
 
 // Two warpgroups form P and dS, each for half of the slice's keys on every step (no row maximum is needed, so the halves
 // are independent and a step's P / dS stretch takes half as long); one issuing thread per product: 32 MMAs per step
-// are too many for one.  W_PROD loads the tiles, W_META looks up the per-token biases of each step; W_SD issues S,
-// W_DP dP, W_ACC dV^T, W_DK dK^T.
+// are too many for one.  W_PROD loads the tiles, W_META looks up the per-token biases and row statistics of each step;
+// W_SD issues S, W_DP dP, W_ACC dV^T, W_DK dK^T.
 constexpr int W_PROD = 8, W_SD = 9, W_ACC = 10, W_DP = 11, W_DK = 12, W_META = 13;
 constexpr int THREADS = 512;              // 8 P / dS warps, 6 service warps, 2 idle: whole warpgroups
-constexpr int REGS_SERVICE = 80, REGS_SOFTMAX = 176;     // (the bias and loader warps need more than the issuers)
-static_assert(THREADS == 512 && 256 * (REGS_SOFTMAX - 128) <= 256 * (128 - REGS_SERVICE), "see the dQ kernel");
+__host__ __device__ constexpr int regs_service(int wt) { return wt > 0 ? 96 : 80; }     // (the bias and loader warps need more than the issuers)
+static_assert(THREADS == 512, "two pairs of warpgroups: one pair can take exactly what the other released");
 constexpr uint32_t TMEM_COLS = 512;     // S0 S1 [0,128) dP0 dP1 [128,256) dV^T [256,320) dK^T [320,384)
 constexpr uint32_t COL_DP = 128, COL_DV = 256, COL_DK = 320;
-constexpr uint32_t PS_BYTES = 128 * NKV * 2;       // 16 KiB: P (or dS) of a step, 128 rows of 128 bytes
-enum Bar { KV_FULL = 0, QD_FULL = 1, SD_FULL = 3, ACC_DONE = 5, PDS_FULL = 7, N_BARS = 9 };   // SD_FULL, ACC_DONE: two arrivals (one per issuer)
-struct Misc {
-  unsigned long long bar[N_BARS];
-  uint32_t tmem_base;
-  int abort_flag;
-  int total;                            // number of steps, written with the end marker
-  int tile[2];                          // query tile of the stage's step (-1: no more steps)
-  float bias[2][MAX_TQ];                // per token of the tile: the chunk's bias (-inf: the token does not attend it)
-  alignas(16) float2 stats[2][128];     // the tile's row statistics (a bulk copy)
-};
-constexpr uint32_t OFF_K = 0, OFF_V = OFF_K + KV_TILE_BYTES, OFF_Q = OFF_V + KV_TILE_BYTES,   // Q stage s at OFF_Q + s * 2 * Q_BYTES,
-                   OFF_P = OFF_Q + 4 * Q_BYTES, OFF_DS = OFF_P + PS_BYTES,                   //   its dO tile Q_BYTES behind
-                   OFF_MISC = OFF_DS + PS_BYTES, SMEM = OFF_MISC + sizeof(Misc);
-static_assert(SMEM <= 232448, "one block per SM");
+constexpr uint32_t PS_BYTES = 128 * NKV * 2;       // 16 KiB: one term of P (or dS) of a step, 128 rows of 128 bytes
+constexpr int MAX_STAGES = 4;
+// SD_FULL: both score products of the step (two arrivals).  PDS_FULL: P and dS in shared memory (SEQ: P alone).
+// ACC_DONE: both accumulating products done (SEQ: dK, which follows dV), the step's stage and the P / dS buffers are free.
+enum Bar { KV_FULL = 0, SD_FULL = 1, PDS_FULL = 3, DV_DONE = 5, DS_FULL = 7, QD_FULL = 9, ACC_DONE = 9 + MAX_STAGES, N_BARS = 9 + 2 * MAX_STAGES };
 
+// A stage holds a Q and a dO tile.  head_dim 128: two stages, Q then dO.  head_dim 64: four stages, dO then Q, so that the
+// two tiles read as MN-major A stack to the M = 128 rows that an accumulating product needs: lanes 0-63 of dO^T P are
+// dV^T, lanes 64-127 of Q^T dS are dK^T (the other halves are not used).
+// Two-term P and dS (P2) take four buffers; at head_dim 128 only two fit, so there dS follows P through the same pair
+// once the dV product has read it (SEQ).
+template <int HD, int CPS, int MTQ, bool P2>
+struct Layout {
+  static constexpr int NST = HD == 128 ? 2 : 4;
+  static constexpr bool SEQ = P2 && HD == 128;
+  struct Misc {
+    unsigned long long bar[N_BARS];
+    uint32_t tmem_base;
+    int abort_flag;
+    int total;                            // number of steps, written with the end marker
+    int tile[NST];                        // query tile of the stage's step (-1: no more steps)
+    float bias[NST][CPS][MTQ];            // per token of the tile: the chunk's bias (-inf: the token does not attend it)
+    alignas(16) float2 stats[NST][128];   // log-sum-exp and delta of the tile's rows
+  };
+  static constexpr uint32_t Q_BYTES = 128 * HD * 2, KV_TILE_BYTES = NKV * HD * 2, STAGE = 2 * Q_BYTES;
+  static constexpr uint32_t AT_Q = HD == 128 ? 0 : Q_BYTES, AT_G = HD == 128 ? Q_BYTES : 0;     // inside a stage
+  static constexpr uint32_t OFF_K = 0, OFF_V = OFF_K + KV_TILE_BYTES, OFF_ST = OFF_V + KV_TILE_BYTES,
+                            OFF_P = OFF_ST + NST * STAGE,                        // terms hi (, lo) of P, then of dS
+                            OFF_DS = SEQ ? OFF_P : OFF_P + (P2 ? 2 : 1) * PS_BYTES,
+                            OFF_MISC = OFF_P + (P2 && !SEQ ? 4 : 2) * PS_BYTES, SMEM = OFF_MISC + sizeof(Misc);
+  static_assert(SMEM <= 232448, "one block per SM");
+};
+
+// 8 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
+__device__ __forceinline__ void copy_async8(uint32_t dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void arrive_after_copies(uint32_t bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(THREADS, 1)
 attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                       const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
+  constexpr bool WIDE = WT > 0;
+  constexpr int TPL = WIDE ? WT : 2, MTQ = 32 * TPL;
+  using LY = Layout<HD, CPS, MTQ, P2>;
+  using Misc = typename LY::Misc;
+  constexpr int NST = LY::NST;
+  constexpr bool SEQ = LY::SEQ;
+  constexpr uint32_t Q_BYTES = LY::Q_BYTES, KV_TILE_BYTES = LY::KV_TILE_BYTES, OFF_K = LY::OFF_K, OFF_V = LY::OFF_V;
   extern __shared__ __align__(1024) uint8_t smem[];
-  Misc* misc = reinterpret_cast<Misc*>(smem + OFF_MISC);
+  Misc* misc = reinterpret_cast<Misc*>(smem + LY::OFF_MISC);
   const Dims& dm = a.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sbase = ptx::smem_u32(smem);
@@ -519,17 +592,22 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   const int b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int TQ = a.TQ, g_q = dm.g_q;
   const int k0 = slice * NKV;                                    // first key of the slice
-  const int c = k0 / dm.B;                                       // its chunk
+  const int c = k0 >> dm.log_b;                                       // its first chunk (CPS of them)
 
   if (tid == 0) {
     misc->abort_flag = ((sbase & 1023u) != 0u) ? 1 : 0;
     if (misc->abort_flag) report_error(a.sb, DASH_ERR_CUDA, 120);
     ptx::mbar_init(bar(KV_FULL), 1);
+    for (int s = 0; s < NST; ++s) {
+      // the loader's arrival (with the byte count), the bias warp's, and one per lane of it for the statistics in flight
+      ptx::mbar_init(bar(QD_FULL + s), 34);
+      ptx::mbar_init(bar(ACC_DONE + s), SEQ ? 1 : 2);
+    }
     for (int s = 0; s < 2; ++s) {
-      ptx::mbar_init(bar(QD_FULL + s), 2);     // the loader's arrival (with the byte count) and the bias warp's
       ptx::mbar_init(bar(SD_FULL + s), 2);
-      ptx::mbar_init(bar(ACC_DONE + s), 2);
       ptx::mbar_init(bar(PDS_FULL + s), 256);
+      ptx::mbar_init(bar(DV_DONE + s), 1);
+      ptx::mbar_init(bar(DS_FULL + s), 256);
     }
     ptx::fence_barrier_init();
   }
@@ -547,14 +625,14 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   __syncthreads();
 
   if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_SERVICE));
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(WT)));
   if (warp == W_PROD || warp == W_META) {
     // =========================== producers ===========================
-    // Both warps enumerate the slice's steps in the same order: (i) the tiles of the slice's own chunk that can see it
-    // (tokens from k0 on: bias 0, causal mask in the kernel), (ii) the later tiles one of whose rows routed the chunk,
-    // read 32 tiles at a time from the tile unions.  W_PROD fetches K / V once and the Q / dO tiles and row
-    // statistics of every step; W_META looks up the per-token biases.  A step's stage is free once both accumulating
-    // products of step j-2 have completed.
+    // Both warps enumerate the slice's steps in the same order: (i) the tiles that hold tokens of the slice's own
+    // chunks from k0 on (causal mask in the kernel), (ii) the later tiles one of whose rows routed one of its chunks, read
+    // 32 tiles at a time from the tile unions.  With several blocks per slice, block s takes every n_split-th of them.
+    // W_PROD fetches K / V once and the Q / dO tiles of every step; W_META looks up the per-token biases and the row
+    // statistics.  A step's stage is free once both accumulating products of the step NST before have completed.
     const bool loader = warp == W_PROD;
     if (lane == 0 && loader) {
       ptx::prefetch_tensormap(&tmQ);
@@ -563,84 +641,95 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ptx::prefetch_tensormap(&tmV);
       ptx::mbar_arrive_expect_tx(bar(KV_FULL), 2 * KV_TILE_BYTES);
       ptx::tma_load_4d(sbase + OFF_K, &tmK, bar(KV_FULL), 0, r, k0, b);
-      ptx::tma_load_4d(sbase + OFF_K + KV_TILE_BYTES / 2, &tmK, bar(KV_FULL), 64, r, k0, b);
+      if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_K + KV_TILE_BYTES / 2, &tmK, bar(KV_FULL), 64, r, k0, b);
       ptx::tma_load_4d(sbase + OFF_V, &tmV, bar(KV_FULL), 0, r, k0, b);
-      ptx::tma_load_4d(sbase + OFF_V + KV_TILE_BYTES / 2, &tmV, bar(KV_FULL), 64, r, k0, b);
+      if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_V + KV_TILE_BYTES / 2, &tmV, bar(KV_FULL), 64, r, k0, b);
     }
-    const long long grp_l = (long long)b * dm.h_kv + r;
-    const long long row0 = grp_l * dm.seq_q;
-    const long long list0 = grp_l * dm.list_rows;
-    const long long stat0 = grp_l * a.n_tiles * 128;
-    const uint32_t* tu = a.tile_union + grp_l * a.n_tiles * dm.W;
-    const int wc = c >> 5, bit = c & 31;
+    const long long row0 = (long long)grp * dm.seq_q;
+    const long long list0 = (long long)grp * dm.list_rows;
+    const int wc = c >> 5, bit = c & 31;             // (the slice's chunks share a mask word)
+    // this lane's rows of a tile (lane, lane + 32, ...): their statistics relative to the tile's first token
+    const char* stat_p[4];
+    int stat_t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int m = lane + 32 * k;
+      stat_t[k] = m / g_q;
+      stat_p[k] = reinterpret_cast<const char*>(a.stats.at(b, r, stat_t[k], m % g_q));
+    }
     int j = 0;
     bool ok = true;
     auto stage_free = [&]() {
-      if (j >= 2) ok = wait_on(bar(ACC_DONE + (j & 1)), (uint32_t)((j >> 1) - 1) & 1u);
+      if (j >= NST) ok = wait_on(bar(ACC_DONE + j % NST), (uint32_t)(j / NST - 1) & 1u);
       return ok;
     };
     // ---- the loader's step
     auto load_step = [&](int tile_idx) {
       if (!stage_free()) return;
-      const int st = j & 1;
+      const int st = j % NST;
       if (lane == 0) {
         misc->tile[st] = tile_idx;
         if (tile_idx >= 0) {
           const int i0 = tile_idx * TQ;
-          const uint32_t dst = sbase + OFF_Q + st * 2 * Q_BYTES;
-          ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), 2 * Q_BYTES + 1024);
-          ptx::tma_load_4d(dst, &tmQ, bar(QD_FULL + st), 0, r * g_q, i0, b);
-          ptx::tma_load_4d(dst + Q_BYTES / 2, &tmQ, bar(QD_FULL + st), 64, r * g_q, i0, b);
-          ptx::tma_load_4d(dst + Q_BYTES, &tmDO, bar(QD_FULL + st), 0, r * g_q, i0, b);
-          ptx::tma_load_4d(dst + Q_BYTES + Q_BYTES / 2, &tmDO, bar(QD_FULL + st), 64, r * g_q, i0, b);
-          ptx::bulk_load(ptx::smem_u32(&misc->stats[st][0]), a.stats + stat0 + (long long)tile_idx * 128, 1024, bar(QD_FULL + st));
+          const uint32_t dq = sbase + LY::OFF_ST + st * LY::STAGE + LY::AT_Q, dg = sbase + LY::OFF_ST + st * LY::STAGE + LY::AT_G;
+          ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), 2 * Q_BYTES);
+          ptx::tma_load_4d(dq, &tmQ, bar(QD_FULL + st), 0, r * g_q, i0, b);
+          if constexpr (HD == 128) ptx::tma_load_4d(dq + Q_BYTES / 2, &tmQ, bar(QD_FULL + st), 64, r * g_q, i0, b);
+          ptx::tma_load_4d(dg, &tmDO, bar(QD_FULL + st), 0, r * g_q, i0, b);
+          if constexpr (HD == 128) ptx::tma_load_4d(dg + Q_BYTES / 2, &tmDO, bar(QD_FULL + st), 64, r * g_q, i0, b);
         } else {
           ptx::mbar_arrive(bar(QD_FULL + st));
         }
       }
       ++j;
     };
-    // ---- the bias warp's steps, four at a time: the mask words and prefix counts of all four, then their biases,
-    // then the four hand-overs (lane t owns tokens t and t + 32 of a tile)
-    int pend[4], n_pend = 0;
-    bool pend_own = false;
+    // ---- the bias warp's steps, NB at a time: the mask words and counts of all, then their biases, then the hand-overs
+    // (lane t owns tokens t, t + 32, ... of a tile)
+    constexpr int NB = WIDE || CPS > 1 ? 2 : 4;
+    int pend[NB], n_pend = 0;
     auto flush = [&]() {
-      float bv[4][2];
-      if (pend_own) {
+      float bv[NB][CPS][TPL];
+      uint32_t wd[NB][TPL];
+      int pf[NB][TPL];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          for (int q = 0; q < 2; ++q) bv[u][q] = (u < n_pend && pend[u] * TQ + lane + 32 * q < dm.seq_q) ? 0.f : -INFINITY;
-      } else {
-        uint32_t wd[4][2];
-        int pf[4][2];
+      for (int u = 0; u < NB; ++u)
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int q = 0; q < TPL; ++q) {
+          const int t = lane + 32 * q, i = (u < n_pend ? pend[u] : 0) * TQ + t;
+          const bool live = u < n_pend && t < TQ && i < dm.seq_q && (i >> dm.log_b) > c;      // a token behind the first chunk
+          wd[u][q] = live ? a.mask[(row0 + i) * dm.W + wc] : 0u;
+          pf[u][q] = live && wc > 0 ? a.marks[marks_of(dm, grp, i) + wc - 1] : 0;
+        }
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int t = lane + 32 * q, i = (u < n_pend ? pend[u] : 0) * TQ + t;
-            const bool live = u < n_pend && t < TQ && i < dm.seq_q;
-            wd[u][q] = live ? a.mask[(row0 + i) * dm.W + wc] : 0u;
-            pf[u][q] = live ? a.prefix[(row0 + i) * dm.W + wc] : 0;
+      for (int u = 0; u < NB; ++u)
+#pragma unroll
+        for (int q = 0; q < TPL; ++q) {
+          const int t = lane + 32 * q, i = (u < n_pend ? pend[u] : 0) * TQ + t, own = i >> dm.log_b;
+          const bool live = u < n_pend && t < TQ && i < dm.seq_q;
+#pragma unroll
+          for (int s = 0; s < CPS; ++s) {
+            bv[u][s][q] = live && c + s == own ? 0.f : -INFINITY;
+            if (c + s < own && ((wd[u][q] >> (bit + s)) & 1u))
+              bv[u][s][q] = __ldg(a.blk_bias + list0 + list_row_offset(dm, i) + pf[u][q] + __popc(wd[u][q] & ((1u << (bit + s)) - 1u)));
           }
+        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            bv[u][q] = -INFINITY;
-            if ((wd[u][q] >> bit) & 1u) {
-              const int i = pend[u] * TQ + lane + 32 * q;
-              bv[u][q] = __ldg(a.blk_bias + list0 + list_row_offset(dm, i) + pf[u][q] + __popc(wd[u][q] & ((1u << bit) - 1u)));
-            }
-          }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < NB; ++u) {
         if (u < n_pend && stage_free()) {
-          const int st = j & 1;
-          for (int q = 0; q < 2; ++q) {
-            const int t = lane + 32 * q;
-            if (t < TQ) misc->bias[st][t] = bv[u][q];
+          const int st = j % NST;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (pend[u] * TQ + stat_t[k] < dm.seq_q)
+              copy_async8(ptx::smem_u32(&misc->stats[st][lane + 32 * k]), stat_p[k] + (long long)pend[u] * TQ * a.stats.si);
           }
+#pragma unroll
+          for (int q = 0; q < TPL; ++q) {
+            const int t = lane + 32 * q;
+            if (t < TQ)
+#pragma unroll
+              for (int s = 0; s < CPS; ++s) misc->bias[st][s][t] = bv[u][s][q];
+          }
+          arrive_after_copies(bar(QD_FULL + st));
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + st));
           ++j;
@@ -648,31 +737,35 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
       n_pend = 0;
     };
-    auto meta_step = [&](int tile_idx, bool own) {
-      if (n_pend > 0 && own != pend_own) flush();
-      pend_own = own;
+    int n_seen = 0;
+    auto step = [&](int tile_idx) {
+      if (a.n_split > 1 && n_seen++ % a.n_split != (int)blockIdx.y) return;
+      if (loader) {
+        load_step(tile_idx);
+      } else {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (u == n_pend) pend[u] = tile_idx;
-      if (++n_pend == 4) flush();
+        for (int u = 0; u < NB; ++u)
+          if (u == n_pend) pend[u] = tile_idx;
+        if (++n_pend == NB) flush();
+      }
     };
-    auto step = [&](int tile_idx, bool own) {
-      if (loader) load_step(tile_idx); else meta_step(tile_idx, own);
-    };
-    const int t_own_lo = k0 / TQ, t_first_routed = min(((c + 1) * dm.B + TQ - 1) / TQ, a.n_tiles);
-    for (int tl = t_own_lo; tl < t_first_routed && ok; ++tl) step(tl, true);
+    const int own_end = CPS > 1 ? k0 + NKV : (c + 1) * dm.B;      // behind the last token of the slice's own chunks
+    const int t_first_routed = min((own_end + TQ - 1) / TQ, a.n_tiles);
+    for (int tl = k0 / TQ; tl < t_first_routed && ok; ++tl) step(tl);
     auto union_word = [&](int tl0) -> uint32_t {
       const int tl = tl0 + lane;
-      return tl < a.n_tiles ? __ldg(tu + (long long)tl * dm.W + wc) : 0u;
+      if (tl >= a.n_tiles) return 0u;
+      const int i = min((tl + 1) * TQ, dm.seq_q) - 1;
+      return (uint32_t)__ldg(a.marks + marks_of(dm, grp, i) + ((i >> dm.log_b) >> 5) + wc);
     };
     uint32_t uw = t_first_routed < a.n_tiles ? union_word(t_first_routed) : 0u, uw_n = 0u;
     for (int tl0 = t_first_routed; tl0 < a.n_tiles && ok; tl0 += 32) {
       if (tl0 + 32 < a.n_tiles) uw_n = union_word(tl0 + 32);
-      uint32_t hits = __ballot_sync(0xffffffffu, ((uw >> bit) & 1u) != 0u);
+      uint32_t hits = __ballot_sync(0xffffffffu, ((uw >> bit) & ((1u << CPS) - 1u)) != 0u);
       while (hits != 0u && ok) {
         const int k = __ffs(hits) - 1;
         hits &= hits - 1;
-        step(tl0 + k, false);
+        step(tl0 + k);
       }
       uw = uw_n;
     }
@@ -683,50 +776,42 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       __syncwarp();
       load_step(-1);
     } else if (ok && stage_free()) {
-      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + (j & 1)));
+      arrive_after_copies(bar(QD_FULL + j % NST));
+      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + j % NST));
       ++j;
     }
     if (!ok && lane == 0 && loader) {
       // a wait ran out: let the copies already issued land (bounded) before the block retires
       for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(KV_FULL), 0); ++k) {}
-      for (int s = 0; s < 2; ++s) {
+      for (int s = 0; s < NST; ++s) {
         const int lj = (j - 1 - s);
-        if (lj < 0 || misc->tile[lj & 1] < 0) continue;
-        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL + (lj & 1)), (uint32_t)(lj >> 1) & 1u); ++k) {}
+        if (lj < 0 || misc->tile[lj % NST] < 0) continue;
+        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL + lj % NST), (uint32_t)(lj / NST) & 1u); ++k) {}
       }
     }
+    if (!ok && !loader) asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp == W_SD || warp == W_DP) {
     // =========================== issuers of the score products: S = Q K^T (W_SD), dP = dO V^T (W_DP) ===========================
     if (lane == 0) {
       const bool is_s = warp == W_SD;
       bool ok = wait_on(bar(KV_FULL), 0);
       constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NKV, false, false);
-      const uint64_t kd0 = ptx::smem_desc_sw128(sbase + OFF_K, 16, 1024);
-      const uint64_t vd0 = ptx::smem_desc_sw128(sbase + OFF_V, 16, 1024);
+      const uint64_t bd0 = ptx::smem_desc_sw128(sbase + (is_s ? OFF_K : OFF_V), 16, 1024);
+      const uint32_t col0 = is_s ? 0u : COL_DP;
       for (int j = 0; ok; ++j) {
-        const int buf = j & 1;
-        ok = wait_on(bar(QD_FULL + buf), (uint32_t)(j >> 1) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[buf]) < 0) break;
-        // the warpgroup of this parity has read S / dP of step j-2
+        const int buf = j & 1, st = j % NST;
+        ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
+        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[st]) < 0) break;
+        // the P / dS warps have read S / dP of step j-2
         if (j >= 2) ok = wait_on(bar(PDS_FULL + buf), (uint32_t)((j >> 1) - 1) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint64_t qd = ptx::smem_desc_sw128(sbase + OFF_Q + buf * 2 * Q_BYTES, 16, 1024);
-        const uint64_t gd = ptx::smem_desc_sw128(sbase + OFF_Q + buf * 2 * Q_BYTES + Q_BYTES, 16, 1024);
-        if (is_s) {
+        const uint64_t ad0 = ptx::smem_desc_sw128(sbase + LY::OFF_ST + st * LY::STAGE + (is_s ? LY::AT_Q : LY::AT_G), 16, 1024);
 #pragma unroll
-          for (int k = 0; k < HD / 16; ++k) {
-            const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
-            const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
-            ptx::mma_bf16_ss(tmem + buf * NKV, qd + off_a, kd0 + off_b, IDESC_S, k > 0 ? 1u : 0u);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < HD / 16; ++k) {
-            const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
-            const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
-            ptx::mma_bf16_ss(tmem + COL_DP + buf * NKV, gd + off_a, vd0 + off_b, IDESC_S, k > 0 ? 1u : 0u);
-          }
+        for (int k = 0; k < HD / 16; ++k) {
+          const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
+          const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
+          ptx::mma_bf16_ss(tmem + col0 + buf * NKV, ad0 + off_a, bd0 + off_b, IDESC_S, k > 0 ? 1u : 0u);
         }
         ptx::mma_commit(bar(SD_FULL + buf));
       }
@@ -737,107 +822,112 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     if (lane == 0) {
       const bool is_v = warp == W_ACC;
       constexpr uint32_t IDESC_ACC = ptx::idesc_bf16_f32(128, NKV, true, true);     // A = (Q | dO)^T, B = (dS | P): both MN-major
-      const uint64_t pd0 = ptx::smem_desc_sw128(sbase + OFF_P, PS_BYTES, 1024);
-      const uint64_t sd0 = ptx::smem_desc_sw128(sbase + OFF_DS, PS_BYTES, 1024);
+      const uint64_t bd0 = ptx::smem_desc_sw128(sbase + (is_v ? LY::OFF_P : LY::OFF_DS), PS_BYTES, 1024);
+      const uint32_t d_tmem = tmem + (is_v ? COL_DV : COL_DK);
       bool ok = true;
       for (int j = 0; ok; ++j) {
-        const int buf = j & 1;
-        ok = wait_on(bar(QD_FULL + buf), (uint32_t)(j >> 1) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[buf]) < 0) break;
-        ok = wait_on(bar(PDS_FULL + buf), (uint32_t)(j >> 1) & 1u);
+        const int buf = j & 1, st = j % NST;
+        ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
+        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[st]) < 0) break;
+        ok = wait_on(bar((SEQ && !is_v ? DS_FULL : PDS_FULL) + buf), (uint32_t)(j >> 1) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
-        // (Q | dO) tile [row][d] read as MN-major A: M = d (two blocks of 64, Q_BYTES / 2 apart), K = rows (16 rows = 2048 B)
-        const uint64_t qmn = ptx::smem_desc_sw128(sbase + OFF_Q + buf * 2 * Q_BYTES, Q_BYTES / 2, 1024);
-        const uint64_t gmn = ptx::smem_desc_sw128(sbase + OFF_Q + buf * 2 * Q_BYTES + Q_BYTES, Q_BYTES / 2, 1024);
-        if (is_v) {
+        // tile [row][d] read as MN-major A: M = d (two blocks of 64), K = rows (16 rows = 2048 B); at head_dim 64 the two
+        // blocks are the dO and the Q tile
+        const uint64_t ad0 = ptx::smem_desc_sw128(sbase + LY::OFF_ST + st * LY::STAGE + (HD == 64 ? 0 : is_v ? LY::AT_G : LY::AT_Q),
+                                                  HD == 64 ? Q_BYTES : Q_BYTES / 2, 1024);
+#pragma unroll
+        for (int term = 0; term < (P2 ? 2 : 1); ++term)
 #pragma unroll
           for (int k = 0; k < 128 / 16; ++k) {
             const uint64_t adv = (uint64_t)((k * 16 * 128) >> 4);
-            ptx::mma_bf16_ss(tmem + COL_DV, gmn + adv, pd0 + adv, IDESC_ACC, (j > 0 || k > 0) ? 1u : 0u);
+            ptx::mma_bf16_ss(d_tmem, ad0 + adv, bd0 + adv + (uint64_t)((term * PS_BYTES) >> 4), IDESC_ACC,
+                             (j > 0 || k > 0 || term > 0) ? 1u : 0u);
           }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 128 / 16; ++k) {
-            const uint64_t adv = (uint64_t)((k * 16 * 128) >> 4);
-            ptx::mma_bf16_ss(tmem + COL_DK, qmn + adv, sd0 + adv, IDESC_ACC, (j > 0 || k > 0) ? 1u : 0u);
-          }
-        }
-        ptx::mma_commit(bar(ACC_DONE + buf));
+        ptx::mma_commit(SEQ && is_v ? bar(DV_DONE + buf) : bar(ACC_DONE + st));
       }
     }
     __syncwarp();
   }
   } else {
     // =========================== P, dS: thread = tile row, warpgroup = half of the keys; epilogue: thread = d ===========================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(256 - regs_service(WT)));
+    constexpr int SPH = CPS == 4 ? 2 : 1;                  // chunks in a half of the slice
     const int wg = warp >> 2;
     const int m = (warp & 3) * 32 + lane;
     const int t = m / g_q;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float c1 = dm.sm_scale * LOG2E;
     bool ok = true;
+    // row m of a [128 rows][64 keys] term: 128 bytes, 16-byte pieces swizzled with the row (128-byte swizzle); this
+    // warpgroup's keys are pieces 4 wg .. 4 wg + 3
+    auto store_row = [&](uint32_t off, const uint32_t (&v)[16]) {
+      uint8_t* row = smem + off + m * 128;
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch)
+        *reinterpret_cast<uint4*>(row + (((wg * 4 + ch) ^ (m & 7)) << 4)) = make_uint4(v[ch * 4], v[ch * 4 + 1], v[ch * 4 + 2], v[ch * 4 + 3]);
+    };
     for (int j = 0; ok; ++j) {
-      const int buf = j & 1;
+      const int buf = j & 1, st = j % NST;
       const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-      ok = wait_on(bar(QD_FULL + buf), ph);
+      ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
       if (!ok) break;
-      const int tile_idx = *reinterpret_cast<volatile int*>(&misc->tile[buf]);
+      const int tile_idx = *reinterpret_cast<volatile int*>(&misc->tile[st]);
       if (tile_idx < 0) break;
       const int i_row = tile_idx * TQ + t;
       const bool row_ok = i_row < dm.seq_q;
-      const float2 stat = row_ok ? misc->stats[buf][m] : make_float2(0.f, 0.f);
+      const float2 stat = row_ok ? misc->stats[st][m] : make_float2(0.f, 0.f);
       const float lse2 = stat.x, delta = stat.y;
-      const float bias = row_ok ? misc->bias[buf][t] : -INFINITY;
-      const float off = bias * LOG2E - lse2;
+      float off[SPH];
+#pragma unroll
+      for (int s = 0; s < SPH; ++s) off[s] = row_ok ? misc->bias[st][CPS == 1 ? 0 : wg * SPH + s][t] * LOG2E - lse2 : -INFINITY;
       const int n_vis = i_row - k0 + 1 - wg * 32;            // visible columns of this warpgroup's half
       ok = wait_on(bar(SD_FULL + buf), ph);
       if (!ok) break;
       ptx::tc_fence_after();
-      uint32_t pp[16], dd[16];                               // the row's 32 P and 32 dS values of this half as bf16 pairs
+      uint32_t p_hi[16], p_lo[16], d_hi[16], d_lo[16];       // the row's 32 P and 32 dS values of this half as bf16 pairs
       {
         uint32_t sv[32], gv[32];
         DASH_TMEM_LD32(sv, lane_addr + buf * NKV + wg * 32);
         DASH_TMEM_LD32(gv, lane_addr + COL_DP + buf * NKV + wg * 32);
         ptx::tmem_wait_ld();
+        float p[32], ds[32];
 #pragma unroll
-        for (int cc = 0; cc < 32; cc += 2) {
-          float p[2], ds[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const bool vis = cc + u < n_vis;
-            p[u] = vis ? exp2f(fmaf(__uint_as_float(sv[cc + u]), c1, off)) : 0.f;
-            ds[u] = p[u] * (__uint_as_float(gv[cc + u]) - delta);
-          }
-          __nv_bfloat162 hp = __floats2bfloat162_rn(p[0], p[1]);
-          __nv_bfloat162 hd = __floats2bfloat162_rn(ds[0], ds[1]);
-          pp[cc >> 1] = *reinterpret_cast<uint32_t*>(&hp);
-          dd[cc >> 1] = *reinterpret_cast<uint32_t*>(&hd);
+        for (int cc = 0; cc < 32; ++cc) {
+          p[cc] = cc < n_vis ? exp2f(fmaf(__uint_as_float(sv[cc]), c1, off[cc / (32 / SPH)])) : 0.f;
+          ds[cc] = p[cc] * (__uint_as_float(gv[cc]) - delta);
         }
+        pack_terms<P2>(p, p_hi, p_lo);
+        pack_terms<P2>(ds, d_hi, d_lo);
       }
       // the accumulating products of the step before have read P / dS
-      if (j >= 1) ok = wait_on(bar(ACC_DONE + (buf ^ 1)), (uint32_t)((j - 1) >> 1) & 1u);
+      if (j >= 1) ok = wait_on(bar(ACC_DONE + (j - 1) % NST), (uint32_t)((j - 1) / NST) & 1u);
       if (!ok) break;
-      // row m of the [128 rows][64 keys] tiles: 128 bytes, 16-byte pieces swizzled with the row (128-byte swizzle); this
-      // warpgroup's keys are pieces 4 wg .. 4 wg + 3
-      uint8_t* prow = smem + OFF_P + m * 128;
-      uint8_t* drow = smem + OFF_DS + m * 128;
-#pragma unroll
-      for (int ch = 0; ch < 4; ++ch) {
-        const int phys = ((wg * 4 + ch) ^ (m & 7)) << 4;
-        *reinterpret_cast<uint4*>(prow + phys) = make_uint4(pp[ch * 4], pp[ch * 4 + 1], pp[ch * 4 + 2], pp[ch * 4 + 3]);
-        *reinterpret_cast<uint4*>(drow + phys) = make_uint4(dd[ch * 4], dd[ch * 4 + 1], dd[ch * 4 + 2], dd[ch * 4 + 3]);
+      store_row(LY::OFF_P, p_hi);
+      if constexpr (P2) store_row(LY::OFF_P + PS_BYTES, p_lo);
+      if constexpr (!SEQ) {
+        store_row(LY::OFF_DS, d_hi);
+        if constexpr (P2) store_row(LY::OFF_DS + PS_BYTES, d_lo);
       }
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(PDS_FULL + buf));
+      if constexpr (SEQ) {
+        ok = wait_on(bar(DV_DONE + buf), ph);
+        if (!ok) break;
+        store_row(LY::OFF_DS, d_hi);
+        store_row(LY::OFF_DS + PS_BYTES, d_lo);
+        ptx::fence_proxy_async_smem();
+        ptx::mbar_arrive(bar(DS_FULL + buf));
+      }
     }
     // epilogue: dV^T, dK^T [d = TMEM lane][key = column] -> dV, dK [batch][key][KV head][d]; one warpgroup each
     const int n_done = ok ? *reinterpret_cast<volatile int*>(&misc->total) : 0;
-    if (ok && n_done > 0) ok = wait_on(bar(ACC_DONE + ((n_done - 1) & 1)), (uint32_t)((n_done - 1) >> 1) & 1u);
-    if (ok) {
+    if (ok && n_done > 0) ok = wait_on(bar(ACC_DONE + (n_done - 1) % NST), (uint32_t)((n_done - 1) / NST) & 1u);
+    const bool mine = HD == 128 || (wg == 0 ? m < 64 : m >= 64);      // (whole warps)
+    if (ok && mine && (n_done > 0 || a.n_split == 1)) {
       ptx::tc_fence_after();
-      const int d = m;
+      const int d = HD == 128 ? m : m & 63;
       float* out = wg == 0 ? a.dV : a.dK;
       const float mul = wg == 0 ? 1.f : dm.sm_scale;
 #pragma unroll 1
@@ -853,8 +943,10 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
         for (int cc = 0; cc < 32; ++cc) {
           const int key = k0 + half * 32 + cc;
-          if (key < dm.seq_kv)
-            out[(((long long)b * dm.seq_kv + key) * dm.h_kv + r) * HD + d] = __uint_as_float(v[cc]) * mul;
+          if (key < dm.seq_kv) {
+            float* o = out + (((long long)b * dm.seq_kv + key) * dm.h_kv + r) * HD + d;
+            if (a.n_split > 1) atomicAdd(o, __uint_as_float(v[cc]) * mul); else *o = __uint_as_float(v[cc]) * mul;
+          }
         }
       }
     }
@@ -871,85 +963,113 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 
 }  // namespace dkv
 
-// [batch, tokens, heads, 128] bf16 tensor with element strides s[3]; box = 64 x box_heads x box_tokens x 1.
-bool make_map(CUtensorMap* out, const void* base, long long tokens, int heads, int batch, const long long* s,
+// [batch, tokens, heads, hd] bf16 tensor with element strides s[3]; box = 64 x box_heads x box_tokens x 1.
+bool make_map(CUtensorMap* out, const void* base, int hd, long long tokens, int heads, int batch, const long long* s,
               int box_heads, int box_tokens) {
-  cuuint64_t dims[4] = {(cuuint64_t)HD, (cuuint64_t)heads, (cuuint64_t)tokens, (cuuint64_t)batch};
+  cuuint64_t dims[4] = {(cuuint64_t)hd, (cuuint64_t)heads, (cuuint64_t)tokens, (cuuint64_t)batch};
   auto st = [](long long e) { return (cuuint64_t)((e > 0 ? e : 8) * 2); };
   cuuint64_t strides[3] = {st(s[2]), st(s[1]), st(s[0])};
   cuuint32_t box[4] = {64u, (cuuint32_t)box_heads, (cuuint32_t)box_tokens, 1u};
   return encode_bf16_sw128_4d(out, base, dims, strides, box);
 }
 
+struct Maps {
+  CUtensorMap q, g, k, v, kc, vc;      // kc, vc: one chunk per box (the dQ kernel packs chunks below 64 tokens)
+};
+
+// dK / dV, then dQ / dbias (which overwrites what the first one reads: see the top of the file)
+template <int HD, int CPS, int WT, bool P2>
+cudaError_t launch_kernels(const BwdArgs& a, const Maps& m, cudaStream_t st) {
+  const long long groups = (long long)a.dm.batch * a.dm.h_kv;
+  constexpr int MTQ = 32 * (WT > 0 ? WT : 2);
+  cudaError_t e;
+  {
+    auto kern = dkv::attend_bwd_dkv_kernel<HD, CPS, WT, P2>;
+    constexpr uint32_t smem = dkv::Layout<HD, CPS, MTQ, P2>::SMEM;
+    static std::atomic<unsigned long long> configured{0};
+    if ((e = allow_dynamic_smem(kern, smem, configured)) != cudaSuccess) return e;
+    e = launch_chained(kern, dim3((unsigned)(a.n_slices * groups), a.n_split), dim3(dkv::THREADS), smem, st, m.q, m.g, m.k, m.v, a);
+    count_launch();
+    if (e != cudaSuccess) return e;
+  }
+  const size_t list_bytes = (size_t)groups * (size_t)a.dm.list_rows * sizeof(float);
+  if (list_bytes > 0 && (e = cudaMemsetAsync(a.dbias, 0, list_bytes, st)) != cudaSuccess) return e;
+  auto kern = dq::attend_bwd_dq_kernel<HD, CPS, WT, P2>;
+  constexpr uint32_t smem = dq::Layout<HD, CPS, MTQ>::SMEM;
+  static std::atomic<unsigned long long> configured{0};
+  if ((e = allow_dynamic_smem(kern, smem, configured)) != cudaSuccess) return e;
+  e = launch_chained(kern, dim3((unsigned)(a.n_tiles * groups)), dim3(dq::THREADS), smem, st, m.q, m.g, m.kc, m.vc, a);
+  count_launch();
+  return e;
+}
+
+template <int HD, int CPS>
+cudaError_t launch_two_term(const BwdArgs& a, const Maps& m, cudaStream_t st) {
+  if (a.dm.g_q == 1) return launch_kernels<HD, CPS, 4, true>(a, m, st);
+  if constexpr (CPS > 1) {
+    if (a.TQ > a.dm.B) return launch_kernels<HD, CPS, 2, true>(a, m, st);
+  }
+  return launch_kernels<HD, CPS, 0, true>(a, m, st);
+}
+
 }  // namespace
 
 bool prefill_bwd_sm100_supported(const Dims& dm) {
-  if (!prefill_sm100_supported(dm) || dm.g_q < 2) return false;
-  if (dm.d != 128 || (dm.B != 64 && dm.B != 128)) return false;
-  if (dm.qs[2] % 8 != 0 || dm.qs[1] % 8 != 0) return false;     // 16-byte stores of dQ rows
-  return true;
+  if (!prefill_sm100_supported(dm)) return false;
+  return dm.qs[2] % 8 == 0 && dm.qs[1] % 8 == 0;      // 16-byte stores of dQ rows
 }
 
-cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, const void* Q, const void* K, const void* V, const void* dO,
-                                            const uint32_t* mask, const float* blk_bias, float2* stats, int* prefix,
-                                             void* dQ, float* dK, float* dV, float* dbias, StatusBlock* sb,
-                                            cudaStream_t st) {
-  // 1. forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written), tile-major
-  const long long tile_rows = (long long)((dm.seq_q + 128 / dm.g_q - 1) / (128 / dm.g_q)) * 128;
-  RowStats rs;
-  rs.base = reinterpret_cast<char*>(stats);
-  rs.sh = sizeof(float2);
-  rs.si = rs.sh * dm.g_q;
-  rs.sr = rs.sh * tile_rows;
-  rs.sb = rs.sr * dm.h_kv;
-  cudaError_t e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, rs, dO);
-  if (e != cudaSuccess) return e;
-  // 2. routed-chunk counts before every mask word
-  const long long rows = (long long)dm.batch * dm.h_kv * dm.seq_q;
-  e = launch_chained(mask_prefix_kernel, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, dm, mask, prefix);
-  count_launch();
-  if (e != cudaSuccess) return e;
-
+cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n_sm, const void* Q, const void* K, const void* V,
+                                            const void* dO, const uint32_t* mask, const float* blk_bias, void* dQ, float* dK,
+                                            float* dV, float* dbias, StatusBlock* sb, cudaStream_t st) {
   BwdArgs a;
   a.dm = dm;
   a.TQ = 128 / dm.g_q;
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
   a.n_slices = (dm.seq_kv + NKV - 1) / NKV;
   a.wait_limit = test_hooks().wait_limit_cycles;
-  a.mask = mask; a.blk_bias = blk_bias; a.stats = stats; a.prefix = prefix;
-  // the tile unions sit behind the prefix counts in the same scratch region
-  uint32_t* tile_union = reinterpret_cast<uint32_t*>(prefix + rows * dm.W);
-  a.tile_union = tile_union;
-  {
-    const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
-    e = launch_chained(tile_union_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
-                       mask, tile_union);
-    count_launch();
-    if (e != cudaSuccess) return e;
-  }
+  a.mask = mask; a.blk_bias = blk_bias; a.marks = reinterpret_cast<int*>(dbias);
   a.dQ = (__nv_bfloat16*)dQ; a.dK = dK; a.dV = dV; a.dbias = dbias; a.sb = sb;
-  CUtensorMap tq, tg, tk, tv;
-  if (!make_map(&tq, Q, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
-  if (!make_map(&tg, dO, dm.seq_q, dm.h_q, dm.batch, dm.os, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
-  if (!make_map(&tk, K, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, NKV)) return cudaErrorInvalidValue;
-  if (!make_map(&tv, V, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, NKV)) return cudaErrorInvalidValue;
-  const int groups = dm.batch * dm.h_kv;
-  {
-    static std::atomic<unsigned long long> configured{0};
-    if ((e = allow_dynamic_smem(dq::attend_bwd_dq_kernel, dq::SMEM, configured)) != cudaSuccess) return e;
-    e = launch_chained(dq::attend_bwd_dq_kernel, dim3((unsigned)((long long)a.n_tiles * groups)), dim3(dq::THREADS),
-                       dq::SMEM, st, tq, tg, tk, tv, a);
-    count_launch();
-    if (e != cudaSuccess) return e;
+  // a row's statistics at the start of its dQ row
+  a.stats.base = reinterpret_cast<char*>(dQ);
+  a.stats.sb = dm.qs[0] * 2; a.stats.si = dm.qs[1] * 2; a.stats.sh = dm.qs[2] * 2; a.stats.sr = a.stats.sh * dm.g_q;
+  // A slice's walk is a chain of one tile after another (one block per SM).  Where the slices alone leave SMs idle, several
+  // blocks share a slice's tiles and add their sums with atomics; with one bf16 term dK and dV keep one owner per element.
+  a.n_split = 1;
+  cudaError_t e = cudaSuccess;
+  if (two_term) {
+    const long long blocks = (long long)a.n_slices * dm.batch * dm.h_kv;
+    a.n_split = (int)std::max<long long>(1, std::min<long long>({2 * n_sm / blocks, a.n_tiles / 4, 16}));
+    if (a.n_split > 1) {
+      const size_t kv_bytes = (size_t)dm.batch * dm.seq_kv * dm.h_kv * dm.d * sizeof(float);
+      if ((e = cudaMemsetAsync(dK, 0, kv_bytes, st)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(dV, 0, kv_bytes, st)) != cudaSuccess) return e;
+    }
   }
-  {
-    static std::atomic<unsigned long long> configured{0};
-    if ((e = allow_dynamic_smem(dkv::attend_bwd_dkv_kernel, dkv::SMEM, configured)) != cudaSuccess) return e;
-    e = launch_chained(dkv::attend_bwd_dkv_kernel, dim3((unsigned)((long long)a.n_slices * groups)), dim3(dkv::THREADS),
-                       dkv::SMEM, st, tq, tg, tk, tv, a);
-    count_launch();
+  // forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written)
+  e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, a.stats, dO);
+  if (e != cudaSuccess) return e;
+  const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
+  e = launch_chained(list_marks_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
+                     mask, a.marks);
+  count_launch();
+  if (e != cudaSuccess) return e;
+
+  Maps m;
+  const int box_kv = dm.B < NKV ? dm.B : NKV;
+  if (!make_map(&m.q, Q, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
+  if (!make_map(&m.g, dO, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.os, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
+  if (!make_map(&m.k, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, NKV)) return cudaErrorInvalidValue;
+  if (!make_map(&m.v, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, NKV)) return cudaErrorInvalidValue;
+  if (!make_map(&m.kc, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, box_kv)) return cudaErrorInvalidValue;
+  if (!make_map(&m.vc, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, box_kv)) return cudaErrorInvalidValue;
+  if (!two_term) {
+    if (dm.d != 128 || dm.B < NKV || dm.g_q < 2) return cudaErrorInvalidValue;
+    return launch_kernels<128, 1, 0, false>(a, m, st);
   }
-  return e;
+  if (dm.d == 128)
+    return dm.B >= NKV ? launch_two_term<128, 1>(a, m, st) : dm.B == 32 ? launch_two_term<128, 2>(a, m, st) : launch_two_term<128, 4>(a, m, st);
+  return dm.B >= NKV ? launch_two_term<64, 1>(a, m, st) : dm.B == 32 ? launch_two_term<64, 2>(a, m, st) : launch_two_term<64, 4>(a, m, st);
 }
 
 }  // namespace dash

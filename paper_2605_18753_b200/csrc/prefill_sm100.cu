@@ -139,7 +139,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   const int b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int TQ = a.TQ, g_q = dm.g_q;
   const int i0 = tile * TQ;
-  const int c_own = i0 / dm.B;                        // own chunk of the tile's first token (WIDE: of that one only)
+  const int c_own = i0 >> dm.log_b;                        // own chunk of the tile's first token (WIDE: of that one only)
   const int sub_per_blk = dm.B / NKV;                 // 64-token steps per chunk (1 or 2)
   const int own_steps = WIDE ? (TQ + NKV - 1) / NKV   // steps over the tile's own tokens
                              : (i0 % dm.B) / NKV + 1; // steps of the own chunk the tile can see
@@ -208,7 +208,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
         for (int t = lane; t < TQ; t += 32)
 #pragma unroll
           for (int s = 0; s < CPS; ++s)
-            misc->bias[sub][s][t] = (WIDE ? (kv0 + s * W) / dm.B == (i0 + t) / dm.B : s == 0) ? 0.f : -INFINITY;
+            misc->bias[sub][s][t] = (WIDE ? (kv0 + s * W) >> dm.log_b == (i0 + t) >> dm.log_b : s == 0) ? 0.f : -INFINITY;
 #pragma unroll
         for (int s = 0; s < CPS; ++s)
           if (lane == s) misc->kvbase[sub][s] = kvs[s];

@@ -29,11 +29,11 @@ struct TileWalk {
     lane = lane_;
     rows = mask + (row0 + i0) * dm.W;
     n_live = min(TQ, dm.seq_q - i0);
-    c_first = i0 / dm.B;
-    n_words = ((WIDE ? (i0 + n_live - 1) / dm.B : c_first) >> 5) + 1;
+    c_first = i0 >> dm.log_b;
+    n_words = ((WIDE ? (i0 + n_live - 1) >> dm.log_b : c_first) >> 5) + 1;
     if constexpr (WIDE) {
 #pragma unroll
-      for (int q = 0; q < TPL; ++q) co[q] = (i0 + lane + 32 * q) / dm.B;
+      for (int q = 0; q < TPL; ++q) co[q] = (i0 + lane + 32 * q) >> dm.log_b;
     }
   }
   // Number of chunks in the union.  Four mask words per sweep: a lane's loads are in flight together (one L2 round trip
