@@ -7,6 +7,7 @@
 // keys for the logits and head_dim slices for the output.  Every warp's state is merged in shared
 // memory, every block writes one partial (m, l, O) per head, and a second kernel merges the partials in
 // split order, so results do not depend on scheduling.  Only the selected chunks' K and V rows are read.
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -21,10 +22,6 @@ static bool decode_use_sm100(const Dims& dm) {
   return need > 0 && need <= DEC_MAX_SPLITS;
 }
 
-// Split count: thread blocks are handed out in waves of one per SM (the tensor-core kernel fills an SM's
-// shared memory), so the time is about ceil(groups * s / SMs) waves of (1/s of a group's work + a fixed cost per
-// block, about 2 % of a long group's work: list staging, first loads, partial write).  At 128 groups on 148 SMs
-// s = 5 leaves a fifth wave a third full, s = 8 fills seven waves almost exactly (measured: 0.155 vs 0.150 ms).
 // SM count of the current device, cached per device (a process may drive several GPUs).
 int current_sm_count() {
   static std::atomic<int> cached[64];
@@ -38,17 +35,38 @@ int current_sm_count() {
   return n;
 }
 
-int decode_num_splits(const Dims& dm) {
-  const int n_sm = current_sm_count();
-  const int groups = dm.batch * dm.h_kv;
-  int lo = 1;
-  if (decode_use_sm100(dm)) lo = max(lo, decode_sm100_min_splits(dm));   // a block owns at most 512 sub-blocks there
-  const int hi = max(lo, min(DEC_MAX_SPLITS, 16));
+// Split count of the CUDA-core kernel: waves of one block per SM, each ceil(groups * s / SMs) long (1 / s of a group's
+// work plus a fixed cost per block, about 2 % of a long group's work).
+static int splits_cuda_cores(const Dims& dm) {
+  const int n_sm = current_sm_count(), groups = dm.batch * dm.h_kv;
+  const int lo = decode_use_sm100(dm) ? decode_sm100_min_splits(dm) : 1, hi = max(lo, 16);
   int best = lo;
   double best_cost = 1e30;
   for (int s = lo; s <= hi; ++s) {
     const long long waves = ((long long)groups * s + n_sm - 1) / n_sm;
     const double cost = (double)waves * (1.0 / s + 0.02);
+    if (cost < best_cost - 1e-12) { best_cost = cost; best = s; }
+  }
+  return best;
+}
+
+// Split count of the tensor-core kernel (two blocks per SM).  In units of a group's whole work: a block takes 1 / s plus a
+// fixed cost f (list staging, first loads, partial results, about twelve 64-token sub-blocks' worth of a group that
+// selects the usual part of its cache), the merge 0.2 f per split.  Blocks that all fit at once end with the slowest group
+// (x 1.3: the groups' lists differ in length); more of them keep the SMs full until the last 0.8 block.  The constants
+// are a fit to thirteen shapes (8 to 384 groups, caches of 1408 to 131072 tokens) timed at 1 to 32 splits: the choice is
+// within 2.6 % of each shape's best on average (16 x 131072 tokens, 8 KV heads: 169 us at 11; one cache of 42405: 29 us at
+// 16, the former limit, 25 at 32).
+int decode_num_splits(const Dims& dm) {
+  if (!decode_use_sm100(dm)) return splits_cuda_cores(dm);
+  const double resident = 2.0 * current_sm_count(), groups = (double)dm.batch * dm.h_kv;
+  const double f = std::min(0.1, std::max(0.01, 12.0 * 64.0 / dm.seq_kv));
+  const int lo = decode_sm100_min_splits(dm);     // a block owns at most 512 sub-blocks
+  int best = lo;
+  double best_cost = 1e30;
+  for (int s = lo; s <= DEC_MAX_SPLITS; ++s) {
+    const double waves = groups * s / resident;
+    const double cost = (1.0 / s + f) * (waves <= 1.0 ? 1.3 : waves + 0.8) + 0.2 * f * s;
     if (cost < best_cost - 1e-12) { best_cost = cost; best = s; }
   }
   return best;
@@ -234,7 +252,7 @@ template <typename T, int D>
 static cudaError_t launch_dec(const Dims& dm, const void* Q, const void* K, const void* V, const int* kv_len,
                               const int* count, const int* blk_idx, const float* blk_bias, void* O,
                               float* partials, StatusBlock* sb, cudaStream_t st) {
-  const int ns = decode_num_splits(dm);
+  const int ns = splits_cuda_cores(dm);
   dim3 grid(ns, dm.h_kv, dm.batch);
   cudaError_t e = cudaSuccess;
 #define DASH_DEC(G)                                                                                              \
@@ -340,7 +358,7 @@ extern "C" int dash_attn_attend_decode_static(const dash_params* p, const void* 
   if (dm.T_s > 0 && (!blk_idx || !blk_bias)) return DASH_ERR_INVALID_ARG;
   const uintptr_t bits = (uintptr_t)Q | (uintptr_t)Kcache | (uintptr_t)Vcache | (uintptr_t)O;
   if (bits & 15) return DASH_ERR_INVALID_ARG;
-  if (decode_partial_bytes(dm) > DECODE_STATIC_MAX_FLOATS * sizeof(float)) return DASH_ERR_TOO_LARGE;
+  if ((size_t)dm.batch * dm.h_q * splits_cuda_cores(dm) * (dm.d + 2) > DECODE_STATIC_MAX_FLOATS) return DASH_ERR_TOO_LARGE;
   if ((rc = validate_device()) != DASH_OK) return rc;
   float* scratch = nullptr;
   if (decode_static_scratch(&scratch) != cudaSuccess) return DASH_ERR_CUDA;

@@ -1,8 +1,9 @@
 // Stage 2, decode, on TMA + tcgen05 for sm_100a (Eq. 7 / Proposition 1; Algorithm 3; split-KV of Section 3.5).
 //
 // HBM-bound: per (batch, KV head) only the routed chunks' K and V rows are read, once, by bulk tensor
-// copies into a 3-deep shared-memory ring (64 KiB per step = 128 KV tokens), so enough bytes are in flight
-// to cover DRAM latency without occupying threads.  The arithmetic is tiny (g_q <= 16 query rows per KV
+// copies into a shared-memory ring of three 32 KiB tiles (K and V of a step of 128 KV tokens in turn), two blocks per SM,
+// so enough bytes are in flight to cover DRAM latency without occupying threads, and one block's set-up and partial
+// results pass under the other one's stream.  The arithmetic is tiny (g_q <= 16 query rows per KV
 // head) and rides on the tensor cores in "transposed" form so that the KV tokens fill the MMA's M:
 //     S^T[128 keys x 16 heads] = K_tile[128 x d] * Q^T[d x 16]          (heads padded to N = 16)
 //     O^T[d = 128 x 16 heads] += V_tile^T[128 x 128 keys] * P^T[128 keys x 16]
@@ -25,21 +26,19 @@ namespace {
 constexpr int HD_MAX = 128;             // the shared-memory layout is the one of head_dim 128 (head_dim 64 fills half a tile)
 constexpr int SUB = 64;                 // KV tokens per sub-block (one TMA box pair)
 constexpr int STEP = 128;               // KV tokens per step = MMA M
-constexpr int NST = 3;                  // K/V ring depth
+constexpr int NSL = 3;                  // ring of K and V tiles: tile 2j = K of step j, 2j + 1 = its V
 constexpr int NH = 16;                  // heads padded to the MMA N
 constexpr int DEC_THREADS = 192;
 constexpr int MAX_RANGE = 512;          // sub-blocks one thread block can own
 constexpr uint32_t TILE_BYTES = STEP * HD_MAX * 2;   // 32 KiB: two regions (d halves) of 128 rows x 128 B
 constexpr uint32_t QT_BYTES = NH * HD_MAX * 2;       // 4 KiB: two regions of 16 rows x 128 B
 constexpr uint32_t PT_BYTES = NH * STEP * 2;     // 4 KiB: two regions (key halves) of 16 rows x 128 B
-constexpr uint32_t OFF_K = 0;
-constexpr uint32_t OFF_V = OFF_K + NST * TILE_BYTES;
-constexpr uint32_t OFF_QT = OFF_V + NST * TILE_BYTES;
+constexpr uint32_t OFF_KV = 0;
+constexpr uint32_t OFF_QT = OFF_KV + NSL * TILE_BYTES;
 constexpr uint32_t OFF_PT = OFF_QT + QT_BYTES;
 constexpr uint32_t OFF_MISC = OFF_PT + PT_BYTES;
 constexpr uint32_t TMEM_COLS = 64;      // S^T buffers at columns 0 and 16, O^T at 32
-enum BarD { Q_READY = 0, S_FULL = 1, P_FULL = 3, P_EMPTY = 5, RED_BAR = 6, LRED_BAR = 8, K_FULL = 9, K_EMPTY = 9 + NST,
-            V_FULL = 9 + 2 * NST, V_EMPTY = 9 + 3 * NST, N_BARS = 9 + 4 * NST };
+enum BarD { Q_READY = 0, S_FULL = 1, P_FULL = 3, P_EMPTY = 5, RED_BAR = 6, LRED_BAR = 8, FULL = 9, EMPTY = 9 + NSL, N_BARS = 9 + 2 * NSL };
 // CPS = routed chunks per 64-token sub-block: 1 for chunks of 64 / 128 tokens, 2 / 4 for chunks of 32 / 16 (a
 // sub-block then gathers that many chunks of the list, each fetched by its own TMA box and carrying its own bias).
 template <int CPS>
@@ -48,21 +47,21 @@ struct MiscT {
   unsigned long long bar[N_BARS];
   uint32_t tmem_base;
   int abort_flag;
-  float bias2[NST][2][CPS];
-  int nvalid[NST][2];
+  float bias2[NSL][2][CPS];   // of the step whose V tile is in the slot
+  int nvalid[NSL][2];
   float red[2][4][NH];
   float lred[4][NH];
   int is_last;               // this block saw the last arrival of its (batch, KV head)
   int idx_s[RANGE][CPS];     // first KV token of each chunk slot of each owned sub-block (paged cache: inside its page)
   int pg_s[RANGE][CPS];      // outermost TMA coordinate of the slot: the sequence, or the physical page
   float bias_s[RANGE][CPS];
-  int nval_s[RANGE];         // valid rows of the sub-block
+  unsigned short nval_s[RANGE];   // valid rows of the sub-block
 };
 constexpr size_t MISC_BYTES = sizeof(MiscT<1>) > sizeof(MiscT<2>)
                                   ? (sizeof(MiscT<1>) > sizeof(MiscT<4>) ? sizeof(MiscT<1>) : sizeof(MiscT<4>))
                                   : (sizeof(MiscT<2>) > sizeof(MiscT<4>) ? sizeof(MiscT<2>) : sizeof(MiscT<4>));
 constexpr uint32_t DEC_SMEM = OFF_MISC + (uint32_t)MISC_BYTES;   // one size for every instantiation
-static_assert(DEC_SMEM <= 232448, "shared memory budget");
+static_assert(DEC_SMEM <= 115712, "two blocks per SM");
 
 struct DecodeArgs {
   Dims dm;
@@ -97,7 +96,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t* r) {
 // (N = 32): rows 0-63 / columns 0-15 hold V_a^T P_a^T and rows 64-127 / columns 16-31 hold V_b^T P_b^T (the other two
 // quadrants are not used); the two are added when the partial is written.
 template <int G, int CPS, int HD>
-__global__ void __launch_bounds__(DEC_THREADS, 1)
+__global__ void __launch_bounds__(DEC_THREADS, 2)
 decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a) {
   using MiscD = MiscT<CPS>;
   constexpr int W = SUB / CPS;          // rows of one chunk slot inside a sub-block
@@ -126,11 +125,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::mbar_init(bar(RED_BAR), 128);
     ptx::mbar_init(bar(RED_BAR + 1), 128);
     ptx::mbar_init(bar(LRED_BAR), 128);
-    for (int s = 0; s < NST; ++s) {
-      ptx::mbar_init(bar(K_FULL + s), 1);
-      ptx::mbar_init(bar(K_EMPTY + s), 1);
-      ptx::mbar_init(bar(V_FULL + s), 1);
-      ptx::mbar_init(bar(V_EMPTY + s), 1);
+    for (int s = 0; s < NSL; ++s) {
+      ptx::mbar_init(bar(FULL + s), 1);
+      ptx::mbar_init(bar(EMPTY + s), 1);
     }
     ptx::fence_barrier_init();
   }
@@ -184,7 +181,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             DASH_CHECK(!dm.page_table || (unsigned)misc->pg_s[k][s] < (unsigned)dm.num_pages, a.sb, 313, misc->pg_s[k][s] = 0);
             misc->bias_s[k][s] = a.blk_bias[loff + e];
           }
-          misc->nval_s[k] = m * dm.B;
+          misc->nval_s[k] = (unsigned short)(m * dm.B);
         } else {
           // the own chunk (shorter than a sub-block): the rows behind it are fetched but marked invalid
 #pragma unroll
@@ -193,7 +190,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             DASH_CHECK(!dm.page_table || (unsigned)misc->pg_s[k][s] < (unsigned)dm.num_pages, a.sb, 315, misc->pg_s[k][s] = 0);
             misc->bias_s[k][s] = 0.f;
           }
-          misc->nval_s[k] = L - c_own * dm.B;
+          misc->nval_s[k] = (unsigned short)(L - c_own * dm.B);
         }
         continue;
       }
@@ -214,7 +211,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
       kv_locate(dm, b, tok0, &misc->pg_s[k][0], &misc->idx_s[k][0]);
       DASH_CHECK(!dm.page_table || (unsigned)misc->pg_s[k][0] < (unsigned)dm.num_pages, a.sb, 314, misc->pg_s[k][0] = 0);
-      misc->bias_s[k][0] = bs; misc->nval_s[k] = nv;
+      misc->bias_s[k][0] = bs; misc->nval_s[k] = (unsigned short)nv;
     }
     __syncwarp();
     if (lane == 0) {
@@ -239,10 +236,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
           }
         };
-        ok = ptx::mbar_wait(bar(K_EMPTY + s), ph, abort_flag);
+        auto advance = [&]() { if (++s == NSL) { s = 0; ph ^= 1; } };
+        ok = ptx::mbar_wait(bar(EMPTY + s), ph, abort_flag);
         if (!ok) break;
-        load_tile(&tmK, sbase + OFF_K + s * TILE_BYTES, bar(K_FULL + s));
-        ok = ptx::mbar_wait(bar(V_EMPTY + s), ph, abort_flag);
+        load_tile(&tmK, sbase + OFF_KV + s * TILE_BYTES, bar(FULL + s));
+        advance();
+        ok = ptx::mbar_wait(bar(EMPTY + s), ph, abort_flag);
         if (!ok) break;
 #pragma unroll
         for (int q = 0; q < CPS; ++q) {
@@ -251,14 +250,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         }
         misc->nvalid[s][0] = misc->nval_s[k0];
         misc->nvalid[s][1] = (k1 != k0) ? misc->nval_s[k1] : 0;
-        load_tile(&tmV, sbase + OFF_V + s * TILE_BYTES, bar(V_FULL + s));
-        if (++s == NST) { s = 0; ph ^= 1; }
+        load_tile(&tmV, sbase + OFF_KV + s * TILE_BYTES, bar(FULL + s));
+        advance();
       }
       if (!ok) {
-        for (int q = 0; q < NST; ++q) {
-          for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(K_FULL + q), 0) && !ptx::mbar_try_wait(bar(K_FULL + q), 1); ++k) {}
-          for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(V_FULL + q), 0) && !ptx::mbar_try_wait(bar(V_FULL + q), 1); ++k) {}
-        }
+        for (int q = 0; q < NSL; ++q)
+          for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(FULL + q), 0) && !ptx::mbar_try_wait(bar(FULL + q), 1); ++k) {}
       }
     }
   } else if (warp == 5) {
@@ -266,16 +263,18 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (lane == 0 && n_steps > 0) {
       constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NH, false, false);
       constexpr uint32_t IDESC_O = ptx::idesc_bf16_f32(128, HD == 128 ? NH : 2 * NH, true, false);
-      const uint64_t kd0 = ptx::smem_desc_sw128(sbase + OFF_K, 16, 1024);
+      const uint64_t kd0 = ptx::smem_desc_sw128(sbase + OFF_KV, 16, 1024);
       const uint64_t qd0 = ptx::smem_desc_sw128(sbase + OFF_QT, 16, 1024);
       // MN-major A: the two MN blocks of 64 are the d halves, 16 KiB apart (head_dim 128), or the two 64-key
       // sub-blocks of the step, 8 KiB apart (head_dim 64)
-      const uint64_t vd0 = ptx::smem_desc_sw128(sbase + OFF_V, HD == 128 ? TILE_BYTES / 2 : SUB * 128, 1024);
+      const uint64_t vd0 = ptx::smem_desc_sw128(sbase + OFF_KV, HD == 128 ? TILE_BYTES / 2 : SUB * 128, 1024);
       const uint64_t pd0 = ptx::smem_desc_sw128(sbase + OFF_PT, 16, 1024);
       bool ok = ptx::mbar_wait(bar(Q_READY), 0, abort_flag);
-      int ks = 0, kph = 0;
+      // tile 2j (K) and 2j + 1 (V) of the ring
+      int ks = 0, kph = 0, vs = 1, vph = 0;
+      auto next_step = [](int& slot, int& phase) { slot += 2; if (slot >= NSL) { slot -= NSL; phase ^= 1; } };
       auto issue_s = [&](int j) -> bool {
-        if (!ptx::mbar_wait(bar(K_FULL + ks), kph, abort_flag)) return false;
+        if (!ptx::mbar_wait(bar(FULL + ks), kph, abort_flag)) return false;
         ptx::tc_fence_after();
         const uint64_t kd = kd0 + (uint64_t)((ks * TILE_BYTES) >> 4);
 #pragma unroll
@@ -285,16 +284,15 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           ptx::mma_bf16_ss(tmem + (j & 1) * NH, ad, bd, IDESC_S, k > 0 ? 1u : 0u);
         }
         ptx::mma_commit(bar(S_FULL + (j & 1)));
-        ptx::mma_commit(bar(K_EMPTY + ks));
-        if (++ks == NST) { ks = 0; kph ^= 1; }
+        ptx::mma_commit(bar(EMPTY + ks));
+        next_step(ks, kph);
         return true;
       };
       if (ok) ok = issue_s(0);
-      int vs = 0, vph = 0;
       for (int j = 0; j < n_steps && ok; ++j) {
         if (j + 1 < n_steps) ok = issue_s(j + 1);
         if (!ok) break;
-        ok = ptx::mbar_wait(bar(V_FULL + vs), vph, abort_flag) && ptx::mbar_wait(bar(P_FULL + (j & 1)), (j >> 1) & 1, abort_flag);
+        ok = ptx::mbar_wait(bar(FULL + vs), vph, abort_flag) && ptx::mbar_wait(bar(P_FULL + (j & 1)), (j >> 1) & 1, abort_flag);
         if (!ok) break;
         ptx::tc_fence_after();
         const uint64_t vd = vd0 + (uint64_t)((vs * TILE_BYTES) >> 4);
@@ -306,9 +304,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           const uint64_t bd = pd0 + (uint64_t)(((HD == 128 ? (k >> 2) * (PT_BYTES / 2) : 0) + (k & 3) * 32) >> 4);
           ptx::mma_bf16_ss(tmem + 2 * NH, ad, bd, IDESC_O, (j > 0 || k > 0) ? 1u : 0u);
         }
-        ptx::mma_commit(bar(V_EMPTY + vs));
+        ptx::mma_commit(bar(EMPTY + vs));
         ptx::mma_commit(bar(P_EMPTY));
-        if (++vs == NST) { vs = 0; vph ^= 1; }
+        next_step(vs, vph);
       }
     }
     __syncwarp();
@@ -334,9 +332,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     for (int h = 0; h < G; ++h) { m[h] = -INFINITY; l[h] = 0.f; }
     const int half = tid >> 6, row = tid & 63;
     bool ok = true;
-    int vs = 0, vph = 0;
+    int vs = 1, vph = 0;
     for (int j = 0; j < n_steps && ok; ++j) {
-      ok = ptx::mbar_wait(bar(V_FULL + vs), vph, abort_flag);     // step metadata visible, V tile landed
+      ok = ptx::mbar_wait(bar(FULL + vs), vph, abort_flag);     // step metadata visible, V tile landed
       if (!ok) break;
       const float b2 = misc->bias2[vs][half][CPS > 1 ? row / W : 0] * 1.4426950408889634f;
       const int nval = misc->nvalid[vs][half];
@@ -399,7 +397,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
       // rows past the end of the sequence may hold anything (even NaN): zero their V rows, since 0 * NaN = NaN
       if (!valid && nval > 0 && nval < SUB) {
-        uint8_t* vrow = smem + OFF_V + vs * TILE_BYTES + tid * 128;
+        uint8_t* vrow = smem + OFF_KV + vs * TILE_BYTES + tid * 128;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           *reinterpret_cast<uint4*>(vrow + (q << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -409,7 +407,8 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(P_FULL + (j & 1)));
-      if (++vs == NST) { vs = 0; vph ^= 1; }
+      vs += 2;
+      if (vs >= NSL) { vs -= NSL; vph ^= 1; }
     }
 
     // ---------------- partial (m, l, O) of this split
@@ -478,22 +477,32 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int h = warp; h < G; h += DEC_THREADS / 32) {
         const long long bh = (long long)b * dm.h_q + (long long)r * G + h;
         const float* p = a.partials + bh * n_split * (HD + 2);
-        float M = -INFINITY;
-        for (int s = 0; s < n_split; ++s) M = fmaxf(M, __ldcg(p + s * (HD + 2)));
-        float Lsum = 0.f, acc[VPL];
+        // lane s holds the weight of split s (at most 32 splits); the partial outputs are summed in split order, eight
+        // loads in flight (one after another they cost a round trip to L2 each: 3.5 us at 16 splits)
+        const float ms = lane < n_split ? __ldcg(p + lane * (HD + 2)) : -INFINITY;
+        const float ls = lane < n_split ? __ldcg(p + lane * (HD + 2) + 1) : 0.f;
+        const float M = warp_max(ms);
+        const float w = ms > -INFINITY ? __expf(ms - M) : 0.f;
+        const float Lsum = warp_sum(w * ls);
+        float acc[VPL];
 #pragma unroll
         for (int v = 0; v < VPL; ++v) acc[v] = 0.f;
-        for (int s = 0; s < n_split; ++s) {
-          const float ms = __ldcg(p + s * (HD + 2));
-          if (ms == -INFINITY) continue;
-          const float w = __expf(ms - M);
-          Lsum += w * __ldcg(p + s * (HD + 2) + 1);
-          const float2* po = reinterpret_cast<const float2*>(p + s * (HD + 2) + 2 + lane * VPL);   // 8-byte aligned
-          const float2 oa = __ldcg(po);
-          acc[0] += w * oa.x; acc[1] += w * oa.y;
-          if constexpr (VPL == 4) {
-            const float2 ob = __ldcg(po + 1);
-            acc[2] += w * ob.x; acc[3] += w * ob.y;
+        for (int s0 = 0; s0 < n_split; s0 += 8) {
+          float2 o[8][VPL / 2];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (s0 + u < n_split) {
+              const float2* po = reinterpret_cast<const float2*>(p + (s0 + u) * (HD + 2) + 2 + lane * VPL);   // 8-byte aligned
+#pragma unroll
+              for (int v = 0; v < VPL / 2; ++v) o[u][v] = __ldcg(po + v);
+            }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float wu = __shfl_sync(0xffffffffu, w, (s0 + u) & 31);
+            if (s0 + u < n_split) {
+#pragma unroll
+              for (int v = 0; v < VPL / 2; ++v) { acc[2 * v] += wu * o[u][v].x; acc[2 * v + 1] += wu * o[u][v].y; }
+            }
           }
         }
         const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
