@@ -80,7 +80,7 @@ __device__ __forceinline__ void score_rows(const float (&q)[G][D / 32], const fl
 // from the row's mean and variance (closed forms for alpha = 2 and 1.5, as in the prefill kernel); either side of the
 // root is a valid start: from the left the iterates rise monotonically, from the right one step lands on the left.
 template <int RPL>
-__device__ __noinline__ float entmax_tau(const float* x, int n_cand, int e_int, float e, int lane) {
+__device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_int, float e, int lane) {
   constexpr int MAX_NEWTON = 64, MAX_NEWTON_GENERIC = 400;
   float xr[RPL];
   float mxg = -INFINITY;
