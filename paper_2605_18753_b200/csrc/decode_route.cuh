@@ -91,13 +91,7 @@ __device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_in
     mxg = fmaxf(mxg, xr[u]);
   }
   for (int c = lane + 32 * RPL; c < n_cand; c += 32) mxg = fmaxf(mxg, x[c]);
-  {
-    // maximum through the integer warp reduction (one instruction instead of five shuffles): floats map to signed
-    // integers of the same order by flipping the magnitude bits of the negative ones
-    const int i = __float_as_int(mxg);
-    const int o = __reduce_max_sync(0xffffffffu, i ^ ((i >> 31) & 0x7fffffff));
-    mxg = __int_as_float(o ^ ((o >> 31) & 0x7fffffff));
-  }
+  mxg = warp_max(mxg);
   // moments about the maximum
   float s1 = 0.f, s2 = 0.f;
 #pragma unroll

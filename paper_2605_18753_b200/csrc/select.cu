@@ -5,23 +5,20 @@
 //   1. Chunk logits x = gamma(alpha-1) <q, kbar_c>/sqrt(d) for every row and candidate chunk are computed
 //      in fp32 and kept in shared memory (they are never written to HBM, unlike Algorithm 2 step 1).
 //   2. One warp per token: for each head of the group, the threshold tau is found by Newton's method on
-//      f(tau) = sum [x - tau]_+^e - 1 (e = 1/(alpha-1)), started at max(x) - 1 where f >= 0.  f is convex
-//      and decreasing, so the iterates rise monotonically to the root and never pass it; for alpha = 2
-//      the iteration is finite.  For alpha in {2, 1.5, 1.25} the powers are products (no exp/log).
+//      f(tau) = sum [x - tau]_+^e - 1 (e = 1/(alpha-1); entmax_tau in decode_route.cuh, the row in registers).  For alpha
+//      in {2, 1.5, 1.25} the powers are products (no exp/log).
 //   3. Group weights w_c = mean_h [x_hc - tau_h]_+^e, support bit = (max_h (x_hc - tau_h) > 0), 32 chunks
 //      per ballot = one mask word (Algorithm 2 steps 7-13); log w in a scaled form; mu = mean log w;
 //      bias = (log w - mu)/sigma compacted into the row's list (steps 15-19), the own chunk's bit is set.
 // With a local window of L chunks the last L chunks before the own one are not scored: their bits are set and
 // they close the row's list with bias 0 (they take no part in tau, w or mu).
-#include "common.cuh"
+#include "decode_route.cuh"
 
 namespace dash {
 
 constexpr int SEL_THREADS = 256;
 constexpr int SEL_CT = 64;          // candidate chunks per staged tile of summaries
 constexpr int SEL_SMEM_BUDGET = 200 * 1024;
-constexpr int SEL_MAX_NEWTON = 64;
-constexpr int SEL_MAX_NEWTON_GENERIC = 400;
 
 struct SelectPlan {
   int TQ;         // tokens per block
@@ -34,7 +31,10 @@ static bool plan_select(const Dims& dm, SelectPlan* pl) {
   if (dm.g_q > 32) return false;
   int tq = 1;
   if (!dm.decode) {
-    while (tq * 2 * dm.g_q <= 32 && tq * 2 <= dm.B) tq *= 2;
+    // more tokens per block read each summary tile for more rows, but a small problem must not leave SMs without a block:
+    // two blocks per SM (148 of them) come first (1024 tokens, one head: 18 us in blocks of 32 tokens, now 8)
+    const long long tokens = (long long)dm.batch * dm.h_kv * dm.seq_q;
+    while (tq * 2 * dm.g_q <= 32 && tq * 2 <= dm.B && tokens / (tq * 2) >= 2 * 148) tq *= 2;
   }
   const int max_cand = (dm.decode || !dm.causal) ? dm.T_s : min(dm.T_s, (dm.seq_q - 1) / dm.B);
   const int xs = ((max_cand + SEL_CT - 1) / SEL_CT) * SEL_CT + 4;
@@ -158,7 +158,6 @@ select_kernel(Dims dm, int TQ, int xs_stride, int token_base, const T* __restric
   // ---- one warp per token: thresholds, group weights, mask words, bias list
   const int e_int = dm.e_int;
   const float e = dm.e;
-  const int max_it = e_int ? SEL_MAX_NEWTON : SEL_MAX_NEWTON_GENERIC;
   const float log_gq = logf((float)g_q);
   for (int t = warp; t < TQ; t += SEL_THREADS / 32) {
     const int i = i0 + t;
@@ -169,28 +168,8 @@ select_kernel(Dims dm, int TQ, int xs_stride, int token_base, const T* __restric
     for (int hh = 0; hh < g_q; ++hh) {
       const float* x = x0 + (size_t)hh * xs_stride;
       float tau = 0.f;
-      if (n_cand > 0) {
-        float mx = -INFINITY;
-        for (int c = lane; c < n_cand; c += 32) mx = fmaxf(mx, x[c]);
-        mx = warp_max(mx);
-        tau = mx - 1.f;
-        for (int it = 0; it < max_it; ++it) {
-          float f = 0.f, g = 0.f;
-          for (int c = lane; c < n_cand; c += 32) {
-            const float m = x[c] - tau;
-            if (m > 0.f) {
-              f += pow_e(m, e_int, e);
-              g += pow_em1(m, e_int, e);
-            }
-          }
-          f = warp_sum(f) - 1.f;
-          g = warp_sum(g);
-          if (!(f > NEWTON_F_TOL)) break;
-          const float nt = tau + newton_delta(f + 1.f, g, e_int, e);
-          if (!(nt > tau)) break;
-          tau = nt;
-        }
-      }
+      if (n_cand > 128) tau = entmax_tau<16>(x, n_cand, e_int, e, lane);
+      else if (n_cand > 0) tau = entmax_tau<4>(x, n_cand, e_int, e, lane);
       if (lane == 0) {
         taus[t * g_q + hh] = tau;
         if (tau_out) tau_out[((long long)b * dm.h_q + r * g_q + hh) * dm.seq_q + (dm.decode ? 0 : i)] = tau;
