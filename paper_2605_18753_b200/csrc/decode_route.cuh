@@ -76,9 +76,7 @@ __device__ __forceinline__ void score_rows(const float (&q)[G][D / 32], const fl
 
 // Entmax threshold of one row of n > 0 logits in shared memory, by one warp, no barrier inside the iteration: a lane keeps
 // its share of the row (RPL logits; anything beyond 32 * RPL is re-read) in registers over all passes, a pass is the
-// lane's sums, two warp sums and the step.  The start is the larger of the all-active root and the normal-tail estimate
-// from the row's mean and variance (closed forms for alpha = 2 and 1.5, as in the prefill kernel); either side of the
-// root is a valid start: from the left the iterates rise monotonically, from the right one step lands on the left.
+// lane's sums, two warp sums and the step.
 template <int RPL>
 __device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_int, float e, int lane) {
   constexpr int MAX_NEWTON = 64, MAX_NEWTON_GENERIC = 400;
@@ -107,23 +105,7 @@ __device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_in
   }
   s1 = warp_sum(s1);
   s2 = warp_sum(s2);
-  float tau;
-  {
-    const float n = (float)n_cand;
-    float t = -1.f;
-    if (e_int == 1) {
-      t = (s1 - 1.f) / n;
-    } else if (e_int == 2) {
-      const float mean = s1 / n, ss = s2 - s1 * mean;
-      if (ss < 1.f) t = mean - sqrtf((1.f - ss) / n);
-      if (n_cand >= 8 && ss > 0.f) {
-        const float L = -__logf(fminf(fmaxf(ss, 0.3334f), 1e7f));
-        const float z = fmaf(fmaf(fmaf(fmaf(-8.93074e-05f, L, -0.0037117f), L, -0.0612527f), L, -0.717421f), L, -0.499476f);
-        t = fmaxf(t, fmaf(z, sqrtf(ss / n), mean));
-      }
-    }
-    tau = mxg + fminf(fmaxf(t, -1.f), -1e-6f);
-  }
+  float tau = mxg + entmax_start((float)n_cand, s1, s2, e_int);
   auto newton = [&](auto ei_tag) {
     constexpr int EI = decltype(ei_tag)::value;
     const int max_it = EI ? MAX_NEWTON : MAX_NEWTON_GENERIC;
