@@ -21,8 +21,6 @@
 #pragma once
 #include <cuda.h>
 
-#include <type_traits>
-
 #include "common.cuh"
 #include "select_sm100.cuh"
 #include "sm100_ptx.cuh"
@@ -91,7 +89,9 @@ __device__ __forceinline__ void add_powers(float2 m, float2& F, float2& G) {
 
 // WIDE: the tile spans several chunks (chunks shorter than 128 / g_q tokens); tiles inside one chunk compile with one
 // candidate count for all rows.
-template <int NST, int G, int CS, int HD, bool WIDE>
+// EI: the exponent 1 / (alpha - 1) as a compile-time constant (1, 2, 4 for alpha = 2, 1.5, 1.25; 0: any other, powf at run
+// time), so that the per-candidate loops hold no tests of it and every kernel has the registers of its own body only.
+template <int NST, int G, int CS, int HD, bool WIDE, int EI>
 __global__ void __launch_bounds__(sel_threads(NST), NST == 1 ? 2 : 1)
 select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKB, SelectTcArgs a) {
   using SP = SmemPlan<NST>;
@@ -231,7 +231,6 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int n_row = WIDE ? min(max(c_row - dm.local_blocks, 0), n_cand) : n_cand;
     const int l_row = WIDE ? (CS > 1 ? max(0, min(CCOLS, n_row - c_lo)) : n_row) : n_loc;
     const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
-    const int e_int = dm.e_int;
     const float e = dm.e, xs = dm.x_scale;
     const int n_chunks = (n_loc + 31) / 32;
     const int per_part = (n_chunks + SPLIT - 1) / SPLIT;
@@ -296,11 +295,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // Newton on f(tau) = sum [x - tau]_+^e - 1 (steps taken on f^(1/e), see newton_delta), convex and decreasing.
     // From the left of the root the iterates rise monotonically and never pass it; from the right one step lands
     // on the left (start: entmax_start).
-    // The body below runs with the exponent as a compile-time constant (1, 2, 4 for alpha = 2, 1.5, 1.25; 0: any other, powf
-    // at run time): the per-candidate loops hold no tests of it.
-    auto solve = [&](auto ei_tag) {
-    constexpr int EI_STATIC = decltype(ei_tag)::value;
-    constexpr int ei = EI_STATIC;
+    constexpr int ei = EI;
     const int max_it = ei ? MAX_NEWTON : MAX_NEWTON_GENERIC;
     auto newton_step = [&](float f, float g, bool& done) {
       if (done) return;
@@ -352,7 +347,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (WIDE && n_row == 0) { tau = 0.f; done = true; }
       for (int it = 0; it < max_it; ++it) {
         float f[4] = {0.f, 0.f, 0.f, 0.f}, g[4] = {0.f, 0.f, 0.f, 0.f};
-        if constexpr (EI_STATIC > 0) {
+        if constexpr (EI > 0) {
           // two candidates per packed instruction, four chains of pairs
           float2 fv[4], gv[4];
 #pragma unroll
@@ -366,7 +361,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 float2 mm = __fadd2_rn(make_float2(xr[k][c], xr[k][c + 1]), ntau);
                 mm.x = fmaxf(mm.x, 0.f);
                 mm.y = fmaxf(mm.y, 0.f);
-                add_powers<EI_STATIC>(mm, fv[(c >> 1) & 3], gv[(c >> 1) & 3]);
+                add_powers<EI>(mm, fv[(c >> 1) & 3], gv[(c >> 1) & 3]);
               }
             }
           }
@@ -456,7 +451,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (WIDE && n_row == 0) { tau = 0.f; done = true; }
       for (int it = 0; it < max_it && ok; ++it) {
         float f[4] = {0.f, 0.f, 0.f, 0.f}, g[4] = {0.f, 0.f, 0.f, 0.f};
-        if constexpr (EI_STATIC > 0) {
+        if constexpr (EI > 0) {
           // two candidates per packed instruction (scale and shift, then the sums)
           float2 fv[4], gv[4];
 #pragma unroll
@@ -469,7 +464,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
               float2 mm = __ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), xs2, ntau);
               mm.x = fmaxf(mm.x, 0.f);
               mm.y = fmaxf(mm.y, 0.f);
-              add_powers<EI_STATIC>(mm, fv[(c >> 1) & 3], gv[(c >> 1) & 3]);
+              add_powers<EI>(mm, fv[(c >> 1) & 3], gv[(c >> 1) & 3]);
             }
           });
 #pragma unroll
@@ -628,13 +623,6 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         base += __popc(bits);
       }
     }
-    };
-    switch (e_int) {
-      case 1: solve(std::integral_constant<int, 1>{}); break;
-      case 2: solve(std::integral_constant<int, 2>{}); break;
-      case 4: solve(std::integral_constant<int, 4>{}); break;
-      default: solve(std::integral_constant<int, 0>{}); break;
-    }
     ptx::tc_fence_before();
   }
 
@@ -647,10 +635,10 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   if (CS > 1) ptx::cluster_sync_all();     // nobody leaves while a peer may still write into its shared memory
 }
 
-template <int NST, int G, int CS, int HD, bool WIDE>
-static cudaError_t launch_band(const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a, long long clusters,
-                               cudaStream_t st) {
-  auto kern = select_sm100_kernel<NST, G, CS, HD, WIDE>;
+template <int NST, int G, int CS, int HD, bool WIDE, int EI>
+static cudaError_t launch_exponent(const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a, long long clusters,
+                                   cudaStream_t st) {
+  auto kern = select_sm100_kernel<NST, G, CS, HD, WIDE, EI>;
   static std::atomic<unsigned long long> configured{0};
   if (cudaError_t e = allow_dynamic_smem(kern, SmemPlan<NST>::TOTAL, configured); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -670,6 +658,17 @@ static cudaError_t launch_band(const CUtensorMap& tq, const CUtensorMap& tkb, co
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tq, tkb, a);
   count_launch();
   return e;
+}
+
+template <int NST, int G, int CS, int HD, bool WIDE>
+static cudaError_t launch_band(const CUtensorMap& tq, const CUtensorMap& tkb, const SelectTcArgs& a, long long clusters,
+                               cudaStream_t st) {
+  switch (a.dm.e_int) {
+    case 1: return launch_exponent<NST, G, CS, HD, WIDE, 1>(tq, tkb, a, clusters, st);
+    case 2: return launch_exponent<NST, G, CS, HD, WIDE, 2>(tq, tkb, a, clusters, st);
+    case 4: return launch_exponent<NST, G, CS, HD, WIDE, 4>(tq, tkb, a, clusters, st);
+    default: return launch_exponent<NST, G, CS, HD, WIDE, 0>(tq, tkb, a, clusters, st);
+  }
 }
 
 template <int NST, int CS, int HD>
