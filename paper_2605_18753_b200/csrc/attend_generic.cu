@@ -18,9 +18,6 @@
 
 namespace dash {
 
-__device__ inline float2 load2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-__device__ inline float2 load2(const __nv_bfloat16* p) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p)); }
-
 // Floats of a block's dynamic shared memory: a slice's probabilities per warp in the walk, the warps' outputs at the end.
 template <int D, int R, int NW> constexpr int buf_floats() { return NW * R * (D > 32 ? D : 32); }
 

@@ -13,85 +13,81 @@
 //   w_c = mean_h p_hc                        =>  dp_hc = dw_c / g_q
 //   p_h = entmax(z_h), z_hc = gamma <q_h, kbar_c>/sqrt(d)   =>  dz_h by the Jacobian above
 //   dq_h = gamma/sqrt(d) sum_c dz_hc kbar_c (written, fp32);   dkbar_c += gamma/sqrt(d) sum_h dz_hc q_h (atomic, fp32)
-// Only routed chunks are touched (two sweeps over the row's list, four entries at a time; the chunk logits are
-// recomputed from Q and Kbar).
+// Only routed chunks are touched, SEG list entries at a time.  Margins: eight chunks at once, four lanes per summary row
+// (lane l reads the 16-byte pieces (l mod 4) + 4 j of the chunk l div 4, so that a query piece read from shared memory
+// serves eight chunks and two shuffles per head finish a dot product); they stay in shared memory until the whole list
+// has been seen, which fixes dz.  Then lanes own head_dim slices: dq_h += dz_hc kbar_c, dkbar_c by vector reductions (the L2
+// atomic units count requests, not bytes).  8192 tokens, 32/8 heads, chunks of 64: 690 us with two sweeps of butterfly
+// reductions over the list, now 450.
 //
-// summaries_bwd_kernel: one warp per (batch, KV head, chunk): Eq. 3, kbar_c = sum_t a_t k_t with
+// summaries_bwd_kernel: four warps per (batch, KV head, chunk), a quarter of its rows each: Eq. 3, kbar_c = sum_t a_t k_t with
 // a = softmax(<qbar, k_t>/sqrt(d)) (a_t = 1/B without a summary query): dk_t += a_t dkbar_c + ds_t qbar/sqrt(d),
-// ds_t = a_t (<k_t, dkbar_c> - sum_u a_u <k_u, dkbar_c>), dqbar += sum_t ds_t k_t / sqrt(d).
+// ds_t = a_t (<k_t, dkbar_c> - sum_u a_u <k_u, dkbar_c>), dqbar += sum_t ds_t k_t / sqrt(d).  The B logits and products of the
+// chunk meet in shared memory.
 #include "common.cuh"
 
 namespace dash {
 
 constexpr int RB_WARPS = 4;
 
-// Sums V values that every lane holds across the warp with the halving exchange (V - 1 + log2(32 / V) ... shuffles
-// instead of 5 V): value v ends up complete in lane v * (32 / V) as x[0]; then every value is broadcast, so that all
-// lanes hold all V sums (another V shuffles).  V must be a power of two <= 32.
+// 4 or 2 consecutive floats added to global memory in one request.
 template <int V>
-__device__ __forceinline__ void warp_sum_all(float (&x)[V], int lane) {
-  float y[V];
-#pragma unroll
-  for (int k = 0; k < V; ++k) y[k] = x[k];
-#pragma unroll
-  for (int width = 16, live = V; width >= 1; width >>= 1) {
-    if (live > 1) {
-      const bool upper = (lane & width) != 0;
-      const int half = live / 2;
-#pragma unroll
-      for (int k = 0; k < V / 2; ++k) {
-        if (k < half) {
-          const float mine = upper ? y[k + half] : y[k];
-          const float give = upper ? y[k] : y[k + half];
-          y[k] = mine + __shfl_xor_sync(0xffffffffu, give, width);
-        }
-      }
-      live = half;
-    } else {
-      y[0] += __shfl_xor_sync(0xffffffffu, y[0], width);
-    }
+__device__ __forceinline__ void add_global(float* p, const float (&x)[V]) {
+  if constexpr (V == 4)
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
+  else
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x[0]), "f"(x[1]) : "memory");
+}
+template <int V, typename T>
+__device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
+  if constexpr (V == 4) {
+    const float4 f = load4(p);
+    x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
+  } else {
+    const float2 f = load2(p);
+    x[0] = f.x; x[1] = f.y;
   }
-  // the lane bits were consumed from the top: value v sits in the lane whose top log2(V) bits spell v
-#pragma unroll
-  for (int v = 0; v < V; ++v) x[v] = __shfl_sync(0xffffffffu, y[0], v * (32 / V));
 }
 
-// G (heads per KV head) is a template parameter so that the per-head arrays live in registers; the row's routed chunks
-// are taken NB at a time: their summary rows are fetched together and the NB * G dot products are reduced together.
+// G (heads per KV head) is a template parameter so that the per-head sums live in registers.
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(RB_WARPS * 32)
 route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
                  const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
                  float* __restrict__ dQr, float* __restrict__ dKbar) {
   constexpr int VPL = D / 32;
-  constexpr int NB = G <= 8 ? 4 : 2;           // entries per batch: NB * G <= 32 values per reduction
-  const int lane = threadIdx.x & 31;
-  const long long gw = (long long)blockIdx.x * RB_WARPS + (threadIdx.x >> 5);
+  constexpr int SEG = G <= 8 ? 64 : 32;        // list entries held at a time
+  __shared__ __align__(16) float q_s[RB_WARPS][G][D];
+  __shared__ __align__(16) float m_s[RB_WARPS][SEG][G];      // margins, then dz
+  __shared__ float dw_s[RB_WARPS][SEG];
+  __shared__ int c_s[RB_WARPS][SEG];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long gw = (long long)blockIdx.x * RB_WARPS + warp;
   const long long total = (long long)dm.batch * dm.h_kv * dm.seq_q;
   if (gw >= total) return;
   const int i = (int)(gw % dm.seq_q);
-  const int r = (int)((gw / dm.seq_q) % dm.h_kv);
-  const int b = (int)(gw / ((long long)dm.seq_q * dm.h_kv));
-  const long long grp = (long long)b * dm.h_kv + r;
+  const long long grp = gw / dm.seq_q;
+  const int r = (int)(grp % dm.h_kv), b = (int)(grp / dm.h_kv);
   // fp32 gradient of Q from the routing: [batch, seq_q, h_q, d], every row written (zeros where nothing is routed)
   float* dq_out = dQr + (((long long)b * dm.seq_q + i) * dm.h_q + (long long)r * G) * D + lane * VPL;
-  const int c_own = i / dm.B;
+  const int c_own = i >> dm.log_b;
   const int n_local = min(dm.local_blocks, c_own);              // window chunks close the list and carry no gradient
   const int n_routed = count[grp * dm.seq_q + i] - n_local;
-  float q[G][VPL], dq[G][VPL];
+  float dq[G][VPL];
 #pragma unroll
   for (int h = 0; h < G; ++h)
 #pragma unroll
     for (int v = 0; v < VPL; ++v) dq[h][v] = 0.f;
   if (n_routed > 0) {
     const long long loff = grp * dm.list_rows + list_row_offset(dm, i);
-    const float* kb = Kbar + grp * dm.T_s * D + lane * VPL;
+    const float* kb = Kbar + grp * dm.T_s * D;
     float th[G];
 #pragma unroll
     for (int h = 0; h < G; ++h) {
-      const T* qp = Q + (long long)b * dm.qs[0] + (long long)i * dm.qs[1] + (long long)(r * G + h) * dm.qs[2] + lane * VPL;
+      float x[VPL];
+      load_vec<VPL>(Q + (long long)b * dm.qs[0] + (long long)i * dm.qs[1] + (long long)(r * G + h) * dm.qs[2] + lane * VPL, x);
 #pragma unroll
-      for (int v = 0; v < VPL; ++v) q[h][v] = to_f32<T>(qp[v]);
+      for (int v = 0; v < VPL; ++v) q_s[warp][h][lane * VPL + v] = x[v];
       th[h] = tau[((long long)b * dm.h_q + r * G + h) * dm.seq_q + i];
     }
     float dmean = 0.f;
@@ -99,101 +95,116 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
     dmean = warp_sum(dmean) / (float)n_routed;
     const float e = dm.e;
     const int e_int = dm.e_int;
-    // One batch: entries k0 .. k0 + NB - 1 (those beyond the list repeat the last one and are ignored by the caller).
-    // kv: their summary rows; m: the margins m_h = x_scale <q_h, kbar_c> - tau_h (clamped at 0) of every entry and head;
-    // dw: the gradient w.r.t. the entry's group weight.
-    auto batch = [&](int k0, int (&c)[NB], float (&kv)[NB][VPL], float (&m)[NB][G], float (&dw)[NB]) {
-      float db[NB];
+    float A[G], S[G];                          // per head A_h = sum_c s_hc dw_c / g_q and S_h = sum_c s_hc
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        const int k = min(k0 + u, n_routed - 1);
-        c[u] = blk_idx[loff + k];
-        db[u] = dbias[loff + k];
+    for (int h = 0; h < G; ++h) A[h] = S[h] = 0.f;
+    // Margins m_hc = x_scale <q_h, kbar_c> - tau_h (clamped at 0) and weight gradients dw_c of entries [k0, k0 + n)
+    auto margins = [&](int k0, int n, bool sum) {
+      __syncwarp();
+      for (int k = lane; k < n; k += 32) {
+        c_s[warp][k] = blk_idx[loff + k0 + k];
+        dw_s[warp][k] = (dbias[loff + k0 + k] - dmean) * dm.inv_sigma;
       }
+      __syncwarp();
+      for (int e0 = 0; e0 < n; e0 += 8) {
+        const int k = e0 + (lane >> 2);
+        const bool live = k < n;
+        const float* kp = kb + (long long)c_s[warp][min(k, n - 1)] * D + 4 * (lane & 3);
+        float x[G];
 #pragma unroll
-      for (int u = 0; u < NB; ++u)
+        for (int h = 0; h < G; ++h) x[h] = 0.f;
+        float4 kv[D / 16];
 #pragma unroll
-        for (int v = 0; v < VPL; ++v) kv[u][v] = kb[(long long)c[u] * D + v];
-      float part[NB * G];
+        for (int j = 0; j < D / 16; ++j) kv[j] = load4(kp + 16 * j);
 #pragma unroll
-      for (int u = 0; u < NB; ++u)
+        for (int j = 0; j < D / 16; ++j)
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-          float s = 0.f;
-#pragma unroll
-          for (int v = 0; v < VPL; ++v) s = fmaf(q[h][v], kv[u][v], s);
-          part[u * G + h] = s;
-        }
-      warp_sum_all<NB * G>(part, lane);
-#pragma unroll
-      for (int u = 0; u < NB; ++u) {
+          for (int h = 0; h < G; ++h) {
+            const float4 qv = load4(&q_s[warp][h][16 * j + 4 * (lane & 3)]);
+            x[h] = fmaf(qv.x, kv[j].x, x[h]); x[h] = fmaf(qv.y, kv[j].y, x[h]);
+            x[h] = fmaf(qv.z, kv[j].z, x[h]); x[h] = fmaf(qv.w, kv[j].w, x[h]);
+          }
         float w = 0.f;
 #pragma unroll
         for (int h = 0; h < G; ++h) {
-          m[u][h] = fmaxf(part[u * G + h] * dm.x_scale - th[h], 0.f);
-          w += pow_e(m[u][h], e_int, e);
+          x[h] += __shfl_xor_sync(0xffffffffu, x[h], 1);
+          x[h] += __shfl_xor_sync(0xffffffffu, x[h], 2);
+          x[h] = fmaxf(x[h] * dm.x_scale - th[h], 0.f);
+          w += pow_e(x[h], e_int, e);
         }
         w /= (float)G;
-        dw[u] = w > 0.f ? (db[u] - dmean) * dm.inv_sigma / w : 0.f;
-      }
-    };
-    // sweep 1: per head A_h = sum_c s_hc dw_c / g_q and S_h = sum_c s_hc
-    float A[G], S[G];
-#pragma unroll
-    for (int h = 0; h < G; ++h) A[h] = S[h] = 0.f;
-    for (int k0 = 0; k0 < n_routed; k0 += NB) {
-      int c[NB];
-      float kv[NB][VPL], m[NB][G], dw[NB];
-      batch(k0, c, kv, m, dw);
-#pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        if (k0 + u < n_routed) {
+        const float dw = live && w > 0.f ? dw_s[warp][k] / (w * (float)G) : 0.f;
+        if (live && sum) {
 #pragma unroll
           for (int h = 0; h < G; ++h) {
-            const float s = pow_em1(m[u][h], e_int, e);
-            A[h] += s * dw[u] / (float)G;
+            const float s = pow_em1(x[h], e_int, e);
+            A[h] = fmaf(s, dw, A[h]);
             S[h] += s;
           }
         }
+        __syncwarp();                           // (everybody has read dw_s of these entries)
+        if (live && (lane & 3) == 0) {
+          dw_s[warp][k] = dw;                   // from here on the gradient w.r.t. every head's weight
+#pragma unroll
+          for (int h = 0; h < G; ++h) m_s[warp][k][h] = x[h];
+        }
       }
-    }
-    // sweep 2: dz_hc, then dq_h and dkbar_c
+      __syncwarp();
+    };
+    for (int k0 = 0; k0 < n_routed; k0 += SEG) margins(k0, min(SEG, n_routed - k0), true);
+    // (the four lanes of a chunk hold the same sums)
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        A[h] += __shfl_xor_sync(0xffffffffu, A[h], o);
+        S[h] += __shfl_xor_sync(0xffffffffu, S[h], o);
+      }
     const float zscale = dm.x_scale / (1.f / e);       // gamma / sqrt(d) = x_scale / (alpha - 1)
-    for (int k0 = 0; k0 < n_routed; k0 += NB) {
-      int c[NB];
-      float kv[NB][VPL], m[NB][G], dw[NB];
-      batch(k0, c, kv, m, dw);
 #pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        if (k0 + u < n_routed) {
-          float dkb[VPL];
+    for (int h = 0; h < G; ++h) A[h] = S[h] > 0.f ? A[h] / S[h] : 0.f;
+    for (int k0 = 0; k0 < n_routed; k0 += SEG) {
+      const int n = min(SEG, n_routed - k0);
+      if (n_routed > SEG) margins(k0, n, false);
+      // dz_hc = s_hc (dw_c / g_q - A_h / S_h), scaled
+      for (int k = lane; k < n; k += 32) {
+        const float dw = dw_s[warp][k];
 #pragma unroll
-          for (int v = 0; v < VPL; ++v) dkb[v] = 0.f;
+        for (int h = 0; h < G; ++h)
+          m_s[warp][k][h] = S[h] > 0.f ? pow_em1(m_s[warp][k][h], e_int, e) * (dw - A[h]) * zscale : 0.f;
+      }
+      __syncwarp();
+      constexpr int NB = 4;
+      for (int e0 = 0; e0 < n; e0 += NB) {
+        float kv[NB][VPL];
+        int c[NB];
 #pragma unroll
-          for (int h = 0; h < G; ++h) {
-            const float s = pow_em1(m[u][h], e_int, e);
-            const float dz = S[h] > 0.f ? s * (dw[u] / (float)G - A[h] / S[h]) : 0.f;
+        for (int u = 0; u < NB; ++u) {
+          c[u] = c_s[warp][min(e0 + u, n - 1)];
+          load_vec<VPL>(kb + (long long)c[u] * D + lane * VPL, kv[u]);
+        }
 #pragma unroll
-            for (int v = 0; v < VPL; ++v) {
-              dq[h][v] = fmaf(dz, kv[u][v], dq[h][v]);
-              dkb[v] = fmaf(dz, q[h][v], dkb[v]);
+        for (int u = 0; u < NB; ++u) {
+          if (e0 + u < n) {
+            float dkb[VPL];
+#pragma unroll
+            for (int v = 0; v < VPL; ++v) dkb[v] = 0.f;
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+              const float dz = m_s[warp][e0 + u][h];
+              float qv[VPL];
+              load_vec<VPL>(&q_s[warp][h][lane * VPL], qv);
+#pragma unroll
+              for (int v = 0; v < VPL; ++v) {
+                dq[h][v] = fmaf(dz, kv[u][v], dq[h][v]);
+                dkb[v] = fmaf(dz, qv[v], dkb[v]);
+              }
             }
+            add_global<VPL>(dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL, dkb);
           }
-          float* dst = dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL;
-          // one vector reduction per lane (16 or 8 bytes): a quarter / half of the requests of scalar atomic adds, and
-          // the requests, not the bytes, are what the L2 atomic units count
-          if constexpr (VPL == 4)
-            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(dkb[0] * zscale), "f"(dkb[1] * zscale),
-                         "f"(dkb[2] * zscale), "f"(dkb[3] * zscale) : "memory");
-          else
-            asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(dkb[0] * zscale), "f"(dkb[1] * zscale) : "memory");
         }
       }
     }
-#pragma unroll
-    for (int h = 0; h < G; ++h)
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) dq[h][v] *= zscale;
   }
 #pragma unroll
   for (int h = 0; h < G; ++h)
@@ -201,81 +212,112 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
     for (int v = 0; v < VPL; ++v) dq_out[(long long)h * D + v] = dq[h][v];
 }
 
+constexpr int SB_SPLIT = 4;      // warps that share a chunk = a block
+
 template <typename T, int D>
-__global__ void __launch_bounds__(RB_WARPS * 32)
+__global__ void __launch_bounds__(SB_SPLIT * 32)
 summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__ qbar, long long qbar_chunk_stride,
                      const float* __restrict__ dKbar, float* __restrict__ dK, float* __restrict__ dqbar) {
-  constexpr int VPL = D / 32;
-  const int lane = threadIdx.x & 31;
-  const long long gw = (long long)blockIdx.x * RB_WARPS + (threadIdx.x >> 5);
-  const long long total = (long long)dm.batch * dm.h_kv * dm.T_s;
-  if (gw >= total) return;
-  const int c = (int)(gw % dm.T_s);
-  const int r = (int)((gw / dm.T_s) % dm.h_kv);
-  const int b = (int)(gw / ((long long)dm.T_s * dm.h_kv));
+  constexpr int VPL = D / 32, NB = 4;
+  __shared__ float s_s[128], da_s[128];      // logits and <k_t, dkbar> of the chunk's tokens
+  __shared__ float red[SB_SPLIT][D];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = (int)(blockIdx.x % dm.T_s);
+  const long long grp = blockIdx.x / dm.T_s;
+  const int r = (int)(grp % dm.h_kv), b = (int)(grp / dm.h_kv);
+  const int rows = dm.B / SB_SPLIT, t0 = warp * rows;          // this warp's tokens of the chunk (4 .. 32)
   const T* kp = K + (long long)b * dm.ks[0] + (long long)c * dm.B * dm.ks[1] + (long long)r * dm.ks[2] + lane * VPL;
   float* dkp = dK + (((long long)b * dm.seq_kv + (long long)c * dm.B) * dm.h_kv + r) * D + lane * VPL;
   const long long gtok = (long long)dm.h_kv * D;
   float g[VPL];
+  load_vec<VPL>(dKbar + (grp * dm.T_s + c) * D + lane * VPL, g);
+  // dk rows of four tokens at a time: read, add, write
+  auto add_rows = [&](int t, auto&& delta) {
+    float x[NB][VPL];
 #pragma unroll
-  for (int v = 0; v < VPL; ++v) g[v] = dKbar[(((long long)b * dm.h_kv + r) * dm.T_s + c) * D + lane * VPL + v];
+    for (int u = 0; u < NB; ++u) load_vec<VPL>(dkp + (long long)(t + u) * gtok, x[u]);
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      delta(u, x[u]);
+      if constexpr (VPL == 4)
+        store4(dkp + (long long)(t + u) * gtok, make_float4(x[u][0], x[u][1], x[u][2], x[u][3]));
+      else
+        *reinterpret_cast<float2*>(dkp + (long long)(t + u) * gtok) = make_float2(x[u][0], x[u][1]);
+    }
+  };
   if (qbar == nullptr) {
     const float inv = 1.f / (float)dm.B;
-    for (int t = 0; t < dm.B; ++t)
+    for (int t = t0; t < t0 + rows; t += NB)
+      add_rows(t, [&](int, float (&x)[VPL]) {
 #pragma unroll
-      for (int v = 0; v < VPL; ++v) dkp[(long long)t * gtok + v] += g[v] * inv;
+        for (int v = 0; v < VPL; ++v) x[v] = fmaf(g[v], inv, x[v]);
+      });
     return;
   }
   float qv[VPL];
-  const float* qp = qbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL;
+  load_vec<VPL>(qbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, qv);
+  for (int t = t0; t < t0 + rows; t += NB) {
+    float kv[NB][VPL], s[NB], da[NB];
 #pragma unroll
-  for (int v = 0; v < VPL; ++v) qv[v] = qp[v];
-  // pass 1: softmax statistics of s_t = <qbar, k_t>/sqrt(d) and sum_t a_t <k_t, g>
-  float mx = -INFINITY;
-  for (int t = 0; t < dm.B; ++t) {
-    float s = 0.f;
+    for (int u = 0; u < NB; ++u) load_vec<VPL>(kp + (long long)(t + u) * dm.ks[1], kv[u]);
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) s = fmaf(qv[v], to_f32<T>(kp[(long long)t * dm.ks[1] + v]), s);
-    mx = fmaxf(mx, warp_sum(s) * dm.sm_scale);
-  }
-  float l = 0.f, ada = 0.f;
-  for (int t = 0; t < dm.B; ++t) {
-    float s = 0.f, da = 0.f;
+    for (int u = 0; u < NB; ++u) {
+      s[u] = da[u] = 0.f;
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const float kvv = to_f32<T>(kp[(long long)t * dm.ks[1] + v]);
-      s = fmaf(qv[v], kvv, s);
-      da = fmaf(g[v], kvv, da);
+      for (int v = 0; v < VPL; ++v) {
+        s[u] = fmaf(qv[v], kv[u][v], s[u]);
+        da[u] = fmaf(g[v], kv[u][v], da[u]);
+      }
     }
-    const float p = __expf(warp_sum(s) * dm.sm_scale - mx);
-    l += p;
-    ada += p * warp_sum(da);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+        da[u] += __shfl_xor_sync(0xffffffffu, da[u], o);
+      }
+#pragma unroll
+    for (int u = 0; u < NB; ++u)
+      if (lane == u) { s_s[t + u] = s[u] * dm.sm_scale; da_s[t + u] = da[u]; }
   }
-  ada /= l;
-  // pass 2: dk_t and dqbar
+  __syncthreads();
+  // softmax statistics and sum_t a_t <k_t, g>, by every warp for itself
+  float mx = -INFINITY, l = 0.f, ada = 0.f;
+  for (int t = lane; t < dm.B; t += 32) mx = fmaxf(mx, s_s[t]);
+  mx = warp_max(mx);
+  for (int t = lane; t < dm.B; t += 32) {
+    const float p = __expf(s_s[t] - mx);
+    l += p;
+    ada = fmaf(p, da_s[t], ada);
+  }
+  const float inv_l = 1.f / warp_sum(l);
+  ada = warp_sum(ada) * inv_l;
   float dqb[VPL];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) dqb[v] = 0.f;
-  for (int t = 0; t < dm.B; ++t) {
-    float kvv[VPL], s = 0.f, da = 0.f;
+  for (int t = t0; t < t0 + rows; t += NB) {
+    float kv[NB][VPL];
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      kvv[v] = to_f32<T>(kp[(long long)t * dm.ks[1] + v]);
-      s = fmaf(qv[v], kvv[v], s);
-      da = fmaf(g[v], kvv[v], da);
-    }
-    const float a = __expf(warp_sum(s) * dm.sm_scale - mx) / l;
-    const float dst = a * (warp_sum(da) - ada);
+    for (int u = 0; u < NB; ++u) load_vec<VPL>(kp + (long long)(t + u) * dm.ks[1], kv[u]);
+    add_rows(t, [&](int u, float (&x)[VPL]) {
+      const float a = __expf(s_s[t + u] - mx) * inv_l, dst = a * (da_s[t + u] - ada);
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      dkp[(long long)t * gtok + v] += a * g[v] + dst * qv[v] * dm.sm_scale;
-      dqb[v] = fmaf(dst, kvv[v], dqb[v]);
-    }
+      for (int v = 0; v < VPL; ++v) {
+        x[v] += a * g[v] + dst * qv[v] * dm.sm_scale;
+        dqb[v] = fmaf(dst, kv[u][v], dqb[v]);
+      }
+    });
   }
   if (dqbar) {
-    float* dq = dqbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL;
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) atomicAdd(dq + v, dqb[v] * dm.sm_scale);
+    for (int v = 0; v < VPL; ++v) red[warp][lane * VPL + v] = dqb[v] * dm.sm_scale;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int v = 0; v < VPL; ++v)
+        dqb[v] = (red[0][lane * VPL + v] + red[1][lane * VPL + v]) + (red[2][lane * VPL + v] + red[3][lane * VPL + v]);
+      add_global<VPL>(dqbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, dqb);
+    }
   }
 }
 
@@ -318,9 +360,9 @@ cudaError_t launch_summaries_bwd(const Dims& dm, const void* K, const float* qba
   }
   const long long total = (long long)dm.batch * dm.h_kv * dm.T_s;
   if (total == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((total + RB_WARPS - 1) / RB_WARPS);
+  const unsigned grid = (unsigned)total;
 #define DASH_SB(T, D) \
-  summaries_bwd_kernel<T, D><<<grid, RB_WARPS * 32, 0, st>>>(dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
+  summaries_bwd_kernel<T, D><<<grid, SB_SPLIT * 32, 0, st>>>(dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
   if (dm.dtype == DASH_BF16) {
     if (dm.d == 128) DASH_SB(__nv_bfloat16, 128); else DASH_SB(__nv_bfloat16, 64);
   } else {
