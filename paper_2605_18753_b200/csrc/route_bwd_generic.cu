@@ -51,7 +51,7 @@ __device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
 
 // G (heads per KV head) is a template parameter so that the per-head sums live in registers.
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(RB_WARPS * 32)
+__global__ void __launch_bounds__(RB_WARPS * 32, G <= 4 ? 5 : 1)
 route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
                  const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
                  float* __restrict__ dQr, float* __restrict__ dKbar) {
@@ -73,21 +73,28 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
   const int c_own = i >> dm.log_b;
   const int n_local = min(dm.local_blocks, c_own);              // window chunks close the list and carry no gradient
   const int n_routed = count[grp * dm.seq_q + i] - n_local;
-  float dq[G][VPL];
+  // (pairs of floats: one instruction for two products)
+  float2 dq[G][VPL / 2];
 #pragma unroll
   for (int h = 0; h < G; ++h)
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) dq[h][v] = 0.f;
+    for (int v = 0; v < VPL / 2; ++v) dq[h][v] = make_float2(0.f, 0.f);
   if (n_routed > 0) {
     const long long loff = grp * dm.list_rows + list_row_offset(dm, i);
     const float* kb = Kbar + grp * dm.T_s * D;
+    // the queries stay in registers for the second part where those suffice (shared memory costs four wavefronts a read)
+    constexpr bool Q_REGS = G <= 4;
+    [[maybe_unused]] float qr[Q_REGS ? G : 1][VPL];
     float th[G];
 #pragma unroll
     for (int h = 0; h < G; ++h) {
       float x[VPL];
       load_vec<VPL>(Q + (long long)b * dm.qs[0] + (long long)i * dm.qs[1] + (long long)(r * G + h) * dm.qs[2] + lane * VPL, x);
 #pragma unroll
-      for (int v = 0; v < VPL; ++v) q_s[warp][h][lane * VPL + v] = x[v];
+      for (int v = 0; v < VPL; ++v) {
+        q_s[warp][h][lane * VPL + v] = x[v];
+        if (Q_REGS) qr[Q_REGS ? h : 0][v] = x[v];
+      }
       th[h] = tau[((long long)b * dm.h_q + r * G + h) * dm.seq_q + i];
     }
     float dmean = 0.f;
@@ -111,19 +118,24 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
         const bool live = k < n;
         const float* kp = kb + (long long)c_s[warp][min(k, n - 1)] * D + 4 * (lane & 3);
         float x[G];
+        {
+          float2 xp[G];
 #pragma unroll
-        for (int h = 0; h < G; ++h) x[h] = 0.f;
-        float4 kv[D / 16];
+          for (int h = 0; h < G; ++h) xp[h] = make_float2(0.f, 0.f);
+          float4 kv[D / 16];
 #pragma unroll
-        for (int j = 0; j < D / 16; ++j) kv[j] = load4(kp + 16 * j);
+          for (int j = 0; j < D / 16; ++j) kv[j] = load4(kp + 16 * j);
 #pragma unroll
-        for (int j = 0; j < D / 16; ++j)
+          for (int j = 0; j < D / 16; ++j)
 #pragma unroll
-          for (int h = 0; h < G; ++h) {
-            const float4 qv = load4(&q_s[warp][h][16 * j + 4 * (lane & 3)]);
-            x[h] = fmaf(qv.x, kv[j].x, x[h]); x[h] = fmaf(qv.y, kv[j].y, x[h]);
-            x[h] = fmaf(qv.z, kv[j].z, x[h]); x[h] = fmaf(qv.w, kv[j].w, x[h]);
-          }
+            for (int h = 0; h < G; ++h) {
+              const float4 qv = load4(&q_s[warp][h][16 * j + 4 * (lane & 3)]);
+              xp[h] = __ffma2_rn(make_float2(qv.x, qv.y), make_float2(kv[j].x, kv[j].y), xp[h]);
+              xp[h] = __ffma2_rn(make_float2(qv.z, qv.w), make_float2(kv[j].z, kv[j].w), xp[h]);
+            }
+#pragma unroll
+          for (int h = 0; h < G; ++h) x[h] = xp[h].x + xp[h].y;
+        }
         float w = 0.f;
 #pragma unroll
         for (int h = 0; h < G; ++h) {
@@ -186,21 +198,26 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
           if (e0 + u < n) {
-            float dkb[VPL];
+            float2 dkb[VPL / 2];
 #pragma unroll
-            for (int v = 0; v < VPL; ++v) dkb[v] = 0.f;
+            for (int v = 0; v < VPL / 2; ++v) dkb[v] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int h = 0; h < G; ++h) {
               const float dz = m_s[warp][e0 + u][h];
-              float qv[VPL];
-              load_vec<VPL>(&q_s[warp][h][lane * VPL], qv);
+              const float2 dz2 = make_float2(dz, dz);
+              [[maybe_unused]] float qs[VPL];
+              if constexpr (!Q_REGS) load_vec<VPL>(&q_s[warp][h][lane * VPL], qs);
 #pragma unroll
-              for (int v = 0; v < VPL; ++v) {
-                dq[h][v] = fmaf(dz, kv[u][v], dq[h][v]);
-                dkb[v] = fmaf(dz, qv[v], dkb[v]);
+              for (int v = 0; v < VPL / 2; ++v) {
+                const float2 qv = Q_REGS ? make_float2(qr[Q_REGS ? h : 0][2 * v], qr[Q_REGS ? h : 0][2 * v + 1]) : make_float2(qs[2 * v], qs[2 * v + 1]);
+                dq[h][v] = __ffma2_rn(dz2, make_float2(kv[u][2 * v], kv[u][2 * v + 1]), dq[h][v]);
+                dkb[v] = __ffma2_rn(dz2, qv, dkb[v]);
               }
             }
-            add_global<VPL>(dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL, dkb);
+            float out[VPL];
+#pragma unroll
+            for (int v = 0; v < VPL / 2; ++v) { out[2 * v] = dkb[v].x; out[2 * v + 1] = dkb[v].y; }
+            add_global<VPL>(dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL, out);
           }
         }
       }
@@ -208,8 +225,10 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
   }
 #pragma unroll
   for (int h = 0; h < G; ++h)
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) dq_out[(long long)h * D + v] = dq[h][v];
+    if constexpr (VPL == 4)
+      store4(dq_out + (long long)h * D, make_float4(dq[h][0].x, dq[h][0].y, dq[h][1].x, dq[h][1].y));
+    else
+      *reinterpret_cast<float2*>(dq_out + (long long)h * D) = dq[h][0];
 }
 
 constexpr int SB_SPLIT = 4;      // warps that share a chunk = a block
