@@ -18,7 +18,7 @@
 // serves eight chunks and two shuffles per head finish a dot product); they stay in shared memory until the whole list
 // has been seen, which fixes dz.  Then lanes own head_dim slices: dq_h += dz_hc kbar_c, dkbar_c by vector reductions (the L2
 // atomic units count requests, not bytes).  8192 tokens, 32/8 heads, chunks of 64: 690 us with two sweeps of butterfly
-// reductions over the list, now 450.
+// reductions over the list, now 435.
 //
 // summaries_bwd_kernel: four warps per (batch, KV head, chunk), a quarter of its rows each: Eq. 3, kbar_c = sum_t a_t k_t with
 // a = softmax(<qbar, k_t>/sqrt(d)) (a_t = 1/B without a summary query): dk_t += a_t dkbar_c + ds_t qbar/sqrt(d),
@@ -51,7 +51,7 @@ __device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
 
 // G (heads per KV head) is a template parameter so that the per-head sums live in registers.
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(RB_WARPS * 32, G <= 4 ? 5 : 1)
+__global__ void __launch_bounds__(RB_WARPS * 32, D == 128 && G <= 4 ? 5 : 1)
 route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
                  const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
                  float* __restrict__ dQr, float* __restrict__ dKbar) {
