@@ -418,6 +418,10 @@ int dash_attn_fwd_decode(const dash_params* p, const void* Q, const void* Kcache
   if ((rc = check_device()) != DASH_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   StatusBlock* sb = at<StatusBlock>(workspace, wl.status);
+  if (decode_fused_supported(dm)) {
+    StageRange nv("dash_attn: decode step");
+    return cuda_status(launch_decode_fused(dm, Q, Kcache, Vcache, Kbar, kv_len, O, sb, st));
+  }
   int* count = at<int>(workspace, wl.count);
   int* idx = at<int>(workspace, wl.blk_idx);
   float* bias = at<float>(workspace, wl.blk_bias);
@@ -448,6 +452,10 @@ int dash_attn_fwd_decode_paged(const dash_params* p, const void* Q, const void* 
   if ((rc = check_device()) != DASH_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   StatusBlock* sb = at<StatusBlock>(workspace, wl.status);
+  if (decode_fused_supported(dm)) {
+    StageRange nv("dash_attn: decode step");
+    return cuda_status(launch_decode_fused(dm, Q, Kpool, Vpool, Kbar, kv_len, O, sb, st));
+  }
   int* count = at<int>(workspace, wl.count);
   int* idx = at<int>(workspace, wl.blk_idx);
   float* bias = at<float>(workspace, wl.blk_bias);

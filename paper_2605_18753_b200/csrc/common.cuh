@@ -307,6 +307,10 @@ int decode_sm100_min_splits(const Dims& dm);
 cudaError_t launch_decode_sm100(const Dims& dm, int n_split, const void* Q, const void* K, const void* V,
                                 const int* kv_len, const int* count, const int* blk_idx, const float* blk_bias,
                                 float* partials, void* O, StatusBlock* sb, cudaStream_t st);
+// the whole decode step (routing and attention) in one launch, for few groups and short caches
+bool decode_fused_supported(const Dims& dm);
+cudaError_t launch_decode_fused(const Dims& dm, const void* Q, const void* K, const void* V, const float* Kbar, const int* kv_len,
+                                void* O, StatusBlock* sb, cudaStream_t st);
 bool prefill_sm100_supported(const Dims& dm);
 // inputs_stable: Q, K, V were not written by the kernel launched just before on the stream
 cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const void* K, const void* V,

@@ -1,5 +1,6 @@
 // Stage 1 of a decode step inside a thread block (Eq. 2, Eq. 4, Algorithm 2, Proposition 1): chunk logits of one query row
-// per head of a group, their entmax thresholds, and the group's routed list (used by the kernels of select_decode.cu).
+// per head of a group, their entmax thresholds, and the group's routed list (used by the kernels of
+// select_decode.cu and, for few groups, by the one of decode_sm100.cu).
 #pragma once
 
 #include <type_traits>
@@ -33,12 +34,24 @@ __device__ __forceinline__ void warp_reduce_many(float (&x)[V], int lane) {
   }
 }
 
+// The group's query rows, scaled.
+template <typename T, int D, int G>
+__device__ __forceinline__ void load_query(const Dims& dm, const T* Q, int b, int r, int lane, float (&q)[G][D / 32]) {
+  constexpr int VPL = D / 32;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const T* qp = Q + (long long)b * dm.qs[0] + (long long)(r * G + g) * dm.qs[2] + lane * VPL;
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) q[g][v] = to_f32<T>(qp[v]) * dm.x_scale;
+  }
+}
+
 // Logits of candidates [c_begin, c_end), one warp per summary row, RB rows in flight per warp (warp `warp` of `n_warps`):
-// out[g * pitch + c - c_begin].  q: the group's query rows, VPL elements per lane, scaled by x_scale; kb: the lane's share
+// store(g, c, logit).  q: the group's query rows, VPL elements per lane, scaled by x_scale; kb: the lane's share
 // of summary row 0.
-template <int D, int G>
+template <int D, int G, typename Store>
 __device__ __forceinline__ void score_rows(const float (&q)[G][D / 32], const float* kb, int c_begin, int c_end, int warp, int n_warps,
-                                           int lane, float* out, long long pitch) {
+                                           int lane, Store&& store) {
   constexpr int VPL = D / 32;                 // floats per lane of one summary row
   constexpr int RB = (G <= 8) ? 4 : 2;        // rows per iteration: RB * G values reduced together (<= 32)
   for (int c0 = c_begin + warp * RB; c0 < c_end; c0 += n_warps * RB) {
@@ -69,7 +82,7 @@ __device__ __forceinline__ void score_rows(const float (&q)[G][D / 32], const fl
     constexpr int STRIDE = 32 / (RB * G);
     if (lane % STRIDE == 0) {
       const int v = lane / STRIDE, u = v / G, g = v % G;
-      if (c0 + u < c_end) out[(long long)g * pitch + c0 + u - c_begin] = part[0];
+      if (c0 + u < c_end) store(g, c0 + u, part[0]);
     }
   }
 }

@@ -13,9 +13,15 @@
 // 64-token sub-blocks, one thread block each; the block that sees the last arrival of its (batch, KV head)
 // merges the partial (m, l, O) of all splits in split order (or, without a workspace, a separate merge kernel does).
 // Every wait is bounded (DASH_ERR_TIMEOUT in the status word).
+//
+// FUSED: the whole decode step in one launch, a cluster of eight blocks per (batch, KV head), for few groups with caches of
+// up to 512 chunks, where a step is launches and round trips to L2 (one 8K cache: 13.4 us as routing and attention kernels).
+// Each block scores an eighth of the candidates and hands its logits to all eight through distributed shared memory, every
+// block routes the group for itself (decode_route.cuh) and attends its eighth of the list, and the partial results meet
+// through distributed shared memory as well.
 #include <cuda.h>
 
-#include "common.cuh"
+#include "decode_route.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 
@@ -51,7 +57,7 @@ struct MiscT {
   int nvalid[NSL][2];
   float red[2][4][NH];
   float lred[4][NH];
-  int is_last;               // this block saw the last arrival of its (batch, KV head)
+  int is_last;               // this block saw the last arrival of its (batch, KV head); FUSED: length of the list
   int idx_s[RANGE][CPS];     // first KV token of each chunk slot of each owned sub-block (paged cache: inside its page)
   int pg_s[RANGE][CPS];      // outermost TMA coordinate of the slot: the sequence, or the physical page
   float bias_s[RANGE][CPS];
@@ -63,8 +69,21 @@ constexpr size_t MISC_BYTES = sizeof(MiscT<1>) > sizeof(MiscT<2>)
 constexpr uint32_t DEC_SMEM = OFF_MISC + (uint32_t)MISC_BYTES;   // one size for every instantiation
 static_assert(DEC_SMEM <= 115712, "two blocks per SM");
 
+// FUSED: blocks per cluster, most chunks of a cache, and where the logits, the lists and (after the walk) the partial results
+// sit in the ring of tiles
+constexpr int FUSED_CS = 8, FUSED_MAX_CHUNKS = 512;
+constexpr uint32_t OFF_LIST = OFF_KV + 2 * TILE_BYTES;
+struct ListS {
+  int chunk[FUSED_MAX_CHUNKS];
+  float bias[FUSED_MAX_CHUNKS];
+  float taus[32], wsum[32];
+  int wcnt[33];
+};
+static_assert(NH * (FUSED_MAX_CHUNKS + 64) * 4 <= 2 * TILE_BYTES && sizeof(ListS) <= TILE_BYTES, "logits and lists fit the ring");
+
 struct DecodeArgs {
   Dims dm;
+  const float* Kbar;     // FUSED only
   int n_split;
   const int* kv_len;
   const int* count;
@@ -95,7 +114,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t* r) {
 // stacked along M instead: A = [V_a^T ; V_b^T] (two MN blocks of 64, 8 KiB apart), K = 64 keys, B = [P_a^T | P_b^T]
 // (N = 32): rows 0-63 / columns 0-15 hold V_a^T P_a^T and rows 64-127 / columns 16-31 hold V_b^T P_b^T (the other two
 // quadrants are not used); the two are added when the partial is written.
-template <int G, int CPS, int HD>
+template <int G, int CPS, int HD, bool FUSED>
 __global__ void __launch_bounds__(DEC_THREADS, 2)
 decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a) {
   using MiscD = MiscT<CPS>;
@@ -108,7 +127,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   auto bar = [&](int i) { return ptx::smem_u32(&misc->bar[i]); };
   volatile int* abort_flag = &misc->abort_flag;
   const int split = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
-  const int n_split = a.n_split;
+  const int n_split = FUSED ? FUSED_CS : a.n_split;      // (a cluster is the blocks of one group: split = rank)
 
   if (tid == 0) {
     misc->abort_flag = 0;
@@ -137,6 +156,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::tc_fence_before();
   }
   __syncthreads();
+  if constexpr (FUSED) ptx::cluster_sync_all();      // every block runs before anybody writes into its shared memory
   ptx::tc_fence_after();
   const uint32_t tmem = misc->tmem_base;
 
@@ -151,7 +171,33 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int c_own = (L - 1) / dm.B;
   const long long grp = (long long)b * dm.h_kv + r;
   const int spb = CPS > 1 ? 1 : dm.B / SUB;                     // sub-blocks per routed chunk (chunks >= 64 tokens)
-  int n_routed = a.count[grp];
+  ListS* list = reinterpret_cast<ListS*>(smem + OFF_LIST);
+  int n_routed;
+  if constexpr (FUSED) {
+    const int n_vis = min(c_own, dm.T_s), n_cand = max(n_vis - dm.local_blocks, 0);
+    const int stride = route_stride(n_vis), share = (n_cand + FUSED_CS - 1) / FUSED_CS;
+    float* X = reinterpret_cast<float*>(smem + OFF_KV);       // [G][stride]
+    if (split * share < n_cand) {
+      float q[G][HD / 32];
+      load_query<__nv_bfloat16, HD, G>(dm, a.Q, b, r, lane, q);
+      const float* kb = a.Kbar + grp * dm.T_s * HD + lane * (HD / 32);
+      score_rows<HD, G>(q, kb, split * share, min(n_cand, (split + 1) * share), warp, DEC_THREADS / 32, lane, [&](int g, int c, float x) {
+        const uint32_t at = sbase + OFF_KV + (uint32_t)(g * stride + c) * 4;
+#pragma unroll
+        for (int k = 0; k < FUSED_CS; ++k) ptx::st_cluster_f32(ptx::map_to_rank(at, k), x);
+      });
+    }
+    __syncwarp();
+    ptx::cluster_sync_all();
+    route_group<G, DEC_THREADS / 32, 16>(
+        dm, X, stride, n_cand, n_vis, (n_vis + 31) / 32, list->taus, list->wsum, list->wcnt, warp, lane, [](int, uint32_t) {},
+        [&](int n) { if (tid == 0) misc->is_last = n; }, [&](int pos, int c, float bias) { list->chunk[pos] = c; list->bias[pos] = bias; });
+    ptx::fence_proxy_async_smem();       // the ring is TMA's from here on
+    __syncthreads();
+    n_routed = misc->is_last;            // (not in the ring: the producer may already be refilling that)
+  } else {
+    n_routed = a.count[grp];
+  }
   DASH_CHECK(n_routed >= 0 && n_routed <= min(c_own, dm.T_s), a.sb, 310, n_routed = 0);
   const int n_routed_sub = CPS > 1 ? (n_routed + CPS - 1) / CPS : n_routed * spb;
   const int own_tokens = L - c_own * dm.B;                       // 1 .. B
@@ -175,11 +221,11 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
           for (int s = 0; s < CPS; ++s) {
             const int e = e0 + min(s, m - 1);
-            int cc = a.blk_idx[loff + e];
+            int cc = FUSED ? list->chunk[e] : a.blk_idx[loff + e];
             DASH_CHECK(cc >= 0 && cc < c_own, a.sb, 311, cc = 0);
             kv_locate(dm, b, cc * dm.B, &misc->pg_s[k][s], &misc->idx_s[k][s]);
             DASH_CHECK(!dm.page_table || (unsigned)misc->pg_s[k][s] < (unsigned)dm.num_pages, a.sb, 313, misc->pg_s[k][s] = 0);
-            misc->bias_s[k][s] = a.blk_bias[loff + e];
+            misc->bias_s[k][s] = FUSED ? list->bias[e] : a.blk_bias[loff + e];
           }
           misc->nval_s[k] = (unsigned short)(m * dm.B);
         } else {
@@ -198,10 +244,10 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       float bs;
       if (it < n_routed_sub) {
         const int e = it / spb, sub = it % spb;
-        int cc = a.blk_idx[loff + e];
+        int cc = FUSED ? list->chunk[e] : a.blk_idx[loff + e];
         DASH_CHECK(cc >= 0 && cc < c_own, a.sb, 312, cc = 0);
         tok0 = cc * dm.B + sub * SUB;
-        bs = a.blk_bias[loff + e];
+        bs = FUSED ? list->bias[e] : a.blk_bias[loff + e];
         nv = SUB;
       } else {
         const int sub = it - n_routed_sub;
@@ -446,14 +492,15 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const long long pbase = (((long long)b * dm.h_q + (long long)r * G) * n_split + split) * (HD + 2);
 #pragma unroll
     for (int h = 0; h < G; ++h) {
-      float* pp = a.partials + pbase + (long long)h * n_split * (HD + 2);
-      if (tid < HD) pp[2 + tid] = (n_steps > 0) ? __uint_as_float(o[h]) : 0.f;   // thread tid holds O^T[d = tid][h]
+      // (m, l, O); FUSED: O, m, l in this block's own ring, whose tiles have all been consumed
+      float* pp = FUSED ? reinterpret_cast<float*>(smem + OFF_KV) + h * (HD + 4) : a.partials + pbase + (long long)h * n_split * (HD + 2);
+      if (tid < HD) pp[(FUSED ? 0 : 2) + tid] = (n_steps > 0) ? __uint_as_float(o[h]) : 0.f;   // thread tid holds O^T[d = tid][h]
       if (tid == h) {
-        pp[0] = (n_steps > 0) ? m[h] * 0.6931471805599453f : -INFINITY;   // the merge works in natural-log units
-        pp[1] = misc->lred[0][h] + misc->lred[1][h] + misc->lred[2][h] + misc->lred[3][h];
+        pp[FUSED ? HD : 0] = (n_steps > 0) ? m[h] * 0.6931471805599453f : -INFINITY;   // the merge works in natural-log units
+        pp[FUSED ? HD + 1 : 1] = misc->lred[0][h] + misc->lred[1][h] + misc->lred[2][h] + misc->lred[3][h];
       }
     }
-    __threadfence();        // the partial is visible device-wide before this block counts itself as arrived
+    if constexpr (!FUSED) __threadfence();        // the partial is visible device-wide before this block counts itself as arrived
     ptx::tc_fence_before();
   }
 
@@ -462,7 +509,42 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
   }
-  if (a.O != nullptr) {
+  if constexpr (FUSED) {
+    // ---------------- rank k merges the heads k, k + 8 from all eight blocks' partial results, in rank order
+    __syncwarp();
+    ptx::cluster_sync_all();
+    constexpr int VPL = HD / 32;
+    for (int h = split + FUSED_CS * warp; h < G; h += FUSED_CS * (DEC_THREADS / 32)) {
+      const uint32_t at = sbase + OFF_KV + (uint32_t)h * (HD + 4) * 4;
+      const uint32_t mine = ptx::map_to_rank(at, lane & (FUSED_CS - 1));
+      const float ms = ptx::ld_cluster_f32(mine + HD * 4), ls = ptx::ld_cluster_f32(mine + HD * 4 + 4);
+      float2 o[FUSED_CS][VPL / 2];
+#pragma unroll
+      for (int k = 0; k < FUSED_CS; ++k)
+#pragma unroll
+        for (int v = 0; v < VPL / 2; ++v) o[k][v] = ptx::ld_cluster_f32x2(ptx::map_to_rank(at, k) + (lane * VPL + 2 * v) * 4);
+      const float w = ms > -INFINITY ? __expf(ms - warp_max(ms)) : 0.f;
+      const float Lsum = warp_sum(lane < FUSED_CS ? w * ls : 0.f);
+      float2 acc[VPL / 2];
+#pragma unroll
+      for (int v = 0; v < VPL / 2; ++v) acc[v] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < FUSED_CS; ++k) {
+        const float wk = __shfl_sync(0xffffffffu, w, k);
+#pragma unroll
+        for (int v = 0; v < VPL / 2; ++v) { acc[v].x += wk * o[k][v].x; acc[v].y += wk * o[k][v].y; }
+      }
+      const float inv = Lsum > 0.f ? 1.f / Lsum : 0.f;
+      __nv_bfloat16* op = a.O + (long long)b * dm.os[0] + (long long)(r * G + h) * dm.os[2] + lane * VPL;
+#pragma unroll
+      for (int v = 0; v < VPL / 2; ++v) {
+        op[2 * v] = __float2bfloat16_rn(acc[v].x * inv);
+        op[2 * v + 1] = __float2bfloat16_rn(acc[v].y * inv);
+      }
+    }
+    __syncwarp();
+    ptx::cluster_sync_all();      // nobody leaves while a peer may still read its shared memory
+  } else if (a.O != nullptr) {
     // ---------------- the last split of this (batch, KV head) to arrive merges all of them, in split order
     int* counter = arrival_counters(a.sb) + grp;
     if (tid == 0) {
@@ -541,41 +623,75 @@ int decode_sm100_min_splits(const Dims& dm) {
   return (max_items + MAX_RANGE - 1) / MAX_RANGE;
 }
 
+template <int G, int CPS, int HD, bool FUSED>
+static cudaError_t launch_one(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeArgs& a, cudaStream_t st) {
+  auto kern = decode_sm100_kernel<G, CPS, HD, FUSED>;
+  static std::atomic<unsigned long long> configured{0};
+  if (cudaError_t e = allow_dynamic_smem(kern, DEC_SMEM, configured); e != cudaSuccess) return e;
+  const dim3 grid(FUSED ? FUSED_CS : a.n_split, a.dm.h_kv, a.dm.batch);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(DEC_THREADS);
+  cfg.dynamicSmemBytes = DEC_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_chained
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = FUSED_CS;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = FUSED ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tk, tv, a);
+  count_launch();
+  return e;
+}
+
+template <int CPS, int HD, bool FUSED>
+static cudaError_t launch_group_size(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeArgs& a, cudaStream_t st) {
+  switch (a.dm.g_q) {
+    case 1: return launch_one<1, CPS, HD, FUSED>(tk, tv, a, st);
+    case 2: return launch_one<2, CPS, HD, FUSED>(tk, tv, a, st);
+    case 4: return launch_one<4, CPS, HD, FUSED>(tk, tv, a, st);
+    case 8: return launch_one<8, CPS, HD, FUSED>(tk, tv, a, st);
+    case 16: return launch_one<16, CPS, HD, FUSED>(tk, tv, a, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <bool FUSED>
+static cudaError_t launch_any(DecodeArgs& a, const void* K, const void* V, cudaStream_t st) {
+  const Dims& dm = a.dm;
+  CUtensorMap tk, tv;
+  if (!make_kv_map(&tk, K, dm, dm.ks) || !make_kv_map(&tv, V, dm, dm.vs)) return cudaErrorInvalidValue;
+  if (dm.d == 128)
+    return dm.B >= SUB ? launch_group_size<1, 128, FUSED>(tk, tv, a, st) : dm.B == 32 ? launch_group_size<2, 128, FUSED>(tk, tv, a, st)
+                                                                                     : launch_group_size<4, 128, FUSED>(tk, tv, a, st);
+  return dm.B >= SUB ? launch_group_size<1, 64, FUSED>(tk, tv, a, st) : dm.B == 32 ? launch_group_size<2, 64, FUSED>(tk, tv, a, st)
+                                                                                   : launch_group_size<4, 64, FUSED>(tk, tv, a, st);
+}
+
 cudaError_t launch_decode_sm100(const Dims& dm, int n_split, const void* Q, const void* K, const void* V,
                                 const int* kv_len, const int* count, const int* blk_idx, const float* blk_bias,
                                 float* partials, void* O, StatusBlock* sb, cudaStream_t st) {
-  DecodeArgs a;
+  DecodeArgs a = {};
   a.O = (__nv_bfloat16*)O;
   a.dm = dm; a.n_split = n_split; a.kv_len = kv_len; a.count = count; a.blk_idx = blk_idx; a.blk_bias = blk_bias;
   a.Q = (const __nv_bfloat16*)Q; a.partials = partials; a.sb = sb;
-  CUtensorMap tk, tv;
-  if (!make_kv_map(&tk, K, dm, dm.ks) || !make_kv_map(&tv, V, dm, dm.vs)) return cudaErrorInvalidValue;
-  dim3 grid(n_split, dm.h_kv, dm.batch);
-  cudaError_t le = cudaSuccess;
-#define DASH_DEC_HD(G, C, H)                                                                                    \
-  {                                                                                                             \
-    static std::atomic<unsigned long long> configured{0};                                                       \
-    cudaError_t e = allow_dynamic_smem(decode_sm100_kernel<G, C, H>, DEC_SMEM, configured);                     \
-    if (e != cudaSuccess) return e;                                                                             \
-    le = launch_chained(decode_sm100_kernel<G, C, H>, grid, dim3(DEC_THREADS), DEC_SMEM, st, tk, tv, a);        \
-  }
-#define DASH_DEC_TC(G, C) \
-  if (dm.d == 128) DASH_DEC_HD(G, C, 128) else DASH_DEC_HD(G, C, 64)
-#define DASH_DEC_G(C)                                  \
-  switch (dm.g_q) {                                    \
-    case 1: DASH_DEC_TC(1, C); break;                  \
-    case 2: DASH_DEC_TC(2, C); break;                  \
-    case 4: DASH_DEC_TC(4, C); break;                  \
-    case 8: DASH_DEC_TC(8, C); break;                  \
-    case 16: DASH_DEC_TC(16, C); break;                \
-    default: return cudaErrorInvalidValue;             \
-  }
-  if (dm.B >= SUB) { DASH_DEC_G(1) } else if (dm.B == 32) { DASH_DEC_G(2) } else { DASH_DEC_G(4) }
-#undef DASH_DEC_G
-#undef DASH_DEC_TC
-#undef DASH_DEC_HD
-  count_launch();
-  return le;
+  return launch_any<false>(a, K, V, st);
+}
+
+// One launch for the step where all clusters fit the GPU at once (two blocks on each of 148 SMs).
+bool decode_fused_supported(const Dims& dm) {
+  return decode_sm100_min_splits(dm) > 0 && dm.T_s >= 1 && dm.T_s <= FUSED_MAX_CHUNKS && (long long)dm.batch * dm.h_kv * FUSED_CS <= 2 * 148;
+}
+
+cudaError_t launch_decode_fused(const Dims& dm, const void* Q, const void* K, const void* V, const float* Kbar, const int* kv_len,
+                                void* O, StatusBlock* sb, cudaStream_t st) {
+  DecodeArgs a = {};
+  a.O = (__nv_bfloat16*)O;
+  a.dm = dm; a.Kbar = Kbar; a.kv_len = kv_len; a.Q = (const __nv_bfloat16*)Q; a.sb = sb;
+  return launch_any<true>(a, K, V, st);
 }
 
 }  // namespace dash

@@ -52,18 +52,6 @@ __device__ __forceinline__ void route_to_global(const Dims& dm, float* X, int st
                            });
 }
 
-// The group's query rows, scaled.
-template <typename T, int D, int G>
-__device__ __forceinline__ void load_query(const Dims& dm, const T* Q, int b, int r, int lane, float (&q)[G][D / 32]) {
-  constexpr int VPL = D / 32;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const T* qp = Q + (long long)b * dm.qs[0] + (long long)(r * G + g) * dm.qs[2] + lane * VPL;
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) q[g][v] = to_f32<T>(qp[v]) * dm.x_scale;
-  }
-}
-
 template <typename T, int D, int G>
 __global__ void __launch_bounds__(SL_WARPS * 32, G * D <= 1024 ? 4 : 2)
 decode_select_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ kv_len, RouteOut out) {
@@ -86,7 +74,7 @@ decode_select_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__
     float q[G][D / 32];
     load_query<T, D, G>(dm, Q, b, r, lane, q);
     const float* kb = Kbar + ((long long)b * dm.h_kv + r) * dm.T_s * D + lane * (D / 32);
-    score_rows<D, G>(q, kb, 0, n_cand, warp, SL_WARPS, lane, X, stride);
+    score_rows<D, G>(q, kb, 0, n_cand, warp, SL_WARPS, lane, [&](int g, int c, float x) { X[(size_t)g * stride + c] = x; });
   }
   __syncthreads();
   route_to_global<G, SL_WARPS, 16>(dm, X, stride, n_cand, n_vis, c_own, taus, wsum, wcnt, out, b, r, warp, lane);
@@ -109,7 +97,8 @@ decode_scores_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__
   float q[G][D / 32];
   load_query<T, D, G>(dm, Q, b, r, lane, q);
   const float* kb = Kbar + ((long long)b * dm.h_kv + r) * dm.T_s * D + lane * (D / 32);
-  score_rows<D, G>(q, kb, c_begin, c_end, warp, SC_WARPS, lane, xs + ((long long)b * dm.h_kv + r) * G * dm.T_s + c_begin, dm.T_s);
+  float* xo = xs + ((long long)b * dm.h_kv + r) * G * dm.T_s;
+  score_rows<D, G>(q, kb, c_begin, c_end, warp, SC_WARPS, lane, [&](int g, int c, float x) { xo[(long long)g * dm.T_s + c] = x; });
 }
 
 template <int G>
