@@ -523,7 +523,8 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int k = 0; k < FUSED_CS; ++k)
 #pragma unroll
         for (int v = 0; v < VPL / 2; ++v) o[k][v] = ptx::ld_cluster_f32x2(ptx::map_to_rank(at, k) + (lane * VPL + 2 * v) * 4);
-      const float w = ms > -INFINITY ? __expf(ms - warp_max(ms)) : 0.f;
+      const float M = warp_max(ms);           // (by all lanes, whatever their split holds: a warp-wide instruction)
+      const float w = ms > -INFINITY ? __expf(ms - M) : 0.f;
       const float Lsum = warp_sum(lane < FUSED_CS ? w * ls : 0.f);
       float2 acc[VPL / 2];
 #pragma unroll
