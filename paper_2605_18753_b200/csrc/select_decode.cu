@@ -4,7 +4,7 @@
 // Caches of up to 512 chunks take one kernel, one block per (batch, KV head):
 //   decode_select_kernel  streams kbar with fully coalesced row reads (one warp per row, several rows in flight), keeps the
 //                         scaled chunk logits x = gamma(alpha-1) <q, kbar_c>/sqrt(d) of the g_q heads in shared memory and
-//                         routes the group (decode_route.cuh).  Four blocks per SM: one group's routing, which moves
+//                         routes the group (decode_route.cuh).  Two to four blocks per SM: one group's routing, which moves
 //                         nothing, passes under other groups' streams.
 // Longer caches are split in two:
 //   decode_scores_kernel  many thread blocks per (batch, KV head) write the logits to a small fp32 scratch (b * h_q * T_s
@@ -23,7 +23,6 @@ constexpr int SC_WARPS = 8;
 constexpr int SC_ROWS_PER_BLOCK = 256;   // summary rows one thread block scores
 constexpr int RT_THREADS = 512;      // 128 registers per thread: a Newton warp keeps 64 logits per lane in registers
 constexpr int RT_LOADS = 4;           // logits per head a thread requests per sweep (2048 candidates: one sweep)
-constexpr int SL_WARPS = 8;
 constexpr int SL_MAX_CHUNKS = 512;    // a Newton warp keeps 16 logits per lane: 64 registers, four blocks per SM
 
 struct RouteOut {
@@ -52,8 +51,8 @@ __device__ __forceinline__ void route_to_global(const Dims& dm, float* X, int st
                            });
 }
 
-template <typename T, int D, int G>
-__global__ void __launch_bounds__(SL_WARPS * 32, G * D <= 1024 ? 4 : 2)
+template <typename T, int D, int G, int NW>
+__global__ void __launch_bounds__(NW * 32, (G * D <= 1024 ? 32 : 16) / NW)
 decode_select_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ kv_len, RouteOut out) {
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -74,10 +73,10 @@ decode_select_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__
     float q[G][D / 32];
     load_query<T, D, G>(dm, Q, b, r, lane, q);
     const float* kb = Kbar + ((long long)b * dm.h_kv + r) * dm.T_s * D + lane * (D / 32);
-    score_rows<D, G>(q, kb, 0, n_cand, warp, SL_WARPS, lane, [&](int g, int c, float x) { X[(size_t)g * stride + c] = x; });
+    score_rows<D, G>(q, kb, 0, n_cand, warp, NW, lane, [&](int g, int c, float x) { X[(size_t)g * stride + c] = x; });
   }
   __syncthreads();
-  route_to_global<G, SL_WARPS, 16>(dm, X, stride, n_cand, n_vis, c_own, taus, wsum, wcnt, out, b, r, warp, lane);
+  route_to_global<G, NW, 16>(dm, X, stride, n_cand, n_vis, c_own, taus, wsum, wcnt, out, b, r, warp, lane);
 }
 
 template <typename T, int D, int G>
@@ -160,9 +159,12 @@ static cudaError_t launch_group_size(const Dims& dm, const void* Q, const float*
                                      float* scratch, cudaStream_t st) {
   const size_t smem = route_smem(dm);
   // one block per group up to 512 chunks: a launch and the logits' way through L2 saved
+  // (sixteen warps instead of eight where rows are long: a row is one block's chain of loads)
   if (dm.T_s <= SL_MAX_CHUNKS) {
-    cudaError_t e = launch_chained(decode_select_kernel<T, D, G>, dim3(dm.h_kv, dm.batch), dim3(SL_WARPS * 32), smem, st, dm,
-                                   (const T*)Q, Kbar, kv_len, out);
+    const dim3 grid(dm.h_kv, dm.batch);
+    cudaError_t e = dm.T_s > SL_MAX_CHUNKS / 4
+                        ? launch_chained(decode_select_kernel<T, D, G, 16>, grid, dim3(16 * 32), smem, st, dm, (const T*)Q, Kbar, kv_len, out)
+                        : launch_chained(decode_select_kernel<T, D, G, 8>, grid, dim3(8 * 32), smem, st, dm, (const T*)Q, Kbar, kv_len, out);
     count_launch();
     return e;
   }
