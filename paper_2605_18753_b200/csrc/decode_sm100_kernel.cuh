@@ -134,6 +134,13 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int split = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
   const int n_split = FUSED ? NC : a.n_split;      // (a cluster is the blocks of one group: split = rank)
 
+  // A block of a short list lives for a few round trips to memory, so independent ones start together: the length (the
+  // caller's input, not a product of the chain) and the descriptors here, the list's length and the status word behind the wait.
+  int L = a.kv_len ? a.kv_len[b] : dm.seq_kv;
+  if (tid == 128) {
+    ptx::prefetch_tensormap(&tmK);
+    ptx::prefetch_tensormap(&tmV);
+  }
   if (tid == 0) {
     misc->abort_flag = 0;
     if ((sbase & 1023u) != 0u) {
@@ -166,18 +173,18 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const uint32_t tmem = misc->tmem_base;
 
   // barriers and tensor memory are set up; everything below reads what the routing kernels wrote
-  int L = a.kv_len ? a.kv_len[b] : dm.seq_kv;   // the caller's input, not a product of the chain: read it before the wait
   chain_wait();
   chain_release();
+  const long long grp = (long long)b * dm.h_kv + r;
+  int n_routed = 0;
+  if constexpr (!FUSED) n_routed = a.count[grp];
   // an error already in the status word makes every role leave at its first wait (see the prefill kernel)
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
   L = max(1, min(L, dm.seq_kv));
-  const int c_own = (L - 1) / dm.B;
-  const long long grp = (long long)b * dm.h_kv + r;
+  const int c_own = (L - 1) >> dm.log_b;
   const int spb = CPS > 1 ? 1 : dm.B / SUB;                     // sub-blocks per routed chunk (chunks >= 64 tokens)
   ListS* list = reinterpret_cast<ListS*>(smem + OFF_LIST);
-  int n_routed;
   if constexpr (FUSED) {
     const int n_vis = min(c_own, dm.T_s), n_cand = max(n_vis - dm.local_blocks, 0);
     const int stride = route_stride(n_vis), share = (n_cand + NC - 1) / NC;
@@ -200,8 +207,6 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::fence_proxy_async_smem();       // the ring is TMA's from here on
     __syncthreads();
     n_routed = misc->is_last;            // (not in the ring: the producer may already be refilling that)
-  } else {
-    n_routed = a.count[grp];
   }
   DASH_CHECK(n_routed >= 0 && n_routed <= min(c_own, dm.T_s), a.sb, 310, n_routed = 0);
   const int n_routed_sub = CPS > 1 ? (n_routed + CPS - 1) / CPS : n_routed * spb;
@@ -266,8 +271,6 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
     __syncwarp();
     if (lane == 0) {
-      ptx::prefetch_tensormap(&tmK);
-      ptx::prefetch_tensormap(&tmV);
       bool ok = true;
       int s = 0, ph = 1;
       for (int j = 0; j < n_steps && ok; ++j) {

@@ -51,7 +51,7 @@ __device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
 
 // G (heads per KV head) is a template parameter so that the per-head sums live in registers.
 template <typename T, int D, int G>
-__global__ void __launch_bounds__(RB_WARPS * 32, D == 128 && G <= 4 ? 5 : 1)
+__global__ void __launch_bounds__(RB_WARPS * 32, G > 4 ? 1 : D == 128 ? 5 : 7)
 route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
                  const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
                  float* __restrict__ dQr, float* __restrict__ dKbar) {
