@@ -24,6 +24,12 @@ cudaError_t launch_decode_sm100(const Dims& dm, int n_split, const void* Q, cons
   a.O = (__nv_bfloat16*)O;
   a.dm = dm; a.n_split = n_split; a.kv_len = kv_len; a.count = count; a.blk_idx = blk_idx; a.blk_bias = blk_bias;
   a.Q = (const __nv_bfloat16*)Q; a.partials = partials; a.sb = sb;
+  // Every block at once: more and shorter splits are the shorter chain, and every group keeps the grid's.  In waves, what a block
+  // costs beside its share counts.  (The separate merge kernel, O null, reads every split's slot.)
+  a.resident = 2 * current_sm_count();
+  const bool waves = (long long)n_split * dm.batch * dm.h_kv > a.resident;
+  a.least = O && waves ? 8 : 0;
+  if (a.least == 0) a.resident = 1 << 30;
   return launch_any<0>(a, K, V, st);
 }
 

@@ -32,6 +32,7 @@ struct DecodeArgs {
   Dims dm;
   const float* Kbar;     // FUSED only
   int n_split;
+  int resident, least;   // blocks that are resident at once; sub-blocks a split has at least, where a group may use fewer splits than the grid has (0: it may not)
   const int* kv_len;
   const int* count;
   const int* blk_idx;
@@ -132,11 +133,36 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   auto bar = [&](int i) { return ptx::smem_u32(&misc->bar[i]); };
   volatile int* abort_flag = &misc->abort_flag;
   const int split = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
-  const int n_split = FUSED ? NC : a.n_split;      // (a cluster is the blocks of one group: split = rank)
+  int n_split = FUSED ? NC : a.n_split;      // (a cluster is the blocks of one group: split = rank)
 
   // A block of a short list lives for a few round trips to memory, so independent ones start together: the length (the
   // caller's input, not a product of the chain) and the descriptors here, the list's length and the status word behind the wait.
   int L = a.kv_len ? a.kv_len[b] : dm.seq_kv;
+  L = max(1, min(L, dm.seq_kv));
+  const int c_own = (L - 1) >> dm.log_b;
+  const long long grp = (long long)b * dm.h_kv + r;
+  const int spb = CPS > 1 ? 1 : dm.B / SUB;                     // sub-blocks per routed chunk (chunks >= 64 tokens)
+  const int own_tokens = L - c_own * dm.B;                       // 1 .. B
+  int n_routed = 0, n_routed_sub = 0, n_items = 0;
+  auto list_size = [&]() {
+    DASH_CHECK(n_routed >= 0 && n_routed <= min(c_own, dm.T_s), a.sb, 310, n_routed = 0);
+    n_routed_sub = CPS > 1 ? (n_routed + CPS - 1) / CPS : n_routed * spb;
+    n_items = n_routed_sub + (own_tokens + SUB - 1) / SUB;
+  };
+  // A short list takes fewer splits than the grid has: a block costs about six sub-blocks of streaming beside its share
+  // (48 paged sequences of 1K to 32K, lists of 20 chunks on average and up to 128).  A surplus block leaves at once, one that
+  // is not among the first before it has set anything up.
+  bool waited = false;
+  if constexpr (!FUSED) {
+    if ((long long)blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z) >= a.resident) {
+      chain_wait();
+      waited = true;
+      n_routed = a.count[grp];
+      list_size();
+      if (a.least > 0) n_split = max(1, min(n_split, n_items / a.least));
+      if (split >= n_split) return;
+    }
+  }
   if (tid == 128) {
     ptx::prefetch_tensormap(&tmK);
     ptx::prefetch_tensormap(&tmV);
@@ -173,17 +199,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const uint32_t tmem = misc->tmem_base;
 
   // barriers and tensor memory are set up; everything below reads what the routing kernels wrote
-  chain_wait();
+  if (!waited) chain_wait();
   chain_release();
-  const long long grp = (long long)b * dm.h_kv + r;
-  int n_routed = 0;
-  if constexpr (!FUSED) n_routed = a.count[grp];
+  if (!FUSED && !waited) n_routed = a.count[grp];
   // an error already in the status word makes every role leave at its first wait (see the prefill kernel)
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
-  L = max(1, min(L, dm.seq_kv));
-  const int c_own = (L - 1) >> dm.log_b;
-  const int spb = CPS > 1 ? 1 : dm.B / SUB;                     // sub-blocks per routed chunk (chunks >= 64 tokens)
   ListS* list = reinterpret_cast<ListS*>(smem + OFF_LIST);
   if constexpr (FUSED) {
     const int n_vis = min(c_own, dm.T_s), n_cand = max(n_vis - dm.local_blocks, 0);
@@ -208,10 +229,19 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __syncthreads();
     n_routed = misc->is_last;            // (not in the ring: the producer may already be refilling that)
   }
-  DASH_CHECK(n_routed >= 0 && n_routed <= min(c_own, dm.T_s), a.sb, 310, n_routed = 0);
-  const int n_routed_sub = CPS > 1 ? (n_routed + CPS - 1) / CPS : n_routed * spb;
-  const int own_tokens = L - c_own * dm.B;                       // 1 .. B
-  const int n_items = n_routed_sub + (own_tokens + SUB - 1) / SUB;
+  if (!waited) {
+    list_size();
+    if constexpr (!FUSED) {
+      if (a.least > 0) n_split = max(1, min(n_split, n_items / a.least));
+      if (split >= n_split) {
+        if (warp == 5) {
+          ptx::tc_fence_after();
+          ptx::tmem_dealloc(tmem, TMEM_COLS);
+        }
+        return;
+      }
+    }
+  }
   const int per = (n_items + n_split - 1) / n_split;
   const int lo = min(n_items, split * per), hi = min(n_items, lo + per);
   const int n_own = hi - lo;                                     // <= MAX_RANGE by the host's choice of n_split
@@ -497,18 +527,19 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + comb[tid * NH + h]);
       }
     }
-    const long long pbase = (((long long)b * dm.h_q + (long long)r * G) * n_split + split) * (HD + 2);
+    const int pitch = a.n_split;             // partial results of a head
+    const long long pbase = (((long long)b * dm.h_q + (long long)r * G) * pitch + split) * (HD + 2);
 #pragma unroll
     for (int h = 0; h < G; ++h) {
       // (m, l, O); FUSED: O, m, l in this block's own ring, whose tiles have all been consumed
-      float* pp = FUSED ? reinterpret_cast<float*>(smem + OFF_KV) + h * (HD + 4) : a.partials + pbase + (long long)h * n_split * (HD + 2);
+      float* pp = FUSED ? reinterpret_cast<float*>(smem + OFF_KV) + h * (HD + 4) : a.partials + pbase + (long long)h * pitch * (HD + 2);
       if (tid < HD) pp[(FUSED ? 0 : 2) + tid] = (n_steps > 0) ? __uint_as_float(o[h]) : 0.f;   // thread tid holds O^T[d = tid][h]
       if (tid == h) {
         pp[FUSED ? HD : 0] = (n_steps > 0) ? m[h] * 0.6931471805599453f : -INFINITY;   // the merge works in natural-log units
         pp[FUSED ? HD + 1 : 1] = misc->lred[0][h] + misc->lred[1][h] + misc->lred[2][h] + misc->lred[3][h];
       }
     }
-    if constexpr (!FUSED) __threadfence();        // the partial is visible device-wide before this block counts itself as arrived
+    if (!FUSED && n_split > 1) __threadfence();        // the partial is visible device-wide before this block counts itself as arrived
     ptx::tc_fence_before();
   }
 
@@ -557,8 +588,8 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     // ---------------- the last split of this (batch, KV head) to arrive merges all of them, in split order
     int* counter = arrival_counters(a.sb) + grp;
     if (tid == 0) {
-      const bool last = atomicAdd(counter, 1) == n_split - 1;
-      if (last) *counter = 0;          // every split has arrived: the counter is ready for the next launch
+      const bool last = n_split == 1 || atomicAdd(counter, 1) == n_split - 1;
+      if (last && n_split > 1) *counter = 0;          // every split has arrived: the counter is ready for the next launch
       misc->is_last = last ? 1 : 0;
     }
     __syncthreads();
@@ -567,7 +598,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       constexpr int VPL = HD / 32;
       for (int h = warp; h < G; h += DEC_THREADS / 32) {
         const long long bh = (long long)b * dm.h_q + (long long)r * G + h;
-        const float* p = a.partials + bh * n_split * (HD + 2);
+        const float* p = a.partials + bh * a.n_split * (HD + 2);
         // lane s holds the weight of split s (at most 32 splits); the partial outputs are summed in split order, eight
         // loads in flight (one after another they cost a round trip to L2 each: 3.5 us at 16 splits)
         const float ms = lane < n_split ? __ldcg(p + lane * (HD + 2)) : -INFINITY;
