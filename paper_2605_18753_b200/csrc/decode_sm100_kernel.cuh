@@ -200,7 +200,6 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
   // barriers and tensor memory are set up; everything below reads what the routing kernels wrote
   if (!waited) chain_wait();
-  chain_release();
   if (!FUSED && !waited) n_routed = a.count[grp];
   // an error already in the status word makes every role leave at its first wait (see the prefill kernel)
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
@@ -544,6 +543,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   }
 
   __syncthreads();
+  // Not before: blocks of the next kernel that arrive while most of this grid still streams pile up on the SMs that were free
+  // first, and stay there (3 caches of 104448 tokens with lists of 8 to 47 chunks: 31.4 us a step instead of 24).
+  chain_release();
   if (warp == 5) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
