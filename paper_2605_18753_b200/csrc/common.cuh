@@ -250,6 +250,12 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
+
+// Zeroes n floats (16-byte aligned, n a multiple of 4) as a link of the chain: a memset node would break it (two gaps of a
+// microsecond or two around it).
+__device__ inline void zero_floats(float* p, long long n, long long thread, long long threads) {
+  for (long long k = thread * 4; k < n; k += threads * 4) *reinterpret_cast<float4*>(p + k) = make_float4(0.f, 0.f, 0.f, 0.f);
+}
 #endif
 
 void count_launch();

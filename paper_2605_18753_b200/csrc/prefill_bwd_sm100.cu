@@ -17,7 +17,7 @@
 //                           dQ += dS K accumulated in tensor memory; dbias from the row sums of dS.
 // What passes between them needs no scratch of its own: a row's statistics sit in the first eight bytes of its dQ row until
 // the dQ kernel, which owns the row, overwrites them; the counts and unions sit in the rows' regions of dbias (a row with
-// own chunk c has c entries there, and c >= 2 floor(c / 32) + 1), which is zeroed behind the dK / dV kernel.
+// own chunk c has c entries there, and c >= 2 floor(c / 32) + 1), which the dQ kernel's block zeroes for its own rows first.
 //
 // bf16 operands, fp32 accumulation.  P2 instantiations (the entry point that takes every shape, which computed P and dS in
 // fp32 when it ran on CUDA cores) carry P and dS as two bf16 terms (hi + lo, 16 bits of mantissa) through every product;
@@ -67,10 +67,15 @@ __device__ __forceinline__ long long marks_of(const Dims& dm, long long grp, int
 }
 
 __global__ void __launch_bounds__(256)
-list_marks_kernel(Dims dm, int TQ, int n_tiles, const uint32_t* __restrict__ mask, int* __restrict__ marks) {
+list_marks_kernel(Dims dm, int TQ, int n_tiles, const uint32_t* __restrict__ mask, int* __restrict__ marks, float* zero_a, float* zero_b,
+                  long long zero_n) {
   chain_wait();
   chain_release();
-  const long long warp_id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const long long thread = (long long)blockIdx.x * blockDim.x + threadIdx.x, warp_id = thread >> 5;
+  if (zero_n > 0) {            // dK, dV: several blocks of the next kernel add to them
+    zero_floats(zero_a, zero_n, thread, (long long)gridDim.x * blockDim.x);
+    zero_floats(zero_b, zero_n, thread, (long long)gridDim.x * blockDim.x);
+  }
   const int lane = threadIdx.x & 31;
   if (warp_id >= (long long)dm.batch * dm.h_kv * n_tiles) return;
   const long long grp = warp_id / n_tiles;
@@ -218,6 +223,12 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const uint32_t tmem = misc->tmem_base;
   chain_wait();
   chain_release();
+  {
+    // this tile's rows' list regions follow each other: their dbias starts from zero (the marks have been read)
+    const long long at = (long long)grp * dm.list_rows, lo = list_row_offset(dm, i0),
+                    hi = i0 + TQ < dm.seq_q ? list_row_offset(dm, i0 + TQ) : dm.list_rows;
+    for (long long k = lo + tid; k < hi; k += THREADS) a.dbias[at + k] = 0.f;
+  }
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
 
@@ -992,8 +1003,6 @@ cudaError_t launch_kernels(const BwdArgs& a, const Maps& m, cudaStream_t st) {
     count_launch();
     if (e != cudaSuccess) return e;
   }
-  const size_t list_bytes = (size_t)groups * (size_t)a.dm.list_rows * sizeof(float);
-  if (list_bytes > 0 && (e = cudaMemsetAsync(a.dbias, 0, list_bytes, st)) != cudaSuccess) return e;
   auto kern = dq::attend_bwd_dq_kernel<HD, CPS, WT, P2>;
   constexpr uint32_t smem = dq::Layout<HD, CPS, MTQ>::SMEM;
   static std::atomic<unsigned long long> configured{0};
@@ -1040,18 +1049,13 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   if (two_term) {
     const long long blocks = (long long)a.n_slices * dm.batch * dm.h_kv;
     a.n_split = (int)std::max<long long>(1, std::min<long long>({2 * n_sm / blocks, a.n_tiles / 4, 16}));
-    if (a.n_split > 1) {
-      const size_t kv_bytes = (size_t)dm.batch * dm.seq_kv * dm.h_kv * dm.d * sizeof(float);
-      if ((e = cudaMemsetAsync(dK, 0, kv_bytes, st)) != cudaSuccess) return e;
-      if ((e = cudaMemsetAsync(dV, 0, kv_bytes, st)) != cudaSuccess) return e;
-    }
   }
   // forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written)
   e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, a.stats, dO);
   if (e != cudaSuccess) return e;
   const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
   e = launch_chained(list_marks_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
-                     mask, a.marks);
+                     mask, a.marks, dK, dV, a.n_split > 1 ? (long long)dm.batch * dm.seq_kv * dm.h_kv * dm.d : 0LL);
   count_launch();
   if (e != cudaSuccess) return e;
 

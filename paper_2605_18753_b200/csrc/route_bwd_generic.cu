@@ -30,6 +30,18 @@ namespace dash {
 
 constexpr int RB_WARPS = 4;
 
+__global__ void __launch_bounds__(256) zero_kernel(float* p, long long n) {
+  chain_wait();
+  chain_release();
+  zero_floats(p, n, (long long)blockIdx.x * 256 + threadIdx.x, (long long)gridDim.x * 256);
+}
+static cudaError_t launch_zero(float* p, size_t bytes, cudaStream_t st) {
+  const long long n = (long long)(bytes / sizeof(float)), blocks = (n + 1023) / 1024;
+  cudaError_t e = launch_chained(zero_kernel, dim3((unsigned)(blocks < 2 * 148 ? blocks : 2 * 148)), dim3(256), 0, st, p, n);
+  count_launch();
+  return e;
+}
+
 // 4 or 2 consecutive floats added to global memory in one request.
 template <int V>
 __device__ __forceinline__ void add_global(float* p, const float (&x)[V]) {
@@ -64,6 +76,8 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long gw = (long long)blockIdx.x * RB_WARPS + warp;
   const long long total = (long long)dm.batch * dm.h_kv * dm.seq_q;
+  chain_wait();
+  chain_release();
   if (gw >= total) return;
   const int i = (int)(gw % dm.seq_q);
   const long long grp = gw / dm.seq_q;
@@ -240,6 +254,8 @@ summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__
   constexpr int VPL = D / 32, NB = 4;
   __shared__ float s_s[128], da_s[128];      // logits and <k_t, dkbar> of the chunk's tokens
   __shared__ float red[SB_SPLIT][D];
+  chain_wait();
+  chain_release();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = (int)(blockIdx.x % dm.T_s);
   const long long grp = blockIdx.x / dm.T_s;
@@ -344,13 +360,14 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
                              const float* tau, const float* dbias, float* dQr, float* dKbar, cudaStream_t st) {
   const size_t kb_bytes = (size_t)dm.batch * dm.h_kv * (size_t)dm.T_s * dm.d * sizeof(float);
   if (kb_bytes > 0) {
-    cudaError_t e = cudaMemsetAsync(dKbar, 0, kb_bytes, st);
+    cudaError_t e = launch_zero(dKbar, kb_bytes, st);
     if (e != cudaSuccess) return e;
   }
   const long long total = (long long)dm.batch * dm.h_kv * dm.seq_q;
   const unsigned grid = (unsigned)((total + RB_WARPS - 1) / RB_WARPS);
+  cudaError_t le = cudaSuccess;
 #define DASH_RB(T, D, GV) \
-  route_bwd_kernel<T, D, GV><<<grid, RB_WARPS * 32, 0, st>>>(dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar)
+  le = launch_chained(route_bwd_kernel<T, D, GV>, dim3(grid), dim3(RB_WARPS * 32), 0, st, dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar)
 #define DASH_RB_G(T, D)                   \
   switch (dm.g_q) {                       \
     case 1: DASH_RB(T, D, 1); break;      \
@@ -368,20 +385,21 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
 #undef DASH_RB_G
 #undef DASH_RB
   count_launch();
-  return cudaGetLastError();
+  return le;
 }
 
 cudaError_t launch_summaries_bwd(const Dims& dm, const void* K, const float* qbar, long long qbar_chunk_stride,
                                  const float* dKbar, float* dK, float* dqbar, size_t dqbar_bytes, cudaStream_t st) {
   if (dqbar && dqbar_bytes > 0) {
-    cudaError_t e = cudaMemsetAsync(dqbar, 0, dqbar_bytes, st);
+    cudaError_t e = launch_zero(dqbar, dqbar_bytes, st);
     if (e != cudaSuccess) return e;
   }
   const long long total = (long long)dm.batch * dm.h_kv * dm.T_s;
   if (total == 0) return cudaSuccess;
   const unsigned grid = (unsigned)total;
+  cudaError_t le = cudaSuccess;
 #define DASH_SB(T, D) \
-  summaries_bwd_kernel<T, D><<<grid, SB_SPLIT * 32, 0, st>>>(dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
+  le = launch_chained(summaries_bwd_kernel<T, D>, dim3(grid), dim3(SB_SPLIT * 32), 0, st, dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
   if (dm.dtype == DASH_BF16) {
     if (dm.d == 128) DASH_SB(__nv_bfloat16, 128); else DASH_SB(__nv_bfloat16, 64);
   } else {
@@ -389,7 +407,7 @@ cudaError_t launch_summaries_bwd(const Dims& dm, const void* K, const float* qba
   }
 #undef DASH_SB
   count_launch();
-  return cudaGetLastError();
+  return le;
 }
 
 }  // namespace dash
