@@ -163,9 +163,11 @@ __device__ __forceinline__ float pow_em1(float m, int e_int, float e) {
 constexpr float NEWTON_F_TOL = 4e-6f;
 
 // Start of that iteration, relative to the row's maximum, from the number of candidates n and the sums s1, s2 of (x - max)
-// and (x - max)^2.  Either side of the root is a valid start (from the left the iterates rise monotonically, from the
-// right one step lands on the left), so a row that is far from the assumptions costs a pass at worst.  Two guesses, the
-// larger is taken:
+// and (x - max)^2.  From the left of the root the iterates rise monotonically; from the right one step lands on the left, as
+// long as the start lies below the maximum (at the maximum no candidate is active and there is no step to take).  The
+// largest of n margins with sum m^e = 1 is at least n^(-1/e), so the root is at most max - n^(-1/e), and that bounds the
+// start: a row that is far from the assumptions below costs a pass at worst.  Where even that distance is lost when it is
+// added to a large maximum, the iteration itself steps back (newton_next).  Two guesses, the larger is taken:
 //   the root with every candidate taken as active (closed form for e = 1 and 2), a lower bound;
 //   the root were the candidates normal with the row's mean and deviation s: n s^e G_e(z) = 1 with z = (tau - mean) / s and
 //   G_e(z) = E[(N(0,1) - z)_+^e].  z is smooth in ln G: quartics hold it within 0.09 over G in [1e-6, 1] (e = 1), 0.07
@@ -194,7 +196,8 @@ __device__ __forceinline__ float entmax_start(float n, float s1, float s2, int e
       t = fmaxf(t, fmaf(z, sqrtf(ss / n), mean));
     }
   }
-  return fminf(fmaxf(t, -1.f), -1e-6f);
+  const float most = e_int == 1 ? 1.f / n : e_int == 2 ? rsqrtf(n) : e_int == 4 ? rsqrtf(sqrtf(n)) : 1.f;      // n^(-1/e)
+  return fminf(fmaxf(t, -1.f), -most);
 }
 
 // Newton step for the threshold, taken on h(tau) = F(tau)^(1/e) - 1 with F = sum [x - tau]_+^e (G = sum [x - tau]_+^(e-1)):
@@ -209,6 +212,14 @@ __device__ __forceinline__ float newton_delta(float F, float G, int e_int, float
   if (e_int == 2) return (F - sqrtf(F)) / G;
   if (e_int == 4) return (F - F * rsqrtf(sqrtf(F))) / G;    // F^(3/4)
   return (F - __powf(F, 1.f - 1.f / e)) / G;
+}
+
+// The next iterate, or `tau` itself once there is nothing left to do (F at its tolerance, or a step below the spacing of
+// floats).  G = 0: tau is on the maximum, because a start just below it was rounded there (|max| above about 2^23 n^(-1/e));
+// max - 1, where every row has F >= 1, goes on from the left.  G is NaN where the row holds one: no step.
+__device__ __forceinline__ float newton_next(float tau, float F, float G, int e_int, float e) {
+  if (fabsf(F - 1.f) <= NEWTON_F_TOL || !(G >= 0.f)) return tau;
+  return G > 0.f ? tau + newton_delta(F, G, e_int, e) : tau - 1.f;
 }
 
 // ---- chained launches (programmatic dependent launch).  The kernels of one forward pass run back to back on one

@@ -137,8 +137,7 @@ __device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_in
       }
       const float f = warp_sum((F[0] + F[1]) + (F[2] + F[3]));
       const float gs = warp_sum((Gs[0] + Gs[1]) + (Gs[2] + Gs[3]));
-      if (fabsf(f - 1.f) <= NEWTON_F_TOL || !(gs > 0.f)) break;
-      const float nt = tau + newton_delta(f, gs, EI, e);
+      const float nt = newton_next(tau, f, gs, EI, e);
       if (nt == tau) break;
       tau = nt;
     }

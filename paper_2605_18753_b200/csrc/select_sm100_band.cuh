@@ -299,8 +299,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const int max_it = ei ? MAX_NEWTON : MAX_NEWTON_GENERIC;
     auto newton_step = [&](float f, float g, bool& done) {
       if (done) return;
-      if (fabsf(f - 1.f) <= NEWTON_F_TOL || !(g > 0.f)) { done = true; return; }
-      const float nt = tau + newton_delta(f, g, ei, e);
+      const float nt = newton_next(tau, f, g, ei, e);
       if (nt == tau) done = true; else tau = nt;
     };
     constexpr bool CAN_HOLD = CS == 1 && SPLIT == 1;   // one thread per row: a short row can live in its registers
