@@ -3,18 +3,18 @@
 
 namespace dash {
 
-// Splits needed so that no thread block owns more than MAX_RANGE sub-blocks (0: shape not served here).
+// Splits needed so that no thread block owns more sub-blocks than its list holds (0: shape not served here).
 int decode_sm100_min_splits(const Dims& dm) {
   if (!dm.decode || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128)) return 0;
   if (dm.B != 16 && dm.B != 32 && dm.B != 64 && dm.B != 128) return 0;
   if (dm.qs[2] % 8 != 0 || tensor_map_encoder() == nullptr) return 0;
   if (dm.B < SUB) {
-    const int cps = SUB / dm.B, range = MAX_RANGE / cps;
+    const int cps = SUB / dm.B, range = max_range(dm.g_q) / cps;
     const int max_items = (dm.T_s + cps - 1) / cps + 1;
     return (max_items + range - 1) / range;
   }
-  const int max_items = (dm.T_s + 1) * (dm.B / SUB);
-  return (max_items + MAX_RANGE - 1) / MAX_RANGE;
+  const int max_items = (dm.T_s + 1) * (dm.B / SUB), range = max_range(dm.g_q);
+  return (max_items + range - 1) / range;
 }
 
 cudaError_t launch_decode_sm100(const Dims& dm, int n_split, const void* Q, const void* K, const void* V,

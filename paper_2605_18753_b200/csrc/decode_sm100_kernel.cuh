@@ -9,6 +9,10 @@
 //     O^T[d = 128 x 16 heads] += V_tile^T[128 x 128 keys] * P^T[128 keys x 16]
 // One softmax thread per key row (= TMEM lane of S^T); the per-head running maximum is shared through a
 // small shared-memory reduction, the accumulator O^T is only 16 TMEM columns, so rescaling it is cheap.
+// P enters its product as two bf16 terms (hi + lo, 16 bits of mantissa): with one, the weight of a split's own maximum was the
+// only exact one, so every change of the split count moved the output by 2e-3, and fewer splits meant a larger error
+// (48 paged caches, against float64: 2.07e-3 in up to 16 splits, 2.10e-3 in as few as the lists need, 1.66e-3 = the rounding
+// of the output now).  Up to eight heads leave half of the MMA's N = 16 free: the lo terms take it, at no further product.
 // The routed list (plus the row's own, possibly partial, chunk) is cut into n_split contiguous ranges of
 // 64-token sub-blocks, one thread block each; the block that sees the last arrival of its (batch, KV head)
 // merges the partial (m, l, O) of all splits in split order (or, without a workspace, a separate merge kernel does).
@@ -51,21 +55,22 @@ constexpr int STEP = 128;               // KV tokens per step = MMA M
 constexpr int NSL = 3;                  // ring of K and V tiles: tile 2j = K of step j, 2j + 1 = its V
 constexpr int NH = 16;                  // heads padded to the MMA N
 constexpr int DEC_THREADS = 192;
-constexpr int MAX_RANGE = 512;          // sub-blocks one thread block can own
+// sub-blocks one thread block can own (a second tile of P terms leaves less room for their list)
+__host__ __device__ constexpr int max_range(int g) { return g > 8 ? 288 : 512; }
 constexpr uint32_t TILE_BYTES = STEP * HD_MAX * 2;   // 32 KiB: two regions (d halves) of 128 rows x 128 B
 constexpr uint32_t QT_BYTES = NH * HD_MAX * 2;       // 4 KiB: two regions of 16 rows x 128 B
 constexpr uint32_t PT_BYTES = NH * STEP * 2;     // 4 KiB: two regions (key halves) of 16 rows x 128 B
 constexpr uint32_t OFF_KV = 0;
 constexpr uint32_t OFF_QT = OFF_KV + NSL * TILE_BYTES;
 constexpr uint32_t OFF_PT = OFF_QT + QT_BYTES;
-constexpr uint32_t OFF_MISC = OFF_PT + PT_BYTES;
+__host__ __device__ constexpr uint32_t off_misc(int g) { return OFF_PT + (g > 8 ? 2 : 1) * PT_BYTES; }     // the lo terms: rows 8 .. 15 of P^T, or a tile of their own
 constexpr uint32_t TMEM_COLS = 64;      // S^T buffers at columns 0 and 16, O^T at 32
 enum BarD { Q_READY = 0, S_FULL = 1, P_FULL = 3, P_EMPTY = 5, RED_BAR = 6, LRED_BAR = 8, FULL = 9, EMPTY = 9 + NSL, N_BARS = 9 + 2 * NSL };
 // CPS = routed chunks per 64-token sub-block: 1 for chunks of 64 / 128 tokens, 2 / 4 for chunks of 32 / 16 (a
 // sub-block then gathers that many chunks of the list, each fetched by its own TMA box and carrying its own bias).
-template <int CPS>
+template <int CPS, int G>
 struct MiscT {
-  static constexpr int RANGE = MAX_RANGE / CPS;   // sub-blocks one thread block can own
+  static constexpr int RANGE = max_range(G) / CPS;   // sub-blocks one thread block can own
   unsigned long long bar[N_BARS];
   uint32_t tmem_base;
   int abort_flag;
@@ -79,11 +84,12 @@ struct MiscT {
   float bias_s[RANGE][CPS];
   unsigned short nval_s[RANGE];   // valid rows of the sub-block
 };
-constexpr size_t MISC_BYTES = sizeof(MiscT<1>) > sizeof(MiscT<2>)
-                                  ? (sizeof(MiscT<1>) > sizeof(MiscT<4>) ? sizeof(MiscT<1>) : sizeof(MiscT<4>))
-                                  : (sizeof(MiscT<2>) > sizeof(MiscT<4>) ? sizeof(MiscT<2>) : sizeof(MiscT<4>));
-constexpr uint32_t DEC_SMEM = OFF_MISC + (uint32_t)MISC_BYTES;   // one size for every instantiation
-static_assert(DEC_SMEM <= 115712, "two blocks per SM");
+template <int CPS, int G>
+constexpr uint32_t dec_smem() {
+  constexpr uint32_t bytes = off_misc(G) + (uint32_t)sizeof(MiscT<CPS, G>);
+  static_assert(bytes <= 115712, "two blocks per SM");
+  return bytes;
+}
 
 // FUSED: most chunks of a cache, and where the logits, the lists and (after the walk) the partial results
 // sit in the ring of tiles
@@ -123,10 +129,10 @@ __global__ void __launch_bounds__(DEC_THREADS, 2)
 decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a) {
   constexpr bool FUSED = CS > 0;
   constexpr int NC = FUSED ? CS : 1;
-  using MiscD = MiscT<CPS>;
+  using MiscD = MiscT<CPS, G>;
   constexpr int W = SUB / CPS;          // rows of one chunk slot inside a sub-block
   extern __shared__ __align__(1024) uint8_t smem[];
-  MiscD* misc = reinterpret_cast<MiscD*>(smem + OFF_MISC);
+  MiscD* misc = reinterpret_cast<MiscD*>(smem + off_misc(G));
   const Dims& dm = a.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t sbase = ptx::smem_u32(smem);
@@ -243,7 +249,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   }
   const int per = (n_items + n_split - 1) / n_split;
   const int lo = min(n_items, split * per), hi = min(n_items, lo + per);
-  const int n_own = hi - lo;                                     // <= MAX_RANGE by the host's choice of n_split
+  const int n_own = hi - lo;                                     // <= max_range(G) by the host's choice of n_split
   const int n_steps = (n_own + 1) / 2;
 
   const long long loff = grp * dm.list_rows;
@@ -386,6 +392,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           // region of 32 rows (sub-block a's heads, then sub-block b's), 64 keys long
           const uint64_t bd = pd0 + (uint64_t)(((HD == 128 ? (k >> 2) * (PT_BYTES / 2) : 0) + (k & 3) * 32) >> 4);
           ptx::mma_bf16_ss(tmem + 2 * NH, ad, bd, IDESC_O, (j > 0 || k > 0) ? 1u : 0u);
+          if constexpr (G > 8) ptx::mma_bf16_ss(tmem + 2 * NH, ad, bd + (uint64_t)(PT_BYTES >> 4), IDESC_O, 1u);     // the lo terms
         }
         ptx::mma_commit(bar(EMPTY + vs));
         ptx::mma_commit(bar(P_EMPTY));
@@ -397,7 +404,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     // ---------------- softmax: thread = key row of the step = TMEM lane of S^T; also lane d of O^T
     const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
     const float c1 = dm.sm_scale * 1.4426950408889634f;
-    // Q^T tile: 16 rows (heads, zero beyond G) x 128 d, K-major, 128-byte swizzle; P^T rows beyond G stay zero
+    // Q^T tile: 16 rows (heads, zero beyond G) x 128 d, K-major, 128-byte swizzle; P^T rows of no head stay zero
     for (int ch = tid; ch < NH * 16; ch += 128) {
       const int h = ch >> 4, c16 = ch & 15;            // 16-byte chunk c16 of head h: d = c16*8 .. +7
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -450,12 +457,13 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         corr[h] = exp2f(m[h] - mn);     // 0 while nothing has been accumulated
         m[h] = mn;
       }
-      __nv_bfloat16 pb[G];
+      __nv_bfloat16 pb[G], pl[G];      // P = pb + pl
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         const float p = valid ? exp2f(x[h] - m[h]) : 0.f;
         l[h] = l[h] * corr[h] + p;
         pb[h] = __float2bfloat16_rn(p);
+        pl[h] = __float2bfloat16_rn(p - __bfloat162float(pb[h]));
       }
       // the previous step's PV must be done before P^T is overwritten and before O^T is rescaled
       ok = ptx::mbar_wait(bar(P_EMPTY), (j & 1) ^ 1, abort_flag);
@@ -468,7 +476,10 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         tmem_ld16(o, o_addr);
         ptx::tmem_wait_ld();
 #pragma unroll
-        for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) * corr[h]);
+        for (int h = 0; h < G; ++h) {
+          o[h] = __float_as_uint(__uint_as_float(o[h]) * corr[h]);
+          if constexpr (G <= 8) o[8 + h] = __float_as_uint(__uint_as_float(o[8 + h]) * corr[h]);
+        }
         tmem_st16(o_addr, o);
         ptx::tmem_wait_st();
       }
@@ -477,6 +488,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int h = 0; h < G; ++h) {
         const uint32_t off = half * (PT_BYTES / 2) + h * 128 + ((((row >> 3) & 7) ^ (h & 7)) << 4) + (row & 7) * 2;
         *reinterpret_cast<__nv_bfloat16*>(smem + OFF_PT + off) = pb[h];
+        *reinterpret_cast<__nv_bfloat16*>(smem + OFF_PT + off + (G <= 8 ? 8 * 128 : PT_BYTES)) = pl[h];      // (row 8 + h: the swizzle of row h)
       }
       // rows past the end of the sequence may hold anything (even NaN): zero their V rows, since 0 * NaN = NaN
       if (!valid && nval > 0 && nval < SUB) {
@@ -510,6 +522,10 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (ok && n_steps > 0) {
       tmem_ld16(o, lane_addr + 2 * NH + ((HD == 64 && (tid >> 6)) ? NH : 0));
       ptx::tmem_wait_ld();
+    }
+    if constexpr (G <= 8) {
+#pragma unroll
+      for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + __uint_as_float(o[8 + h]));
     }
     if constexpr (HD == 64) {
       // O^T[d][h] = (sub-block a's part in lane d) + (sub-block b's part in lane 64 + d): the upper lanes hand theirs
@@ -653,12 +669,13 @@ template <int G, int CPS, int HD, int CS>
 static cudaError_t launch_one(const CUtensorMap& tk, const CUtensorMap& tv, const DecodeArgs& a, cudaStream_t st) {
   auto kern = decode_sm100_kernel<G, CPS, HD, CS>;
   static std::atomic<unsigned long long> configured{0};
-  if (cudaError_t e = allow_dynamic_smem(kern, DEC_SMEM, configured); e != cudaSuccess) return e;
+  constexpr uint32_t smem = dec_smem<CPS, G>();
+  if (cudaError_t e = allow_dynamic_smem(kern, smem, configured); e != cudaSuccess) return e;
   const dim3 grid(CS > 0 ? CS : a.n_split, a.dm.h_kv, a.dm.batch);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(DEC_THREADS);
-  cfg.dynamicSmemBytes = DEC_SMEM;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_chained
