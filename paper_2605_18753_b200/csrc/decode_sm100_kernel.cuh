@@ -490,8 +490,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         *reinterpret_cast<__nv_bfloat16*>(smem + OFF_PT + off) = pb[h];
         *reinterpret_cast<__nv_bfloat16*>(smem + OFF_PT + off + (G <= 8 ? 8 * 128 : PT_BYTES)) = pl[h];      // (row 8 + h: the swizzle of row h)
       }
-      // rows past the end of the sequence may hold anything (even NaN): zero their V rows, since 0 * NaN = NaN
-      if (!valid && nval > 0 && nval < SUB) {
+      // rows past the end of the sequence may hold anything (even NaN): zero their V rows, since 0 * NaN = NaN (also in the
+      // half that repeats an odd tail's last sub-block, all of whose rows are invalid)
+      if (!valid) {
         uint8_t* vrow = smem + OFF_KV + vs * TILE_BYTES + tid * 128;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
