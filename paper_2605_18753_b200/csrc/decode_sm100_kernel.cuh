@@ -274,11 +274,15 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           }
           misc->nval_s[k] = (unsigned short)(m * dm.B);
         } else {
-          // the own chunk (shorter than a sub-block): the rows behind it are fetched but marked invalid
+          // the own chunk (shorter than a sub-block) repeats in every slot, all but the first marked invalid: the chunk behind it
+          // may lie in a page that the table does not hold
+          int pg, tok;
+          kv_locate(dm, b, c_own * dm.B, &pg, &tok);
+          DASH_CHECK(!dm.page_table || (unsigned)pg < (unsigned)dm.num_pages, a.sb, 315, pg = 0);
 #pragma unroll
           for (int s = 0; s < CPS; ++s) {
-            kv_locate(dm, b, c_own * dm.B + s * W, &misc->pg_s[k][s], &misc->idx_s[k][s]);
-            DASH_CHECK(!dm.page_table || (unsigned)misc->pg_s[k][s] < (unsigned)dm.num_pages, a.sb, 315, misc->pg_s[k][s] = 0);
+            misc->pg_s[k][s] = pg;
+            misc->idx_s[k][s] = tok;
             misc->bias_s[k][s] = 0.f;
           }
           misc->nval_s[k] = (unsigned short)(L - c_own * dm.B);
