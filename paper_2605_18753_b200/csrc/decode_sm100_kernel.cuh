@@ -495,13 +495,13 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         *reinterpret_cast<__nv_bfloat16*>(smem + OFF_PT + off + (G <= 8 ? 8 * 128 : PT_BYTES)) = pl[h];      // (row 8 + h: the swizzle of row h)
       }
       // rows past the end of the sequence may hold anything (even NaN): zero their V rows, since 0 * NaN = NaN (also in the
-      // half that repeats an odd tail's last sub-block, all of whose rows are invalid)
-      if (!valid) {
-        uint8_t* vrow = smem + OFF_KV + vs * TILE_BYTES + tid * 128;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          *reinterpret_cast<uint4*>(vrow + (q << 4)) = make_uint4(0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>(vrow + TILE_BYTES / 2 + (q << 4)) = make_uint4(0u, 0u, 0u, 0u);
+      // half that repeats an odd tail's last sub-block, all of whose rows are invalid).  By the whole warp, a row's 16-byte
+      // pieces in adjacent lanes: one row per lane would be 32 ways of bank conflict
+      if (const int first = nval - (row & 32); first < 32) {      // this warp's rows from `first` on
+        for (int q = max(first, 0) * 8 + lane; q < 32 * 8; q += 32) {
+          uint8_t* piece = smem + OFF_KV + vs * TILE_BYTES + warp * (32 * 128) + q * 16;
+          *reinterpret_cast<uint4*>(piece) = make_uint4(0u, 0u, 0u, 0u);
+          if constexpr (HD == 128) *reinterpret_cast<uint4*>(piece + TILE_BYTES / 2) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
       ptx::fence_proxy_async_smem();
