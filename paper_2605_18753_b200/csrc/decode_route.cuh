@@ -9,6 +9,16 @@
 
 namespace dash {
 
+// A sequence's length is read behind chain_wait(): the kernel before this one on the stream may be the caller's, and may be
+// writing it.  Its line is brought into L2 before the wait (a prefetch reads no value: what a later read finds there is
+// current), by one thread of the block; 48 paged caches take 88.8 us a step without that and 87 with.
+__device__ __forceinline__ void warm_length(const int* kv_len, int b) {
+  if (kv_len && threadIdx.x == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(kv_len + b));
+}
+__device__ __forceinline__ int sequence_length(const Dims& dm, const int* kv_len, int b) {
+  return max(1, min(kv_len ? kv_len[b] : dm.seq_kv, dm.seq_kv));
+}
+
 // Sum V values held by every lane across the warp with the halving butterfly: the number of live values halves per step;
 // value v ends up (fully reduced) in lane (v * 32 / V), as x[0], for V | 32.
 template <int V>

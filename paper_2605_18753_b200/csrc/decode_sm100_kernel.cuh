@@ -141,15 +141,21 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int split = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
   int n_split = FUSED ? NC : a.n_split;      // (a cluster is the blocks of one group: split = rank)
 
-  // A block of a short list lives for a few round trips to memory, so independent ones start together: the length (the
-  // caller's input, not a product of the chain) and the descriptors here, the list's length and the status word behind the wait.
-  int L = a.kv_len ? a.kv_len[b] : dm.seq_kv;
-  L = max(1, min(L, dm.seq_kv));
-  const int c_own = (L - 1) >> dm.log_b;
+  // A block of a short list lives for a few round trips to memory, so independent ones start together: the descriptors here,
+  // the lengths of sequence and list and the status word behind the wait.
+  warm_length(a.kv_len, b);
   const long long grp = (long long)b * dm.h_kv + r;
   const int spb = CPS > 1 ? 1 : dm.B / SUB;                     // sub-blocks per routed chunk (chunks >= 64 tokens)
-  const int own_tokens = L - c_own * dm.B;                       // 1 .. B
+  int L = 0, c_own = 0, own_tokens = 0;                          // own_tokens: 1 .. B
   int n_routed = 0, n_routed_sub = 0, n_items = 0;
+  auto read_lengths = [&]() {
+    const int len = a.kv_len ? a.kv_len[b] : dm.seq_kv, status = a.sb ? *reinterpret_cast<volatile int*>(&a.sb->status) : 0;
+    if constexpr (!FUSED) n_routed = a.count[grp];
+    L = max(1, min(len, dm.seq_kv));
+    c_own = (L - 1) >> dm.log_b;
+    own_tokens = L - c_own * dm.B;
+    return status;
+  };
   auto list_size = [&]() {
     DASH_CHECK(n_routed >= 0 && n_routed <= min(c_own, dm.T_s), a.sb, 310, n_routed = 0);
     n_routed_sub = CPS > 1 ? (n_routed + CPS - 1) / CPS : n_routed * spb;
@@ -159,11 +165,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   // (48 paged sequences of 1K to 32K, lists of 20 chunks on average and up to 128).  A surplus block leaves at once, one that
   // is not among the first before it has set anything up.
   bool waited = false;
+  int status = 0;
   if constexpr (!FUSED) {
     if ((long long)blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z) >= a.resident) {
       chain_wait();
       waited = true;
-      n_routed = a.count[grp];
+      status = read_lengths();
       list_size();
       if (a.least > 0) n_split = max(1, min(n_split, n_items / a.least));
       if (split >= n_split) return;
@@ -205,10 +212,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const uint32_t tmem = misc->tmem_base;
 
   // barriers and tensor memory are set up; everything below reads what the routing kernels wrote
-  if (!waited) chain_wait();
-  if (!FUSED && !waited) n_routed = a.count[grp];
+  if (!waited) {
+    chain_wait();
+    status = read_lengths();
+  }
   // an error already in the status word makes every role leave at its first wait (see the prefill kernel)
-  if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
+  if (status != 0) *abort_flag = 1;
   __syncthreads();
   ListS* list = reinterpret_cast<ListS*>(smem + OFF_LIST);
   if constexpr (FUSED) {

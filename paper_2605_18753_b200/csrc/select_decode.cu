@@ -57,10 +57,10 @@ decode_select_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__
   extern __shared__ __align__(16) float sm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = blockIdx.x, b = blockIdx.y;
-  int L = kv_len ? kv_len[b] : dm.seq_kv;     // the caller's input, not a product of the chain: read it before the wait
+  warm_length(kv_len, b);
   chain_wait();
   chain_release();
-  L = max(1, min(L, dm.seq_kv));
+  const int L = sequence_length(dm, kv_len, b);
   const int c_own = (L - 1) >> dm.log_b;
   const int n_vis = min(c_own, dm.T_s);                 // chunks before the own one: candidates, then the window
   const int n_cand = max(n_vis - dm.local_blocks, 0);   // scored by entmax
@@ -85,10 +85,10 @@ decode_scores_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__
                      float* __restrict__ xs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = blockIdx.y, b = blockIdx.z;
-  int L = kv_len ? kv_len[b] : dm.seq_kv;     // the caller's input, not a product of the chain: read it before the wait
+  warm_length(kv_len, b);
   chain_wait();
   chain_release();
-  L = max(1, min(L, dm.seq_kv));
+  const int L = sequence_length(dm, kv_len, b);
   const int n_cand = max(min((L - 1) >> dm.log_b, dm.T_s) - dm.local_blocks, 0);   // window chunks are not scored
   const int c_begin = blockIdx.x * SC_ROWS_PER_BLOCK;
   const int c_end = min(n_cand, c_begin + SC_ROWS_PER_BLOCK);
@@ -106,10 +106,10 @@ decode_route_kernel(Dims dm, const float* __restrict__ xs, const int* __restrict
   extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r = blockIdx.x, b = blockIdx.y;
-  int L = kv_len ? kv_len[b] : dm.seq_kv;     // the caller's input, not a product of the chain: read it before the wait
+  warm_length(kv_len, b);
   chain_wait();
   chain_release();
-  L = max(1, min(L, dm.seq_kv));
+  const int L = sequence_length(dm, kv_len, b);
   const int c_own = (L - 1) >> dm.log_b;
   const int n_vis = min(c_own, dm.T_s);
   const int n_cand = max(n_vis - dm.local_blocks, 0);

@@ -69,3 +69,33 @@ def test_decode_step_replays_from_a_cuda_graph():
     B.dash_attn_fwd_decode(p, q, Kc, Vc, kbar, kl, O, ws)
     torch.cuda.synchronize()
     assert torch.equal(O, replayed) and not torch.equal(O, eager)
+
+
+@pytest.mark.parametrize("batch,seq", [(2, 2048), (48, 2048), (2, 64 * 700)])      # one launch; two kernels; scores, routing and attention apart
+def test_decode_sees_the_length_that_the_kernel_before_it_wrote(batch, seq):
+    """kv_len advances on the stream right before every step, as a serving loop does it, with nothing in between."""
+    w = synth.workload("decode_128k", batch=batch, seq=seq)
+    di = synth.make_decode_inputs(w, DEV)
+    Q, K, V, full = di["Q"], di["K"], di["V"], di["kv_len"]
+    O = torch.empty_like(Q)
+    p = B.params_for_decode(Q, K, V, O, block=w.block, alpha=w.alpha, gamma=w.gamma, sigma=w.sigma)
+    kbar, ws = B.alloc_kbar(p), B.alloc_workspace(p)
+    B.dash_attn_block_summaries(p, K, kbar, kv_len=full)
+    lengths = [seq - 700 + 97 * s for s in range(8)]
+    want = []
+    for n in lengths:
+        kv = torch.full_like(full, n)
+        torch.cuda.synchronize()
+        B.dash_attn_fwd_decode(p, Q, K, V, kbar, kv, O, ws)
+        want.append(O.clone())
+    kv = torch.full_like(full, lengths[0] - 97)
+    for k in range(5):
+        got = []
+        kv.fill_(lengths[0] - 97)
+        for _ in lengths:
+            kv.add_(97)
+            B.dash_attn_fwd_decode(p, Q, K, V, kbar, kv, O, ws)
+            got.append(O.clone())
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+    assert B.dash_attn_last_status(ws) == 0
