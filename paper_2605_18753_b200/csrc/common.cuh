@@ -65,6 +65,12 @@ __host__ __device__ inline long long list_row_offset(const Dims& dm, int i) {
   return ((c * (c - 1)) >> 1 << dm.log_b) + (long long)(i & (dm.B - 1)) * c;
 }
 
+// Tensors with a broadcast dimension (stride 0 over an extent above 1, as an expanded batch or expanded KV heads have) take the
+// CUDA-core kernels: the tensor-core kernels fetch their tiles through tensor maps, which have no stride of 0.
+inline bool broadcasts(const long long* s, int batch, int tokens, int heads) {
+  return (s[0] == 0 && batch > 1) || (s[1] == 0 && tokens > 1) || (s[2] == 0 && heads > 1);
+}
+
 // Workspace: 256-byte header (status word first), then regions carved by the host.
 struct StatusBlock {
   int status;        // dash_status written by kernels (first error wins)

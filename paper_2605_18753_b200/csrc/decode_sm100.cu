@@ -8,6 +8,7 @@ int decode_sm100_min_splits(const Dims& dm) {
   if (!dm.decode || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128)) return 0;
   if (dm.B != 16 && dm.B != 32 && dm.B != 64 && dm.B != 128) return 0;
   if (dm.qs[2] % 8 != 0 || tensor_map_encoder() == nullptr) return 0;
+  if (broadcasts(dm.ks, dm.batch, dm.seq_kv, dm.h_kv) || broadcasts(dm.vs, dm.batch, dm.seq_kv, dm.h_kv)) return 0;
   if (dm.B < SUB) {
     const int cps = SUB / dm.B, range = max_range(dm.g_q) / cps;
     const int max_items = (dm.T_s + cps - 1) / cps + 1;

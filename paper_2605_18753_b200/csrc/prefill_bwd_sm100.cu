@@ -1024,7 +1024,7 @@ cudaError_t launch_two_term(const BwdArgs& a, const Maps& m, cudaStream_t st) {
 }  // namespace
 
 bool prefill_bwd_sm100_supported(const Dims& dm) {
-  if (!prefill_sm100_supported(dm)) return false;
+  if (!prefill_sm100_supported(dm) || broadcasts(dm.os, dm.batch, dm.seq_q, dm.h_q)) return false;      // (os: dO)
   return dm.qs[2] % 8 == 0 && dm.qs[1] % 8 == 0;      // 16-byte stores of dQ rows
 }
 

@@ -622,6 +622,9 @@ bool prefill_sm100_supported(const Dims& dm) {
   if (dm.decode || !dm.causal || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128)) return false;
   if (dm.B != 16 && dm.B != 32 && dm.B != 64 && dm.B != 128) return false;
   if (dm.os[2] % 8 != 0 || dm.os[1] % 8 != 0) return false;
+  if (broadcasts(dm.qs, dm.batch, dm.seq_q, dm.h_q) || broadcasts(dm.ks, dm.batch, dm.seq_kv, dm.h_kv) ||
+      broadcasts(dm.vs, dm.batch, dm.seq_kv, dm.h_kv))
+    return false;
   return tensor_map_encoder() != nullptr;
 }
 

@@ -28,7 +28,7 @@ __global__ void kbar_split_kernel(const float* __restrict__ kbar, __nv_bfloat16*
 // holds 512 candidates per row in tensor memory; clusters of 2 or 4 blocks extend that to 1024 / 2048.
 int select_sm100_token_limit(const Dims& dm) {
   if (dm.decode || !dm.causal || dm.dtype != DASH_BF16 || (dm.d != 64 && dm.d != 128) || dm.T_s < 1) return 0;
-  if (tensor_map_encoder() == nullptr) return 0;
+  if (tensor_map_encoder() == nullptr || broadcasts(dm.qs, dm.batch, dm.seq_q, dm.h_q)) return 0;
   // own chunk index <= 2048, in whole tiles
   const int tq = 128 / dm.g_q;
   const long long lim = (long long)(SELECT_MAX_CS * SELECT_CLUSTER_COLS + 1) * dm.B / tq * tq;
