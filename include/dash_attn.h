@@ -200,7 +200,9 @@ int dash_attn_attend_decode_static(const dash_params* p, const void* Q, const vo
  * mask / blk_bias as written by dash_attn_select for the same parameters.  bf16 tensors (causal) run on tensor cores with
  * P and dS carried as two bf16 terms each, fp32 and the non-causal mode on CUDA cores (one warp per row and head); either
  * way some sums are formed by fp32 atomics, so last bits vary from run to run.  No workspace: what the kernels hand to each
- * other sits in dQ and dbias until those get their values.  dash_attn_bwd_select_prefill and dash_attn_bwd_block_summaries carry dbias on through the routing. */
+ * other sits in dQ and dbias until those get their values (neither may overlap an input), and there is no status word: where a
+ * bounded device-side wait runs out, the rows and keys concerned come back as NaN in every gradient.
+ * dash_attn_bwd_select_prefill and dash_attn_bwd_block_summaries carry dbias on through the routing. */
 int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void* K, const void* V, const void* dO,
                                  const uint32_t* mask, const float* blk_bias, void* dQ, float* dK, float* dV,
                                  float* dbias, void* stream);
@@ -216,7 +218,8 @@ int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void
  * P and dS enter the dQ / dK / dV products rounded to bf16.
  *   bwd_workspace   device scratch of at least dash_attn_bwd_workspace_bytes(p) bytes, 256-byte aligned, owned by the
  *                   caller; it opens with a status word like the forward workspace's (dash_attn_last_status and
- *                   dash_attn_reset_status accept it): a bounded wait that runs out leaves DASH_ERR_TIMEOUT there.
+ *                   dash_attn_reset_status accept it): a bounded wait that runs out leaves DASH_ERR_TIMEOUT there
+ *                   (and NaN in the gradients concerned).
  * Other arguments, layouts and dtypes as for dash_attn_bwd_attend_prefill. */
 size_t dash_attn_bwd_workspace_bytes(const dash_params* p);
 int dash_attn_bwd_attend_prefill_tc(const dash_params* p, const void* Q, const void* K, const void* V, const void* dO,

@@ -87,6 +87,9 @@ constexpr int ARRIVAL_COUNTERS = 4096;
 constexpr size_t STATUS_REGION_BYTES = 256 + ARRIVAL_COUNTERS * sizeof(int);
 __host__ __device__ inline int* arrival_counters(StatusBlock* sb) { return reinterpret_cast<int*>(sb + 1); }
 
+// What a block of the backward pass leaves where a wait of it ran out: statistics and gradients that cannot be taken for
+// values, whether or not the call has a status word.
+__device__ inline float gave_up() { return __int_as_float(0x7fffffff); }      // NaN
 __device__ inline void report_error(StatusBlock* sb, int status, int detail) {
   if (!sb) return;
   if (atomicCAS(&sb->status, 0, status) == 0) sb->detail = detail;

@@ -18,6 +18,8 @@
 // What passes between them needs no scratch of its own: a row's statistics sit in the first eight bytes of its dQ row until
 // the dQ kernel, which owns the row, overwrites them; the counts and unions sit in the rows' regions of dbias (a row with
 // own chunk c has c entries there, and c >= 2 floor(c / 32) + 1), which the dQ kernel's block zeroes for its own rows first.
+// A block whose wait ran out writes NaN in the place of its statistics or gradients: the entry point without a status word has
+// no other way to say so, and what the buffers held as scratch must not pass for gradients.
 //
 // bf16 operands, fp32 accumulation.  P2 instantiations (the entry point that takes every shape, which computed P and dS in
 // fp32 when it ran on CUDA cores) carry P and dS as two bf16 terms (hi + lo, 16 bits of mantissa) through every product;
@@ -515,6 +517,17 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
   }
+  if (misc->abort_flag) {
+    // nothing of what the gradient buffers held as scratch may pass for a gradient
+    const __nv_bfloat162 nan2 = __floats2bfloat162_rn(gave_up(), gave_up());
+    for (int k = tid; k < 128 * HD / 2; k += THREADS) {
+      const int m = k / (HD / 2), i = i0 + m / g_q;
+      if (i < dm.seq_q)
+        *reinterpret_cast<__nv_bfloat162*>(a.dQ + (long long)b * dm.qs[0] + (long long)i * dm.qs[1] + (long long)(r * g_q + m % g_q) * dm.qs[2] + 2 * (k % (HD / 2))) = nan2;
+    }
+    const long long at = (long long)grp * dm.list_rows, hi = i0 + TQ < dm.seq_q ? list_row_offset(dm, i0 + TQ) : dm.list_rows;
+    for (long long k = list_row_offset(dm, i0) + tid; k < hi; k += THREADS) a.dbias[at + k] = gave_up();
+  }
   if (tid == 0 && misc->abort_flag) report_error(a.sb, DASH_ERR_TIMEOUT, 111);
 }
 
@@ -968,6 +981,13 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   if (warp == W_SD) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
+  }
+  if (misc->abort_flag) {
+    for (int k = tid; k < NKV * HD; k += THREADS) {
+      const int key = k0 + k / HD;
+      const long long at = (((long long)b * dm.seq_kv + key) * dm.h_kv + r) * HD + k % HD;
+      if (key < dm.seq_kv) a.dK[at] = a.dV[at] = gave_up();      // (what other blocks add to it does not change it)
+    }
   }
   if (tid == 0 && misc->abort_flag) report_error(a.sb, DASH_ERR_TIMEOUT, 121);
 }

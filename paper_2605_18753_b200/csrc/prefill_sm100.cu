@@ -595,6 +595,10 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   }
 
   __syncthreads();
+  if (P2 && a.stats.base && misc->abort_flag) {       // the kernels behind this one carry it on to every gradient of these rows
+    for (int m = tid; m < 128; m += PF_THREADS)
+      if (i0 + m / g_q < dm.seq_q) *a.stats.at(b, r, i0 + m / g_q, m % g_q) = make_float2(gave_up(), gave_up());
+  }
   if (release_late) chain_release();
   if (warp == 5) {
     ptx::tc_fence_after();

@@ -93,3 +93,44 @@ def test_bounded_wait_really_runs_out_and_the_kernel_returns():
     B.dash_attn_fwd_prefill(p, Q, K, V, O, ws)
     assert B.dash_attn_last_status(ws) == 0
     assert torch.equal(O, good)
+
+
+@pytest.mark.parametrize("kw", [dict(h_q=4, h_kv=4, head_dim=64, block=32), dict(h_q=8, h_kv=2, head_dim=128, block=64),
+                                dict(h_q=4, h_kv=2, head_dim=64, block=16)])
+def test_backward_without_a_status_word_says_nan_when_a_wait_runs_out(kw):
+    """dash_attn_bwd_attend_prefill has no workspace.  The statistics pass is told not to load its first K tile and to give up
+    after 2e5 cycles: every gradient of every row and key must then be NaN (the buffers held statistics, counts and bit masks
+    meanwhile), and the next call must be right again."""
+    from tests.test_gpu_parity import _wl
+    w = _wl(seq=300, gamma=2.0, seed=55, **kw)
+    inp = synth.make_prefill_inputs(w, DEV)
+    Q, K, V = inp["Q"], inp["K"], inp["V"]
+    dO = torch.randn(Q.shape, device=DEV, generator=torch.Generator(DEV).manual_seed(56)).to(Q.dtype)
+    p = B.params_for_prefill(Q, K, V, dO, block=w.block, alpha=w.alpha, gamma=w.gamma, sigma=w.sigma)
+    ws, kbar, rt = B.alloc_workspace(p), B.alloc_kbar(p), B.alloc_routing(p)
+    B.dash_attn_block_summaries(p, K, kbar)
+    B.dash_attn_select(p, Q, kbar, rt["mask"], rt["count"], rt["blk_idx"], rt["blk_bias"], ws)
+
+    def grads():
+        out = (torch.zeros_like(Q), torch.zeros(w.batch, w.seq, w.h_kv, w.head_dim, device=DEV),
+               torch.zeros(w.batch, w.seq, w.h_kv, w.head_dim, device=DEV), torch.zeros_like(rt["blk_bias"]))
+        B.dash_attn_bwd_attend_prefill(p, Q, K, V, dO, rt["mask"], rt["blk_bias"], *out)
+        torch.cuda.synchronize()
+        return out
+
+    good = grads()
+    assert all(torch.isfinite(t.float()).all() for t in good)
+    try:
+        B.dash_attn_test_hooks(wait_limit_cycles=200_000, skip_own_k_load=1)
+        dQ, dK, dV, dbias = grads()
+    finally:
+        B.dash_attn_test_hooks()
+    assert torch.isnan(dQ.float()).all() and torch.isnan(dK).all() and torch.isnan(dV).all()
+    count = rt["count"].cpu()
+    for r in range(w.h_kv):
+        for i in range(w.block, w.seq, 7):
+            at = B.dash_attn_list_offset(p, 0, r, i)
+            assert torch.isnan(dbias[at:at + int(count[0, r, i])]).all()
+    again = grads()
+    for a, b in zip(again, good):
+        assert torch.allclose(a.float(), b.float(), rtol=1e-2, atol=1e-4)
