@@ -25,6 +25,8 @@
  *     the workspace; dash_attn_last_status() synchronises the stream and returns it.
  *   - Tensors are strided: stride arrays give element strides of (batch, token, head); the head_dim
  *     axis is contiguous.  Base pointers must be 16-byte aligned, strides multiples of 8 elements.
+ *     (The fp32 buffers of the routing and summary backward calls need the alignment of a float only; 16-byte aligned
+ *     ones are faster.)
  *     A stride of 0 repeats (expanded batches or heads); such tensors take the CUDA-core kernels.
  *   - 0-based positions.  Chunk of token j is j / block.  T_s = seq_kv / block complete chunks have
  *     summaries; T_a = ceil(seq_kv / block) chunks exist; W = ceil(T_a / 32) mask words per row.

@@ -337,7 +337,6 @@ int dash_attn_bwd_select_prefill(const dash_params* p, const void* Q, const floa
   if (dm.decode || !dm.causal) return DASH_ERR_UNSUPPORTED;
   if (!Q || !count || !dQ_route || !aligned16(Q)) return DASH_ERR_INVALID_ARG;
   if (dm.T_s > 0 && (!Kbar || !blk_idx || !tau || !dbias || !dKbar)) return DASH_ERR_INVALID_ARG;
-  if (!aligned16(dQ_route) || (dm.T_s > 0 && (!aligned16(Kbar) || !aligned16(dKbar)))) return DASH_ERR_INVALID_ARG;
   if ((rc = check_device()) != DASH_OK) return rc;
   StageRange nv("dash_attn: stage 1 routing, backward");
   return cuda_status(launch_route_bwd(dm, Q, Kbar, count, blk_idx, tau, dbias, dQ_route, dKbar, (cudaStream_t)stream));
@@ -351,8 +350,7 @@ int dash_attn_bwd_block_summaries(const dash_params* p, const void* K, const flo
   if (dm.decode) return DASH_ERR_UNSUPPORTED;
   if (!K || !dK || !aligned16(K)) return DASH_ERR_INVALID_ARG;
   if (dm.T_s > 0 && !dKbar) return DASH_ERR_INVALID_ARG;
-  if (!aligned16(dK) || (dm.T_s > 0 && !aligned16(dKbar))) return DASH_ERR_INVALID_ARG;
-  if (qbar && (!aligned16(qbar) || (dqbar && !aligned16(dqbar)) || qbar_chunk_stride < 0 || qbar_chunk_stride % 4 != 0)) return DASH_ERR_INVALID_ARG;
+  if (qbar && (qbar_chunk_stride < 0 || qbar_chunk_stride % 4 != 0)) return DASH_ERR_INVALID_ARG;
   if ((rc = check_device()) != DASH_OK) return rc;
   const size_t dq_bytes = !qbar ? 0 : (qbar_chunk_stride == 0 ? (size_t)dm.h_kv * dm.d
                                                                : (size_t)dm.T_s * (size_t)qbar_chunk_stride) * sizeof(float);

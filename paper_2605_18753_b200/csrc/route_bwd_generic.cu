@@ -24,35 +24,56 @@
 // a = softmax(<qbar, k_t>/sqrt(d)) (a_t = 1/B without a summary query): dk_t += a_t dkbar_c + ds_t qbar/sqrt(d),
 // ds_t = a_t (<k_t, dkbar_c> - sum_u a_u <k_u, dkbar_c>), dqbar += sum_t ds_t k_t / sqrt(d).  The B logits and products of the
 // chunk meet in shared memory.
+#include <initializer_list>
+
 #include "common.cuh"
 
 namespace dash {
 
 constexpr int RB_WARPS = 4;
 
-__global__ void __launch_bounds__(256) zero_kernel(float* p, long long n) {
+// The fp32 buffers of these two entry points may sit anywhere a float may (a view into a flat gradient buffer): VEC, 16-byte
+// accesses, only where all of a call's are 16-byte aligned.
+static bool all_aligned16(std::initializer_list<const void*> ptrs) {
+  for (const void* p : ptrs)
+    if (reinterpret_cast<uintptr_t>(p) & 15) return false;
+  return true;
+}
+
+__global__ void __launch_bounds__(256) zero_kernel(float* p, long long n, bool vec) {
   chain_wait();
   chain_release();
-  zero_floats(p, n, (long long)blockIdx.x * 256 + threadIdx.x, (long long)gridDim.x * 256);
+  const long long thread = (long long)blockIdx.x * 256 + threadIdx.x, threads = (long long)gridDim.x * 256;
+  if (vec) {
+    zero_floats(p, n, thread, threads);
+  } else {
+    for (long long k = thread; k < n; k += threads) p[k] = 0.f;
+  }
 }
 static cudaError_t launch_zero(float* p, size_t bytes, cudaStream_t st) {
   const long long n = (long long)(bytes / sizeof(float)), blocks = (n + 1023) / 1024;
-  cudaError_t e = launch_chained(zero_kernel, dim3((unsigned)(blocks < 2 * 148 ? blocks : 2 * 148)), dim3(256), 0, st, p, n);
+  cudaError_t e = launch_chained(zero_kernel, dim3((unsigned)(blocks < 2 * 148 ? blocks : 2 * 148)), dim3(256), 0, st, p, n, all_aligned16({p}));
   count_launch();
   return e;
 }
 
-// 4 or 2 consecutive floats added to global memory in one request.
-template <int V>
+// 4 or 2 consecutive floats added to global memory, in one request where they are aligned.
+template <int V, bool VEC>
 __device__ __forceinline__ void add_global(float* p, const float (&x)[V]) {
-  if constexpr (V == 4)
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) atomicAdd(p + v, x[v]);
+  } else if constexpr (V == 4)
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
   else
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(x[0]), "f"(x[1]) : "memory");
 }
-template <int V, typename T>
+template <int V, bool VEC = true, typename T>
 __device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
-  if constexpr (V == 4) {
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) x[v] = p[v];
+  } else if constexpr (V == 4) {
     const float4 f = load4(p);
     x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
   } else {
@@ -61,8 +82,20 @@ __device__ __forceinline__ void load_vec(const T* p, float (&x)[V]) {
   }
 }
 
+template <int V, bool VEC>
+__device__ __forceinline__ void store_vec(float* p, const float (&x)[V]) {
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) p[v] = x[v];
+  } else if constexpr (V == 4) {
+    store4(p, make_float4(x[0], x[1], x[2], x[3]));
+  } else {
+    *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+  }
+}
+
 // G (heads per KV head) is a template parameter so that the per-head sums live in registers.
-template <typename T, int D, int G>
+template <typename T, int D, int G, bool VEC>
 __global__ void __launch_bounds__(RB_WARPS * 32, G > 4 ? 1 : D == 128 ? 5 : 7)
 route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
                  const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
@@ -138,7 +171,8 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
           for (int h = 0; h < G; ++h) xp[h] = make_float2(0.f, 0.f);
           float4 kv[D / 16];
 #pragma unroll
-          for (int j = 0; j < D / 16; ++j) kv[j] = load4(kp + 16 * j);
+          for (int j = 0; j < D / 16; ++j)
+            kv[j] = VEC ? load4(kp + 16 * j) : make_float4(kp[16 * j], kp[16 * j + 1], kp[16 * j + 2], kp[16 * j + 3]);
 #pragma unroll
           for (int j = 0; j < D / 16; ++j)
 #pragma unroll
@@ -207,7 +241,7 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
           c[u] = c_s[warp][min(e0 + u, n - 1)];
-          load_vec<VPL>(kb + (long long)c[u] * D + lane * VPL, kv[u]);
+          load_vec<VPL, VEC>(kb + (long long)c[u] * D + lane * VPL, kv[u]);
         }
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
@@ -231,23 +265,24 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
             float out[VPL];
 #pragma unroll
             for (int v = 0; v < VPL / 2; ++v) { out[2 * v] = dkb[v].x; out[2 * v + 1] = dkb[v].y; }
-            add_global<VPL>(dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL, out);
+            add_global<VPL, VEC>(dKbar + (grp * dm.T_s + c[u]) * D + lane * VPL, out);
           }
         }
       }
     }
   }
 #pragma unroll
-  for (int h = 0; h < G; ++h)
-    if constexpr (VPL == 4)
-      store4(dq_out + (long long)h * D, make_float4(dq[h][0].x, dq[h][0].y, dq[h][1].x, dq[h][1].y));
-    else
-      *reinterpret_cast<float2*>(dq_out + (long long)h * D) = dq[h][0];
+  for (int h = 0; h < G; ++h) {
+    float x[VPL];
+#pragma unroll
+    for (int v = 0; v < VPL / 2; ++v) { x[2 * v] = dq[h][v].x; x[2 * v + 1] = dq[h][v].y; }
+    store_vec<VPL, VEC>(dq_out + (long long)h * D, x);
+  }
 }
 
 constexpr int SB_SPLIT = 4;      // warps that share a chunk = a block
 
-template <typename T, int D>
+template <typename T, int D, bool VEC>
 __global__ void __launch_bounds__(SB_SPLIT * 32)
 summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__ qbar, long long qbar_chunk_stride,
                      const float* __restrict__ dKbar, float* __restrict__ dK, float* __restrict__ dqbar) {
@@ -265,19 +300,16 @@ summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__
   float* dkp = dK + (((long long)b * dm.seq_kv + (long long)c * dm.B) * dm.h_kv + r) * D + lane * VPL;
   const long long gtok = (long long)dm.h_kv * D;
   float g[VPL];
-  load_vec<VPL>(dKbar + (grp * dm.T_s + c) * D + lane * VPL, g);
+  load_vec<VPL, VEC>(dKbar + (grp * dm.T_s + c) * D + lane * VPL, g);
   // dk rows of four tokens at a time: read, add, write
   auto add_rows = [&](int t, auto&& delta) {
     float x[NB][VPL];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) load_vec<VPL>(dkp + (long long)(t + u) * gtok, x[u]);
+    for (int u = 0; u < NB; ++u) load_vec<VPL, VEC>(dkp + (long long)(t + u) * gtok, x[u]);
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       delta(u, x[u]);
-      if constexpr (VPL == 4)
-        store4(dkp + (long long)(t + u) * gtok, make_float4(x[u][0], x[u][1], x[u][2], x[u][3]));
-      else
-        *reinterpret_cast<float2*>(dkp + (long long)(t + u) * gtok) = make_float2(x[u][0], x[u][1]);
+      store_vec<VPL, VEC>(dkp + (long long)(t + u) * gtok, x[u]);
     }
   };
   if (qbar == nullptr) {
@@ -290,7 +322,7 @@ summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__
     return;
   }
   float qv[VPL];
-  load_vec<VPL>(qbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, qv);
+  load_vec<VPL, VEC>(qbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, qv);
   for (int t = t0; t < t0 + rows; t += NB) {
     float kv[NB][VPL], s[NB], da[NB];
 #pragma unroll
@@ -351,7 +383,7 @@ summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__
 #pragma unroll
       for (int v = 0; v < VPL; ++v)
         dqb[v] = (red[0][lane * VPL + v] + red[1][lane * VPL + v]) + (red[2][lane * VPL + v] + red[3][lane * VPL + v]);
-      add_global<VPL>(dqbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, dqb);
+      add_global<VPL, VEC>(dqbar + (long long)c * qbar_chunk_stride + (long long)r * D + lane * VPL, dqb);
     }
   }
 }
@@ -366,8 +398,11 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
   const long long total = (long long)dm.batch * dm.h_kv * dm.seq_q;
   const unsigned grid = (unsigned)((total + RB_WARPS - 1) / RB_WARPS);
   cudaError_t le = cudaSuccess;
+  const bool vec = all_aligned16({Kbar, dQr, dKbar});
+#define DASH_RB_V(T, D, GV, V) \
+  le = launch_chained(route_bwd_kernel<T, D, GV, V>, dim3(grid), dim3(RB_WARPS * 32), 0, st, dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar)
 #define DASH_RB(T, D, GV) \
-  le = launch_chained(route_bwd_kernel<T, D, GV>, dim3(grid), dim3(RB_WARPS * 32), 0, st, dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar)
+  if (vec) DASH_RB_V(T, D, GV, true); else DASH_RB_V(T, D, GV, false)
 #define DASH_RB_G(T, D)                   \
   switch (dm.g_q) {                       \
     case 1: DASH_RB(T, D, 1); break;      \
@@ -384,6 +419,7 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
   }
 #undef DASH_RB_G
 #undef DASH_RB
+#undef DASH_RB_V
   count_launch();
   return le;
 }
@@ -398,14 +434,18 @@ cudaError_t launch_summaries_bwd(const Dims& dm, const void* K, const float* qba
   if (total == 0) return cudaSuccess;
   const unsigned grid = (unsigned)total;
   cudaError_t le = cudaSuccess;
+  const bool vec = all_aligned16({qbar, dKbar, dK, dqbar});
+#define DASH_SB_V(T, D, V) \
+  le = launch_chained(summaries_bwd_kernel<T, D, V>, dim3(grid), dim3(SB_SPLIT * 32), 0, st, dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
 #define DASH_SB(T, D) \
-  le = launch_chained(summaries_bwd_kernel<T, D>, dim3(grid), dim3(SB_SPLIT * 32), 0, st, dm, (const T*)K, qbar, qbar_chunk_stride, dKbar, dK, dqbar)
+  do { if (vec) DASH_SB_V(T, D, true); else DASH_SB_V(T, D, false); } while (0)
   if (dm.dtype == DASH_BF16) {
     if (dm.d == 128) DASH_SB(__nv_bfloat16, 128); else DASH_SB(__nv_bfloat16, 64);
   } else {
     if (dm.d == 128) DASH_SB(float, 128); else DASH_SB(float, 64);
   }
 #undef DASH_SB
+#undef DASH_SB_V
   count_launch();
   return le;
 }
