@@ -249,8 +249,8 @@ static cudaError_t launch_tiles(const Dims& dm, const void* Q, const void* K, co
 template <typename T, int D>
 static cudaError_t launch_size(const Dims& dm, const void* Q, const void* K, const void* V, const uint32_t* mask,
                                const float* blk_bias, void* O, cudaStream_t st) {
-  // with fewer than two eight-row tiles per SM (148 of them) the SMs that hold the longest tiles are what the kernel takes
-  const bool few = (long long)dm.batch * dm.seq_q * dm.h_q <= 8LL * 2 * 148;
+  // with fewer than two eight-row tiles per SM the SMs that hold the longest tiles are what the kernel takes
+  const bool few = (long long)dm.batch * dm.seq_q * dm.h_q <= 8LL * 2 * current_sm_count();
   return few ? launch_tiles<T, D, 4, 8>(dm, Q, K, V, mask, blk_bias, O, st) : launch_tiles<T, D, 8, 8>(dm, Q, K, V, mask, blk_bias, O, st);
 }
 

@@ -34,8 +34,9 @@ cudaError_t launch_decode_sm100(const Dims& dm, int n_split, const void* Q, cons
   return launch_any<0>(a, K, V, st);
 }
 
-// Blocks per cluster of the fused step (0: not taken): the most of 8, 4, 2 with which all clusters are resident at once (two
-// blocks on each of 148 SMs).  In a second wave nothing hides a cluster's serial parts: 104 groups of 4671 tokens take 19 us
+// Blocks per cluster of the fused step (0: not taken): the most of 8, 4, 2 with which the grid is no larger than two blocks per
+// SM.  (A measured line: a cluster sits inside one GPC, so the last few of that many clusters may have to wait for others.)  In
+// a second wave nothing hides a cluster's serial parts: 104 groups of 4671 tokens take 19 us
 // as two kernels and would take 31 in three waves of clusters of eight.  A block's share of the longest possible list is
 // bounded as well: lists differ in length, and one long list in two shares is what the step waits for (39 sequences of
 // 33597 tokens, 2 KV heads, chunks of 128: 92 us as two kernels, 138 in clusters of two).
@@ -44,7 +45,7 @@ static int fused_cluster(const Dims& dm) {
   if (need == 0 || dm.T_s < 1 || dm.T_s > FUSED_MAX_CHUNKS) return 0;
   const int most = dm.T_s * (dm.B > SUB ? dm.B / SUB : 1) / (dm.B < SUB ? SUB / dm.B : 1);     // sub-blocks of the longest list
   for (int cs = 8; cs >= 2 && cs >= need; cs /= 2)
-    if ((long long)dm.batch * dm.h_kv * cs <= 2 * 148) return most <= 128 * cs ? cs : 0;
+    if ((long long)dm.batch * dm.h_kv * cs <= 2 * current_sm_count()) return most <= 128 * cs ? cs : 0;
   return 0;
 }
 bool decode_fused_supported(const Dims& dm) { return fused_cluster(dm) > 0; }

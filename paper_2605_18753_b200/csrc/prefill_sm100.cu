@@ -94,6 +94,7 @@ struct PrefillArgs {
   int TQ;            // tokens per tile
   int n_tiles;       // tiles per (batch, KV head)
   int early_loads;   // 1: Q, K, V are not written by the kernel before this one on the stream (their first loads may precede chain_wait)
+  int resident;      // blocks that the device holds at once
   int inject;        // test hook: 1 = the K producer never loads the own chunk's keys (the waits for them run out)
   long long wait_limit;   // cycles a bounded wait may spin
   const uint32_t* mask;
@@ -224,7 +225,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   chain_wait();
   // The next kernel's blocks: at once where this grid takes several waves (they come with its last one), else only when this
   // block is done, for they would all settle on the SMs that have none of the few blocks (500 tokens: 24.7 -> 23.6 us a forward).
-  const bool release_late = gridDim.x <= 2 * 148;
+  const bool release_late = (int)gridDim.x <= a.resident;
   if (!release_late) chain_release();
   // a workspace whose status word already holds an error makes every role leave at its first wait: after one
   // block's wait has run out, the rest of the grid retires in microseconds instead of a wait limit each
@@ -679,6 +680,7 @@ cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const voi
   a.TQ = 128 / dm.g_q;
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
   a.early_loads = inputs_stable ? 1 : 0;
+  a.resident = 2 * current_sm_count();
   a.inject = test_hooks().skip_own_k_load;
   a.wait_limit = test_hooks().wait_limit_cycles;
   a.mask = mask;

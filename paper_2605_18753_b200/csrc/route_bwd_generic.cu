@@ -51,8 +51,8 @@ __global__ void __launch_bounds__(256) zero_kernel(float* p, long long n, bool v
   }
 }
 static cudaError_t launch_zero(float* p, size_t bytes, cudaStream_t st) {
-  const long long n = (long long)(bytes / sizeof(float)), blocks = (n + 1023) / 1024;
-  cudaError_t e = launch_chained(zero_kernel, dim3((unsigned)(blocks < 2 * 148 ? blocks : 2 * 148)), dim3(256), 0, st, p, n, all_aligned16({p}));
+  const long long n = (long long)(bytes / sizeof(float)), blocks = (n + 1023) / 1024, most = 2 * current_sm_count();
+  cudaError_t e = launch_chained(zero_kernel, dim3((unsigned)(blocks < most ? blocks : most)), dim3(256), 0, st, p, n, all_aligned16({p}));
   count_launch();
   return e;
 }

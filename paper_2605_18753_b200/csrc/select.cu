@@ -32,9 +32,10 @@ static bool plan_select(const Dims& dm, SelectPlan* pl) {
   int tq = 1;
   if (!dm.decode) {
     // more tokens per block read each summary tile for more rows, but a small problem must not leave SMs without a block:
-    // two blocks per SM (148 of them) come first (1024 tokens, one head: 18 us in blocks of 32 tokens, now 8)
+    // two blocks per SM come first (1024 tokens, one head: 18 us in blocks of 32 tokens, now 8)
     const long long tokens = (long long)dm.batch * dm.h_kv * dm.seq_q;
-    while (tq * 2 * dm.g_q <= 32 && tq * 2 <= dm.B && tokens / (tq * 2) >= 2 * 148) tq *= 2;
+    const int blocks = 2 * current_sm_count();
+    while (tq * 2 * dm.g_q <= 32 && tq * 2 <= dm.B && tokens / (tq * 2) >= blocks) tq *= 2;
   }
   const int max_cand = (dm.decode || !dm.causal) ? dm.T_s : min(dm.T_s, (dm.seq_q - 1) / dm.B);
   const int xs = ((max_cand + SEL_CT - 1) / SEL_CT) * SEL_CT + 4;

@@ -162,8 +162,8 @@ cudaError_t launch_summaries(const Dims& dm, const void* K, const float* qbar, l
   if (num_blocks <= 0) return cudaSuccess;
   const long long plane_elems = (long long)dm.batch * dm.h_kv * dm.T_s * dm.d;
   const long long total = (long long)dm.batch * dm.h_kv * num_blocks;
-  // four warps per chunk up to sixteen warps per SM (148 of them)
-  const int split = total < 16 * 148 ? 4 : 1;
+  // four warps per chunk up to sixteen warps per SM
+  const int split = total < 16 * current_sm_count() ? 4 : 1;
   const unsigned grid = (unsigned)((total * split + SUM_WARPS - 1) / SUM_WARPS);
   const dim3 block(SUM_WARPS * 32);
   cudaError_t le = cudaSuccess;
