@@ -33,7 +33,8 @@
  *   - Query head h uses KV head h / (h_q / h_kv) (Section 3.2).
  *   - Which kernels run: bf16 tensors take the TMA / tcgen05 kernels (head_dim 64 or 128, every chunk size; prefill
  *     and decode take every group size g_q = h_q / h_kv); fp32 tensors and the non-causal mode take CUDA-core
- *     kernels that compute the same thing.
+ *     kernels that compute the same thing.  O carries the rounding of the weights to bf16 (2^-9) in a bf16 prefill
+ *     with g_q >= 2; decode and g_q = 1 carry them as two bf16 terms (2^-17).
  *     The choice is made from the parameters alone, never from the data, and is the same on every call.
  *   - causal = 1 is the paper's setting and the one the tensor-core kernels serve.  causal = 0 (prefill only;
  *     the paper does not define it) is read as: every complete chunk is a candidate of every row; the
@@ -200,7 +201,7 @@ int dash_attn_attend_decode_static(const dash_params* p, const void* Q, const vo
  *          stay zero): the quantity a backward of Stage 1 continues from.
  *   dO     incoming gradient of O, dtype p->dtype, strides p->o_stride.
  * mask / blk_bias as written by dash_attn_select for the same parameters.  bf16 tensors (causal) run on tensor cores with
- * P and dS carried as two bf16 terms each, fp32 and the non-causal mode on CUDA cores (one warp per row and head); either
+ * P and dS carried as two bf16 terms each (within 2^-17 of every weight, sums in fp32), fp32 and the non-causal mode on CUDA cores (one warp per row and head); either
  * way some sums are formed by fp32 atomics, so last bits vary from run to run.  No workspace: what the kernels hand to each
  * other sits in dQ and dbias until those get their values (neither may overlap an input), and there is no status word: where a
  * bounded device-side wait runs out, the rows and keys concerned come back as NaN in every gradient.
@@ -238,7 +239,7 @@ int dash_attn_bwd_attend_prefill_tc(const dash_params* p, const void* Q, const v
  *   dQ_route   fp32, contiguous [batch, seq_q, h_q, head_dim]: the part of dL/dQ that flows through the routing; the
  *              caller adds it to the Stage-2 part (every row is written, zeros where nothing is routed).
  *   dKbar      fp32 [batch, h_kv, T_s, head_dim]: gradient w.r.t. the summaries; zeroed, then accumulated (atomics).
- * CUDA-core correctness path.  Rows whose support holds a chunk sitting on the threshold have no gradient in the
+ * CUDA cores, one warp per row.  Rows whose support holds a chunk sitting on the threshold have no gradient in the
  * mathematical sense (the map is piecewise differentiable); the kernel then returns the one-sided value of Eq. 2. */
 int dash_attn_bwd_select_prefill(const dash_params* p, const void* Q, const float* Kbar, const int32_t* count,
                                  const int32_t* blk_idx, const float* tau, const float* dbias, float* dQ_route,

@@ -137,9 +137,9 @@ def strerror(code: int) -> str:
     return lib().dash_attn_strerror(int(code)).decode()
 
 
-# A short decode step is three kernels of a few microseconds, so what a call costs here counts: plain integers go to
+# A short decode step is one or two kernels of a few microseconds, so what a call costs here counts: plain integers go to
 # ctypes (the declared argument types convert them), and the stream handle is read without building a torch.cuda.Stream
-# object (3.4 -> 0.1 us a call; a decode step's issue 14.3 -> 9.7 us).
+# object (3.4 -> 0.1 us a call; a decode step's issue 14.3 -> 10.3 us).
 def _ptr(t):
     return t if t is None or isinstance(t, int) else t.data_ptr()
 

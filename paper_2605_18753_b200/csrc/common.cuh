@@ -144,7 +144,8 @@ __device__ inline float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// One instruction on sm_100a instead of five shuffles and maxima.
+// One instruction on sm_100a instead of five shuffles and maxima.  Every lane of the warp must take part: inside a branch that
+// some lanes do not enter (a conditional expression is one) the warp waits for them for ever.
 __device__ inline float warp_max(float v) {
   float m;
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));

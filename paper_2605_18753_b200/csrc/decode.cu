@@ -36,7 +36,9 @@ int current_sm_count() {
 }
 
 // Split count of the CUDA-core kernel: waves of one block per SM, each ceil(groups * s / SMs) long (1 / s of a group's
-// work plus a fixed cost per block, about 2 % of a long group's work).
+// work plus a fixed cost per block, about 2 % of a long group's work), at most 16 up to caches of 2^19 tokens; longer bf16 caches
+// keep the lower bound of the tensor-core kernel, whose blocks own a limited share of the list, so that blocks stay of about
+// one size there.
 static int splits_cuda_cores(const Dims& dm) {
   const int n_sm = current_sm_count(), groups = dm.batch * dm.h_kv;
   const int lo = decode_use_sm100(dm) ? decode_sm100_min_splits(dm) : 1, hi = max(lo, 16);
@@ -289,7 +291,7 @@ cudaError_t launch_attend_decode_ex(const Dims& dm, const void* Q, const void* K
                                     const int* count, const int* blk_idx, const float* blk_bias, void* O,
                                     float* partials, StatusBlock* sb, cudaStream_t st) {
   if (decode_use_sm100(dm)) {
-    // bf16, head_dim 128, chunks of 64 or 128: TMA-fed tensor-core split kernel, then the common merge
+    // bf16: TMA-fed tensor-core split kernel, then the common merge
     const int ns = decode_num_splits(dm);
     // with a workspace (status block + arrival counters) the last split of each group merges in the same kernel
     const bool fused = sb != nullptr && dm.batch * dm.h_kv <= ARRIVAL_COUNTERS;

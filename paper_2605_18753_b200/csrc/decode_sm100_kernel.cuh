@@ -16,10 +16,11 @@
 // The routed list (plus the row's own, possibly partial, chunk) is cut into n_split contiguous ranges of
 // 64-token sub-blocks, one thread block each; the block that sees the last arrival of its (batch, KV head)
 // merges the partial (m, l, O) of all splits in split order (or, without a workspace, a separate merge kernel does).
-// Every wait is bounded (DASH_ERR_TIMEOUT in the status word).
+// Every wait on an mbarrier is bounded (DASH_ERR_TIMEOUT in the status word).  The fused step's cluster barriers have no limit
+// and need none: every thread of a cluster reaches all of them, also after a wait of its block has run out.
 //
-// FUSED: the whole decode step in one launch, a cluster of CS blocks per (batch, KV head), where all clusters fit the GPU at
-// once and caches have up to 512 chunks: such a step is launches and round trips to L2.  Each block scores its share of
+// FUSED: the whole decode step in one launch, a cluster of CS blocks per (batch, KV head), where the grid is at most
+// two blocks per SM and caches have up to 512 chunks: such a step is launches and round trips to L2.  Each block scores its share of
 // the candidates and hands its logits to all of them through distributed shared memory, every block routes the group for
 // itself (decode_route.cuh) and attends its share of the list, and the partial results meet through distributed shared memory
 // as well.  One 8K cache, 8 KV heads: 13.4 us as routing and attention kernels, 9.3 fused.

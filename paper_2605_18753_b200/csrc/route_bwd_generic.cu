@@ -1,4 +1,4 @@
-// Backward of Stage 1 (routing) and Stage 0 (chunk summaries), prefill, CUDA-core correctness path.
+// Backward of Stage 1 (routing) and Stage 0 (chunk summaries), prefill, on CUDA cores.
 //
 // Section 3.5 notes that the backward pass can reuse the forward pass's bit mask because the alpha-entmax Jacobian is
 // sparse; the appendix ("The alpha-entmax mapping") states that the Jacobian has a closed form where the support is
