@@ -19,9 +19,9 @@ def test_cluster_sizes_and_waves(batch, h_kv):
 
 
 @pytest.mark.parametrize("chunks", [512, 513])
-# (eight heads, not sixteen: from 64 rows on the harness wants four fifths of the groups free of chunks inside the 1e-4 band
-# around the threshold, and one of the four groups holds one)
-@pytest.mark.parametrize("g_q,head_dim", [(1, 128), (8, 64)])
-def test_longest_fused_cache(chunks, g_q, head_dim):
-    w = P._wl(kind="decode", batch=2, seq=chunks * 16 + 5, h_q=2 * g_q, h_kv=2, head_dim=head_dim, block=16, seed=71)
-    P._decode_case(w, [chunks * 16 + 5, 700], local_blocks=1)
+# (sixteen heads: one KV head and three sequences, because from 64 rows on the harness wants four fifths of the groups free of
+# chunks inside the 1e-4 band around the threshold, which so many heads seldom are)
+@pytest.mark.parametrize("g_q,head_dim,h_kv,batch", [(1, 128, 2, 2), (8, 64, 2, 2), (16, 64, 1, 3), (16, 128, 1, 3)])
+def test_longest_fused_cache(chunks, g_q, head_dim, h_kv, batch):
+    w = P._wl(kind="decode", batch=batch, seq=chunks * 16 + 5, h_q=h_kv * g_q, h_kv=h_kv, head_dim=head_dim, block=16, seed=71)
+    P._decode_case(w, [chunks * 16 + 5, 700, chunks * 8][:batch], local_blocks=1)

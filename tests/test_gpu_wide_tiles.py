@@ -15,4 +15,4 @@ def test_tiles_over_several_chunks(g_q, block, extra, local_blocks):
     for tiles, head_dim in ((1, 64), (5, 128)):
         seq = tiles * max(tile, block) + extra
         w = P._wl(seq=seq, h_q=2 * g_q, h_kv=2, head_dim=head_dim, block=block, dtype="bf16", gamma=2.0, seed=40 + tiles)
-        P._fwd_prefill_case(w, range(seq), local_blocks=local_blocks, min_clean=0.5)
+        P._fwd_prefill_case(w, range(seq), local_blocks=local_blocks)
