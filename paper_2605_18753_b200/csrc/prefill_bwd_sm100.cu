@@ -550,6 +550,11 @@ constexpr uint32_t TMEM_COLS = 512;     // S0 S1 [0,128) dP0 dP1 [128,256) dV^T 
 constexpr uint32_t COL_DP = 128, COL_DV = 256, COL_DK = 320;
 constexpr uint32_t PS_BYTES = 128 * NKV * 2;       // 16 KiB: one term of P (or dS) of a step, 128 rows of 128 bytes
 constexpr int MAX_STAGES = 4;
+// Two-term kernels take their sums out of tensor memory every FLUSH steps and add them up in registers: the tensor cores cut the
+// low bits of an accumulator off at every product, so that a sum left there loses about half a unit per product, the longer
+// the walk the more.  dK against float64, 16 heads per KV head, d 64 (relative 2-norm): 1500 tokens 1.3e-5 -> 2.5e-6, 6000
+// tokens 2.8e-4 -> 2.3e-6, which is the two terms' own 2^-18; 2 x 1500 tokens, 8/2 heads: 152.9 -> 154.7 us the whole backward.
+constexpr int FLUSH = 2;
 // SD_FULL: both score products of the step (two arrivals).  PDS_FULL: P and dS in shared memory (SEQ: P alone).
 // ACC_DONE: both accumulating products done (SEQ: dK, which follows dV), the step's stage and the P / dS buffers are free.
 enum Bar { KV_FULL = 0, SD_FULL = 1, PDS_FULL = 3, DV_DONE = 5, DS_FULL = 7, QD_FULL = 9, ACC_DONE = 9 + MAX_STAGES, N_BARS = 9 + 2 * MAX_STAGES };
@@ -866,7 +871,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           for (int k = 0; k < 128 / 16; ++k) {
             const uint64_t adv = (uint64_t)((k * 16 * 128) >> 4);
             ptx::mma_bf16_ss(d_tmem, ad0 + adv, bd0 + adv + (uint64_t)((term * PS_BYTES) >> 4), IDESC_ACC,
-                             (j > 0 || k > 0 || term > 0) ? 1u : 0u);
+                             ((P2 ? j % FLUSH : j) > 0 || k > 0 || term > 0) ? 1u : 0u);
           }
         ptx::mma_commit(SEQ && is_v ? bar(DV_DONE + buf) : bar(ACC_DONE + st));
       }
@@ -882,6 +887,25 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const int t = m / g_q;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float c1 = dm.sm_scale * LOG2E;
+    const bool mine = HD == 128 || (wg == 0 ? m < 64 : m >= 64);      // this thread's lane holds sums (whole warps)
+    const uint32_t sum_addr = lane_addr + (wg == 0 ? COL_DV : COL_DK);
+    [[maybe_unused]] float sums[P2 ? NKV : 1];                        // dV or dK of row d = lane, one per key
+    if constexpr (P2) {
+#pragma unroll
+      for (int cc = 0; cc < NKV; ++cc) sums[cc] = 0.f;
+    }
+    [[maybe_unused]] auto take_sums = [&]() {
+      if constexpr (P2) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          uint32_t v[32];
+          DASH_TMEM_LD32(v, sum_addr + half * 32);
+          ptx::tmem_wait_ld();
+#pragma unroll
+          for (int cc = 0; cc < 32; ++cc) sums[half * 32 + cc] += __uint_as_float(v[cc]);
+        }
+      }
+    };
     bool ok = true;
     // row m of a [128 rows][64 keys] term: 128 bytes, 16-byte pieces swizzled with the row (128-byte swizzle); this
     // warpgroup's keys are pieces 4 wg .. 4 wg + 3
@@ -933,6 +957,12 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         store_row(LY::OFF_DS, d_hi);
         if constexpr (P2) store_row(LY::OFF_DS + PS_BYTES, d_lo);
       }
+      if constexpr (P2) {
+        if (j > 0 && j % FLUSH == 0 && mine) {         // (every product so far is done, and the next ones wait for this step's P)
+          ptx::tc_fence_after();
+          take_sums();
+        }
+      }
       ptx::fence_proxy_async_smem();
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(PDS_FULL + buf));
@@ -948,29 +978,33 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // epilogue: dV^T, dK^T [d = TMEM lane][key = column] -> dV, dK [batch][key][KV head][d]; one warpgroup each
     const int n_done = ok ? *reinterpret_cast<volatile int*>(&misc->total) : 0;
     if (ok && n_done > 0) ok = wait_on(bar(ACC_DONE + (n_done - 1) % NST), (uint32_t)((n_done - 1) / NST) & 1u);
-    const bool mine = HD == 128 || (wg == 0 ? m < 64 : m >= 64);      // (whole warps)
     if (ok && mine && (n_done > 0 || a.n_split == 1)) {
       ptx::tc_fence_after();
       const int d = HD == 128 ? m : m & 63;
-      float* out = wg == 0 ? a.dV : a.dK;
+      float* out = (wg == 0 ? a.dV : a.dK) + (((long long)b * dm.seq_kv + k0) * dm.h_kv + r) * HD + d;
       const float mul = wg == 0 ? 1.f : dm.sm_scale;
+      const long long pitch = (long long)dm.h_kv * HD;
+      auto put = [&](int key, float x) {
+        if (k0 + key >= dm.seq_kv) return;
+        if (a.n_split > 1) atomicAdd(out + key * pitch, x * mul); else out[key * pitch] = x * mul;
+      };
+      if constexpr (P2) {
+        if (n_done > 0) take_sums();
+#pragma unroll
+        for (int cc = 0; cc < NKV; ++cc) put(cc, sums[cc]);
+      } else {
 #pragma unroll 1
-      for (int half = 0; half < 2; ++half) {
-        uint32_t v[32];
-        if (n_done > 0) {
-          DASH_TMEM_LD32(v, lane_addr + (wg == 0 ? COL_DV : COL_DK) + half * 32);
-          ptx::tmem_wait_ld();
-        } else {
+        for (int half = 0; half < 2; ++half) {
+          uint32_t v[32];
+          if (n_done > 0) {
+            DASH_TMEM_LD32(v, sum_addr + half * 32);
+            ptx::tmem_wait_ld();
+          } else {
 #pragma unroll
-          for (int cc = 0; cc < 32; ++cc) v[cc] = 0u;
-        }
-#pragma unroll
-        for (int cc = 0; cc < 32; ++cc) {
-          const int key = k0 + half * 32 + cc;
-          if (key < dm.seq_kv) {
-            float* o = out + (((long long)b * dm.seq_kv + key) * dm.h_kv + r) * HD + d;
-            if (a.n_split > 1) atomicAdd(o, __uint_as_float(v[cc]) * mul); else *o = __uint_as_float(v[cc]) * mul;
+            for (int cc = 0; cc < 32; ++cc) v[cc] = 0u;
           }
+#pragma unroll
+          for (int cc = 0; cc < 32; ++cc) put(half * 32 + cc, __uint_as_float(v[cc]));
         }
       }
     }
