@@ -27,6 +27,8 @@
  *     axis is contiguous.  Base pointers must be 16-byte aligned, strides multiples of 8 elements.
  *     (The fp32 buffers of the routing and summary backward calls need the alignment of a float only; 16-byte aligned
  *     ones are faster.)
+ *     Keys and values are taken to be finite: a NaN or an infinity in one reaches the rows that attend it, and may reach
+ *     other rows of a prefill or backward tile (128 rows; 4 or 8 on CUDA cores) that share the tile's keys and values.
  *     A stride of 0 repeats (expanded batches or heads); such tensors take the CUDA-core kernels.
  *   - 0-based positions.  Chunk of token j is j / block.  T_s = seq_kv / block complete chunks have
  *     summaries; T_a = ceil(seq_kv / block) chunks exist; W = ceil(T_a / 32) mask words per row.
