@@ -342,8 +342,7 @@ bool prefill_sm100_supported(const Dims& dm);
 // inputs_stable: Q, K, V were not written by the kernel launched just before on the stream
 cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const void* K, const void* V,
                                         const uint32_t* mask, const float* blk_bias, void* O, StatusBlock* sb,
-                                        bool inputs_stable, cudaStream_t st, const RowStats& stats = RowStats(),
-                                        const void* dO = nullptr);
+                                        bool inputs_stable, cudaStream_t st);
 // Stage 2 backward on tensor cores (bf16, causal).  two_term: every shape, P and dS as two bf16 terms; else head_dim 128,
 // chunks of 64 or 128 tokens, g_q >= 2, one term.  The gradient buffers double as its scratch.
 bool prefill_bwd_sm100_supported(const Dims& dm);

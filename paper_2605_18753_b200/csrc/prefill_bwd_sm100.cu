@@ -4,7 +4,7 @@
 // With P = softmax of the row's logits l_j = <q,k_j>/sqrt(d) + bias_c(j) over its selected tokens, dP = dO V^T,
 // delta = <O, dO> per row and dS = P o (dP - delta):
 //     dQ = dS K / sqrt(d),   dK = dS^T Q / sqrt(d),   dV = P^T dO,   dbias_c = sum of dS over the chunk's tokens.
-// Three launches behind the forward kernel run in "statistics" mode (it leaves the log-sum-exp and delta of every row):
+// Three launches behind the statistics pass (prefill_bwd_stats_sm100.cu; it leaves the log-sum-exp and delta of every row):
 //   list_marks_kernel       per row, the number of routed chunks in the mask words before each word (so that a row's
 //                           list entry for a chunk can be found from one word of its mask), and per query tile the OR of
 //                           its rows' mask words (which chunks any of its rows routed);
@@ -27,40 +27,19 @@
 //
 // Bound by the chain of a step (tile landed -> S, dP -> P, dS -> accumulating products), one block per SM.  2 x 1500 tokens,
 // 8/2 heads, d 64, chunks of 32: 2.02 ms on CUDA cores (one warp per row and head, two vector reductions per token and
-// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: 2.0 ms (statistics 0.40, dK / dV 1.04, dQ 0.55).
+// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: statistics 0.40 -> 0.39, dK / dV 1.05, dQ 0.59 -> 0.56 ms.
 #include <cuda.h>
 
 #include <algorithm>
 
-#include "common.cuh"
-#include "sm100_ptx.cuh"
+#include "bwd_sm100.cuh"
 #include "tensor_map.cuh"
-#include "tile_walk.cuh"
 
 namespace dash {
 
 namespace {
 
-constexpr int NKV = 64;                 // keys per step / per slice
-constexpr float LOG2E = 1.4426950408889634f;
-
-struct BwdArgs {
-  Dims dm;
-  int TQ;             // tokens per query tile
-  int n_tiles;        // query tiles per (batch, KV head)
-  int n_slices;       // 64-key slices per (batch, KV head)
-  int n_split;        // blocks that share a slice's query tiles (1: they write dK / dV, more: they add to them)
-  long long wait_limit;
-  const uint32_t* mask;
-  const float* blk_bias;
-  RowStats stats;
-  int* marks;         // counts and unions, in the layout of the lists
-  __nv_bfloat16* dQ;
-  float* dK;
-  float* dV;
-  float* dbias;
-  StatusBlock* sb;
-};
+constexpr int NKV = BWD_NKV;
 
 // Where a row's counts start (entry w - 1: routed chunks in mask words 0 .. w - 1), and the unions of the tile whose last
 // row it is (behind the counts, one per mask word).
@@ -139,34 +118,29 @@ __device__ __forceinline__ void pack_terms(const float (&x)[32], uint32_t (&hi)[
 // ===================================================================================================================
 namespace dq {
 
-// Two warpgroups form dS, each for half of a step's 64 columns (no row maximum is needed: the log-sum-exp is known), so
-// a step's exponentials take half as long.  One issuing thread per product (S, dP, dQ): a thread issues an MMA every
-// 60-80 clocks whatever its size, and 20 per step through one thread would be the kernel's pace.
-constexpr int W_KPROD = 8, W_S = 9, W_VPROD = 10, W_DP = 11, W_DQ = 12;
-constexpr int THREADS = 512;              // 8 dS warps, 5 service warps, 3 idle: whole warpgroups, so that the registers can be re-divided
-// registers per thread after the re-division (128 each at launch); wide tiles keep more per producer lane
-__host__ __device__ constexpr int regs_service(int wt, int cps) { return wt > 2 || (wt > 0 && cps > 2) ? 96 : wt > 0 || cps > 1 ? 80 : 56; }
-static_assert(THREADS == 512, "two pairs of warpgroups: one pair can take exactly what the other released");
-constexpr int KST = 3;                  // K / V ring and S / dP ring: stage = step mod 3, held until the step's dQ product is done
+// Warps as in the statistics pass (bwd_sm100.cuh): three warpgroups form dS, taking the steps in turn; one issuing thread per
+// product (S, dP, dQ): a thread issues an MMA every 60-80 clocks whatever its size, and 20 per step through one thread would be
+// the kernel's pace.  A V tile is free when its dP product is done, a K tile and a step record when the step's dQ product is:
+// rings of their own, so that a step's tiles have landed by the time its S / dP slot is free.
+constexpr int THREADS = BWD_ROW_THREADS;
+constexpr int KST = 5, VST = 3;         // ring of K tiles and step records; ring of V tiles and of S / dP slots
 constexpr uint32_t TMEM_COLS = 512;     // S [0,192) dP [192,384) dQ [384,512)
 constexpr uint32_t COL_DP = 192, COL_DQ = 384;
-enum Bar { QD_FULL = 0, META, S_FULL = 2, DP_FULL = 5, DS_FULL = 8, V_FULL = 11, K_FULL = 14, KV_FREE = 17, N_BARS = 20 };
+enum Bar { QD_FULL = 0, META_READY, SD_FULL = 2, DS_FULL = 5, KV_FULL = 8, K_FREE = 13, N_BARS = 18 };
 template <int CPS, int MTQ>
 struct MiscT {
   unsigned long long bar[N_BARS];
   uint32_t tmem_base;
   int n_steps;
   int abort_flag;
-  int kvbase[KST][CPS];
-  float bias[KST][CPS][MTQ];
-  int pos[KST][CPS][MTQ];               // the chunk's position in the token's list (-1: none: own chunk or not routed)
+  StepMeta<CPS, MTQ, KST, true> meta;
 };
 template <int HD, int CPS, int MTQ>
 struct Layout {
   static constexpr uint32_t Q_BYTES = 128 * HD * 2;          // HD = 128: 32 KiB, two 128x64 regions
   static constexpr uint32_t KV_TILE_BYTES = NKV * HD * 2;
   static constexpr uint32_t OFF_Q = 0, OFF_DO = OFF_Q + Q_BYTES, OFF_K = OFF_DO + Q_BYTES, OFF_V = OFF_K + KST * KV_TILE_BYTES,
-                            OFF_MISC = OFF_V + KST * KV_TILE_BYTES, SMEM = OFF_MISC + sizeof(MiscT<CPS, MTQ>);
+                            OFF_MISC = OFF_V + VST * KV_TILE_BYTES, SMEM = OFF_MISC + sizeof(MiscT<CPS, MTQ>);
   static_assert(SMEM <= 232448, "one block per SM");
 };
 
@@ -174,8 +148,7 @@ template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(THREADS, 1)
 attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
-  constexpr bool WIDE = WT > 0;
-  constexpr int TPL = WIDE ? WT : 2, MTQ = 32 * TPL, W = NKV / CPS;
+  constexpr int MTQ = 32 * (WT > 0 ? WT : 2), W = NKV / CPS;
   using LY = Layout<HD, CPS, MTQ>;
   using Misc = MiscT<CPS, MTQ>;
   constexpr uint32_t Q_BYTES = LY::Q_BYTES, KV_TILE_BYTES = LY::KV_TILE_BYTES, OFF_Q = LY::OFF_Q, OFF_DO = LY::OFF_DO,
@@ -196,26 +169,23 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   const int b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int TQ = a.TQ, g_q = dm.g_q;
   const int i0 = tile * TQ;
-  const int c_own = i0 >> dm.log_b;
-  const int sub_per_blk = dm.B / NKV;
-  const int own_steps = WIDE ? (TQ + NKV - 1) / NKV : (i0 % dm.B) / NKV + 1;
 
   if (tid == 0) {
     misc->abort_flag = ((sbase & 1023u) != 0u) ? 1 : 0;
     if (misc->abort_flag) report_error(a.sb, DASH_ERR_CUDA, 110);
     ptx::mbar_init(bar(QD_FULL), 1);
-    ptx::mbar_init(bar(META), 1);
+    ptx::mbar_init(bar(META_READY), 1);
+    for (int s = 0; s < VST; ++s) {
+      ptx::mbar_init(bar(SD_FULL + s), 2);
+      ptx::mbar_init(bar(DS_FULL + s), 128);
+    }
     for (int s = 0; s < KST; ++s) {
-      ptx::mbar_init(bar(S_FULL + s), 1);
-      ptx::mbar_init(bar(DP_FULL + s), 1);
-      ptx::mbar_init(bar(DS_FULL + s), 256);
-      ptx::mbar_init(bar(K_FULL + s), 1);
-      ptx::mbar_init(bar(V_FULL + s), 1);
-      ptx::mbar_init(bar(KV_FREE + s), 1);
+      ptx::mbar_init(bar(KV_FULL + s), 1 + 32);
+      ptx::mbar_init(bar(K_FREE + s), 1);
     }
     ptx::fence_barrier_init();
   }
-  if (warp == W_S) {
+  if (warp == BWD_W_S) {
     ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), TMEM_COLS);
     ptx::tmem_relinquish();
     ptx::tc_fence_before();
@@ -234,22 +204,10 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
 
-  auto load_packed = [&](const CUtensorMap* tm, uint32_t dst, uint32_t barrier, const int* kvs) {
-    ptx::mbar_arrive_expect_tx(barrier, KV_TILE_BYTES);
-#pragma unroll
-    for (int s = 0; s < CPS; ++s) {
-      const uint32_t d = dst + s * W * 128;
-      ptx::tma_load_4d(d, tm, barrier, 0, r, kvs[s], b);
-      if constexpr (HD == 128) ptx::tma_load_4d(d + KV_TILE_BYTES / 2, tm, barrier, 64, r, kvs[s], b);
-    }
-  };
-
-  if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(WT, CPS)));
-  if (warp == W_KPROD || warp == W_VPROD) {
-    // =========================== producers: the forward kernel's walk ===========================
-    const bool do_k = (warp == W_KPROD), do_v = (warp == W_VPROD);
-    if (lane == 0 && do_k) {
+  if (warp >= BWD_W_PROD) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(bwd_regs_service(WT, CPS)));
+  if (warp == BWD_W_PROD) {
+    if (lane == 0) {
       ptx::prefetch_tensormap(&tmQ);
       ptx::prefetch_tensormap(&tmDO);
       ptx::prefetch_tensormap(&tmK);
@@ -260,96 +218,25 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       ptx::tma_load_4d(sbase + OFF_DO, &tmDO, bar(QD_FULL), 0, r * g_q, i0, b);
       if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_DO + Q_BYTES / 2, &tmDO, bar(QD_FULL), 64, r * g_q, i0, b);
     }
-    // own chunks first (steps 0 .. own_steps-1 <= 2 go to stages 0 / 1, which are free), as in the forward kernel
-    for (int sub = 0; sub < own_steps; ++sub) {
-      int kvs[CPS];
-      const int kv0 = WIDE ? i0 + sub * NKV : c_own * dm.B + sub * NKV;
-#pragma unroll
-      for (int s = 0; s < CPS; ++s) kvs[s] = WIDE && kv0 + s * W < i0 + TQ ? kv0 + s * W : kv0;
-      if (do_k) {
-        if (lane == 0) load_packed(&tmK, sbase + OFF_K + sub * KV_TILE_BYTES, bar(K_FULL + sub), kvs);
-      } else {
-        for (int t = lane; t < TQ; t += 32)
-#pragma unroll
-          for (int s = 0; s < CPS; ++s) {
-            misc->bias[sub][s][t] = (WIDE ? (kv0 + s * W) >> dm.log_b == (i0 + t) >> dm.log_b : s == 0) ? 0.f : -INFINITY;
-            misc->pos[sub][s][t] = -1;
+    produce_steps<HD, CPS, WT, KST, VST, true>(
+        a, &tmK, &tmV, grp, i0, lane, sbase + OFF_K, sbase + OFF_V, &misc->bar[KV_FULL], &misc->meta, false,
+        [&](int j) {
+          return wait_on(bar(SD_FULL + j % VST), (uint32_t)(j / VST - 1) & 1u) &&
+                 (j < KST || wait_on(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u));
+        },
+        [&](int n) {
+          if (lane == 0) {
+            misc->n_steps = n;
+            ptx::mbar_arrive(bar(META_READY));
           }
-#pragma unroll
-        for (int s = 0; s < CPS; ++s)
-          if (lane == s) misc->kvbase[sub][s] = kvs[s];
-        __syncwarp();
-        if (lane == 0) load_packed(&tmV, sbase + OFF_V + sub * KV_TILE_BYTES, bar(V_FULL + sub), kvs);
-      }
-    }
-    TileWalk<CPS, WIDE, TPL> walk(dm, a.mask, (long long)grp * dm.seq_q, i0, TQ, lane);
-    const int total = walk.count();
-    const int n_steps = (CPS > 1 ? (total + CPS - 1) / CPS : total * sub_per_blk) + own_steps;
-    if (lane == 0 && do_k) {
-      misc->n_steps = n_steps;
-      ptx::mbar_arrive(bar(META));
-    }
-    const float* list[TPL];
-#pragma unroll
-    for (int q = 0; q < TPL; ++q)
-      list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
-    walk.start();
-    bool ok = true;
-    int last_j[KST];
-#pragma unroll
-    for (int s = 0; s < KST; ++s) last_j[s] = s < own_steps ? s : -1;
-    for (int j = own_steps; j < n_steps && ok;) {
-      int cs[CPS], pos[CPS][TPL];
-      float bvs[CPS][TPL];
-      walk.next(cs, pos);
-      if (do_v) {
-#pragma unroll
-        for (int s = 0; s < CPS; ++s)
-#pragma unroll
-          for (int q = 0; q < TPL; ++q) bvs[s][q] = pos[s][q] >= 0 ? __ldg(list[q] + pos[s][q]) : -INFINITY;
-      }
-      for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk) && ok; ++sub, ++j) {
-        int kvs[CPS];
-#pragma unroll
-        for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
-        const int st = j % KST;
-        if (j >= KST) ok = wait_on(bar(KV_FREE + st), (uint32_t)(j / KST - 1) & 1u);   // every product of step j-3 has read the stage
-        if (!ok) break;
-        if (do_k) {
-          if (lane == 0) load_packed(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kvs);
-        } else {
-#pragma unroll
-          for (int s = 0; s < CPS; ++s) {
-#pragma unroll
-            for (int q = 0; q < TPL; ++q) {
-              const int t = lane + 32 * q;
-              if (t < TQ) { misc->bias[st][s][t] = bvs[s][q]; misc->pos[st][s][t] = pos[s][q]; }
-            }
-            if (lane == s) misc->kvbase[st][s] = kvs[s];
-          }
-          __syncwarp();
-          if (lane == 0) load_packed(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kvs);
-        }
-#pragma unroll
-        for (int s = 0; s < KST; ++s)
-          if (s == st) last_j[s] = j;
-      }
-    }
-    if (!ok && lane == 0) {
-      for (int s = 0; s < KST; ++s) {
-        if (last_j[s] < 0) continue;
-        const uint32_t full = bar((do_k ? K_FULL : V_FULL) + s), parity = (uint32_t)(last_j[s] / KST) & 1u;
-        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(full, parity); ++k) {}
-      }
-      if (do_k)
-        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL), 0); ++k) {}
-    }
-  } else if (warp == W_S || warp == W_DP) {
-    // =========================== issuers of S = Q K^T (warp W_S) and dP = dO V^T (warp W_DP) ===========================
-    // Ring slot j mod 3 of S / dP is free when the K / V stage of the same index is: both wait for the dQ product of
-    // step j-3 (the producers do, before they refill the stage).
+        });
+    if (lane == 0 && *abort_flag)
+      for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL), 0); ++k) {}
+  } else if (warp == BWD_W_S || warp == BWD_W_DP) {
+    // =========================== issuers of S = Q K^T and dP = dO V^T ===========================
+    // Slot j mod 3 of S / dP is free once the dQ product of step j-3 is done (which reads dS from it).
     if (lane == 0) {
-      const bool is_s = warp == W_S;
+      const bool is_s = warp == BWD_W_S;
       bool ok = wait_on(bar(QD_FULL), 0);
       int n_steps = 0x7fffffff;            // known from step 1 on; step 0 (the own chunk) always exists
       constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NKV, false, false);
@@ -358,27 +245,27 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const uint32_t col0 = is_s ? 0u : COL_DP;
       for (int j = 0; j < n_steps && ok; ++j) {
         if (j == 1) {
-          ok = wait_on(bar(META), 0);
+          ok = wait_on(bar(META_READY), 0);
           if (!ok) break;
           n_steps = misc->n_steps;
           if (j >= n_steps) break;
         }
-        const int st = j % KST;
-        ok = wait_on(bar((is_s ? K_FULL : V_FULL) + st), (uint32_t)(j / KST) & 1u);
+        ok = wait_on(bar(KV_FULL + j % KST), (uint32_t)(j / KST) & 1u);
+        if (ok && j >= VST) ok = wait_on(bar(K_FREE + (j - VST) % KST), (uint32_t)((j - VST) / KST) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint64_t bd = bd0 + (uint64_t)((st * KV_TILE_BYTES) >> 4);
+        const uint64_t bd = bd0 + (uint64_t)(((is_s ? j % KST : j % VST) * KV_TILE_BYTES) >> 4);
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) {
           const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
           const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
-          ptx::mma_bf16_ss(tmem + col0 + st * NKV, ad0 + off_a, bd + off_b, IDESC_S, k > 0 ? 1u : 0u);
+          ptx::mma_bf16_ss(tmem + col0 + (j % VST) * NKV, ad0 + off_a, bd + off_b, IDESC_S, k > 0 ? 1u : 0u);
         }
-        ptx::mma_commit(bar((is_s ? S_FULL : DP_FULL) + st));
+        ptx::mma_commit(bar(SD_FULL + j % VST));
       }
     }
     __syncwarp();
-  } else if (warp == W_DQ) {
+  } else {
     // =========================== issuer of dQ += dS K ===========================
     if (lane == 0) {
       bool ok = true;
@@ -387,33 +274,32 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const uint64_t kmn0 = ptx::smem_desc_sw128(sbase + OFF_K, KV_TILE_BYTES / 2, 1024);   // K as MN-major B
       for (int j = 0; j < n_steps && ok; ++j) {
         if (j == 1) {
-          ok = wait_on(bar(META), 0);
+          ok = wait_on(bar(META_READY), 0);
           if (!ok) break;
           n_steps = misc->n_steps;
           if (j >= n_steps) break;
         }
-        const int st = j % KST;
-        ok = wait_on(bar(DS_FULL + st), (uint32_t)(j / KST) & 1u);
+        const int slot = j % VST;
+        ok = wait_on(bar(DS_FULL + slot), (uint32_t)(j / VST) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint64_t kmn = kmn0 + (uint64_t)((st * KV_TILE_BYTES) >> 4);
+        const uint64_t kmn = kmn0 + (uint64_t)(((j % KST) * KV_TILE_BYTES) >> 4);
         // dS of keys 16k .. 16k+15: eight packed columns, keys 0-31 at columns 0-15 and keys 32-63 at columns 32-47 of the
         // step's S slot; the remainders, with two-term dS, 16 columns behind
 #pragma unroll
         for (int term = 0; term < (P2 ? 2 : 1); ++term)
 #pragma unroll
           for (int k = 0; k < NKV / 16; ++k)
-            ptx::mma_bf16_ts(tmem + COL_DQ, tmem + st * NKV + (k >> 1) * 32 + term * 16 + (k & 1) * 8,
+            ptx::mma_bf16_ts(tmem + COL_DQ, tmem + slot * NKV + (k >> 1) * 32 + term * 16 + (k & 1) * 8,
                              kmn + (uint64_t)((k * 16 * 128) >> 4), IDESC_DQ, (j > 0 || k > 0 || term > 0) ? 1u : 0u);
-        ptx::mma_commit(bar(KV_FREE + st));
+        ptx::mma_commit(bar(K_FREE + j % KST));
       }
     }
     __syncwarp();
   }
   } else {
-    // =========================== dS / epilogue: thread = tile row, warpgroup = column half ===========================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(256 - regs_service(WT, CPS)));
-    constexpr int SPH = CPS == 4 ? 2 : 1;                  // chunk slots in a half of the columns
+    // =========================== dS / epilogue: thread = tile row, warpgroup wg takes the steps wg, wg + 3, ... ===========================
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(bwd_regs_row(WT, CPS)));
     const int wg = warp >> 2;
     const int m = (warp & 3) * 32 + lane;
     const int t = m / g_q, hh = m % g_q;
@@ -425,72 +311,87 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const float lse2 = stat.x, delta = stat.y;
     float* drow = a.dbias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i_row, dm.seq_q - 1));
     bool ok = true;
-    int n_steps = 0x7fffffff;              // known from step 1 on; step 0 (the own chunk) always exists
-    for (int j = 0; j < n_steps && ok; ++j) {
-      if (j == 1) {
-        ok = wait_on(bar(META), 0);
-        if (!ok) break;
-        n_steps = misc->n_steps;
-        if (j >= n_steps) break;
-      }
-      const int st = j % KST;
-      const uint32_t ph = (uint32_t)(j / KST) & 1u;
-      ok = wait_on(bar(V_FULL + st), ph);                  // bias / pos / kvbase of the step visible
+    int n_steps = 1;                       // step 0 always exists; the others are known with the walk
+    if (wg > 0) {
+      ok = wait_on(bar(META_READY), 0);
+      n_steps = ok ? misc->n_steps : 0;
+    }
+    for (int j = wg; j < n_steps && ok; j += BWD_ROW_WG) {
+      const int slot = j % VST, rec = j % KST;
+      ok = wait_on(bar(KV_FULL + rec), (uint32_t)(j / KST) & 1u);      // the step's record is visible
       if (!ok) break;
-      float off[SPH];                                      // -inf: the row did not route the chunk
-      int pos[SPH], n_vis[SPH];                            // causal: column c of the half visible iff c < n_vis
+      float off[CPS];                                      // -inf: the row did not route the chunk
+      int pos[CPS], n_vis[CPS];                            // causal: column c of the slot visible iff c < n_vis
+      bool any = false;
 #pragma unroll
-      for (int s = 0; s < SPH; ++s) {
-        const int slot = CPS == 1 ? 0 : wg * SPH + s;
-        off[s] = row_ok ? misc->bias[st][slot][t] * LOG2E - lse2 : -INFINITY;
-        pos[s] = misc->pos[st][slot][t];
-        n_vis[s] = i_row - misc->kvbase[st][slot] + 1 + (CPS == 1 ? -wg * 32 : s * W);
+      for (int s = 0; s < CPS; ++s) {
+        off[s] = row_ok ? misc->meta.bias[rec][s][t] * LOG2E - lse2 : -INFINITY;
+        pos[s] = misc->meta.pos[rec][s][t];
+        n_vis[s] = i_row - misc->meta.kvbase[rec][s] + 1;
+        any = any || !(off[s] == -INFINITY);
       }
-      ok = wait_on(bar(S_FULL + st), ph) && wait_on(bar(DP_FULL + st), ph);
+      any = __any_sync(0xffffffffu, any);                  // a warp none of whose rows routed a chunk of the step only writes zeros
+      ok = wait_on(bar(SD_FULL + slot), (uint32_t)(j / VST) & 1u);
       if (!ok) break;
       ptx::tc_fence_after();
-      float rowsum[SPH];
-      {
-        uint32_t sv[32], gv[32];
-        DASH_TMEM_LD32(sv, lane_addr + st * NKV + wg * 32);
-        DASH_TMEM_LD32(gv, lane_addr + COL_DP + st * NKV + wg * 32);
-        ptx::tmem_wait_ld();
-        float ds[32];
+      float rowsum[CPS];
 #pragma unroll
-        for (int s = 0; s < SPH; ++s) {
-          rowsum[s] = 0.f;
+      for (int s = 0; s < CPS; ++s) rowsum[s] = 0.f;
 #pragma unroll
-          for (int c = s * (32 / SPH); c < (s + 1) * (32 / SPH); ++c) {
-            const float p = c < n_vis[s] ? exp2f(fmaf(__uint_as_float(sv[c]), c1, off[s])) : 0.f;
+      for (int half = 0; half < 2; ++half) {               // 32 columns at a time
+        uint32_t hi[16], lo[16];
+        if (any) {
+          uint32_t sv[32], gv[32];
+          DASH_TMEM_LD32(sv, lane_addr + slot * NKV + half * 32);
+          DASH_TMEM_LD32(gv, lane_addr + COL_DP + slot * NKV + half * 32);
+          DASH_TMEM_WAIT_LD32(sv);
+          DASH_TMEM_WAIT_LD32(gv);
+          float ds[32];
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            const int s = (half * 32 + c) / W;
+            const float p = half * 32 + c - s * W < n_vis[s] ? exp2f(fmaf(__uint_as_float(sv[c]), c1, off[s])) : 0.f;
             ds[c] = p * (__uint_as_float(gv[c]) - delta);
             rowsum[s] += ds[c];
           }
+          // dS -> the first 16 columns of this half of the step's S slot (two bf16 per column), the remainders behind them
+          pack_terms<P2>(ds, hi, lo);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0u;
         }
-        // dS row -> the first 16 columns of this warpgroup's own half of the step's S buffer (two bf16 per column), the
-        // remainders behind them: the other warpgroup's scores, in the other 32 columns, are never touched
-        uint32_t hi[16], lo[16];
-        pack_terms<P2>(ds, hi, lo);
-        ptx::tmem_st_n<16>(lane_addr + st * NKV + wg * 32, hi);
-        if constexpr (P2) ptx::tmem_st_n<16>(lane_addr + st * NKV + wg * 32 + 16, lo);
+        ptx::tmem_st_n<16>(lane_addr + slot * NKV + half * 32, hi);
+        if constexpr (P2) ptx::tmem_st_n<16>(lane_addr + slot * NKV + half * 32 + 16, lo);
       }
       ptx::tmem_wait_st();
       ptx::tc_fence_before();
-      ptx::mbar_arrive(bar(DS_FULL + st));
+      ptx::mbar_arrive(bar(DS_FULL + slot));
       // dbias of the (token, chunk): the row sums of the group's heads (adjacent lanes) added up
+      if (any) {
 #pragma unroll
-      for (int s = 0; s < SPH; ++s) {
-        for (int o = 1; o < g_q; o <<= 1) rowsum[s] += __shfl_xor_sync(0xffffffffu, rowsum[s], o);
-        if (hh == 0 && pos[s] >= 0 && row_ok) atomicAdd(drow + pos[s], rowsum[s]);
+        for (int s = 0; s < CPS; ++s) {
+          for (int o = 1; o < g_q; o <<= 1) rowsum[s] += __shfl_xor_sync(0xffffffffu, rowsum[s], o);
+          if (hh == 0 && pos[s] >= 0 && row_ok) atomicAdd(drow + pos[s], rowsum[s]);
+        }
+      }
+      if (j == 0) {
+        ok = wait_on(bar(META_READY), 0);
+        n_steps = ok ? misc->n_steps : 0;
       }
     }
-    // epilogue: dQ / sqrt(d) -> global; each warpgroup takes half of the row's columns
-    if (ok && n_steps > 0) ok = wait_on(bar(KV_FREE + ((n_steps - 1) % KST)), (uint32_t)((n_steps - 1) / KST) & 1u);
-    if (ok && n_steps > 0) {
+    // epilogue: dQ / sqrt(d) -> global; the warpgroups share the row's columns
+    if (ok) {
+      ok = wait_on(bar(META_READY), 0);
+      n_steps = ok ? misc->n_steps : 0;
+    }
+    // (a warpgroup has seen the scores of step n-3 or a later one, or none where n < 3: the phase before this one is over)
+    if (ok) ok = wait_on(bar(K_FREE + ((n_steps - 1) % KST)), (uint32_t)((n_steps - 1) / KST) & 1u);
+    if (ok) {
       ptx::tc_fence_after();
       __nv_bfloat16* op = a.dQ + (long long)b * dm.qs[0] + (long long)i_row * dm.qs[1] + (long long)(r * g_q + hh) * dm.qs[2];
       const float sc = dm.sm_scale;
 #pragma unroll 1
-      for (int q = wg * (HD / 64); q < (wg + 1) * (HD / 64); ++q) {
+      for (int q = wg; q < HD / 32; q += BWD_ROW_WG) {
         uint32_t o[32];
         DASH_TMEM_LD32(o, lane_addr + COL_DQ + q * 32);
         ptx::tmem_wait_ld();
@@ -513,7 +414,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   }
 
   __syncthreads();
-  if (warp == W_S) {
+  if (warp == BWD_W_S) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
   }
@@ -585,14 +486,6 @@ struct Layout {
                             OFF_MISC = OFF_P + (P2 && !SEQ ? 4 : 2) * PS_BYTES, SMEM = OFF_MISC + sizeof(Misc);
   static_assert(SMEM <= 232448, "one block per SM");
 };
-
-// 8 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
-__device__ __forceinline__ void copy_async8(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void arrive_after_copies(uint32_t bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
 
 template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -1038,13 +931,9 @@ bool make_map(CUtensorMap* out, const void* base, int hd, long long tokens, int 
   return encode_bf16_sw128_4d(out, base, dims, strides, box);
 }
 
-struct Maps {
-  CUtensorMap q, g, k, v, kc, vc;      // kc, vc: one chunk per box (the dQ kernel packs chunks below 64 tokens)
-};
-
 // dK / dV, then dQ / dbias (which overwrites what the first one reads: see the top of the file)
 template <int HD, int CPS, int WT, bool P2>
-cudaError_t launch_kernels(const BwdArgs& a, const Maps& m, cudaStream_t st) {
+cudaError_t launch_kernels(const BwdArgs& a, const BwdMaps& m, cudaStream_t st) {
   const long long groups = (long long)a.dm.batch * a.dm.h_kv;
   constexpr int MTQ = 32 * (WT > 0 ? WT : 2);
   cudaError_t e;
@@ -1067,7 +956,7 @@ cudaError_t launch_kernels(const BwdArgs& a, const Maps& m, cudaStream_t st) {
 }
 
 template <int HD, int CPS>
-cudaError_t launch_two_term(const BwdArgs& a, const Maps& m, cudaStream_t st) {
+cudaError_t launch_two_term(const BwdArgs& a, const BwdMaps& m, cudaStream_t st) {
   if (a.dm.g_q == 1) return launch_kernels<HD, CPS, 4, true>(a, m, st);
   if constexpr (CPS > 1) {
     if (a.TQ > a.dm.B) return launch_kernels<HD, CPS, 2, true>(a, m, st);
@@ -1090,6 +979,7 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   a.TQ = 128 / dm.g_q;
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
   a.n_slices = (dm.seq_kv + NKV - 1) / NKV;
+  a.inject = test_hooks().skip_own_k_load;
   a.wait_limit = test_hooks().wait_limit_cycles;
   a.mask = mask; a.blk_bias = blk_bias; a.marks = reinterpret_cast<int*>(dbias);
   a.dQ = (__nv_bfloat16*)dQ; a.dK = dK; a.dV = dV; a.dbias = dbias; a.sb = sb;
@@ -1104,16 +994,7 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
     const long long blocks = (long long)a.n_slices * dm.batch * dm.h_kv;
     a.n_split = (int)std::max<long long>(1, std::min<long long>({2 * n_sm / blocks, a.n_tiles / 4, 16}));
   }
-  // forward recomputation in statistics mode: log-sum-exp and delta of every row (O itself is not written)
-  e = launch_attend_prefill_sm100(dm, Q, K, V, mask, blk_bias, nullptr, sb, false, st, a.stats, dO);
-  if (e != cudaSuccess) return e;
-  const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
-  e = launch_chained(list_marks_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
-                     mask, a.marks, dK, dV, a.n_split > 1 ? (long long)dm.batch * dm.seq_kv * dm.h_kv * dm.d : 0LL);
-  count_launch();
-  if (e != cudaSuccess) return e;
-
-  Maps m;
+  BwdMaps m;
   const int box_kv = dm.B < NKV ? dm.B : NKV;
   if (!make_map(&m.q, Q, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
   if (!make_map(&m.g, dO, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.os, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
@@ -1121,6 +1002,13 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   if (!make_map(&m.v, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, NKV)) return cudaErrorInvalidValue;
   if (!make_map(&m.kc, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, box_kv)) return cudaErrorInvalidValue;
   if (!make_map(&m.vc, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, box_kv)) return cudaErrorInvalidValue;
+  if ((e = launch_attend_bwd_stats(a, m, st)) != cudaSuccess) return e;
+  const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
+  e = launch_chained(list_marks_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
+                     mask, a.marks, dK, dV, a.n_split > 1 ? (long long)dm.batch * dm.seq_kv * dm.h_kv * dm.d : 0LL);
+  count_launch();
+  if (e != cudaSuccess) return e;
+
   if (!two_term) {
     if (dm.d != 128 || dm.B < NKV || dm.g_q < 2) return cudaErrorInvalidValue;
     return launch_kernels<128, 1, 0, false>(a, m, st);

@@ -99,20 +99,14 @@ struct PrefillArgs {
   long long wait_limit;   // cycles a bounded wait may spin
   const uint32_t* mask;
   const float* blk_bias;
-  __nv_bfloat16* O;          // may be null when only the row statistics are wanted
-  // Row statistics for the backward pass (base null: not wanted): the log-sum-exp of the row's logits in the log2 domain
-  // and delta = <O_row, dO_row> (dO: strides of O), both from the fp32 accumulator.
-  RowStats stats;
-  const __nv_bfloat16* dO;
+  __nv_bfloat16* O;
   StatusBlock* sb;
 };
 
 // WT > 0: a wide tile, which may span several chunks (chunks shorter than 128 / g_q tokens, or g_q = 1), of at most
 // 32 * WT tokens; tiles inside one chunk (WT = 0, at most 64 tokens) compile without the per-row own chunks.
 // P2: P enters the P V product as two bf16 terms (P = hi + lo, the remainder in the second half of the step's S columns),
-// so O is accurate to fp32 class instead of bf16 class.  Taken for g_q = 1 and, whatever the group size, when the row
-// statistics for the backward pass are wanted (delta = <O, dO> feeds the gradient of the routing, which amplifies its
-// error).
+// so O is accurate to fp32 class instead of bf16 class.  Taken for g_q = 1.
 template <int HD, int CPS, int WT, bool P2>
 __global__ void __launch_bounds__(PF_THREADS, 2)
 attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -553,30 +547,14 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
     if (ok && n_steps > 0) {
       ptx::tc_fence_after();
       const float inv = l > 0.f ? 1.f / l : 0.f;
-      const long long o_off = (long long)b * dm.os[0] + (long long)i_row * dm.os[1] + (long long)(r * g_q + hh) * dm.os[2];
-      __nv_bfloat16* op = a.O + o_off;
+      __nv_bfloat16* op = a.O + (long long)b * dm.os[0] + (long long)i_row * dm.os[1] + (long long)(r * g_q + hh) * dm.os[2];
       const bool row_out = i_row < dm.seq_q;
-      float dot = 0.f;
 #pragma unroll 1
       for (int q = 0; q < HD / 32; ++q) {
         uint32_t o[32];
         DASH_TMEM_LD32(o, lane_addr + 2 * NKV + q * 32);
         ptx::tmem_wait_ld();
-        if (P2 && a.stats.base && row_out) {
-          const __nv_bfloat16* gp = a.dO + o_off + q * 32;
-#pragma unroll
-          for (int c = 0; c < 32; c += 8) {
-            const uint4 gv = *reinterpret_cast<const uint4*>(gp + c);
-            const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&gv);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const float2 gf = __bfloat1622float2(g2[u]);
-              dot = fmaf(__uint_as_float(o[c + 2 * u]), gf.x, dot);
-              dot = fmaf(__uint_as_float(o[c + 2 * u + 1]), gf.y, dot);
-            }
-          }
-        }
-        if (a.O && row_out) {
+        if (row_out) {
 #pragma unroll
           for (int c = 0; c < 32; c += 8) {
             uint4 v;
@@ -590,16 +568,11 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
           }
         }
       }
-      if (P2 && a.stats.base && row_out) *a.stats.at(b, r, i_row, hh) = make_float2(m_used + log2f(l), dot * inv);
     }
     ptx::tc_fence_before();
   }
 
   __syncthreads();
-  if (P2 && a.stats.base && misc->abort_flag) {       // the kernels behind this one carry it on to every gradient of these rows
-    for (int m = tid; m < 128; m += PF_THREADS)
-      if (i0 + m / g_q < dm.seq_q) *a.stats.at(b, r, i0 + m / g_q, m % g_q) = make_float2(gave_up(), gave_up());
-  }
   if (release_late) chain_release();
   if (warp == 5) {
     ptx::tc_fence_after();
@@ -654,13 +627,11 @@ static cudaError_t launch_one(const PrefillArgs& a, const CUtensorMap& tq, const
 template <int HD, int CPS>
 static cudaError_t launch_cps(const PrefillArgs& a, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                               cudaStream_t st) {
-  const bool stats = a.stats.base != nullptr;
   if (a.dm.g_q == 1) return launch_one<HD, CPS, 4, true>(a, tq, tk, tv, st);
   if constexpr (CPS > 1) {
-    if (a.TQ > a.dm.B)
-      return stats ? launch_one<HD, CPS, 2, true>(a, tq, tk, tv, st) : launch_one<HD, CPS, 2, false>(a, tq, tk, tv, st);
+    if (a.TQ > a.dm.B) return launch_one<HD, CPS, 2, false>(a, tq, tk, tv, st);
   }
-  return stats ? launch_one<HD, CPS, 0, true>(a, tq, tk, tv, st) : launch_one<HD, CPS, 0, false>(a, tq, tk, tv, st);
+  return launch_one<HD, CPS, 0, false>(a, tq, tk, tv, st);
 }
 
 template <int HD>
@@ -672,10 +643,8 @@ static cudaError_t launch_hd(const PrefillArgs& a, const CUtensorMap& tq, const 
 
 cudaError_t launch_attend_prefill_sm100(const Dims& dm, const void* Q, const void* K, const void* V,
                                         const uint32_t* mask, const float* blk_bias, void* O, StatusBlock* sb,
-                                        bool inputs_stable, cudaStream_t st, const RowStats& stats, const void* dO) {
+                                        bool inputs_stable, cudaStream_t st) {
   PrefillArgs a;
-  a.stats = stats;
-  a.dO = (const __nv_bfloat16*)dO;
   a.dm = dm;
   a.TQ = 128 / dm.g_q;
   a.n_tiles = (dm.seq_q + a.TQ - 1) / a.TQ;
