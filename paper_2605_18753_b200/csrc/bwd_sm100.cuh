@@ -19,10 +19,12 @@ struct BwdArgs {
   int n_split;        // blocks that share a slice's query tiles (1: they write dK / dV, more: they add to them)
   int inject;         // test hook: 1 = the statistics pass never loads the own chunk's keys (the waits for them run out)
   long long wait_limit;
+  const __nv_bfloat16* Q;
+  const __nv_bfloat16* dO;
   const uint32_t* mask;
   const float* blk_bias;
   RowStats stats;
-  int* marks;         // counts and unions, in the layout of the lists
+  int* marks;         // counts, in the layout of the lists
   __nv_bfloat16* dQ;
   float* dK;
   float* dV;
@@ -31,7 +33,7 @@ struct BwdArgs {
 };
 
 struct BwdMaps {
-  CUtensorMap q, g, k, v, kc, vc;      // kc, vc: one chunk per box (query-tile-stationary kernels pack chunks below 64 tokens)
+  CUtensorMap q, g, k, v, kc, vc;      // q, g: a query tile per box; kc, vc: one chunk per box (query-tile-stationary kernels pack chunks below 64 tokens)
 };
 
 cudaError_t launch_attend_bwd_stats(const BwdArgs& a, const BwdMaps& m, cudaStream_t st);
@@ -53,12 +55,15 @@ constexpr int BWD_ROW_WG = 3, BWD_ROW_THREADS = (BWD_ROW_WG + 1) * 128, BWD_W_PR
 __host__ __device__ constexpr int bwd_regs_service(int wt, int cps) { return wt > 2 || (wt > 0 && cps > 2) ? 104 : wt > 0 || cps > 1 ? 80 : 56; }
 __host__ __device__ constexpr int bwd_regs_row(int wt, int cps) { return (4 * 128 - bwd_regs_service(wt, cps)) / 3 / 8 * 8; }
 
-// 4 or 8 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
+// 4, 8 or 16 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
 __device__ __forceinline__ void copy_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void copy_async8(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void arrive_after_copies(uint32_t bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");

@@ -6,18 +6,17 @@
 //     dQ = dS K / sqrt(d),   dK = dS^T Q / sqrt(d),   dV = P^T dO,   dbias_c = sum of dS over the chunk's tokens.
 // Three launches behind the statistics pass (prefill_bwd_stats_sm100.cu; it leaves the log-sum-exp and delta of every row):
 //   list_marks_kernel       per row, the number of routed chunks in the mask words before each word (so that a row's
-//                           list entry for a chunk can be found from one word of its mask), and per query tile the OR of
-//                           its rows' mask words (which chunks any of its rows routed);
-//   attend_bwd_dkv_kernel   key-slice stationary (64 keys of one KV head): walks the query tiles that attend the slice
-//                           (the tiles of its own chunks, causally masked, then every later tile whose union holds one of
-//                           its chunks), computes S and dP, and accumulates dV^T += dO^T P and dK^T += Q^T dS in tensor
-//                           memory (P and dS pass through shared memory as bf16 MN-major operands);
+//                           list entry for a chunk can be found from one word of its mask);
+//   attend_bwd_dkv_kernel   key-slice stationary (64 keys of one KV head): gathers the tokens that attend the slice (those of
+//                           its own chunks, causally masked, then every later one that routed one of its chunks) into steps
+//                           of 128 (token, head) rows, computes S and dP, and accumulates dV^T += dO^T P and dK^T += Q^T dS
+//                           in tensor memory (P and dS pass through shared memory as bf16 MN-major operands);
 //   attend_bwd_dq_kernel    query-tile stationary, the forward kernel's walk over the union of the tile's routed
 //                           chunks: S = Q K^T and dP = dO V^T into tensor memory, dS (bf16) back into tensor memory,
 //                           dQ += dS K accumulated in tensor memory; dbias from the row sums of dS.
 // What passes between them needs no scratch of its own: a row's statistics sit in the first eight bytes of its dQ row until
-// the dQ kernel, which owns the row, overwrites them; the counts and unions sit in the rows' regions of dbias (a row with
-// own chunk c has c entries there, and c >= 2 floor(c / 32) + 1), which the dQ kernel's block zeroes for its own rows first.
+// the dQ kernel, which owns the row, overwrites them; the counts sit in the rows' regions of dbias (a row with own chunk c has
+// c entries there, and c >= floor(c / 32)), which the dQ kernel's block zeroes for its own rows first.
 // A block whose wait ran out writes NaN in the place of its statistics or gradients: the entry point without a status word has
 // no other way to say so, and what the buffers held as scratch must not pass for gradients.
 //
@@ -27,7 +26,7 @@
 //
 // Bound by the chain of a step (tile landed -> S, dP -> P, dS -> accumulating products), one block per SM.  2 x 1500 tokens,
 // 8/2 heads, d 64, chunks of 32: 2.02 ms on CUDA cores (one warp per row and head, two vector reductions per token and
-// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: statistics 0.40 -> 0.39, dK / dV 1.05, dQ 0.59 -> 0.56 ms.
+// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: statistics 0.39, dK / dV 0.57, dQ 0.56 ms.
 #include <cuda.h>
 
 #include <algorithm>
@@ -41,60 +40,35 @@ namespace {
 
 constexpr int NKV = BWD_NKV;
 
-// Where a row's counts start (entry w - 1: routed chunks in mask words 0 .. w - 1), and the unions of the tile whose last
-// row it is (behind the counts, one per mask word).
+// Where a row's counts start (entry w - 1: routed chunks in mask words 0 .. w - 1).
 __device__ __forceinline__ long long marks_of(const Dims& dm, long long grp, int i) {
   return grp * dm.list_rows + list_row_offset(dm, i);
 }
 
 __global__ void __launch_bounds__(256)
-list_marks_kernel(Dims dm, int TQ, int n_tiles, const uint32_t* __restrict__ mask, int* __restrict__ marks, float* zero_a, float* zero_b,
-                  long long zero_n) {
+list_marks_kernel(Dims dm, const uint32_t* __restrict__ mask, int* __restrict__ marks, float* zero_a, float* zero_b, long long zero_n) {
   chain_wait();
   chain_release();
-  const long long thread = (long long)blockIdx.x * blockDim.x + threadIdx.x, warp_id = thread >> 5;
+  const long long thread = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (zero_n > 0) {            // dK, dV: several blocks of the next kernel add to them
     zero_floats(zero_a, zero_n, thread, (long long)gridDim.x * blockDim.x);
     zero_floats(zero_b, zero_n, thread, (long long)gridDim.x * blockDim.x);
   }
-  const int lane = threadIdx.x & 31;
-  if (warp_id >= (long long)dm.batch * dm.h_kv * n_tiles) return;
-  const long long grp = warp_id / n_tiles;
-  const int i0 = (int)(warp_id % n_tiles) * TQ;
-  const int n_live = min(TQ, dm.seq_q - i0), i_last = i0 + n_live - 1, c_last = i_last / dm.B;
-  if (c_last == 0) return;                      // nothing routed, and no room in the rows' regions
-  const long long last = marks_of(dm, grp, i_last) + (c_last >> 5);
-  int acc[4] = {0, 0, 0, 0}, own[4];
-  long long at[4];
-  uint32_t next[4] = {0u, 0u, 0u, 0u};
-  const uint32_t* row[4];
+  if (thread >= (long long)dm.batch * dm.h_kv * dm.seq_q) return;
+  const long long grp = thread / dm.seq_q;
+  const int i = (int)(thread % dm.seq_q), last_w = (i >> dm.log_b) >> 5;      // (the words before the own chunk's hold routed chunks only)
+  const uint32_t* row = mask + thread * dm.W;
+  int* out = marks + marks_of(dm, grp, i);
+  int acc = 0;
+  for (int w0 = 0; w0 < last_w; w0 += 4) {
+    uint32_t word[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int i = min(i0 + lane + 32 * q, i_last);
-    own[q] = lane + 32 * q < n_live ? i >> dm.log_b : -1;      // -1: no such token
-    at[q] = marks_of(dm, grp, i);
-    row[q] = mask + (grp * dm.seq_q + i) * dm.W;
-    if (own[q] >= 0) next[q] = row[q][0];
-  }
-  const int last_w = c_last >> 5;
-  for (int w = 0; w <= last_w; ++w) {
-    uint32_t u = 0u, word[4];
+    for (int k = 0; k < 4; ++k) word[k] = w0 + k < last_w ? row[w0 + k] : 0u;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      word[q] = next[q];
-      if (w < last_w && own[q] >= 0) next[q] = row[q][w + 1];      // one word ahead
+    for (int k = 0; k < 4; ++k) {
+      acc += __popc(word[k]);
+      if (w0 + k < last_w) out[w0 + k] = acc;
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (own[q] >= 0) {
-        const uint32_t bits = routed_bits(word[q], w, own[q]);
-        if (w > 0 && w <= (own[q] >> 5)) marks[at[q] + w - 1] = acc[q];
-        acc[q] += __popc(bits);
-        u |= bits;
-      }
-    }
-    u = __reduce_or_sync(0xffffffffu, u);
-    if (lane == 0) marks[last + w] = (int)u;
   }
 }
 
@@ -441,16 +415,26 @@ namespace dkv {
 
 // Two warpgroups form P and dS, each for half of the slice's keys on every step (no row maximum is needed, so the halves
 // are independent and a step's P / dS stretch takes half as long); one issuing thread per product: 32 MMAs per step
-// are too many for one.  W_PROD loads the tiles, W_META looks up the per-token biases and row statistics of each step;
-// W_SD issues S, W_DP dP, W_ACC dV^T, W_DK dK^T.
-constexpr int W_PROD = 8, W_SD = 9, W_ACC = 10, W_DP = 11, W_DK = 12, W_META = 13;
-constexpr int THREADS = 512;              // 8 P / dS warps, 6 service warps, 2 idle: whole warpgroups
-__host__ __device__ constexpr int regs_service(int wt) { return wt > 0 ? 96 : 80; }     // (the bias and loader warps need more than the issuers)
-static_assert(THREADS == 512, "two pairs of warpgroups: one pair can take exactly what the other released");
+// are too many for one.  W_SCAN reads the slice's column of the mask and collects the tokens that attend the slice; the
+// loader warps copy their rows, 16 bytes per lane; W_META looks up their biases and statistics.  W_SD issues S, W_DP dP, W_ACC
+// dV^T, W_DK dK^T.
+// 8192 tokens, 32/8 heads, chunks of 64, 29 % of the chunks routed: whole query tiles of 32 tokens, of which one in two has a
+// token for the slice, 87.8 K steps and 1.05 ms; gathered 37.7 K steps and 0.57 ms.  A TMA box per token and half row instead of the
+// copies: 27 clocks of the TMA unit each, 128 of them a step, 0.85 ms.  The seven roles share an instruction cache: with the
+// scanner's and loaders' loops unrolled eight to sixteen times every role slows down, 0.77-1.15 ms.
+constexpr int W_SD = 8, W_ACC = 9, W_DP = 10, W_DK = 11, W_META = 12, W_SCAN = 13;
+// Loaders: four in a warpgroup of their own; two-term kernels, whose P / dS threads keep 64 sums, make do with the two warps left.
+__host__ __device__ constexpr int n_load(bool p2) { return p2 ? 2 : 4; }
+__host__ __device__ constexpr int w_load(bool p2) { return p2 ? 14 : 16; }
+__host__ __device__ constexpr int threads(bool p2) { return p2 ? 512 : 640; }
+// registers per thread after the re-division (at launch: 128 with two terms, 96 with one)
+__host__ __device__ constexpr int regs_service(bool p2, int tpl) { return p2 ? (tpl > 2 ? 96 : 80) : 64; }
+__host__ __device__ constexpr int regs_rows(bool p2, int tpl) { return p2 ? 256 - regs_service(p2, tpl) : 144; }
+static_assert(2 * regs_rows(false, 2) + 3 * regs_service(false, 2) <= 5 * 96, "the block's own pool is all that it can draw from");
 constexpr uint32_t TMEM_COLS = 512;     // S0 S1 [0,128) dP0 dP1 [128,256) dV^T [256,320) dK^T [320,384)
 constexpr uint32_t COL_DP = 128, COL_DV = 256, COL_DK = 320;
 constexpr uint32_t PS_BYTES = 128 * NKV * 2;       // 16 KiB: one term of P (or dS) of a step, 128 rows of 128 bytes
-constexpr int MAX_STAGES = 4;
+constexpr int MAX_STAGES = 4, MAX_SLOTS = 16, SCAN_AHEAD = 16;
 // Two-term kernels take their sums out of tensor memory every FLUSH steps and add them up in registers: the tensor cores cut the
 // low bits of an accumulator off at every product, so that a sum left there loses about half a unit per product, the longer
 // the walk the more.  dK against float64, 16 heads per KV head, d 64 (relative 2-norm): 1500 tokens 1.3e-5 -> 2.5e-6, 6000
@@ -458,7 +442,9 @@ constexpr int MAX_STAGES = 4;
 constexpr int FLUSH = 2;
 // SD_FULL: both score products of the step (two arrivals).  PDS_FULL: P and dS in shared memory (SEQ: P alone).
 // ACC_DONE: both accumulating products done (SEQ: dK, which follows dV), the step's stage and the P / dS buffers are free.
-enum Bar { KV_FULL = 0, SD_FULL = 1, PDS_FULL = 3, DV_DONE = 5, DS_FULL = 7, QD_FULL = 9, ACC_DONE = 9 + MAX_STAGES, N_BARS = 9 + 2 * MAX_STAGES };
+// TOK_FULL / TOK_FREE: a step's tokens are listed / have been read by W_PROD and W_META.
+enum Bar { KV_FULL = 0, SD_FULL = 1, PDS_FULL = 3, DV_DONE = 5, DS_FULL = 7, QD_FULL = 9, ACC_DONE = 9 + MAX_STAGES,
+           TOK_FULL = 9 + 2 * MAX_STAGES, TOK_FREE = TOK_FULL + MAX_SLOTS, N_BARS = TOK_FREE + MAX_SLOTS };
 
 // A stage holds a Q and a dO tile.  head_dim 128: two stages, Q then dO.  head_dim 64: four stages, dO then Q, so that the
 // two tiles read as MN-major A stack to the M = 128 rows that an accumulating product needs: lanes 0-63 of dO^T P are
@@ -469,13 +455,20 @@ template <int HD, int CPS, int MTQ, bool P2>
 struct Layout {
   static constexpr int NST = HD == 128 ? 2 : 4;
   static constexpr bool SEQ = P2 && HD == 128;
+  static constexpr int LOG_RING = MTQ > 64 ? 8 : 7, RING = 1 << LOG_RING;      // tokens that W_SCAN is ahead: 2 steps of MTQ tokens .. 16 of 8
   struct Misc {
     unsigned long long bar[N_BARS];
     uint32_t tmem_base;
     int abort_flag;
     int total;                            // number of steps, written with the end marker
-    int tile[NST];                        // query tile of the stage's step (-1: no more steps)
-    float bias[NST][CPS][MTQ];            // per token of the tile: the chunk's bias (-inf: the token does not attend it)
+    int live[NST];                        // 1: the stage holds a step, -1: no more steps
+    int irow[NST][MTQ];                   // token of each of the step's rows
+    float bias[NST][CPS][MTQ];            // per token of the step: the chunk's bias (-inf: the token does not attend it)
+    // what W_SCAN hands on: tokens (bit 31: a repetition that fills up the last step) and their mask words over the slice's
+    // chunks, step after step; last[slot]: no such step
+    int tok[RING], last[MAX_SLOTS];
+    uint32_t word[RING];
+    uint32_t ahead[SCAN_AHEAD][32];       // mask words that W_SCAN has asked for
     alignas(16) float2 stats[NST][128];   // log-sum-exp and delta of the tile's rows
   };
   static constexpr uint32_t Q_BYTES = 128 * HD * 2, KV_TILE_BYTES = NKV * HD * 2, STAGE = 2 * Q_BYTES;
@@ -487,12 +480,12 @@ struct Layout {
   static_assert(SMEM <= 232448, "one block per SM");
 };
 
-template <int HD, int CPS, int WT, bool P2>
-__global__ void __launch_bounds__(THREADS, 1)
-attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
-                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
-  constexpr bool WIDE = WT > 0;
-  constexpr int TPL = WIDE ? WT : 2, MTQ = 32 * TPL;
+// TPL: tokens per lane of the service warps, a step's tokens being at most 32 * TPL.
+template <int HD, int CPS, int TPL, bool P2>
+__global__ void __launch_bounds__(threads(P2), 1)
+attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
+  constexpr int NLOAD = n_load(P2), W_LOAD = w_load(P2), THREADS = threads(P2);
+  constexpr int MTQ = 32 * TPL;
   using LY = Layout<HD, CPS, MTQ, P2>;
   using Misc = typename LY::Misc;
   constexpr int NST = LY::NST;
@@ -515,15 +508,20 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   const int TQ = a.TQ, g_q = dm.g_q;
   const int k0 = slice * NKV;                                    // first key of the slice
   const int c = k0 >> dm.log_b;                                       // its first chunk (CPS of them)
+  const int log_t = 31 - __clz(TQ), log_slots = LY::LOG_RING - log_t, n_slots = 1 << log_slots;      // a step has TQ tokens; steps in W_SCAN's ring (2 .. 16)
 
   if (tid == 0) {
     misc->abort_flag = ((sbase & 1023u) != 0u) ? 1 : 0;
     if (misc->abort_flag) report_error(a.sb, DASH_ERR_CUDA, 120);
     ptx::mbar_init(bar(KV_FULL), 1);
     for (int s = 0; s < NST; ++s) {
-      // the loader's arrival (with the byte count), the bias warp's, and one per lane of it for the statistics in flight
-      ptx::mbar_init(bar(QD_FULL + s), 34);
+      // one arrival of the first loader, one of W_META, and one per lane of each for the copies in flight
+      ptx::mbar_init(bar(QD_FULL + s), 2 + 32 * (NLOAD + 1));
       ptx::mbar_init(bar(ACC_DONE + s), SEQ ? 1 : 2);
+    }
+    for (int s = 0; s < n_slots; ++s) {
+      ptx::mbar_init(bar(TOK_FULL + s), 1);
+      ptx::mbar_init(bar(TOK_FREE + s), NLOAD + 1);
     }
     for (int s = 0; s < 2; ++s) {
       ptx::mbar_init(bar(SD_FULL + s), 2);
@@ -547,18 +545,88 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   __syncthreads();
 
   if (warp >= 8) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(WT)));
-  if (warp == W_PROD || warp == W_META) {
-    // =========================== producers ===========================
-    // Both warps enumerate the slice's steps in the same order: (i) the tiles that hold tokens of the slice's own
-    // chunks from k0 on (causal mask in the kernel), (ii) the later tiles one of whose rows routed one of its chunks, read
-    // 32 tiles at a time from the tile unions.  With several blocks per slice, block s takes every n_split-th of them.
-    // W_PROD fetches K / V once and the Q / dO tiles of every step; W_META looks up the per-token biases and the row
-    // statistics.  A step's stage is free once both accumulating products of the step NST before have completed.
-    const bool loader = warp == W_PROD;
-    if (lane == 0 && loader) {
-      ptx::prefetch_tensormap(&tmQ);
-      ptx::prefetch_tensormap(&tmDO);
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_service(P2, TPL)));
+  const int wc = c >> 5, bit = c & 31;             // (the slice's chunks share a mask word)
+  const long long row0 = (long long)grp * dm.seq_q;
+  if (warp == W_SCAN) {
+    // =========================== scanner ===========================
+    // The tokens from k0 on, 32 at a time, the mask words of the next groups on their way to shared memory; those that attend the
+    // slice (its own chunks' tokens, and later ones that routed one of them) are appended to the ring.  With several blocks per
+    // slice, block s takes every n_split-th group.  (A short loop on purpose: one warp that runs through unrolled code waits for its
+    // instructions, and pushes the other roles' out of the cache.)
+    const int stride = 32 * a.n_split;
+    bool ok = true;
+    int n = 0, free_slots = n_slots, done = 0;      // tokens so far; steps that may be written; steps handed on
+    auto reserve = [&](int steps) {
+      for (; free_slots < steps && ok; ++free_slots)
+        ok = wait_on(bar(TOK_FREE + (free_slots & (n_slots - 1))), (uint32_t)((free_slots >> log_slots) - 1) & 1u);
+    };
+    auto hand_on = [&](int steps, bool last) {
+      __syncwarp();
+      if (lane == 0)
+        for (int k = done; k < steps; ++k) {
+          misc->last[k & (n_slots - 1)] = last;
+          ptx::mbar_arrive(bar(TOK_FULL + (k & (n_slots - 1))));
+        }
+      done = steps;
+    };
+    const int i_first = k0 + 32 * (int)blockIdx.y + lane;
+    const uint32_t* src = a.mask + (row0 + i_first) * dm.W + wc;
+    const long long src_step = (long long)stride * dm.W;
+    const uint32_t ahead = ptx::smem_u32(&misc->ahead[0][lane]);
+    int i_next = i_first;                           // token whose word is asked for next
+    uint32_t g = 0;                                 // groups looked at
+    auto ask = [&](uint32_t group) {
+      if (i_next < dm.seq_q) copy_async4(ahead + (group & (SCAN_AHEAD - 1)) * 128, src);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      src += src_step;
+      i_next += stride;
+    };
+#pragma unroll 1
+    for (uint32_t k = 0; k < SCAN_AHEAD - 1; ++k) ask(k);
+#pragma unroll 1
+    for (int i = i_first; i - lane < dm.seq_q && ok; i += stride, ++g) {
+      ask(g + SCAN_AHEAD - 1);
+      asm volatile("cp.async.wait_group %0;" ::"n"(SCAN_AHEAD - 1) : "memory");
+      const uint32_t word = misc->ahead[g & (SCAN_AHEAD - 1)][lane];      // (only this lane wrote it)
+      const int own = i >> dm.log_b;
+      bool on = false;
+#pragma unroll
+      for (int s = 0; s < CPS; ++s) on = on || c + s == own || (c + s < own && ((word >> (bit + s)) & 1u));
+      const uint32_t hit = __ballot_sync(0xffffffffu, on && i < dm.seq_q);
+      if (hit == 0u) continue;
+      const int e = (n + __popc(hit & ((1u << lane) - 1u))) & (LY::RING - 1);
+      n += __popc(hit);
+      reserve(((n - 1) >> log_t) + 1);
+      if ((hit >> lane) & 1u) {
+        misc->tok[e] = i;
+        misc->word[e] = word;
+      }
+      if ((n >> log_t) > done) hand_on(n >> log_t, false);
+    }
+    const int steps = (n + TQ - 1) >> log_t;
+    if (ok && steps > done) {                       // fill up the last step with copies of a token whose weights will be zero
+      __syncwarp();
+      const int copy = misc->tok[(done << log_t) & (LY::RING - 1)] | (int)0x80000000;
+#pragma unroll 1
+      for (int e = n + lane; e < steps << log_t; e += 32) {
+        misc->tok[e & (LY::RING - 1)] = copy;
+        misc->word[e & (LY::RING - 1)] = 0u;
+      }
+      hand_on(steps, false);
+    }
+    reserve(steps + 1);
+    if (ok) hand_on(steps + 1, true);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else if (warp >= W_LOAD && warp < W_LOAD + NLOAD) {
+    // =========================== loaders ===========================
+    // The first one fetches K / V, all of them the Q / dO rows of every step's tokens: a lane copies one 16-byte piece of a row, to
+    // where the 128-byte swizzle has it.  A step's stage is free once both accumulating products of the step NST before have
+    // completed.  (cp.async writes through the generic proxy: the issuers fence before their products read the stage.)
+    constexpr int PIECES = HD / 8, RP = 32 / PIECES;      // pieces of a row, rows of a warp's copy
+    constexpr int NR = 16 / (RP * NLOAD);                 // of sixteen rows at a time, a loader copies NR x RP
+    const int w = warp - W_LOAD, p = lane % PIECES;
+    if (w == 0 && lane == 0) {
       ptx::prefetch_tensormap(&tmK);
       ptx::prefetch_tensormap(&tmV);
       ptx::mbar_arrive_expect_tx(bar(KV_FULL), 2 * KV_TILE_BYTES);
@@ -567,151 +635,109 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ptx::tma_load_4d(sbase + OFF_V, &tmV, bar(KV_FULL), 0, r, k0, b);
       if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_V + KV_TILE_BYTES / 2, &tmV, bar(KV_FULL), 64, r, k0, b);
     }
-    const long long row0 = (long long)grp * dm.seq_q;
-    const long long list0 = (long long)grp * dm.list_rows;
-    const int wc = c >> 5, bit = c & 31;             // (the slice's chunks share a mask word)
-    // this lane's rows of a tile (lane, lane + 32, ...): their statistics relative to the tile's first token
-    const char* stat_p[4];
-    int stat_t[4];
+    // (sixteen rows on, a row has the same head of the group and the same place in the swizzle)
+    const char *q0[NR], *g0[NR];
+    uint32_t dst0[NR], tok0[NR];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int m = lane + 32 * k;
-      stat_t[k] = m / g_q;
-      stat_p[k] = reinterpret_cast<const char*>(a.stats.at(b, r, stat_t[k], m % g_q));
+    for (int k = 0; k < NR; ++k) {
+      const int m = (w + k * NLOAD) * RP + lane / PIECES, head = r * g_q + (m & (g_q - 1));
+      q0[k] = reinterpret_cast<const char*>(a.Q + (long long)b * dm.qs[0] + head * dm.qs[2] + p * 8);
+      g0[k] = reinterpret_cast<const char*>(a.dO + (long long)b * dm.os[0] + head * dm.os[2] + p * 8);
+      dst0[k] = sbase + LY::OFF_ST + (p >> 3) * (Q_BYTES / 2) + m * 128 + (((p ^ m) & 7) << 4);
+      tok0[k] = m / g_q;
     }
-    int j = 0;
+    const long long q_tok = dm.qs[1] * 2, g_tok = dm.os[1] * 2;
     bool ok = true;
-    auto stage_free = [&]() {
-      if (j >= NST) ok = wait_on(bar(ACC_DONE + j % NST), (uint32_t)(j / NST - 1) & 1u);
-      return ok;
-    };
-    // ---- the loader's step
-    auto load_step = [&](int tile_idx) {
-      if (!stage_free()) return;
-      const int st = j % NST;
+    for (int j = 0;; ++j) {
+      const int st = j % NST, sl = j & (n_slots - 1);
+      ok = wait_on(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
+      if (ok && j >= NST) ok = wait_on(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      if (!ok) break;
+      const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
+      if (!end) {
+        const int* tok = misc->tok + (sl << log_t);
+        uint32_t at = st * LY::STAGE;
+#pragma unroll 1
+        for (int it = 0; it < 8; ++it, at += 16 * 128, tok += 16 / g_q) {
+          uint32_t i[NR];
+#pragma unroll
+          for (int k = 0; k < NR; ++k) i[k] = (uint32_t)tok[tok0[k]] & 0x7fffffffu;
+#pragma unroll
+          for (int k = 0; k < NR; ++k) {
+            copy_async16(dst0[k] + at + LY::AT_Q, q0[k] + (unsigned long long)i[k] * q_tok);
+            copy_async16(dst0[k] + at + LY::AT_G, g0[k] + (unsigned long long)i[k] * g_tok);
+          }
+        }
+      }
+      arrive_after_copies(bar(QD_FULL + st));
+      __syncwarp();
       if (lane == 0) {
-        misc->tile[st] = tile_idx;
-        if (tile_idx >= 0) {
-          const int i0 = tile_idx * TQ;
-          const uint32_t dq = sbase + LY::OFF_ST + st * LY::STAGE + LY::AT_Q, dg = sbase + LY::OFF_ST + st * LY::STAGE + LY::AT_G;
-          ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), 2 * Q_BYTES);
-          ptx::tma_load_4d(dq, &tmQ, bar(QD_FULL + st), 0, r * g_q, i0, b);
-          if constexpr (HD == 128) ptx::tma_load_4d(dq + Q_BYTES / 2, &tmQ, bar(QD_FULL + st), 64, r * g_q, i0, b);
-          ptx::tma_load_4d(dg, &tmDO, bar(QD_FULL + st), 0, r * g_q, i0, b);
-          if constexpr (HD == 128) ptx::tma_load_4d(dg + Q_BYTES / 2, &tmDO, bar(QD_FULL + st), 64, r * g_q, i0, b);
-        } else {
+        ptx::mbar_arrive(bar(TOK_FREE + sl));
+        if (w == 0) {
+          misc->live[st] = end ? -1 : 1;
+          if (end) misc->total = j;
           ptx::mbar_arrive(bar(QD_FULL + st));
         }
       }
-      ++j;
-    };
-    // ---- the bias warp's steps, NB at a time: the mask words and counts of all, then their biases, then the hand-overs
-    // (lane t owns tokens t, t + 32, ... of a tile)
-    constexpr int NB = WIDE || CPS > 1 ? 2 : 4;
-    int pend[NB], n_pend = 0;
-    auto flush = [&]() {
-      float bv[NB][CPS][TPL];
-      uint32_t wd[NB][TPL];
-      int pf[NB][TPL];
-#pragma unroll
-      for (int u = 0; u < NB; ++u)
-#pragma unroll
-        for (int q = 0; q < TPL; ++q) {
-          const int t = lane + 32 * q, i = (u < n_pend ? pend[u] : 0) * TQ + t;
-          const bool live = u < n_pend && t < TQ && i < dm.seq_q && (i >> dm.log_b) > c;      // a token behind the first chunk
-          wd[u][q] = live ? a.mask[(row0 + i) * dm.W + wc] : 0u;
-          pf[u][q] = live && wc > 0 ? a.marks[marks_of(dm, grp, i) + wc - 1] : 0;
-        }
-#pragma unroll
-      for (int u = 0; u < NB; ++u)
-#pragma unroll
-        for (int q = 0; q < TPL; ++q) {
-          const int t = lane + 32 * q, i = (u < n_pend ? pend[u] : 0) * TQ + t, own = i >> dm.log_b;
-          const bool live = u < n_pend && t < TQ && i < dm.seq_q;
-#pragma unroll
-          for (int s = 0; s < CPS; ++s) {
-            bv[u][s][q] = live && c + s == own ? 0.f : -INFINITY;
-            if (c + s < own && ((wd[u][q] >> (bit + s)) & 1u))
-              bv[u][s][q] = __ldg(a.blk_bias + list0 + list_row_offset(dm, i) + pf[u][q] + __popc(wd[u][q] & ((1u << (bit + s)) - 1u)));
-          }
-        }
-#pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        if (u < n_pend && stage_free()) {
-          const int st = j % NST;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (pend[u] * TQ + stat_t[k] < dm.seq_q)
-              copy_async8(ptx::smem_u32(&misc->stats[st][lane + 32 * k]), stat_p[k] + (long long)pend[u] * TQ * a.stats.si);
-          }
-#pragma unroll
-          for (int q = 0; q < TPL; ++q) {
-            const int t = lane + 32 * q;
-            if (t < TQ)
-#pragma unroll
-              for (int s = 0; s < CPS; ++s) misc->bias[st][s][t] = bv[u][s][q];
-          }
-          arrive_after_copies(bar(QD_FULL + st));
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + st));
-          ++j;
-        }
-      }
-      n_pend = 0;
-    };
-    int n_seen = 0;
-    auto step = [&](int tile_idx) {
-      if (a.n_split > 1 && n_seen++ % a.n_split != (int)blockIdx.y) return;
-      if (loader) {
-        load_step(tile_idx);
-      } else {
-#pragma unroll
-        for (int u = 0; u < NB; ++u)
-          if (u == n_pend) pend[u] = tile_idx;
-        if (++n_pend == NB) flush();
-      }
-    };
-    const int own_end = CPS > 1 ? k0 + NKV : (c + 1) * dm.B;      // behind the last token of the slice's own chunks
-    const int t_first_routed = min((own_end + TQ - 1) / TQ, a.n_tiles);
-    for (int tl = k0 / TQ; tl < t_first_routed && ok; ++tl) step(tl);
-    auto union_word = [&](int tl0) -> uint32_t {
-      const int tl = tl0 + lane;
-      if (tl >= a.n_tiles) return 0u;
-      const int i = min((tl + 1) * TQ, dm.seq_q) - 1;
-      return (uint32_t)__ldg(a.marks + marks_of(dm, grp, i) + ((i >> dm.log_b) >> 5) + wc);
-    };
-    uint32_t uw = t_first_routed < a.n_tiles ? union_word(t_first_routed) : 0u, uw_n = 0u;
-    for (int tl0 = t_first_routed; tl0 < a.n_tiles && ok; tl0 += 32) {
-      if (tl0 + 32 < a.n_tiles) uw_n = union_word(tl0 + 32);
-      uint32_t hits = __ballot_sync(0xffffffffu, ((uw >> bit) & ((1u << CPS) - 1u)) != 0u);
-      while (hits != 0u && ok) {
-        const int k = __ffs(hits) - 1;
-        hits &= hits - 1;
-        step(tl0 + k);
-      }
-      uw = uw_n;
+      if (end) break;
     }
-    if (!loader && ok && n_pend > 0) flush();
-    // the end marker (every role visits every step, so one is enough): both producers arrive on its stage
-    if (ok && loader) {
-      if (lane == 0) misc->total = j;
-      __syncwarp();
-      load_step(-1);
-    } else if (ok && stage_free()) {
-      arrive_after_copies(bar(QD_FULL + j % NST));
-      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + j % NST));
-      ++j;
-    }
-    if (!ok && lane == 0 && loader) {
-      // a wait ran out: let the copies already issued land (bounded) before the block retires
+    // a wait that ran out: the copies already issued land before the block retires
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok && w == 0 && lane == 0)
       for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(KV_FULL), 0); ++k) {}
-      for (int s = 0; s < NST; ++s) {
-        const int lj = (j - 1 - s);
-        if (lj < 0 || misc->tile[lj % NST] < 0) continue;
-        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL + lj % NST), (uint32_t)(lj / NST) & 1u); ++k) {}
+  } else if (warp == W_META) {
+    // =========================== biases and statistics of every step ===========================
+    const long long list0 = (long long)grp * dm.list_rows;
+    bool ok = true;
+    for (int j = 0;; ++j) {
+      const int st = j % NST, sl = j & (n_slots - 1);
+      ok = wait_on(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
+      if (!ok) break;
+      const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
+      uint32_t word[TPL];
+      int tok[TPL], before[TPL], row_tok[4];
+#pragma unroll
+      for (int q = 0; q < TPL; ++q) {
+        const bool in = !end && lane + 32 * q < TQ;
+        const int e = ((j << log_t) + lane + 32 * q) & (LY::RING - 1);
+        tok[q] = in ? misc->tok[e] : (int)0x80000000;
+        word[q] = in ? misc->word[e] : 0u;
+        // routed chunks in the mask words before the slice's
+        before[q] = wc > 0 && tok[q] >= 0 && (tok[q] >> dm.log_b) > c ? a.marks[marks_of(dm, grp, tok[q]) + wc - 1] : 0;
       }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) row_tok[k] = end ? 0 : misc->tok[((j << log_t) + (lane + 32 * k) / g_q) & (LY::RING - 1)] & 0x7fffffff;
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(bar(TOK_FREE + sl));
+      if (j >= NST) ok = wait_on(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      if (!ok) break;
+      if (!end) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          copy_async8(ptx::smem_u32(&misc->stats[st][lane + 32 * k]), a.stats.at(b, r, row_tok[k], (lane + 32 * k) % g_q));
+#pragma unroll
+        for (int q = 0; q < TPL; ++q) {
+          const int t = lane + 32 * q, i = tok[q] & 0x7fffffff, own = i >> dm.log_b;
+          if (t < TQ) {
+            misc->irow[st][t] = i;
+#pragma unroll
+            for (int s = 0; s < CPS; ++s) {
+              const bool routed = tok[q] >= 0 && c + s < own && ((word[q] >> (bit + s)) & 1u);
+              if (routed)
+                copy_async4(ptx::smem_u32(&misc->bias[st][s][t]),
+                            a.blk_bias + list0 + list_row_offset(dm, i) + before[q] + __popc(word[q] & ((1u << (bit + s)) - 1u)));
+              else
+                misc->bias[st][s][t] = tok[q] >= 0 && c + s == own ? 0.f : -INFINITY;
+            }
+          }
+        }
+      }
+      arrive_after_copies(bar(QD_FULL + st));
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + st));
+      if (end) break;
     }
-    if (!ok && !loader) asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp == W_SD || warp == W_DP) {
     // =========================== issuers of the score products: S = Q K^T (W_SD), dP = dO V^T (W_DP) ===========================
     if (lane == 0) {
@@ -723,7 +749,8 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       for (int j = 0; ok; ++j) {
         const int buf = j & 1, st = j % NST;
         ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[st]) < 0) break;
+        if (!ok || *reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
+        ptx::fence_proxy_async_smem();
         // the P / dS warps have read S / dP of step j-2
         if (j >= 2) ok = wait_on(bar(PDS_FULL + buf), (uint32_t)((j >> 1) - 1) & 1u);
         if (!ok) break;
@@ -750,7 +777,8 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       for (int j = 0; ok; ++j) {
         const int buf = j & 1, st = j % NST;
         ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->tile[st]) < 0) break;
+        if (!ok || *reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
+        ptx::fence_proxy_async_smem();
         ok = wait_on(bar((SEQ && !is_v ? DS_FULL : PDS_FULL) + buf), (uint32_t)(j >> 1) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
@@ -773,7 +801,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   }
   } else {
     // =========================== P, dS: thread = tile row, warpgroup = half of the keys; epilogue: thread = d ===========================
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(256 - regs_service(WT)));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_rows(P2, TPL)));
     constexpr int SPH = CPS == 4 ? 2 : 1;                  // chunks in a half of the slice
     const int wg = warp >> 2;
     const int m = (warp & 3) * 32 + lane;
@@ -813,15 +841,13 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t ph = (uint32_t)(j >> 1) & 1u;
       ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
       if (!ok) break;
-      const int tile_idx = *reinterpret_cast<volatile int*>(&misc->tile[st]);
-      if (tile_idx < 0) break;
-      const int i_row = tile_idx * TQ + t;
-      const bool row_ok = i_row < dm.seq_q;
-      const float2 stat = row_ok ? misc->stats[st][m] : make_float2(0.f, 0.f);
+      if (*reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
+      const int i_row = misc->irow[st][t];
+      const float2 stat = misc->stats[st][m];
       const float lse2 = stat.x, delta = stat.y;
       float off[SPH];
 #pragma unroll
-      for (int s = 0; s < SPH; ++s) off[s] = row_ok ? misc->bias[st][CPS == 1 ? 0 : wg * SPH + s][t] * LOG2E - lse2 : -INFINITY;
+      for (int s = 0; s < SPH; ++s) off[s] = misc->bias[st][CPS == 1 ? 0 : wg * SPH + s][t] * LOG2E - lse2;
       const int n_vis = i_row - k0 + 1 - wg * 32;            // visible columns of this warpgroup's half
       ok = wait_on(bar(SD_FULL + buf), ph);
       if (!ok) break;
@@ -935,14 +961,14 @@ bool make_map(CUtensorMap* out, const void* base, int hd, long long tokens, int 
 template <int HD, int CPS, int WT, bool P2>
 cudaError_t launch_kernels(const BwdArgs& a, const BwdMaps& m, cudaStream_t st) {
   const long long groups = (long long)a.dm.batch * a.dm.h_kv;
-  constexpr int MTQ = 32 * (WT > 0 ? WT : 2);
+  constexpr int MTQ = 32 * (WT > 0 ? WT : 2), TPL = WT > 2 ? 4 : 2;
   cudaError_t e;
   {
-    auto kern = dkv::attend_bwd_dkv_kernel<HD, CPS, WT, P2>;
-    constexpr uint32_t smem = dkv::Layout<HD, CPS, MTQ, P2>::SMEM;
+    auto kern = dkv::attend_bwd_dkv_kernel<HD, CPS, TPL, P2>;
+    constexpr uint32_t smem = dkv::Layout<HD, CPS, 32 * TPL, P2>::SMEM;
     static std::atomic<unsigned long long> configured{0};
     if ((e = allow_dynamic_smem(kern, smem, configured)) != cudaSuccess) return e;
-    e = launch_chained(kern, dim3((unsigned)(a.n_slices * groups), a.n_split), dim3(dkv::THREADS), smem, st, m.q, m.g, m.k, m.v, a);
+    e = launch_chained(kern, dim3((unsigned)(a.n_slices * groups), a.n_split), dim3(dkv::threads(P2)), smem, st, m.k, m.v, a);
     count_launch();
     if (e != cudaSuccess) return e;
   }
@@ -981,6 +1007,7 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   a.n_slices = (dm.seq_kv + NKV - 1) / NKV;
   a.inject = test_hooks().skip_own_k_load;
   a.wait_limit = test_hooks().wait_limit_cycles;
+  a.Q = (const __nv_bfloat16*)Q; a.dO = (const __nv_bfloat16*)dO;
   a.mask = mask; a.blk_bias = blk_bias; a.marks = reinterpret_cast<int*>(dbias);
   a.dQ = (__nv_bfloat16*)dQ; a.dK = dK; a.dV = dV; a.dbias = dbias; a.sb = sb;
   // a row's statistics at the start of its dQ row
@@ -1003,9 +1030,9 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   if (!make_map(&m.kc, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, box_kv)) return cudaErrorInvalidValue;
   if (!make_map(&m.vc, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, box_kv)) return cudaErrorInvalidValue;
   if ((e = launch_attend_bwd_stats(a, m, st)) != cudaSuccess) return e;
-  const long long warps = (long long)dm.batch * dm.h_kv * a.n_tiles;
-  e = launch_chained(list_marks_kernel, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0, st, dm, a.TQ, a.n_tiles,
-                     mask, a.marks, dK, dV, a.n_split > 1 ? (long long)dm.batch * dm.seq_kv * dm.h_kv * dm.d : 0LL);
+  const long long rows = (long long)dm.batch * dm.h_kv * dm.seq_q;
+  e = launch_chained(list_marks_kernel, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, dm, mask, a.marks, dK, dV,
+                     a.n_split > 1 ? (long long)dm.batch * dm.seq_kv * dm.h_kv * dm.d : 0LL);
   count_launch();
   if (e != cudaSuccess) return e;
 
