@@ -49,8 +49,9 @@ struct StepMeta {
 
 // Warps of the query-tile-stationary kernels: three warpgroups that take the steps in turn (a thread = a tile row), and one of
 // service warps.  A step costs a thread some 600 clocks of barrier tests, tensor-memory loads and arrivals whatever its
-// width, so a warpgroup takes whole steps, every third one, instead of a share of every step.
-constexpr int BWD_ROW_WG = 3, BWD_ROW_THREADS = (BWD_ROW_WG + 1) * 128, BWD_W_PROD = 12, BWD_W_S = 13, BWD_W_DP = 14, BWD_W_DQ = 15;
+// width, so a warpgroup takes whole steps, every third one, instead of a share of every step.  Tiles and records come from two
+// warps: one that does both needs 900 clocks a step, more than the products take.
+constexpr int BWD_ROW_WG = 3, BWD_ROW_THREADS = (BWD_ROW_WG + 1) * 128, BWD_W_TILES = 12, BWD_W_RECORDS = 13, BWD_W_SD = 14, BWD_W_DQ = 15;
 // Registers per thread after the re-division (128 each at launch): a producer lane of a wide tile looks after more tokens.
 __host__ __device__ constexpr int bwd_regs_service(int wt, int cps) { return wt > 2 || (wt > 0 && cps > 2) ? 104 : wt > 0 || cps > 1 ? 80 : 56; }
 __host__ __device__ constexpr int bwd_regs_row(int wt, int cps) { return (4 * 128 - bwd_regs_service(wt, cps)) / 3 / 8 * 8; }
@@ -69,13 +70,26 @@ __device__ __forceinline__ void arrive_after_copies(uint32_t bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// The forward kernel's walk (own chunks, then the union of the tile's routed chunks, 64 tokens per step) by one warp, which
-// loads Q and dO and fills a ring of DK K tiles and step records and one of DV V tiles.  Step j's barrier is full[j mod DK]: one
-// arrival with the byte count of both tiles, and one from every lane.  `free_for(j)` waits until step j's tiles and record may
-// be overwritten (called for j >= min(DK, DV)); `publish(n)` is told the number of steps.  Biases go from the lists to the
-// record by asynchronous copies, so nothing waits for a list entry.  A walk that was cut short (a wait ran out) lets its
-// copies in flight land (bounded).
-template <int HD, int CPS, int WT, int DK, int DV, bool POS, typename Meta, typename FreeFor, typename Publish>
+// A ring position that is stepped instead of divided: index (below N) and phase parity of step j.
+template <int N>
+struct RingPos {
+  int at = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ void step() {
+    if (++at == N) {
+      at = 0;
+      phase ^= 1u;
+    }
+  }
+};
+
+// The forward kernel's walk (own chunks, then the union of the tile's routed chunks, 64 tokens per step), made by two warps:
+// with TILES one fills a ring of DK K tiles and one of DV V tiles, without it the other a ring of DK step records.  Step j's
+// barrier is full[j mod DK]: of the tiles one arrival with the byte count of both, of the records one and one of every lane.
+// `free_for(j)` waits until step j's tiles and record may be overwritten (called for j >= min(DK, DV)); `publish(n)` is
+// told the number of steps.  Biases go from the lists to the record by asynchronous copies, so nothing waits for a list entry.  A
+// walk that was cut short (a wait ran out) lets its copies in flight land (bounded).
+template <int HD, int CPS, int WT, int DK, int DV, bool TILES, bool POS, typename Meta, typename FreeFor, typename Publish>
 __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMap* tmK, const CUtensorMap* tmV, int grp, int i0, int lane,
                                               uint32_t ring_k, uint32_t ring_v, const unsigned long long* full, Meta* meta,
                                               bool skip_own_k, FreeFor&& free_for, Publish&& publish) {
@@ -86,13 +100,15 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
   const int TQ = a.TQ, b = grp / dm.h_kv, r = grp % dm.h_kv;
   const int c_own = i0 >> dm.log_b, sub_per_blk = dm.B / NKV;
   const int own_steps = WIDE ? (TQ + NKV - 1) / NKV : (i0 % dm.B) / NKV + 1;      // at most 2
-  auto bar_of = [&](int j) { return ptx::smem_u32(full + j % DK); };
-  auto load = [&](int j, const int* kvs, bool with_k) {
-    const uint32_t bar = bar_of(j);
-    ptx::mbar_arrive_expect_tx(bar, 2 * TILE_BYTES);      // (releases the record's plain stores as well)
+  RingPos<DK> pk;
+  RingPos<DV> pv;
+  auto bar_of = [&](int at) { return ptx::smem_u32(full + at); };
+  auto load = [&](const int* kvs, bool with_k) {
+    const uint32_t bar = bar_of(pk.at);
+    ptx::mbar_arrive_expect_tx(bar, 2 * TILE_BYTES);
 #pragma unroll
     for (int s = 0; s < CPS; ++s) {
-      const uint32_t k = ring_k + (j % DK) * TILE_BYTES + s * W * 128, v = ring_v + (j % DV) * TILE_BYTES + s * W * 128;
+      const uint32_t k = ring_k + pk.at * TILE_BYTES + s * W * 128, v = ring_v + pv.at * TILE_BYTES + s * W * 128;
       if (with_k) {
         ptx::tma_load_4d(k, tmK, bar, 0, r, kvs[s], b);
         if constexpr (HD == 128) ptx::tma_load_4d(k + TILE_BYTES / 2, tmK, bar, 64, r, kvs[s], b);
@@ -101,69 +117,85 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
       if constexpr (HD == 128) ptx::tma_load_4d(v + TILE_BYTES / 2, tmV, bar, 64, r, kvs[s], b);
     }
   };
+  auto record_done = [&]() {
+    arrive_after_copies(bar_of(pk.at));
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(bar_of(pk.at));      // (releases the record's plain stores)
+  };
   // own chunks first: their tiles need nothing from the mask
   for (int sub = 0; sub < own_steps; ++sub) {
     int kvs[CPS];
     const int kv0 = WIDE ? i0 + sub * NKV : c_own * dm.B + sub * NKV;
 #pragma unroll
     for (int s = 0; s < CPS; ++s) kvs[s] = WIDE && kv0 + s * W < i0 + TQ ? kv0 + s * W : kv0;
-    for (int t = lane; t < TQ; t += 32)
+    if constexpr (TILES) {
+      if (lane == 0) load(kvs, !skip_own_k);
+    } else {
+      for (int t = lane; t < TQ; t += 32)
 #pragma unroll
-      for (int s = 0; s < CPS; ++s) {
-        meta->bias[sub][s][t] = (WIDE ? (kv0 + s * W) >> dm.log_b == (i0 + t) >> dm.log_b : s == 0) ? 0.f : -INFINITY;
-        if constexpr (POS) meta->pos[sub][s][t] = -1;
-      }
+        for (int s = 0; s < CPS; ++s) {
+          meta->bias[sub][s][t] = (WIDE ? (kv0 + s * W) >> dm.log_b == (i0 + t) >> dm.log_b : s == 0) ? 0.f : -INFINITY;
+          if constexpr (POS) meta->pos[sub][s][t] = -1;
+        }
 #pragma unroll
-    for (int s = 0; s < CPS; ++s)
-      if (lane == s) meta->kvbase[sub][s] = kvs[s];
-    arrive_after_copies(bar_of(sub));
-    __syncwarp();
-    if (lane == 0) load(sub, kvs, !skip_own_k);
+      for (int s = 0; s < CPS; ++s)
+        if (lane == s) meta->kvbase[sub][s] = kvs[s];
+      record_done();
+    }
+    pk.step();
+    pv.step();
   }
   TileWalk<CPS, WIDE, TPL> walk(dm, a.mask, (long long)grp * dm.seq_q, i0, TQ, lane);
   const int total = walk.count();
   const int n_steps = (CPS > 1 ? (total + CPS - 1) / CPS : total * sub_per_blk) + own_steps;
   publish(n_steps);
-  const float* list[TPL];
+  [[maybe_unused]] const float* list[TPL];
+  if constexpr (!TILES) {
 #pragma unroll
-  for (int q = 0; q < TPL; ++q)
-    list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
+    for (int q = 0; q < TPL; ++q)
+      list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
+  }
   walk.start();
   bool ok = true;
-  int last = own_steps - 1;                 // last step whose copies were issued
-  for (int j = own_steps; j < n_steps && ok;) {
+  int j = own_steps;
+  while (j < n_steps && ok) {
     int cs[CPS], pos[CPS][TPL];
-    walk.next(cs, pos);
-    for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk) && ok; ++sub, ++j) {
+    walk.template next<!TILES>(cs, pos);
+    for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk); ++sub) {
       int kvs[CPS];
 #pragma unroll
       for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
       if (j >= (DK < DV ? DK : DV)) ok = free_for(j);
       if (!ok) break;
-      const int ms = j % DK;
+      if constexpr (TILES) {
+        if (lane == 0) load(kvs, true);
+      } else {
+        const int ms = pk.at;
 #pragma unroll
-      for (int s = 0; s < CPS; ++s) {
+        for (int s = 0; s < CPS; ++s) {
 #pragma unroll
-        for (int q = 0; q < TPL; ++q) {
-          const int t = lane + 32 * q;
-          if (t < TQ) {
-            if (pos[s][q] >= 0) copy_async4(ptx::smem_u32(&meta->bias[ms][s][t]), list[q] + pos[s][q]);
-            else meta->bias[ms][s][t] = -INFINITY;
-            if constexpr (POS) meta->pos[ms][s][t] = pos[s][q];
+          for (int q = 0; q < TPL; ++q) {
+            const int t = lane + 32 * q;
+            if (t < TQ) {
+              if (pos[s][q] >= 0) copy_async4(ptx::smem_u32(&meta->bias[ms][s][t]), list[q] + pos[s][q]);
+              else meta->bias[ms][s][t] = -INFINITY;
+              if constexpr (POS) meta->pos[ms][s][t] = pos[s][q];
+            }
           }
+          if (lane == s) meta->kvbase[ms][s] = kvs[s];
         }
-        if (lane == s) meta->kvbase[ms][s] = kvs[s];
+        record_done();
       }
-      arrive_after_copies(bar_of(j));
-      __syncwarp();
-      if (lane == 0) load(j, kvs, true);
-      last = j;
+      pk.step();
+      pv.step();
+      ++j;
     }
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  if (!ok && lane == 0) {
-    for (int j = last; j >= (skip_own_k ? own_steps : 0) && j > last - DK; --j)
-      for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar_of(j), (uint32_t)(j / DK) & 1u); ++k) {}
+  if constexpr (!TILES) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else if (!ok && lane == 0) {
+    for (int last = j - 1; last >= (skip_own_k ? own_steps : 0) && last > j - 1 - DK; --last)
+      for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar_of(last % DK), (uint32_t)(last / DK) & 1u); ++k) {}
   }
 }
 

@@ -92,15 +92,13 @@ __device__ __forceinline__ void pack_terms(const float (&x)[32], uint32_t (&hi)[
 // ===================================================================================================================
 namespace dq {
 
-// Warps as in the statistics pass (bwd_sm100.cuh): three warpgroups form dS, taking the steps in turn; one issuing thread per
-// product (S, dP, dQ): a thread issues an MMA every 60-80 clocks whatever its size, and 20 per step through one thread would be
-// the kernel's pace.  A V tile is free when its dP product is done, a K tile and a step record when the step's dQ product is:
+// Warps as in the statistics pass (bwd_sm100.cuh): three warpgroups form dS, taking the steps in turn.  A V tile is free when its dP product is done, a K tile and a step record when the step's dQ product is:
 // rings of their own, so that a step's tiles have landed by the time its S / dP slot is free.
 constexpr int THREADS = BWD_ROW_THREADS;
 constexpr int KST = 5, VST = 3;         // ring of K tiles and step records; ring of V tiles and of S / dP slots
 constexpr uint32_t TMEM_COLS = 512;     // S [0,192) dP [192,384) dQ [384,512)
 constexpr uint32_t COL_DP = 192, COL_DQ = 384;
-enum Bar { QD_FULL = 0, META_READY, SD_FULL = 2, DS_FULL = 5, KV_FULL = 8, K_FREE = 13, N_BARS = 18 };
+enum Bar { QD_FULL = 0, META_READY, SD_FULL = 2, DS_FULL = 5, KV_FULL = 8, K_FREE = 13, REC_FULL = 18, N_BARS = 23 };
 template <int CPS, int MTQ>
 struct MiscT {
   unsigned long long bar[N_BARS];
@@ -136,6 +134,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
   auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return __all_sync(0xffffffffu, wait_on(barrier, parity)) != 0; };     // a whole warp
 
   const int groups = dm.batch * dm.h_kv;
   const int tile = a.n_tiles - 1 - (int)(blockIdx.x / groups);  // late (long) tiles first
@@ -150,16 +149,17 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     ptx::mbar_init(bar(QD_FULL), 1);
     ptx::mbar_init(bar(META_READY), 1);
     for (int s = 0; s < VST; ++s) {
-      ptx::mbar_init(bar(SD_FULL + s), 2);
+      ptx::mbar_init(bar(SD_FULL + s), 1);
       ptx::mbar_init(bar(DS_FULL + s), 128);
     }
     for (int s = 0; s < KST; ++s) {
-      ptx::mbar_init(bar(KV_FULL + s), 1 + 32);
+      ptx::mbar_init(bar(KV_FULL + s), 1);
+      ptx::mbar_init(bar(REC_FULL + s), 1 + 32);
       ptx::mbar_init(bar(K_FREE + s), 1);
     }
     ptx::fence_barrier_init();
   }
-  if (warp == BWD_W_S) {
+  if (warp == BWD_W_SD) {
     ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), TMEM_COLS);
     ptx::tmem_relinquish();
     ptx::tc_fence_before();
@@ -178,9 +178,9 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
 
-  if (warp >= BWD_W_PROD) {
+  if (warp >= BWD_W_TILES) {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(bwd_regs_service(WT, CPS)));
-  if (warp == BWD_W_PROD) {
+  if (warp == BWD_W_TILES) {
     if (lane == 0) {
       ptx::prefetch_tensormap(&tmQ);
       ptx::prefetch_tensormap(&tmDO);
@@ -192,7 +192,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       ptx::tma_load_4d(sbase + OFF_DO, &tmDO, bar(QD_FULL), 0, r * g_q, i0, b);
       if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_DO + Q_BYTES / 2, &tmDO, bar(QD_FULL), 64, r * g_q, i0, b);
     }
-    produce_steps<HD, CPS, WT, KST, VST, true>(
+    produce_steps<HD, CPS, WT, KST, VST, true, true>(
         a, &tmK, &tmV, grp, i0, lane, sbase + OFF_K, sbase + OFF_V, &misc->bar[KV_FULL], &misc->meta, false,
         [&](int j) {
           return wait_on(bar(SD_FULL + j % VST), (uint32_t)(j / VST - 1) & 1u) &&
@@ -206,70 +206,86 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         });
     if (lane == 0 && *abort_flag)
       for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL), 0); ++k) {}
-  } else if (warp == BWD_W_S || warp == BWD_W_DP) {
-    // =========================== issuers of S = Q K^T and dP = dO V^T ===========================
+  } else if (warp == BWD_W_RECORDS) {
+    produce_steps<HD, CPS, WT, KST, VST, false, true>(
+        a, &tmK, &tmV, grp, i0, lane, 0u, 0u, &misc->bar[REC_FULL], &misc->meta, false,
+        [&](int j) { return j < KST || wait_on(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u); }, [](int) {});
+  } else if (warp == BWD_W_SD) {
+    // =========================== issuer of S = Q K^T and dP = dO V^T ===========================
     // Slot j mod 3 of S / dP is free once the dQ product of step j-3 is done (which reads dS from it).
-    if (lane == 0) {
-      const bool is_s = warp == BWD_W_S;
-      bool ok = wait_on(bar(QD_FULL), 0);
-      int n_steps = 0x7fffffff;            // known from step 1 on; step 0 (the own chunk) always exists
-      constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NKV, false, false);
-      const uint64_t ad0 = ptx::smem_desc_sw128(sbase + (is_s ? OFF_Q : OFF_DO), 16, 1024);
-      const uint64_t bd0 = ptx::smem_desc_sw128(sbase + (is_s ? OFF_K : OFF_V), 16, 1024);
-      const uint32_t col0 = is_s ? 0u : COL_DP;
-      for (int j = 0; j < n_steps && ok; ++j) {
-        if (j == 1) {
-          ok = wait_on(bar(META_READY), 0);
-          if (!ok) break;
-          n_steps = misc->n_steps;
-          if (j >= n_steps) break;
-        }
-        ok = wait_on(bar(KV_FULL + j % KST), (uint32_t)(j / KST) & 1u);
-        if (ok && j >= VST) ok = wait_on(bar(K_FREE + (j - VST) % KST), (uint32_t)((j - VST) / KST) & 1u);
+    bool ok = wait_all(bar(QD_FULL), 0);
+    int n_steps = 0x7fffffff;            // known from step 1 on; step 0 (the own chunk) always exists
+    constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NKV, false, false);
+    const uint64_t qd = ptx::smem_desc_sw128(sbase + OFF_Q, 16, 1024), gd = ptx::smem_desc_sw128(sbase + OFF_DO, 16, 1024);
+    const uint64_t kd0 = ptx::smem_desc_sw128(sbase + OFF_K, 16, 1024), vd0 = ptx::smem_desc_sw128(sbase + OFF_V, 16, 1024);
+    const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
+    RingPos<KST> pk, pf;                 // step j's K tile; step j-3's, whose release frees the slot
+    RingPos<VST> pv;
+    for (int j = 0; j < n_steps && ok; ++j, pk.step(), pv.step()) {
+      if (j == 1) {
+        ok = wait_all(bar(META_READY), 0);
         if (!ok) break;
-        ptx::tc_fence_after();
-        const uint64_t bd = bd0 + (uint64_t)(((is_s ? j % KST : j % VST) * KV_TILE_BYTES) >> 4);
+        n_steps = __shfl_sync(0xffffffffu, misc->n_steps, 0);
+        if (j >= n_steps) break;
+      }
+      ok = wait_all(bar(KV_FULL + pk.at), pk.phase);
+      if (ok && j >= VST) {
+        ok = wait_all(bar(K_FREE + pf.at), pf.phase);
+        pf.step();
+      }
+      if (!ok) break;
+      ptx::tc_fence_after();
+      const uint64_t ktile = (uint64_t)((pk.at * KV_TILE_BYTES) >> 4), vtile = (uint64_t)((pv.at * KV_TILE_BYTES) >> 4);
+      if (ptx::elect_one()) {
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) {
           const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
           const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
-          ptx::mma_bf16_ss(tmem + col0 + (j % VST) * NKV, ad0 + off_a, bd + off_b, IDESC_S, k > 0 ? 1u : 0u);
+          ptx::mma_bf16_ss(d0 + pv.at * NKV, qd + off_a, kd0 + ktile + off_b, IDESC_S, k > 0 ? 1u : 0u);
         }
-        ptx::mma_commit(bar(SD_FULL + j % VST));
+#pragma unroll
+        for (int k = 0; k < HD / 16; ++k) {
+          const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
+          const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
+          ptx::mma_bf16_ss(d0 + COL_DP + pv.at * NKV, gd + off_a, vd0 + vtile + off_b, IDESC_S, k > 0 ? 1u : 0u);
+        }
+        ptx::mma_commit(bar(SD_FULL + pv.at));
       }
+      __syncwarp();
     }
-    __syncwarp();
   } else {
     // =========================== issuer of dQ += dS K ===========================
-    if (lane == 0) {
-      bool ok = true;
-      int n_steps = 0x7fffffff;
-      constexpr uint32_t IDESC_DQ = ptx::idesc_bf16_f32(128, HD, false, true);
-      const uint64_t kmn0 = ptx::smem_desc_sw128(sbase + OFF_K, KV_TILE_BYTES / 2, 1024);   // K as MN-major B
-      for (int j = 0; j < n_steps && ok; ++j) {
-        if (j == 1) {
-          ok = wait_on(bar(META_READY), 0);
-          if (!ok) break;
-          n_steps = misc->n_steps;
-          if (j >= n_steps) break;
-        }
-        const int slot = j % VST;
-        ok = wait_on(bar(DS_FULL + slot), (uint32_t)(j / VST) & 1u);
+    bool ok = true;
+    int n_steps = 0x7fffffff;
+    constexpr uint32_t IDESC_DQ = ptx::idesc_bf16_f32(128, HD, false, true);
+    const uint64_t kmn0 = ptx::smem_desc_sw128(sbase + OFF_K, KV_TILE_BYTES / 2, 1024);   // K as MN-major B
+    const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
+    RingPos<KST> pk;
+    RingPos<VST> pv;
+    for (int j = 0; j < n_steps && ok; ++j, pk.step(), pv.step()) {
+      if (j == 1) {
+        ok = wait_all(bar(META_READY), 0);
         if (!ok) break;
-        ptx::tc_fence_after();
-        const uint64_t kmn = kmn0 + (uint64_t)(((j % KST) * KV_TILE_BYTES) >> 4);
-        // dS of keys 16k .. 16k+15: eight packed columns, keys 0-31 at columns 0-15 and keys 32-63 at columns 32-47 of the
-        // step's S slot; the remainders, with two-term dS, 16 columns behind
+        n_steps = __shfl_sync(0xffffffffu, misc->n_steps, 0);
+        if (j >= n_steps) break;
+      }
+      ok = wait_all(bar(DS_FULL + pv.at), pv.phase);
+      if (!ok) break;
+      ptx::tc_fence_after();
+      const uint64_t kmn = kmn0 + (uint64_t)((pk.at * KV_TILE_BYTES) >> 4);
+      // dS of keys 16k .. 16k+15: eight packed columns, keys 0-31 at columns 0-15 and keys 32-63 at columns 32-47 of the
+      // step's S slot; the remainders, with two-term dS, 16 columns behind
+      if (ptx::elect_one()) {
 #pragma unroll
         for (int term = 0; term < (P2 ? 2 : 1); ++term)
 #pragma unroll
           for (int k = 0; k < NKV / 16; ++k)
-            ptx::mma_bf16_ts(tmem + COL_DQ, tmem + slot * NKV + (k >> 1) * 32 + term * 16 + (k & 1) * 8,
+            ptx::mma_bf16_ts(d0 + COL_DQ, d0 + pv.at * NKV + (k >> 1) * 32 + term * 16 + (k & 1) * 8,
                              kmn + (uint64_t)((k * 16 * 128) >> 4), IDESC_DQ, (j > 0 || k > 0 || term > 0) ? 1u : 0u);
-        ptx::mma_commit(bar(K_FREE + j % KST));
+        ptx::mma_commit(bar(K_FREE + pk.at));
       }
+      __syncwarp();
     }
-    __syncwarp();
   }
   } else {
     // =========================== dS / epilogue: thread = tile row, warpgroup wg takes the steps wg, wg + 3, ... ===========================
@@ -292,7 +308,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     }
     for (int j = wg; j < n_steps && ok; j += BWD_ROW_WG) {
       const int slot = j % VST, rec = j % KST;
-      ok = wait_on(bar(KV_FULL + rec), (uint32_t)(j / KST) & 1u);      // the step's record is visible
+      ok = wait_on(bar(REC_FULL + rec), (uint32_t)(j / KST) & 1u);     // the step's record is visible
       if (!ok) break;
       float off[CPS];                                      // -inf: the row did not route the chunk
       int pos[CPS], n_vis[CPS];                            // causal: column c of the slot visible iff c < n_vis
@@ -388,7 +404,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   }
 
   __syncthreads();
-  if (warp == BWD_W_S) {
+  if (warp == BWD_W_SD) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
   }

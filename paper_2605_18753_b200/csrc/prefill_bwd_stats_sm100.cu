@@ -9,9 +9,9 @@
 // values are in registers.  Three warpgroups take the steps in turn, each under a maximum of its own; a row's three parts meet
 // at the end.
 //
-// Bound by the two score products: at N = 64 each MMA reads its 4 KiB slice of Q or dO again and holds the pipe 48 clocks
-// (768 per step, measured 1022).  8192 tokens, 32/8 heads, d 128: 397 us as a forward pass with two-term P, 385 us; 2 x 1500
-// tokens, 8/2 heads, d 64, chunks of 32: 27 -> 19 us.
+// Bound by the two score products: at N = 64 each MMA reads its 4 KiB slice of Q or dO again and holds the pipe 48 clocks,
+// 768 per step.  8192 tokens, 32/8 heads, d 128: 397 us as a forward pass with two-term P, 385 us with one producer warp (900
+// clocks a step, its pace), 410 with one issuer, 338 us; 2 x 1500 tokens, 8/2 heads, d 64, chunks of 32: 27 -> 18 us.
 #include "bwd_sm100.cuh"
 
 namespace dash {
@@ -23,7 +23,7 @@ constexpr int THREADS = BWD_ROW_THREADS;
 constexpr int RING = 4;                   // K / V tiles, step records, S / dP slots: index = step mod 4
 constexpr uint32_t TMEM_COLS = 512, COL_DP = RING * NKV;      // S [0,256) dP [256,512)
 constexpr float RESCALE_LOG2 = 8.f;       // a running maximum is moved only when it grew by more than this
-enum Bar { QD_FULL = 0, META_READY, SD_FULL = 2, SD_FREE = 6, KV_FULL = 10, N_BARS = 14 };
+enum Bar { QD_FULL = 0, META_READY, SD_FULL = 2, SD_FREE = 6, KV_FULL = 10, REC_FULL = 14, N_BARS = 18 };
 
 template <int HD, int CPS, int MTQ>
 struct Layout {
@@ -58,6 +58,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
   auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return __all_sync(0xffffffffu, wait_on(barrier, parity)) != 0; };     // a whole warp
 
   const int groups = dm.batch * dm.h_kv;
   const int tile = a.n_tiles - 1 - (int)(blockIdx.x / groups);  // late (long) tiles first
@@ -72,13 +73,14 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     ptx::mbar_init(bar(QD_FULL), 1);
     ptx::mbar_init(bar(META_READY), 1);
     for (int s = 0; s < RING; ++s) {
-      ptx::mbar_init(bar(SD_FULL + s), 2);
+      ptx::mbar_init(bar(SD_FULL + s), 1);
       ptx::mbar_init(bar(SD_FREE + s), 128);
-      ptx::mbar_init(bar(KV_FULL + s), 1 + 32);
+      ptx::mbar_init(bar(KV_FULL + s), 1);
+      ptx::mbar_init(bar(REC_FULL + s), 1 + 32);
     }
     ptx::fence_barrier_init();
   }
-  if (warp == BWD_W_S) {
+  if (warp == BWD_W_SD) {
     ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), TMEM_COLS);
     ptx::tmem_relinquish();
     ptx::tc_fence_before();
@@ -91,9 +93,11 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (a.sb && *reinterpret_cast<volatile int*>(&a.sb->status) != 0) *abort_flag = 1;
   __syncthreads();
 
-  if (warp >= BWD_W_PROD) {
+  if (warp >= BWD_W_TILES) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(bwd_regs_service(WT, CPS)));
-    if (warp == BWD_W_PROD) {
+    // everything of a step is free when its warpgroup has taken it (which both products precede)
+    auto step_free = [&](int j) { return wait_on(bar(SD_FREE + j % RING), (uint32_t)(j / RING - 1) & 1u); };
+    if (warp == BWD_W_TILES) {
       if (lane == 0) {
         ptx::prefetch_tensormap(&tmQ);
         ptx::prefetch_tensormap(&tmDO);
@@ -105,10 +109,8 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         ptx::tma_load_4d(sbase + OFF_DO, &tmDO, bar(QD_FULL), 0, r * g_q, i0, b);
         if constexpr (HD == 128) ptx::tma_load_4d(sbase + OFF_DO + Q_BYTES / 2, &tmDO, bar(QD_FULL), 64, r * g_q, i0, b);
       }
-      // everything of a step is free when its warpgroup has taken it (which both products precede)
-      produce_steps<HD, CPS, WT, RING, RING, false>(
-          a, &tmK, &tmV, grp, i0, lane, sbase + LY::OFF_K, sbase + LY::OFF_V, &misc->bar[KV_FULL], &misc->meta, a.inject != 0,
-          [&](int j) { return wait_on(bar(SD_FREE + j % RING), (uint32_t)(j / RING - 1) & 1u); },
+      produce_steps<HD, CPS, WT, RING, RING, true, false>(
+          a, &tmK, &tmV, grp, i0, lane, sbase + LY::OFF_K, sbase + LY::OFF_V, &misc->bar[KV_FULL], &misc->meta, a.inject != 0, step_free,
           [&](int n) {
             if (lane == 0) {
               misc->n_steps = n;
@@ -117,35 +119,49 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           });
       if (lane == 0 && *abort_flag)
         for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL), 0); ++k) {}
-    } else if (warp != BWD_W_DQ && lane == 0) {
-      // issuers of S = Q K^T and dP = dO V^T: 16 MMAs per step are too many for one thread
-      const bool is_s = warp == BWD_W_S;
-      bool ok = wait_on(bar(QD_FULL), 0);
+    } else if (warp == BWD_W_RECORDS) {
+      produce_steps<HD, CPS, WT, RING, RING, false, false>(a, &tmK, &tmV, grp, i0, lane, 0u, 0u, &misc->bar[REC_FULL], &misc->meta,
+                                                           false, step_free, [](int) {});
+    } else {
+      // two issuers of S = Q K^T and dP = dO V^T, of the even and the odd steps: between the products of a step and the next one's
+      // lie some 250 clocks of barrier tests, which the other issuer's products fill
+      const int parity = __shfl_sync(0xffffffffu, warp, 0) == BWD_W_SD ? 0 : 1;
+      bool ok = wait_all(bar(QD_FULL), 0);
       int n_steps = 0x7fffffff;            // known from step 1 on; step 0 (the own chunk) always exists
       constexpr uint32_t IDESC_S = ptx::idesc_bf16_f32(128, NKV, false, false);
-      const uint64_t ad0 = ptx::smem_desc_sw128(sbase + (is_s ? OFF_Q : OFF_DO), 16, 1024);
-      const uint64_t bd0 = ptx::smem_desc_sw128(sbase + (is_s ? LY::OFF_K : LY::OFF_V), 16, 1024);
-      const uint32_t col0 = is_s ? 0u : COL_DP;
-      for (int j = 0; j < n_steps && ok; ++j) {
-        if (j == 1) {
-          ok = wait_on(bar(META_READY), 0);
+      const uint64_t qd = ptx::smem_desc_sw128(sbase + OFF_Q, 16, 1024), gd = ptx::smem_desc_sw128(sbase + OFF_DO, 16, 1024);
+      const uint64_t kd0 = ptx::smem_desc_sw128(sbase + LY::OFF_K, 16, 1024), vd0 = ptx::smem_desc_sw128(sbase + LY::OFF_V, 16, 1024);
+      const uint32_t d0 = __shfl_sync(0xffffffffu, tmem, 0);
+      RingPos<RING> p;
+      if (parity) p.step();
+      for (int j = parity; j < n_steps && ok; j += 2, p.step(), p.step()) {
+        if (j == 1 || j == 2) {
+          ok = wait_all(bar(META_READY), 0);
           if (!ok) break;
-          n_steps = misc->n_steps;
+          n_steps = __shfl_sync(0xffffffffu, misc->n_steps, 0);
           if (j >= n_steps) break;
         }
-        const int st = j % RING;
-        // (the producer refilled the stage only after the threads had taken step j - 4, so the slot is free as well)
-        ok = wait_on(bar(KV_FULL + st), (uint32_t)(j / RING) & 1u);
+        // (the tiles' stage was refilled only after the threads had taken step j - 4, so the slot is free as well)
+        ok = wait_all(bar(KV_FULL + p.at), p.phase);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint64_t bd = bd0 + (uint64_t)((st * KV_TILE_BYTES) >> 4);
+        const uint64_t tile = (uint64_t)((p.at * KV_TILE_BYTES) >> 4);
+        if (ptx::elect_one()) {
 #pragma unroll
-        for (int k = 0; k < HD / 16; ++k) {
-          const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
-          const uint64_t off_b = (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
-          ptx::mma_bf16_ss(tmem + col0 + st * NKV, ad0 + off_a, bd + off_b, IDESC_S, k > 0 ? 1u : 0u);
+          for (int k = 0; k < HD / 16; ++k) {
+            const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
+            const uint64_t off_b = tile + (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
+            ptx::mma_bf16_ss(d0 + p.at * NKV, qd + off_a, kd0 + off_b, IDESC_S, k > 0 ? 1u : 0u);
+          }
+#pragma unroll
+          for (int k = 0; k < HD / 16; ++k) {
+            const uint64_t off_a = (uint64_t)(((k >> 2) * (Q_BYTES / 2) + (k & 3) * 32) >> 4);
+            const uint64_t off_b = tile + (uint64_t)(((k >> 2) * (KV_TILE_BYTES / 2) + (k & 3) * 32) >> 4);
+            ptx::mma_bf16_ss(d0 + COL_DP + p.at * NKV, gd + off_a, vd0 + off_b, IDESC_S, k > 0 ? 1u : 0u);
+          }
+          ptx::mma_commit(bar(SD_FULL + p.at));
         }
-        ptx::mma_commit(bar(SD_FULL + st));
+        __syncwarp();
       }
     }
     __syncwarp();
@@ -168,7 +184,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     for (int j = wg; j < n_steps && ok; j += BWD_ROW_WG) {
       const int st = j % RING;
       const uint32_t ph = (uint32_t)(j / RING) & 1u;
-      ok = wait_on(bar(KV_FULL + st), ph);                    // the step's record is visible
+      ok = wait_on(bar(REC_FULL + st), ph);                   // the step's record is visible
       if (!ok) break;
       float b2[CPS];                                          // bias in the log2 domain (-inf: the row did not route the chunk)
       int n_vis[CPS];                                         // causal: column c of the slot visible iff c < n_vis
@@ -265,7 +281,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     for (int m = tid; m < 128; m += THREADS)
       if (i0 + m / g_q < dm.seq_q) *a.stats.at(b, r, i0 + m / g_q, m % g_q) = make_float2(gave_up(), gave_up());
   }
-  if (warp == BWD_W_S) {
+  if (warp == BWD_W_SD) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, TMEM_COLS);
   }

@@ -89,13 +89,17 @@ struct TileWalk {
   // The next chunks of the union, ascending, at most CPS of them: returns their number m and, for each, the position of
   // the chunk in the lists of this lane's tokens (-1: the token did not route it).  A position is the count of the
   // token's routed bits below the chunk, so nothing walks the lists entry by entry.
+  // (POS = false: chunks only.)
+  template <bool POS = true>
   __device__ __forceinline__ int next(int (&cs)[CPS], int (&pos)[CPS][TPL]) {
     int m = 0;
 #pragma unroll
     for (int s = 0; s < CPS; ++s) {
       while (u == 0u && w < n_words) {
+        if constexpr (POS) {
 #pragma unroll
-        for (int q = 0; q < TPL; ++q) seen[q] += __popc(rw[q]);
+          for (int q = 0; q < TPL; ++q) seen[q] += __popc(rw[q]);
+        }
         if (++w < n_words) take();
       }
       const bool got = u != 0u;
@@ -109,7 +113,7 @@ struct TileWalk {
       }
 #pragma unroll
       for (int q = 0; q < TPL; ++q)
-        pos[s][q] = got && ((rw[q] >> bit) & 1u) ? seen[q] + __popc(rw[q] & ((1u << bit) - 1u)) : -1;
+        if constexpr (POS) pos[s][q] = got && ((rw[q] >> bit) & 1u) ? seen[q] + __popc(rw[q] & ((1u << bit) - 1u)) : -1;
     }
     return m;
   }
