@@ -150,6 +150,7 @@ __device__ __forceinline__ float entmax_tau(const float* x, int n_cand, int e_in
       const float nt = newton_next(tau, f, gs, EI, e);
       if (nt == tau) break;
       tau = nt;
+      if (newton_settled(f, gs, (float)n_cand, EI)) break;
     }
   };
   switch (e_int) {

@@ -301,6 +301,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       if (done) return;
       const float nt = newton_next(tau, f, g, ei, e);
       if (nt == tau) done = true; else tau = nt;
+      if (newton_settled(f, g, (float)n_row, ei)) done = true;
     };
     constexpr bool CAN_HOLD = CS == 1 && SPLIT == 1;   // one thread per row: a short row can live in its registers
     float xr[CAN_HOLD ? 4 : 1][32];                // the whole row, when it has at most 128 candidates
