@@ -280,6 +280,202 @@ route_bwd_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kba
   }
 }
 
+// The same for sixteen consecutive tokens per block, a warp each, whose lists fit in shared memory together: dz stays there, and
+// once all sixteen are done the block goes through the chunks that any of them routed, one warp per chunk, and sends one
+// reduction per chunk instead of one per token and chunk.  The reductions were what bounded the kernel above: the L2's atomic
+// units take about 97 G requests a second whatever their width, and 8192 tokens, 32/8 heads, chunks of 64 send 36 M of them.
+constexpr int RT_TOK = 16;
+template <int G>
+struct RouteTile {      // offsets in dynamic shared memory, for lists of up to `cap` chunks (a multiple of 8)
+  static constexpr size_t ENTRY = 4 * G + 4 + 2 + 2;      // margin or dz per head, dw, chunk id, place of a chunk in the list
+  __host__ __device__ static size_t bytes(int cap, int d, int elem) { return (size_t)RT_TOK * cap * ENTRY + (size_t)RT_TOK * G * d * elem + (size_t)cap * 4; }
+};
+
+template <typename T, int D, int G, bool VEC>
+__global__ void __launch_bounds__(RT_TOK * 32, 2)
+route_bwd_tile_kernel(Dims dm, const T* __restrict__ Q, const float* __restrict__ Kbar, const int* __restrict__ count,
+                      const int* __restrict__ blk_idx, const float* __restrict__ tau, const float* __restrict__ dbias,
+                      float* __restrict__ dQr, float* __restrict__ dKbar, int n_tiles, int cap) {
+  constexpr int VPL = D / 32;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* m_all = reinterpret_cast<float*>(smem);                                  // [token][cap][G]
+  T* q_all = reinterpret_cast<T*>(m_all + (size_t)RT_TOK * cap * G);              // [token][G][D]
+  float* dw_s = reinterpret_cast<float*>(q_all + RT_TOK * G * D) + warp * cap;    // [token][cap]
+  uint32_t* bits_s = reinterpret_cast<uint32_t*>(dw_s - warp * cap + RT_TOK * cap);      // [cap]: the tokens that routed a chunk
+  unsigned short* c_s = reinterpret_cast<unsigned short*>(bits_s + cap) + warp * cap;    // [token][cap]
+  unsigned short* pos_all = c_s - warp * cap + RT_TOK * cap;                      // [token][cap]
+  float* m_s = m_all + (size_t)warp * cap * G;
+  T* q_s = q_all + warp * G * D;
+  for (int c = threadIdx.x; c < cap; c += RT_TOK * 32) bits_s[c] = 0u;
+  chain_wait();
+  chain_release();
+  __syncthreads();
+  const long long grp = blockIdx.x / n_tiles;
+  const int i0 = (int)(blockIdx.x % n_tiles) * RT_TOK, i = i0 + warp;
+  const int r = (int)(grp % dm.h_kv), b = (int)(grp / dm.h_kv);
+  const float* kb = Kbar + grp * dm.T_s * D;
+  const int c_own = i >> dm.log_b;
+  const int n_routed = i < dm.seq_q ? count[grp * dm.seq_q + i] - min(dm.local_blocks, c_own) : 0;      // (window chunks close the list)
+  const float e = dm.e;
+  const int e_int = dm.e_int;
+  float2 dq[G][VPL / 2];
+#pragma unroll
+  for (int h = 0; h < G; ++h)
+#pragma unroll
+    for (int v = 0; v < VPL / 2; ++v) dq[h][v] = make_float2(0.f, 0.f);
+  if (n_routed > 0) {
+    const long long loff = grp * dm.list_rows + list_row_offset(dm, i);
+    float th[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      const T* qp = Q + (long long)b * dm.qs[0] + (long long)i * dm.qs[1] + (long long)(r * G + h) * dm.qs[2] + lane * VPL;
+      if constexpr (VPL == 4 && sizeof(T) == 2) *reinterpret_cast<uint2*>(q_s + h * D + lane * VPL) = *reinterpret_cast<const uint2*>(qp);
+      else
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) q_s[h * D + lane * VPL + v] = qp[v];
+      th[h] = tau[((long long)b * dm.h_q + r * G + h) * dm.seq_q + i];
+    }
+    float dmean = 0.f;
+    for (int k = lane; k < n_routed; k += 32) {
+      const int c = blk_idx[loff + k];
+      const float db = dbias[loff + k];
+      c_s[k] = (unsigned short)c;
+      pos_all[warp * cap + c] = (unsigned short)k;
+      atomicOr(&bits_s[c], 1u << warp);
+      dw_s[k] = db;
+      dmean += db;
+    }
+    dmean = warp_sum(dmean) / (float)n_routed;
+    __syncwarp();
+    // margins, eight chunks at once (as above)
+    float A[G], S[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) A[h] = S[h] = 0.f;
+#pragma unroll 1
+    for (int e0 = 0; e0 < n_routed; e0 += 8) {
+      const int k = e0 + (lane >> 2);
+      const bool live = k < n_routed;
+      const float* kp = kb + (long long)c_s[min(k, n_routed - 1)] * D + 4 * (lane & 3);
+      float2 xp[G];
+#pragma unroll
+      for (int h = 0; h < G; ++h) xp[h] = make_float2(0.f, 0.f);
+      float4 kv[D / 16];
+#pragma unroll
+      for (int j = 0; j < D / 16; ++j)
+        kv[j] = VEC ? load4(kp + 16 * j) : make_float4(kp[16 * j], kp[16 * j + 1], kp[16 * j + 2], kp[16 * j + 3]);
+#pragma unroll
+      for (int j = 0; j < D / 16; ++j)
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+          const float4 qv = load4(q_s + h * D + 16 * j + 4 * (lane & 3));
+          xp[h] = __ffma2_rn(make_float2(qv.x, qv.y), make_float2(kv[j].x, kv[j].y), xp[h]);
+          xp[h] = __ffma2_rn(make_float2(qv.z, qv.w), make_float2(kv[j].z, kv[j].w), xp[h]);
+        }
+      float x[G], w = 0.f;
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        x[h] = xp[h].x + xp[h].y;
+        x[h] += __shfl_xor_sync(0xffffffffu, x[h], 1);
+        x[h] += __shfl_xor_sync(0xffffffffu, x[h], 2);
+        x[h] = fmaxf(x[h] * dm.x_scale - th[h], 0.f);
+        w += pow_e(x[h], e_int, e);
+      }
+      w /= (float)G;
+      const float dw = live && w > 0.f ? (dw_s[k] - dmean) * dm.inv_sigma / (w * (float)G) : 0.f;
+      __syncwarp();                           // (everybody has read dw_s of these entries)
+      if (live) {
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+          const float sp = pow_em1(x[h], e_int, e);
+          A[h] = fmaf(sp, dw, A[h]);
+          S[h] += sp;
+        }
+        if ((lane & 3) == 0) {
+          dw_s[k] = dw;                       // from here on the gradient w.r.t. every head's weight
+#pragma unroll
+          for (int h = 0; h < G; ++h) m_s[k * G + h] = x[h];
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        A[h] += __shfl_xor_sync(0xffffffffu, A[h], o);
+        S[h] += __shfl_xor_sync(0xffffffffu, S[h], o);
+      }
+    const float zscale = dm.x_scale / (1.f / e);       // gamma / sqrt(d) = x_scale / (alpha - 1)
+#pragma unroll
+    for (int h = 0; h < G; ++h) A[h] = S[h] > 0.f ? A[h] / S[h] : 0.f;
+    __syncwarp();
+    // dz_hc = s_hc (dw_c / g_q - A_h / S_h), scaled
+    for (int k = lane; k < n_routed; k += 32) {
+      const float dw = dw_s[k];
+#pragma unroll
+      for (int h = 0; h < G; ++h)
+        m_s[k * G + h] = S[h] > 0.f ? pow_em1(m_s[k * G + h], e_int, e) * (dw - A[h]) * zscale : 0.f;
+    }
+    __syncwarp();
+    constexpr int NB = 4;
+#pragma unroll 1
+    for (int e0 = 0; e0 < n_routed; e0 += NB) {
+      float kv[NB][VPL];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) load_vec<VPL, VEC>(kb + (long long)c_s[min(e0 + u, n_routed - 1)] * D + lane * VPL, kv[u]);
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        if (e0 + u < n_routed) {
+#pragma unroll
+          for (int h = 0; h < G; ++h) {
+            const float dz = m_s[(e0 + u) * G + h];
+#pragma unroll
+            for (int v = 0; v < VPL / 2; ++v) dq[h][v] = __ffma2_rn(make_float2(dz, dz), make_float2(kv[u][2 * v], kv[u][2 * v + 1]), dq[h][v]);
+          }
+        }
+      }
+    }
+  }
+  if (i < dm.seq_q) {
+    float* dq_out = dQr + (((long long)b * dm.seq_q + i) * dm.h_q + (long long)r * G) * D + lane * VPL;
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      float x[VPL];
+#pragma unroll
+      for (int v = 0; v < VPL / 2; ++v) { x[2 * v] = dq[h][v].x; x[2 * v + 1] = dq[h][v].y; }
+      store_vec<VPL, VEC>(dq_out + (long long)h * D, x);
+    }
+  }
+  __syncthreads();
+  // dkbar of the chunks that any of the block's tokens routed
+  const int n_c = min(min(i0 + RT_TOK, dm.seq_q) - 1 >> dm.log_b, dm.T_s);
+#pragma unroll 1
+  for (int c = warp; c < n_c; c += RT_TOK) {
+    uint32_t bits = bits_s[c];
+    if (bits == 0u) continue;
+    float2 dkb[VPL / 2];
+#pragma unroll
+    for (int v = 0; v < VPL / 2; ++v) dkb[v] = make_float2(0.f, 0.f);
+    while (bits) {
+      const int t = __ffs(bits) - 1;
+      bits &= bits - 1;
+      const float* dz = m_all + ((size_t)t * cap + pos_all[t * cap + c]) * G;
+      const T* qp = q_all + t * G * D + lane * VPL;
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        float q[VPL];
+        load_vec<VPL>(qp + h * D, q);
+#pragma unroll
+        for (int v = 0; v < VPL / 2; ++v) dkb[v] = __ffma2_rn(make_float2(dz[h], dz[h]), make_float2(q[2 * v], q[2 * v + 1]), dkb[v]);
+      }
+    }
+    float out[VPL];
+#pragma unroll
+    for (int v = 0; v < VPL / 2; ++v) { out[2 * v] = dkb[v].x; out[2 * v + 1] = dkb[v].y; }
+    add_global<VPL, VEC>(dKbar + (grp * dm.T_s + c) * D + lane * VPL, out);
+  }
+}
+
 constexpr int SB_SPLIT = 4;      // warps that share a chunk = a block
 
 template <typename T, int D, bool VEC>
@@ -388,6 +584,28 @@ summaries_bwd_kernel(Dims dm, const T* __restrict__ K, const float* __restrict__
   }
 }
 
+// Tiles of sixteen tokens: causal lists (no longer than T_s, and the tokens of a tile share their own chunk) of groups of up to
+// eight heads, where two blocks fit on an SM (bf16, four heads, d 128: up to 184 chunks).  Longer lists take a warp per row.
+static int route_tile_cap(const Dims& dm) { return (dm.T_s + 7) / 8 * 8; }
+template <typename T, int D, int G>
+static bool tiles_fit(const Dims& dm) {
+  return dm.causal && G <= 8 && RouteTile<G>::bytes(route_tile_cap(dm), D, sizeof(T)) <= 112 * 1024;
+}
+template <typename T, int D, int G, bool VEC>
+static cudaError_t launch_route_tiles(const Dims& dm, const T* Q, const float* Kbar, const int* count, const int* blk_idx,
+                                      const float* tau, const float* dbias, float* dQr, float* dKbar, cudaStream_t st) {
+  if constexpr (G > 8) {
+    return cudaErrorInvalidValue;
+  } else {
+    static std::atomic<unsigned long long> configured{0};
+    auto kern = route_bwd_tile_kernel<T, D, G, VEC>;
+    if (cudaError_t e = allow_dynamic_smem(kern, 112 * 1024, configured); e != cudaSuccess) return e;
+    const int n_tiles = (dm.seq_q + RT_TOK - 1) / RT_TOK, cap = route_tile_cap(dm);
+    return launch_chained(kern, dim3((unsigned)((long long)dm.batch * dm.h_kv * n_tiles)), dim3(RT_TOK * 32),
+                          RouteTile<G>::bytes(cap, D, sizeof(T)), st, dm, Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar, n_tiles, cap);
+  }
+}
+
 cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, const int* count, const int* blk_idx,
                              const float* tau, const float* dbias, float* dQr, float* dKbar, cudaStream_t st) {
   const size_t kb_bytes = (size_t)dm.batch * dm.h_kv * (size_t)dm.T_s * dm.d * sizeof(float);
@@ -402,7 +620,10 @@ cudaError_t launch_route_bwd(const Dims& dm, const void* Q, const float* Kbar, c
 #define DASH_RB_V(T, D, GV, V) \
   le = launch_chained(route_bwd_kernel<T, D, GV, V>, dim3(grid), dim3(RB_WARPS * 32), 0, st, dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar)
 #define DASH_RB(T, D, GV) \
-  if (vec) DASH_RB_V(T, D, GV, true); else DASH_RB_V(T, D, GV, false)
+  if (tiles_fit<T, D, GV>(dm)) \
+    le = vec ? launch_route_tiles<T, D, GV, true>(dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar, st) \
+             : launch_route_tiles<T, D, GV, false>(dm, (const T*)Q, Kbar, count, blk_idx, tau, dbias, dQr, dKbar, st); \
+  else if (vec) DASH_RB_V(T, D, GV, true); else DASH_RB_V(T, D, GV, false)
 #define DASH_RB_G(T, D)                   \
   switch (dm.g_q) {                       \
     case 1: DASH_RB(T, D, 1); break;      \
