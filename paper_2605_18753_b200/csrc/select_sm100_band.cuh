@@ -515,6 +515,8 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const long long row_id = ((long long)b * dm.h_kv + r) * dm.seq_q + i;
     const long long loff = ((long long)b * dm.h_kv + r) * dm.list_rows + list_row_offset(dm, min(i, dm.seq_q - 1));
     uint32_t* mrow = a.mask + row_id * dm.W;
+    float* list_bias = a.blk_bias + loff;
+    int* list_idx = a.blk_idx ? a.blk_idx + loff : nullptr;
     const float log_gq = logf((float)G);
     float slog = 0.f;
     int nsel = 0;
@@ -543,16 +545,14 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         uint32_t bits = 0;
         uint32_t lwv[OWN];
 #pragma unroll
-        for (int c = 0; c < OWN; ++c) lwv[c] = 0x7f800000u;       // +inf: not routed
-#pragma unroll
-        for (int q = 0; q < OWN; ++q) {
-          if (pe[q] > 0.f) {
-            const float lw = __logf(pe[q]) - log_gq;
-            lwv[q] = __float_as_uint(lw);
-            slog += lw;
-            bits |= 1u << (own0 + q);
-          }
+        for (int q = 0; q < OWN; ++q) {                           // (selects, no branches)
+          const bool on = pe[q] > 0.f;
+          const float lw = __logf(pe[q]) - log_gq;
+          lwv[q] = on ? __float_as_uint(lw) : 0x7f800000u;        // +inf: not routed
+          slog += on ? lw : 0.f;
+          bits |= on ? 1u << q : 0u;
         }
+        bits <<= own0;
 #pragma unroll
         for (int o = 1; o < G; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
         ptx::tmem_st_n<OWN>(lane_addr + k * 32, lwv);            // slot q of this lane = chunk own0 + q of step k
@@ -614,14 +614,13 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 #pragma unroll
         for (int o = 1; o < G; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
         if (row_valid) {
+          int at = base + __popc(bits & ((1u << own0) - 1u));      // place of this lane's first routed chunk
 #pragma unroll
           for (int q = 0; q < OWN; ++q) {
-            if (lwv[q] != 0x7f800000u) {
-              const int c = own0 + q;
-              const long long pos = loff + base + __popc(bits & ((1u << c) - 1u));
-              a.blk_bias[pos] = (__uint_as_float(lwv[q]) - mu) * dm.inv_sigma;
-              if (a.blk_idx) a.blk_idx[pos] = c_lo + k * 32 + c;
-            }
+            const bool on = lwv[q] != 0x7f800000u;
+            if (on) list_bias[at] = (__uint_as_float(lwv[q]) - mu) * dm.inv_sigma;
+            if (on && list_idx) list_idx[at] = c_lo + k * 32 + own0 + q;
+            at += on ? 1 : 0;
           }
         }
         base += __popc(bits);
