@@ -539,7 +539,7 @@ def measure_backward(B, synth, w, dev, flush, iters=3, tensor_cores=False, fwd_s
     if tensor_cores:
         bws = B.alloc_bwd_workspace(p, dev)
         stage2 = lambda: B.dash_attn_bwd_attend_prefill_tc(p, Q, K, V, dO, rt["mask"], rt["blk_bias"], dQ, dK, dV, dbias, bws)
-        kernels = ("Stage 2 on tensor cores (statistics pass of the forward kernel, dQ / dbias kernel, dK / dV kernel); "
+        kernels = ("Stage 2 on tensor cores (row statistics, dQ / dbias kernel, dK / dV kernel); "
                    "routing and summaries on CUDA cores")
     else:
         stage2 = lambda: B.dash_attn_bwd_attend_prefill(p, Q, K, V, dO, rt["mask"], rt["blk_bias"], dQ, dK, dV, dbias)

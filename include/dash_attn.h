@@ -214,10 +214,9 @@ int dash_attn_bwd_attend_prefill(const dash_params* p, const void* Q, const void
 
 /* The same gradients on tensor cores (bf16, head_dim 128, chunks of 64 or 128 tokens, at least two query heads per KV
  * head, causal; anything else returns DASH_ERR_UNSUPPORTED and nothing is enqueued: call dash_attn_bwd_attend_prefill).
- * Four launches: the forward Stage-2 kernel run for its row statistics (log-sum-exp and delta = <O, dO>; O itself is
- * not written, and P enters its P V product as two bf16 terms, so that delta, which the routing's backward amplifies,
- * is accurate to fp32 class), a small kernel over the mask (routed-chunk counts before every mask word; the union
- * of every query tile's mask words), a key-slice-stationary kernel for dK and dV (no atomics: every element has one
+ * Four launches: a kernel for the row statistics (log-sum-exp and delta = sum of P dP, formed in fp32, because the routing's
+ * backward amplifies its error), a small kernel over the mask (routed-chunk counts before every mask word), a
+ * key-slice-stationary kernel for dK and dV that gathers the tokens attending the slice (no atomics: every element has one
  * owner and is written whether or not any row attends it) and a query-tile-stationary kernel for dQ and dbias (dbias is
  * zeroed and then receives a few atomic adds per entry, whose order cannot change the sum beyond the last bit).
  * P and dS enter the dQ / dK / dV products rounded to bf16.

@@ -26,7 +26,7 @@
 //
 // Bound by the chain of a step (tile landed -> S, dP -> P, dS -> accumulating products), one block per SM.  2 x 1500 tokens,
 // 8/2 heads, d 64, chunks of 32: 2.02 ms on CUDA cores (one warp per row and head, two vector reductions per token and
-// row) -> 0.12 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: statistics 0.39, dK / dV 0.57, dQ 0.56 ms.
+// row) -> 0.11 ms; 8192 tokens, 32/8 heads, d 128, chunks of 64, one term: statistics 0.33, dK / dV 0.56, dQ 0.51 ms.
 #include <cuda.h>
 
 #include <algorithm>
