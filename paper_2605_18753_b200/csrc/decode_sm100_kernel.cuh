@@ -438,12 +438,12 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     bool ok = true;
     int vs = 1, vph = 0;
     for (int j = 0; j < n_steps && ok; ++j) {
-      ok = ptx::mbar_wait(bar(FULL + vs), vph, abort_flag);     // step metadata visible, V tile landed
+      ok = ptx::mbar_wait_warp(bar(FULL + vs), vph, abort_flag);     // step metadata visible, V tile landed
       if (!ok) break;
       const float b2 = misc->bias2[vs][half][CPS > 1 ? row / W : 0] * 1.4426950408889634f;
       const int nval = misc->nvalid[vs][half];
       const bool valid = row < nval;
-      ok = ptx::mbar_wait(bar(S_FULL + (j & 1)), (j >> 1) & 1, abort_flag);
+      ok = ptx::mbar_wait_warp(bar(S_FULL + (j & 1)), (j >> 1) & 1, abort_flag);
       if (!ok) break;
       ptx::tc_fence_after();
       uint32_t sr[16];
@@ -458,7 +458,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
       // per-head maxima of the four warps meet through shared memory (bounded mbarrier, not bar.sync)
       ptx::mbar_arrive(bar(RED_BAR + (j & 1)));
-      ok = ptx::mbar_wait(bar(RED_BAR + (j & 1)), (j >> 1) & 1, abort_flag);
+      ok = ptx::mbar_wait_warp(bar(RED_BAR + (j & 1)), (j >> 1) & 1, abort_flag);
       if (!ok) break;
       float corr[G];
       bool changed = false;
@@ -480,7 +480,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         pl[h] = __float2bfloat16_rn(p - __bfloat162float(pb[h]));
       }
       // the previous step's PV must be done before P^T is overwritten and before O^T is rescaled
-      ok = ptx::mbar_wait(bar(P_EMPTY), (j & 1) ^ 1, abort_flag);
+      ok = ptx::mbar_wait_warp(bar(P_EMPTY), (j & 1) ^ 1, abort_flag);
       if (!ok) break;
       ptx::tc_fence_after();
       if (j > 0 && changed) {
@@ -522,7 +522,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
 
     // ---------------- partial (m, l, O) of this split
-    if (ok && n_steps > 0) ok = ptx::mbar_wait(bar(P_EMPTY), (n_steps - 1) & 1, abort_flag);
+    if (ok && n_steps > 0) ok = ptx::mbar_wait_warp(bar(P_EMPTY), (n_steps - 1) & 1, abort_flag);
     ptx::tc_fence_after();
 #pragma unroll
     for (int h = 0; h < G; ++h) {
@@ -530,7 +530,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       if (lane == 0) misc->lred[warp][h] = ls;
     }
     ptx::mbar_arrive(bar(LRED_BAR));
-    ok = ptx::mbar_wait(bar(LRED_BAR), 0, abort_flag) && ok;
+    ok = ptx::mbar_wait_warp(bar(LRED_BAR), 0, abort_flag) && ok;
     uint32_t o[16];
 #pragma unroll
     for (int h = 0; h < 16; ++h) o[h] = 0u;
@@ -551,7 +551,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int h = 0; h < G; ++h) comb[(tid - 64) * NH + h] = __uint_as_float(o[h]);
       }
       ptx::mbar_arrive(bar(LRED_BAR));
-      ok = ptx::mbar_wait(bar(LRED_BAR), 1, abort_flag) && ok;
+      ok = ptx::mbar_wait_warp(bar(LRED_BAR), 1, abort_flag) && ok;
       if (tid < 64) {
 #pragma unroll
         for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + comb[tid * NH + h]);

@@ -133,8 +133,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   auto bar = [&](int i) { return ptx::smem_u32(&misc->bar[i]); };
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
-  auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
-  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return __all_sync(0xffffffffu, wait_on(barrier, parity)) != 0; };     // a whole warp
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait_warp(barrier, parity, abort_flag, wait_limit); };
 
   const int groups = dm.batch * dm.h_kv;
   const int tile = a.n_tiles - 1 - (int)(blockIdx.x / groups);  // late (long) tiles first
@@ -195,8 +194,8 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     produce_steps<HD, CPS, WT, KST, VST, true, true>(
         a, &tmK, &tmV, grp, i0, lane, sbase + OFF_K, sbase + OFF_V, &misc->bar[KV_FULL], &misc->meta, false,
         [&](int j) {
-          return wait_on(bar(SD_FULL + j % VST), (uint32_t)(j / VST - 1) & 1u) &&
-                 (j < KST || wait_on(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u));
+          return wait_all(bar(SD_FULL + j % VST), (uint32_t)(j / VST - 1) & 1u) &&
+                 (j < KST || wait_all(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u));
         },
         [&](int n) {
           if (lane == 0) {
@@ -209,7 +208,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   } else if (warp == BWD_W_RECORDS) {
     produce_steps<HD, CPS, WT, KST, VST, false, true>(
         a, &tmK, &tmV, grp, i0, lane, 0u, 0u, &misc->bar[REC_FULL], &misc->meta, false,
-        [&](int j) { return j < KST || wait_on(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u); }, [](int) {});
+        [&](int j) { return j < KST || wait_all(bar(K_FREE + j % KST), (uint32_t)(j / KST - 1) & 1u); }, [](int) {});
   } else if (warp == BWD_W_SD) {
     // =========================== issuer of S = Q K^T and dP = dO V^T ===========================
     // Slot j mod 3 of S / dP is free once the dQ product of step j-3 is done (which reads dS from it).
@@ -303,12 +302,12 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     bool ok = true;
     int n_steps = 1;                       // step 0 always exists; the others are known with the walk
     if (wg > 0) {
-      ok = wait_on(bar(META_READY), 0);
+      ok = wait_all(bar(META_READY), 0);
       n_steps = ok ? misc->n_steps : 0;
     }
     for (int j = wg; j < n_steps && ok; j += BWD_ROW_WG) {
       const int slot = j % VST, rec = j % KST;
-      ok = wait_on(bar(REC_FULL + rec), (uint32_t)(j / KST) & 1u);     // the step's record is visible
+      ok = wait_all(bar(REC_FULL + rec), (uint32_t)(j / KST) & 1u);    // the step's record is visible
       if (!ok) break;
       float off[CPS];                                      // -inf: the row did not route the chunk
       int pos[CPS], n_vis[CPS];                            // causal: column c of the slot visible iff c < n_vis
@@ -321,7 +320,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         any = any || !(off[s] == -INFINITY);
       }
       any = __any_sync(0xffffffffu, any);                  // a warp none of whose rows routed a chunk of the step only writes zeros
-      ok = wait_on(bar(SD_FULL + slot), (uint32_t)(j / VST) & 1u);
+      ok = wait_all(bar(SD_FULL + slot), (uint32_t)(j / VST) & 1u);
       if (!ok) break;
       ptx::tc_fence_after();
       float rowsum[CPS];
@@ -365,17 +364,17 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         }
       }
       if (j == 0) {
-        ok = wait_on(bar(META_READY), 0);
+        ok = wait_all(bar(META_READY), 0);
         n_steps = ok ? misc->n_steps : 0;
       }
     }
     // epilogue: dQ / sqrt(d) -> global; the warpgroups share the row's columns
     if (ok) {
-      ok = wait_on(bar(META_READY), 0);
+      ok = wait_all(bar(META_READY), 0);
       n_steps = ok ? misc->n_steps : 0;
     }
     // (a warpgroup has seen the scores of step n-3 or a later one, or none where n < 3: the phase before this one is over)
-    if (ok) ok = wait_on(bar(K_FREE + ((n_steps - 1) % KST)), (uint32_t)((n_steps - 1) / KST) & 1u);
+    if (ok) ok = wait_all(bar(K_FREE + ((n_steps - 1) % KST)), (uint32_t)((n_steps - 1) / KST) & 1u);
     if (ok) {
       ptx::tc_fence_after();
       __nv_bfloat16* op = a.dQ + (long long)b * dm.qs[0] + (long long)i_row * dm.qs[1] + (long long)(r * g_q + hh) * dm.qs[2];
@@ -516,6 +515,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
   auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait_warp(barrier, parity, abort_flag, wait_limit); };
 
   const int groups = dm.batch * dm.h_kv;
   const int slice = (int)(blockIdx.x / groups);                  // early slices first: every later token may attend them
@@ -575,7 +575,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     int n = 0, free_slots = n_slots, done = 0;      // tokens so far; steps that may be written; steps handed on
     auto reserve = [&](int steps) {
       for (; free_slots < steps && ok; ++free_slots)
-        ok = wait_on(bar(TOK_FREE + (free_slots & (n_slots - 1))), (uint32_t)((free_slots >> log_slots) - 1) & 1u);
+        ok = wait_all(bar(TOK_FREE + (free_slots & (n_slots - 1))), (uint32_t)((free_slots >> log_slots) - 1) & 1u);
     };
     auto hand_on = [&](int steps, bool last) {
       __syncwarp();
@@ -666,8 +666,8 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     bool ok = true;
     for (int j = 0;; ++j) {
       const int st = j % NST, sl = j & (n_slots - 1);
-      ok = wait_on(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
-      if (ok && j >= NST) ok = wait_on(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      ok = wait_all(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
+      if (ok && j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
       if (!ok) break;
       const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
       if (!end) {
@@ -707,7 +707,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     bool ok = true;
     for (int j = 0;; ++j) {
       const int st = j % NST, sl = j & (n_slots - 1);
-      ok = wait_on(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
+      ok = wait_all(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
       if (!ok) break;
       const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
       uint32_t word[TPL];
@@ -725,7 +725,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       for (int k = 0; k < 4; ++k) row_tok[k] = end ? 0 : misc->tok[((j << log_t) + (lane + 32 * k) / g_q) & (LY::RING - 1)] & 0x7fffffff;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(bar(TOK_FREE + sl));
-      if (j >= NST) ok = wait_on(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      if (j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
       if (!ok) break;
       if (!end) {
 #pragma unroll
@@ -855,7 +855,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int j = 0; ok; ++j) {
       const int buf = j & 1, st = j % NST;
       const uint32_t ph = (uint32_t)(j >> 1) & 1u;
-      ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
+      ok = wait_all(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
       if (!ok) break;
       if (*reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
       const int i_row = misc->irow[st][t];
@@ -865,7 +865,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
       for (int s = 0; s < SPH; ++s) off[s] = misc->bias[st][CPS == 1 ? 0 : wg * SPH + s][t] * LOG2E - lse2;
       const int n_vis = i_row - k0 + 1 - wg * 32;            // visible columns of this warpgroup's half
-      ok = wait_on(bar(SD_FULL + buf), ph);
+      ok = wait_all(bar(SD_FULL + buf), ph);
       if (!ok) break;
       ptx::tc_fence_after();
       uint32_t p_hi[16], p_lo[16], d_hi[16], d_lo[16];       // the row's 32 P and 32 dS values of this half as bf16 pairs
@@ -884,7 +884,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         pack_terms<P2>(ds, d_hi, d_lo);
       }
       // the accumulating products of the step before have read P / dS
-      if (j >= 1) ok = wait_on(bar(ACC_DONE + (j - 1) % NST), (uint32_t)((j - 1) / NST) & 1u);
+      if (j >= 1) ok = wait_all(bar(ACC_DONE + (j - 1) % NST), (uint32_t)((j - 1) / NST) & 1u);
       if (!ok) break;
       store_row(LY::OFF_P, p_hi);
       if constexpr (P2) store_row(LY::OFF_P + PS_BYTES, p_lo);
@@ -902,7 +902,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       ptx::tc_fence_before();
       ptx::mbar_arrive(bar(PDS_FULL + buf));
       if constexpr (SEQ) {
-        ok = wait_on(bar(DV_DONE + buf), ph);
+        ok = wait_all(bar(DV_DONE + buf), ph);
         if (!ok) break;
         store_row(LY::OFF_DS, d_hi);
         store_row(LY::OFF_DS + PS_BYTES, d_lo);
@@ -912,7 +912,7 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
     // epilogue: dV^T, dK^T [d = TMEM lane][key = column] -> dV, dK [batch][key][KV head][d]; one warpgroup each
     const int n_done = ok ? *reinterpret_cast<volatile int*>(&misc->total) : 0;
-    if (ok && n_done > 0) ok = wait_on(bar(ACC_DONE + (n_done - 1) % NST), (uint32_t)((n_done - 1) / NST) & 1u);
+    if (ok && n_done > 0) ok = wait_all(bar(ACC_DONE + (n_done - 1) % NST), (uint32_t)((n_done - 1) / NST) & 1u);
     if (ok && mine && (n_done > 0 || a.n_split == 1)) {
       ptx::tc_fence_after();
       const int d = HD == 128 ? m : m & 63;

@@ -57,8 +57,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   auto bar = [&](int i) { return ptx::smem_u32(&misc->bar[i]); };
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
-  auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
-  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return __all_sync(0xffffffffu, wait_on(barrier, parity)) != 0; };     // a whole warp
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait_warp(barrier, parity, abort_flag, wait_limit); };
 
   const int groups = dm.batch * dm.h_kv;
   const int tile = a.n_tiles - 1 - (int)(blockIdx.x / groups);  // late (long) tiles first
@@ -96,7 +95,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (warp >= BWD_W_TILES) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(bwd_regs_service(WT, CPS)));
     // everything of a step is free when its warpgroup has taken it (which both products precede)
-    auto step_free = [&](int j) { return wait_on(bar(SD_FREE + j % RING), (uint32_t)(j / RING - 1) & 1u); };
+    auto step_free = [&](int j) { return wait_all(bar(SD_FREE + j % RING), (uint32_t)(j / RING - 1) & 1u); };
     if (warp == BWD_W_TILES) {
       if (lane == 0) {
         ptx::prefetch_tensormap(&tmQ);
@@ -178,13 +177,13 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     bool ok = true;
     int n_steps = 1;                                          // step 0 always exists; the others are known with the walk
     if (wg > 0) {
-      ok = wait_on(bar(META_READY), 0);
+      ok = wait_all(bar(META_READY), 0);
       n_steps = ok ? misc->n_steps : 0;
     }
     for (int j = wg; j < n_steps && ok; j += BWD_ROW_WG) {
       const int st = j % RING;
       const uint32_t ph = (uint32_t)(j / RING) & 1u;
-      ok = wait_on(bar(REC_FULL + st), ph);                   // the step's record is visible
+      ok = wait_all(bar(REC_FULL + st), ph);                  // the step's record is visible
       if (!ok) break;
       float b2[CPS];                                          // bias in the log2 domain (-inf: the row did not route the chunk)
       int n_vis[CPS];                                         // causal: column c of the slot visible iff c < n_vis
@@ -195,7 +194,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         n_vis[s] = i_row - misc->meta.kvbase[st][s] + 1;
         any = any || b2[s] > -INFINITY;
       }
-      ok = wait_on(bar(SD_FULL + st), ph);
+      ok = wait_all(bar(SD_FULL + st), ph);
       if (!ok) break;
       if (!__any_sync(0xffffffffu, any)) {                    // none of the warp's rows routed the step's chunks
         ptx::mbar_arrive(bar(SD_FREE + st));
@@ -260,7 +259,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         acc += at.x + at.y;
       }
       if (j == 0) {
-        ok = wait_on(bar(META_READY), 0);
+        ok = wait_all(bar(META_READY), 0);
         n_steps = ok ? misc->n_steps : 0;
       }
     }

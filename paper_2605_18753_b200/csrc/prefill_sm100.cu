@@ -127,6 +127,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
   volatile int* abort_flag = &misc->abort_flag;
   const long long wait_limit = a.wait_limit;
   auto wait_on = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait(barrier, parity, abort_flag, wait_limit); };
+  auto wait_all = [&](uint32_t barrier, uint32_t parity) { return ptx::mbar_wait_warp(barrier, parity, abort_flag, wait_limit); };
 
   const int groups = dm.batch * dm.h_kv;
   const int tile = a.n_tiles - 1 - (int)(blockIdx.x / groups);  // late (long) tiles first
@@ -272,12 +273,11 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
         for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
         const int st = j & 1, prev_ph = ((j >> 1) - 1) & 1;   // stage, and the phase of step j-2 on the completion barriers
         if (do_k) {
-          if (j >= 2) ok = wait_on(bar(S_FULL + st), prev_ph);     // QK of step j-2 has read the stage
+          if (j >= 2) ok = wait_all(bar(S_FULL + st), prev_ph);    // QK of step j-2 has read the stage
           if (!ok) break;
           if (lane == 0) load_packed(&tmK, sbase + OFF_K + st * KV_TILE_BYTES, bar(K_FULL + st), kvs);
         } else {
-          if (j >= 2) ok = wait_on(bar(PV_DONE + st), prev_ph);    // PV of step j-2 has read the stage
-          if (!ok) break;
+          const bool free = j < 2 || wait_on(bar(PV_DONE + st), prev_ph);    // PV of step j-2 has read the stage
 #pragma unroll
           for (int s = 0; s < CPS; ++s) {
 #pragma unroll
@@ -287,7 +287,8 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
             }
             if (lane == s) misc->kvbase[st][s] = kvs[s];
           }
-          __syncwarp();
+          ok = __all_sync(0xffffffffu, free);      // (the record is written, too; nobody reads it if the warp gives up)
+          if (!ok) break;
           if (lane == 0) load_packed(&tmV, sbase + OFF_V + st * KV_TILE_BYTES, bar(V_FULL + st), kvs);
         }
         last_j[st] = j;
@@ -378,21 +379,20 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
 
     for (int j = 0; ok; ++j) {
       if (j == 1) {
-        ok = wait_on(bar(META), 0);
+        ok = wait_all(bar(META), 0);
         if (!ok) break;
         n_steps = misc->n_steps;
       }
       if (j >= n_steps) break;
       const int buf = j & 1;
-      // bias / kvbase of the step visible; the MMA thread relies on this wait for the V tile as well
-      ok = wait_on(bar(V_FULL + buf), (j >> 1) & 1);
-      if (!ok) break;
+      // bias / kvbase of the step visible; the MMA thread relies on this wait for the V tile as well.  (A lane whose wait runs out
+      // here or at the scores stays with its warp, on values of no meaning, until the warp votes before it hands P on.)
+      bool here = wait_on(bar(V_FULL + buf), (j >> 1) & 1);
       float b2s[CPS];                                // per packed chunk: bias in the log2 domain (-inf: not routed)
 #pragma unroll
       for (int s = 0; s < CPS; ++s) b2s[s] = misc->bias[buf][s][t] * 1.4426950408889634f;
       const int kv0 = misc->kvbase[buf][0];
-      ok = wait_on(bar(S_FULL + buf), (j >> 1) & 1);
-      if (!ok) break;
+      here = wait_on(bar(S_FULL + buf), (j >> 1) & 1) && here;
       ptx::tc_fence_after();
       uint32_t sreg[64];
       {
@@ -519,9 +519,13 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
       }
 
       // O is stable once the previous step's PV has completed
-      const bool fix = j > 0 && __any_sync(0xffffffffu, moved);
+      const bool fix = __any_sync(0xffffffffu, moved || !here);
       if (fix) {
-        ok = wait_on(bar(PV_DONE + (buf ^ 1)), ((j - 1) >> 1) & 1);
+        ok = __all_sync(0xffffffffu, here);
+        if (!ok) break;
+      }
+      if (fix && j > 0) {
+        ok = wait_all(bar(PV_DONE + (buf ^ 1)), ((j - 1) >> 1) & 1);
         if (!ok) break;
         ptx::tc_fence_after();
         // rescale this row of the accumulator: O *= 2^(m_old - m_new)
@@ -543,7 +547,7 @@ attend_prefill_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __gri
     }
 
     // epilogue: O / l -> global (row m is 128 contiguous bf16 of token i_row, head r*g_q + hh)
-    if (ok && n_steps > 0) ok = wait_on(bar(PV_DONE + ((n_steps - 1) & 1)), ((n_steps - 1) >> 1) & 1);
+    if (ok && n_steps > 0) ok = wait_all(bar(PV_DONE + ((n_steps - 1) & 1)), ((n_steps - 1) >> 1) & 1);
     if (ok && n_steps > 0) {
       ptx::tc_fence_after();
       const float inv = l > 0.f ? 1.f / l : 0.f;

@@ -242,7 +242,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // 64-chunk blocks while the later ones are still being produced (see solve_streaming)
     const bool row_in_regs = CS == 1 && SPLIT == 1 && n_chunks <= 4;
     if (n_loc > 0 && (row_in_regs || n_cand == 0)) {
-      ok = ptx::mbar_wait(bar(X_FULL), 0, abort_flag);
+      ok = ptx::mbar_wait_warp(bar(X_FULL), 0, abort_flag);
       ptx::tc_fence_after();
     }
     // Cluster all-reduce of two floats per row: every thread writes its pair into slot [parity][its rank][row]
@@ -268,14 +268,14 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if constexpr (CS == 1) {
           *mine = make_float4(va, vb, vc, 0.f);
           ptx::mbar_arrive(mybar);
-          if (!ptx::mbar_wait(mybar, (xround >> 1) & 1, abort_flag)) return false;
+          if (!ptx::mbar_wait_warp(mybar, (xround >> 1) & 1, abort_flag)) return false;
         } else {
           const uint32_t slot = ptx::smem_u32(mine);
 #pragma unroll
           for (int pr = 0; pr < CS; ++pr) ptx::st_cluster_f32x4(ptx::map_to_rank(slot, pr), va, vb, vc, 0.f);
 #pragma unroll
           for (int pr = 0; pr < CS; ++pr) ptx::mbar_arrive_cluster(ptx::map_to_rank(mybar, pr));
-          if (!ptx::mbar_wait_cluster(mybar, (xround >> 1) & 1, abort_flag)) return false;
+          if (!ptx::mbar_wait_cluster_warp(mybar, (xround >> 1) & 1, abort_flag)) return false;
         }
         float sa = 0.f, sb = 0.f, sc = 0.f, mxa = -INFINITY, below = 0.f;
 #pragma unroll
@@ -421,7 +421,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       float s1v[4] = {0.f, 0.f, 0.f, 0.f}, s2v[4] = {0.f, 0.f, 0.f, 0.f};
       for (int k = k_lo; k < k_hi && ok; ++k) {
-        ok = ptx::mbar_wait(bar(CB_DONE + (k >> 1)), 0, abort_flag);
+        ok = ptx::mbar_wait_warp(bar(CB_DONE + (k >> 1)), 0, abort_flag);
         if (!ok) break;
         ptx::tc_fence_after();
         uint32_t v[32];
@@ -440,7 +440,7 @@ select_sm100_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       }
       // the later passes read all of this thread's columns at will: the whole tile must be there
       if (ok && n_loc > 0) {
-        ok = ptx::mbar_wait(bar(X_FULL), 0, abort_flag);
+        ok = ptx::mbar_wait_warp(bar(X_FULL), 0, abort_flag);
         ptx::tc_fence_after();
       }
       float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));

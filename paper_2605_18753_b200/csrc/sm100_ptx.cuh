@@ -36,7 +36,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 
 // Bounded wait: gives up after ~1 s of SM clock (or as soon as another thread of the block has
-// raised *abort_flag), raises the flag itself and returns false.  Never spins forever.
+// raised *abort_flag), raises the flag itself and returns false.  Never spins forever.  For code that one lane runs: it may run out
+// in some lanes of a warp and not in others (mbar_wait_warp).
 constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           long long limit_cycles = WAIT_LIMIT_CYCLES) {
@@ -52,6 +53,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
       }
     }
   }
+}
+
+// The same by a whole converged warp: its lanes go on together or give up together.  A vote, shuffle, warp barrier or
+// tensor-memory access that some lanes reach while others have left the loop has no limit to its own wait, whatever limit the
+// barriers have.  (Voting on every test leaves uniform branches only; a vote on the outcome of mbar_wait cost 1-2 % of a prefill.)
+template <typename Try>
+__device__ __forceinline__ bool warp_wait(Try&& test, volatile int* abort_flag, long long limit_cycles) {
+  if (__all_sync(0xffffffffu, test())) return true;
+  const long long t0 = clock64();
+  for (uint32_t it = 1;; ++it) {
+    if (__all_sync(0xffffffffu, test())) return true;
+    if ((it & 63u) == 0u && __any_sync(0xffffffffu, *abort_flag || clock64() - t0 > limit_cycles)) {
+      *abort_flag = 1;
+      return false;
+    }
+  }
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               long long limit_cycles = WAIT_LIMIT_CYCLES) {
+  return warp_wait([&]() { return mbar_try_wait(bar, parity); }, abort_flag, limit_cycles);
 }
 
 // ---------------------------------------------------------------- thread-block cluster (distributed shared memory)
@@ -102,19 +123,8 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if ((it & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > 2000000000LL) {
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
+__device__ __forceinline__ bool mbar_wait_cluster_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return warp_wait([&]() { return mbar_try_wait_cluster(bar, parity); }, abort_flag, WAIT_LIMIT_CYCLES);
 }
 
 // generic-proxy writes to shared memory -> visible to the async proxy (TMA / tcgen05.mma operand reads)
