@@ -33,7 +33,7 @@ struct BwdArgs {
 };
 
 struct BwdMaps {
-  CUtensorMap q, g, k, v, kc, vc;      // q, g: a query tile per box; kc, vc: one chunk per box (query-tile-stationary kernels pack chunks below 64 tokens)
+  CUtensorMap q, g, qr, gr, k, v, kc, vc;      // q, g: a query tile per box; qr, gr: a run of at most 32 tokens; kc, vc: one chunk per box (query-tile-stationary kernels pack chunks below 64 tokens)
 };
 
 cudaError_t launch_attend_bwd_stats(const BwdArgs& a, const BwdMaps& m, cudaStream_t st);
@@ -56,12 +56,9 @@ constexpr int BWD_ROW_WG = 3, BWD_ROW_THREADS = (BWD_ROW_WG + 1) * 128, BWD_W_TI
 __host__ __device__ constexpr int bwd_regs_service(int wt, int cps) { return wt > 2 || (wt > 0 && cps > 2) ? 104 : wt > 0 || cps > 1 ? 80 : 56; }
 __host__ __device__ constexpr int bwd_regs_row(int wt, int cps) { return (4 * 128 - bwd_regs_service(wt, cps)) / 3 / 8 * 8; }
 
-// 4, 8 or 16 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
+// 4 or 16 bytes global -> shared, asynchronously; the barrier gets one arrival once this thread's copies have landed.
 __device__ __forceinline__ void copy_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy_async8(uint32_t dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void copy_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -85,10 +82,9 @@ struct RingPos {
 
 // The forward kernel's walk (own chunks, then the union of the tile's routed chunks, 64 tokens per step), made by two warps:
 // with TILES one fills a ring of DK K tiles and one of DV V tiles, without it the other a ring of DK step records.  Step j's
-// barrier is full[j mod DK]: of the tiles one arrival with the byte count of both, of the records one and one of every lane.
+// barrier is full[j mod DK], with one arrival: of the tiles with the byte count of both.
 // `free_for(j)` waits until step j's tiles and record may be overwritten (called for j >= min(DK, DV)); `publish(n)` is
-// told the number of steps.  Biases go from the lists to the record by asynchronous copies, so nothing waits for a list entry.  A
-// walk that was cut short (a wait ran out) lets its copies in flight land (bounded).
+// told the number of steps.  A walk that was cut short (a wait ran out) lets its copies in flight land (bounded).
 template <int HD, int CPS, int WT, int DK, int DV, bool TILES, bool POS, typename Meta, typename FreeFor, typename Publish>
 __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMap* tmK, const CUtensorMap* tmV, int grp, int i0, int lane,
                                               uint32_t ring_k, uint32_t ring_v, const unsigned long long* full, Meta* meta,
@@ -103,24 +99,30 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
   RingPos<DK> pk;
   RingPos<DV> pv;
   auto bar_of = [&](int at) { return ptx::smem_u32(full + at); };
+  // (by the whole warp: an elected lane issues, so that the operands are uniform; sixteen copies a step of chunks of 16 tokens)
   auto load = [&](const int* kvs, bool with_k) {
-    const uint32_t bar = bar_of(pk.at);
-    ptx::mbar_arrive_expect_tx(bar, 2 * TILE_BYTES);
+    int at[CPS];
 #pragma unroll
-    for (int s = 0; s < CPS; ++s) {
-      const uint32_t k = ring_k + pk.at * TILE_BYTES + s * W * 128, v = ring_v + pv.at * TILE_BYTES + s * W * 128;
-      if (with_k) {
-        ptx::tma_load_4d(k, tmK, bar, 0, r, kvs[s], b);
-        if constexpr (HD == 128) ptx::tma_load_4d(k + TILE_BYTES / 2, tmK, bar, 64, r, kvs[s], b);
+    for (int s = 0; s < CPS; ++s) at[s] = __shfl_sync(0xffffffffu, kvs[s], 0);
+    if (ptx::elect_one()) {
+      const uint32_t bar = bar_of(pk.at);
+      ptx::mbar_arrive_expect_tx(bar, 2 * TILE_BYTES);
+#pragma unroll
+      for (int s = 0; s < CPS; ++s) {
+        const uint32_t k = ring_k + pk.at * TILE_BYTES + s * W * 128, v = ring_v + pv.at * TILE_BYTES + s * W * 128;
+        if (with_k) {
+          ptx::tma_load_4d(k, tmK, bar, 0, r, at[s], b);
+          if constexpr (HD == 128) ptx::tma_load_4d(k + TILE_BYTES / 2, tmK, bar, 64, r, at[s], b);
+        }
+        ptx::tma_load_4d(v, tmV, bar, 0, r, at[s], b);
+        if constexpr (HD == 128) ptx::tma_load_4d(v + TILE_BYTES / 2, tmV, bar, 64, r, at[s], b);
       }
-      ptx::tma_load_4d(v, tmV, bar, 0, r, kvs[s], b);
-      if constexpr (HD == 128) ptx::tma_load_4d(v + TILE_BYTES / 2, tmV, bar, 64, r, kvs[s], b);
     }
+    __syncwarp();
   };
   auto record_done = [&]() {
-    arrive_after_copies(bar_of(pk.at));
     __syncwarp();
-    if (lane == 0) ptx::mbar_arrive(bar_of(pk.at));      // (releases the record's plain stores)
+    if (lane == 0) ptx::mbar_arrive(bar_of(pk.at));
   };
   // own chunks first: their tiles need nothing from the mask
   for (int sub = 0; sub < own_steps; ++sub) {
@@ -129,7 +131,7 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
 #pragma unroll
     for (int s = 0; s < CPS; ++s) kvs[s] = WIDE && kv0 + s * W < i0 + TQ ? kv0 + s * W : kv0;
     if constexpr (TILES) {
-      if (lane == 0) load(kvs, !skip_own_k);
+      load(kvs, !skip_own_k);
     } else {
       for (int t = lane; t < TQ; t += 32)
 #pragma unroll
@@ -149,27 +151,50 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
   const int total = walk.count();
   const int n_steps = (CPS > 1 ? (total + CPS - 1) / CPS : total * sub_per_blk) + own_steps;
   publish(n_steps);
-  [[maybe_unused]] const float* list[TPL];
-  if constexpr (!TILES) {
-#pragma unroll
-    for (int q = 0; q < TPL; ++q)
-      list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
-  }
   walk.start();
   bool ok = true;
   int j = own_steps;
-  while (j < n_steps && ok) {
-    int cs[CPS], pos[CPS][TPL];
-    walk.template next<!TILES>(cs, pos);
-    for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk); ++sub) {
-      int kvs[CPS];
+  if constexpr (TILES) {
+    while (j < n_steps && ok) {
+      int cs[CPS], pos[CPS][TPL];
+      walk.template next<false>(cs, pos);
+      for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk); ++sub) {
+        int kvs[CPS];
 #pragma unroll
-      for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
-      if (j >= (DK < DV ? DK : DV)) ok = free_for(j);
-      if (!ok) break;
-      if constexpr (TILES) {
-        if (lane == 0) load(kvs, true);
-      } else {
+        for (int s = 0; s < CPS; ++s) kvs[s] = cs[s] * dm.B + sub * NKV;
+        if (j >= (DK < DV ? DK : DV)) ok = free_for(j);
+        if (!ok) break;
+        load(kvs, true);
+        pk.step();
+        pv.step();
+        ++j;
+      }
+    }
+  } else {
+    const float* list[TPL];
+#pragma unroll
+    for (int q = 0; q < TPL; ++q)
+      list[q] = a.blk_bias + (long long)grp * dm.list_rows + list_row_offset(dm, min(i0 + lane + 32 * q, dm.seq_q - 1));
+    // A chunk's biases are asked for before the step before is handed on, and stored when its own turn comes.  (Loads: a warp's 32 list
+    // entries lie in 32 places, and an asynchronous copy of them holds the warp up for some 200 clk, sixteen of them a step in
+    // chunks of 16 with 128 tokens, 6000 clk a step.)
+    int cs[CPS], pos[CPS][TPL];
+    float bias[CPS][TPL];
+    auto ask = [&]() {
+      walk.next(cs, pos);
+#pragma unroll
+      for (int s = 0; s < CPS; ++s)
+#pragma unroll
+        for (int q = 0; q < TPL; ++q) {
+          bias[s][q] = -INFINITY;
+          if (pos[s][q] >= 0) bias[s][q] = __ldg(list[q] + pos[s][q]);
+        }
+    };
+    if (j < n_steps) ask();
+    while (j < n_steps && ok) {
+      for (int sub = 0; sub < (CPS > 1 ? 1 : sub_per_blk); ++sub) {
+        if (j >= DK) ok = free_for(j);
+        if (!ok) break;
         const int ms = pk.at;
 #pragma unroll
         for (int s = 0; s < CPS; ++s) {
@@ -177,23 +202,20 @@ __device__ __forceinline__ void produce_steps(const BwdArgs& a, const CUtensorMa
           for (int q = 0; q < TPL; ++q) {
             const int t = lane + 32 * q;
             if (t < TQ) {
-              if (pos[s][q] >= 0) copy_async4(ptx::smem_u32(&meta->bias[ms][s][t]), list[q] + pos[s][q]);
-              else meta->bias[ms][s][t] = -INFINITY;
+              meta->bias[ms][s][t] = bias[s][q];
               if constexpr (POS) meta->pos[ms][s][t] = pos[s][q];
             }
           }
-          if (lane == s) meta->kvbase[ms][s] = kvs[s];
+          if (lane == s) meta->kvbase[ms][s] = cs[s] * dm.B + sub * NKV;
         }
         record_done();
+        pk.step();
+        ++j;
       }
-      pk.step();
-      pv.step();
-      ++j;
+      if (j < n_steps && ok) ask();
     }
   }
-  if constexpr (!TILES) {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-  } else if (!ok && lane == 0) {
+  if (TILES && !ok && lane == 0) {
     for (int last = j - 1; last >= (skip_own_k ? own_steps : 0) && last > j - 1 - DK; --last)
       for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar_of(last % DK), (uint32_t)(last / DK) & 1u); ++k) {}
   }

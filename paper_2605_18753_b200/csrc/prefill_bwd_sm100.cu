@@ -153,7 +153,7 @@ attend_bwd_dq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     }
     for (int s = 0; s < KST; ++s) {
       ptx::mbar_init(bar(KV_FULL + s), 1);
-      ptx::mbar_init(bar(REC_FULL + s), 1 + 32);
+      ptx::mbar_init(bar(REC_FULL + s), 1);
       ptx::mbar_init(bar(K_FREE + s), 1);
     }
     ptx::fence_barrier_init();
@@ -449,7 +449,7 @@ static_assert(2 * regs_rows(false, 2) + 3 * regs_service(false, 2) <= 5 * 96, "t
 constexpr uint32_t TMEM_COLS = 512;     // S0 S1 [0,128) dP0 dP1 [128,256) dV^T [256,320) dK^T [320,384)
 constexpr uint32_t COL_DP = 128, COL_DV = 256, COL_DK = 320;
 constexpr uint32_t PS_BYTES = 128 * NKV * 2;       // 16 KiB: one term of P (or dS) of a step, 128 rows of 128 bytes
-constexpr int MAX_STAGES = 4, MAX_SLOTS = 16, SCAN_AHEAD = 16;
+constexpr int MAX_STAGES = 4, MAX_SLOTS = 16, AHEAD = 16;
 // Two-term kernels take their sums out of tensor memory every FLUSH steps and add them up in registers: the tensor cores cut the
 // low bits of an accumulator off at every product, so that a sum left there loses about half a unit per product, the longer
 // the walk the more.  dK against float64, 16 heads per KV head, d 64 (relative 2-norm): 1500 tokens 1.3e-5 -> 2.5e-6, 6000
@@ -476,14 +476,15 @@ struct Layout {
     uint32_t tmem_base;
     int abort_flag;
     int total;                            // number of steps, written with the end marker
-    int live[NST];                        // 1: the stage holds a step, -1: no more steps
+    int live[NST];                        // the stage holds a step, 1 with gathered rows, 0 without; -1: no more steps
     int irow[NST][MTQ];                   // token of each of the step's rows
     float bias[NST][CPS][MTQ];            // per token of the step: the chunk's bias (-inf: the token does not attend it)
     // what W_SCAN hands on: tokens (bit 31: a repetition that fills up the last step) and their mask words over the slice's
     // chunks, step after step; last[slot]: no such step
     int tok[RING], last[MAX_SLOTS];
     uint32_t word[RING];
-    uint32_t ahead[SCAN_AHEAD][32];       // mask words that W_SCAN has asked for
+    uint32_t whole[MAX_SLOTS];            // the step's runs that are consecutive tokens (a bit each)
+    uint32_t ahead[AHEAD][32];            // mask words that W_SCAN has asked for
     alignas(16) float2 stats[NST][128];   // log-sum-exp and delta of the tile's rows
   };
   static constexpr uint32_t Q_BYTES = 128 * HD * 2, KV_TILE_BYTES = NKV * HD * 2, STAGE = 2 * Q_BYTES;
@@ -498,7 +499,8 @@ struct Layout {
 // TPL: tokens per lane of the service warps, a step's tokens being at most 32 * TPL.
 template <int HD, int CPS, int TPL, bool P2>
 __global__ void __launch_bounds__(threads(P2), 1)
-attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
+attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
+                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, BwdArgs a) {
   constexpr int NLOAD = n_load(P2), W_LOAD = w_load(P2), THREADS = threads(P2);
   constexpr int MTQ = 32 * TPL;
   using LY = Layout<HD, CPS, MTQ, P2>;
@@ -525,17 +527,19 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   const int k0 = slice * NKV;                                    // first key of the slice
   const int c = k0 >> dm.log_b;                                       // its first chunk (CPS of them)
   const int log_t = 31 - __clz(TQ), log_slots = LY::LOG_RING - log_t, n_slots = 1 << log_slots;      // a step has TQ tokens; steps in W_SCAN's ring (2 .. 16)
+  const int log_run = min(log_t, 5), log_rps = log_t - log_run;      // tokens of a run, runs of a step (1, 2 or 4)
 
   if (tid == 0) {
     misc->abort_flag = ((sbase & 1023u) != 0u) ? 1 : 0;
     if (misc->abort_flag) report_error(a.sb, DASH_ERR_CUDA, 120);
     ptx::mbar_init(bar(KV_FULL), 1);
     for (int s = 0; s < NST; ++s) {
-      // one arrival of the first loader, one of W_META, and one per lane of each for the copies in flight
-      ptx::mbar_init(bar(QD_FULL + s), 2 + 32 * (NLOAD + 1));
+      // one arrival of the first loader, one of W_META, and one per lane of the loaders for the copies in flight
+      ptx::mbar_init(bar(QD_FULL + s), 2 + 32 * NLOAD);
       ptx::mbar_init(bar(ACC_DONE + s), SEQ ? 1 : 2);
     }
     for (int s = 0; s < n_slots; ++s) {
+      misc->last[s] = 0;
       ptx::mbar_init(bar(TOK_FULL + s), 1);
       ptx::mbar_init(bar(TOK_FREE + s), NLOAD + 1);
     }
@@ -566,25 +570,28 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   const long long row0 = (long long)grp * dm.seq_q;
   if (warp == W_SCAN) {
     // =========================== scanner ===========================
-    // The tokens from k0 on, 32 at a time, the mask words of the next groups on their way to shared memory; those that attend the
-    // slice (its own chunks' tokens, and later ones that routed one of them) are appended to the ring.  With several blocks per
-    // slice, block s takes every n_split-th group.  (A short loop on purpose: one warp that runs through unrolled code waits for its
-    // instructions, and pushes the other roles' out of the cache.)
-    const int stride = 32 * a.n_split;
+    // The tokens from k0 on, 32 at a time, the mask words of the next groups on their way; those that attend the
+    // slice (its own chunks' tokens, and later ones that routed one of them) are appended to the ring.  A run of neighbours most of which
+    // attend it goes in as it is, in front of the run that is being gathered: the loader fetches it with one copy per tensor.
+    // With several blocks per slice, block s takes every n_split-th group.  (A short loop on purpose: one warp that runs
+    // through unrolled code waits for its instructions, and pushes the other roles' out of the cache.)
+    const int stride = 32 * a.n_split, R = 1 << log_run;
     bool ok = true;
     int n = 0, free_slots = n_slots, done = 0;      // tokens so far; steps that may be written; steps handed on
+    uint32_t marks = 0u;                            // the open step's runs that are neighbours
     auto reserve = [&](int steps) {
       for (; free_slots < steps && ok; ++free_slots)
         ok = wait_all(bar(TOK_FREE + (free_slots & (n_slots - 1))), (uint32_t)((free_slots >> log_slots) - 1) & 1u);
     };
-    auto hand_on = [&](int steps, bool last) {
+    auto hand_on = [&](int steps) {
       __syncwarp();
       if (lane == 0)
         for (int k = done; k < steps; ++k) {
-          misc->last[k & (n_slots - 1)] = last;
+          misc->whole[k & (n_slots - 1)] = k == done ? marks : 0u;
           ptx::mbar_arrive(bar(TOK_FULL + (k & (n_slots - 1))));
         }
       done = steps;
+      marks = 0u;
     };
     const int i_first = k0 + 32 * (int)blockIdx.y + lane;
     const uint32_t* src = a.mask + (row0 + i_first) * dm.W + wc;
@@ -593,32 +600,66 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     int i_next = i_first;                           // token whose word is asked for next
     uint32_t g = 0;                                 // groups looked at
     auto ask = [&](uint32_t group) {
-      if (i_next < dm.seq_q) copy_async4(ahead + (group & (SCAN_AHEAD - 1)) * 128, src);
+      if (i_next < dm.seq_q) copy_async4(ahead + (group & (AHEAD - 1)) * 128, src);
       asm volatile("cp.async.commit_group;" ::: "memory");
       src += src_step;
       i_next += stride;
     };
 #pragma unroll 1
-    for (uint32_t k = 0; k < SCAN_AHEAD - 1; ++k) ask(k);
+    for (uint32_t k = 0; k < AHEAD - 1; ++k) ask(k);
 #pragma unroll 1
     for (int i = i_first; i - lane < dm.seq_q && ok; i += stride, ++g) {
-      ask(g + SCAN_AHEAD - 1);
-      asm volatile("cp.async.wait_group %0;" ::"n"(SCAN_AHEAD - 1) : "memory");
-      const uint32_t word = misc->ahead[g & (SCAN_AHEAD - 1)][lane];      // (only this lane wrote it)
+      ask(g + AHEAD - 1);
+      asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+      const uint32_t word = misc->ahead[g & (AHEAD - 1)][lane];      // (only this lane wrote it)
       const int own = i >> dm.log_b;
       bool on = false;
 #pragma unroll
       for (int s = 0; s < CPS; ++s) on = on || c + s == own || (c + s < own && ((word >> (bit + s)) & 1u));
       const uint32_t hit = __ballot_sync(0xffffffffu, on && i < dm.seq_q);
       if (hit == 0u) continue;
-      const int e = (n + __popc(hit & ((1u << lane) - 1u))) & (LY::RING - 1);
-      n += __popc(hit);
-      reserve(((n - 1) >> log_t) + 1);
-      if ((hit >> lane) & 1u) {
-        misc->tok[e] = i;
-        misc->word[e] = word;
+      const int n_hit = __popc(hit);
+      // (a gathered row costs about 1.25 rows of a run that is fetched as it is)
+      if (5 * n_hit < 4 * R || i - lane + 32 > dm.seq_q) {
+        const int e = (n + __popc(hit & ((1u << lane) - 1u))) & (LY::RING - 1);
+        n += n_hit;
+        reserve(((n - 1) >> log_t) + 1);
+        if ((hit >> lane) & 1u) {
+          misc->tok[e] = i;
+          misc->word[e] = word;
+        }
+        if ((n >> log_t) > done) hand_on(n >> log_t);
+        continue;
       }
-      if ((n >> log_t) > done) hand_on(n >> log_t, false);
+#pragma unroll 1
+      for (int at = 0; at < 32 && ok; at += R) {
+        const uint32_t bits = (hit >> at) & (0xffffffffu >> (32 - R));
+        const bool here = (unsigned)(lane - at) < (unsigned)R;
+        const int first = n & ~(R - 1), open = n - first;
+        const bool whole = 5 * __popc(bits) >= 4 * R;
+        int e = n + __popc(bits & ((1u << ((lane - at) & 31)) - 1u)), tok = 0;
+        uint32_t w = 0u;
+        if (whole) {                                // the run being gathered moves on by one, and this one takes its place
+          if (lane < open) {
+            tok = misc->tok[(first + lane) & (LY::RING - 1)];
+            w = misc->word[(first + lane) & (LY::RING - 1)];
+          }
+          e = first + lane - at;
+          marks |= 1u << ((first >> log_run) & ((1 << log_rps) - 1));
+        }
+        n += whole ? R : __popc(bits);
+        reserve(((n - 1) >> log_t) + 1);
+        __syncwarp();
+        if (whole && lane < open) {
+          misc->tok[(first + R + lane) & (LY::RING - 1)] = tok;
+          misc->word[(first + R + lane) & (LY::RING - 1)] = w;
+        }
+        if (here && (whole || ((hit >> lane) & 1u))) {
+          misc->tok[e & (LY::RING - 1)] = i;
+          misc->word[e & (LY::RING - 1)] = word;
+        }
+        if ((n >> log_t) > done) hand_on(n >> log_t);
+      }
     }
     const int steps = (n + TQ - 1) >> log_t;
     if (ok && steps > done) {                       // fill up the last step with copies of a token whose weights will be zero
@@ -629,20 +670,26 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         misc->tok[e & (LY::RING - 1)] = copy;
         misc->word[e & (LY::RING - 1)] = 0u;
       }
-      hand_on(steps, false);
+      hand_on(steps);
     }
     reserve(steps + 1);
-    if (ok) hand_on(steps + 1, true);
+    if (ok && lane == 0) {
+      misc->last[steps & (n_slots - 1)] = 1;
+      ptx::mbar_arrive(bar(TOK_FULL + (steps & (n_slots - 1))));
+    }
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp >= W_LOAD && warp < W_LOAD + NLOAD) {
     // =========================== loaders ===========================
-    // The first one fetches K / V, all of them the Q / dO rows of every step's tokens: a lane copies one 16-byte piece of a row, to
-    // where the 128-byte swizzle has it.  A step's stage is free once both accumulating products of the step NST before have
-    // completed.  (cp.async writes through the generic proxy: the issuers fence before their products read the stage.)
+    // The first one fetches K / V and the Q / dO rows of runs of neighbours, all of them the rows of gathered tokens: a lane copies one
+    // 16-byte piece of a row, to where the 128-byte swizzle has it.  A step's stage is free once both accumulating products of the
+    // step NST before have completed.  (cp.async writes through the generic proxy: the issuers fence before their products read
+    // the stage.)
     constexpr int PIECES = HD / 8, RP = 32 / PIECES;      // pieces of a row, rows of a warp's copy
     constexpr int NR = 16 / (RP * NLOAD);                 // of sixteen rows at a time, a loader copies NR x RP
     const int w = warp - W_LOAD, p = lane % PIECES;
     if (w == 0 && lane == 0) {
+      ptx::prefetch_tensormap(&tmQ);
+      ptx::prefetch_tensormap(&tmDO);
       ptx::prefetch_tensormap(&tmK);
       ptx::prefetch_tensormap(&tmV);
       ptx::mbar_arrive_expect_tx(bar(KV_FULL), 2 * KV_TILE_BYTES);
@@ -664,96 +711,153 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
     const long long q_tok = dm.qs[1] * 2, g_tok = dm.os[1] * 2;
     bool ok = true;
+    int n_done = 0;                                       // steps whose copies are under way
     for (int j = 0;; ++j) {
       const int st = j % NST, sl = j & (n_slots - 1);
       ok = wait_all(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
-      if (ok && j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
       if (!ok) break;
       const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
-      if (!end) {
-        const int* tok = misc->tok + (sl << log_t);
-        uint32_t at = st * LY::STAGE;
-#pragma unroll 1
-        for (int it = 0; it < 8; ++it, at += 16 * 128, tok += 16 / g_q) {
-          uint32_t i[NR];
+      const uint32_t whole = end ? 0u : *reinterpret_cast<volatile uint32_t*>(&misc->whole[sl]);
+      const uint32_t tx = 2 * (Q_BYTES >> log_rps) * __popc(whole);
+      int first = misc->tok[sl << log_t];                       // (of the first run)
+      if (j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      if (!ok) break;
+      if (w == 0 && lane == 0) {
+        misc->live[st] = end ? -1 : whole != (2u << ((1 << log_rps) - 1)) - 1u;
+        if (end) misc->total = j;
+        if (whole == 0u) ptx::mbar_arrive(bar(QD_FULL + st));
+        else ptx::mbar_arrive_expect_tx(bar(QD_FULL + st), tx);
+        for (int run = 0; whole >> run; ++run) {
+          if (run > 0) first = misc->tok[(sl << log_t) + (run << log_run)];
+          if (!((whole >> run) & 1u)) continue;
+          const uint32_t dst = sbase + LY::OFF_ST + st * LY::STAGE + run * (128 >> log_rps) * 128;
 #pragma unroll
-          for (int k = 0; k < NR; ++k) i[k] = (uint32_t)tok[tok0[k]] & 0x7fffffffu;
-#pragma unroll
-          for (int k = 0; k < NR; ++k) {
-            copy_async16(dst0[k] + at + LY::AT_Q, q0[k] + (unsigned long long)i[k] * q_tok);
-            copy_async16(dst0[k] + at + LY::AT_G, g0[k] + (unsigned long long)i[k] * g_tok);
+          for (int h = 0; h < HD / 64; ++h) {
+            ptx::tma_load_4d(dst + LY::AT_Q + h * (Q_BYTES / 2), &tmQ, bar(QD_FULL + st), 64 * h, r * g_q, first, b);
+            ptx::tma_load_4d(dst + LY::AT_G + h * (Q_BYTES / 2), &tmDO, bar(QD_FULL + st), 64 * h, r * g_q, first, b);
           }
         }
       }
-      arrive_after_copies(bar(QD_FULL + st));
-      __syncwarp();
-      if (lane == 0) {
-        ptx::mbar_arrive(bar(TOK_FREE + sl));
-        if (w == 0) {
-          misc->live[st] = end ? -1 : 1;
-          if (end) misc->total = j;
-          ptx::mbar_arrive(bar(QD_FULL + st));
-        }
-      }
-      if (end) break;
-    }
-    // a wait that ran out: the copies already issued land before the block retires
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (!ok && w == 0 && lane == 0)
-      for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(KV_FULL), 0); ++k) {}
-  } else if (warp == W_META) {
-    // =========================== biases and statistics of every step ===========================
-    const long long list0 = (long long)grp * dm.list_rows;
-    bool ok = true;
-    for (int j = 0;; ++j) {
-      const int st = j % NST, sl = j & (n_slots - 1);
-      ok = wait_all(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
-      if (!ok) break;
-      const bool end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
-      uint32_t word[TPL];
-      int tok[TPL], before[TPL], row_tok[4];
-#pragma unroll
-      for (int q = 0; q < TPL; ++q) {
-        const bool in = !end && lane + 32 * q < TQ;
-        const int e = ((j << log_t) + lane + 32 * q) & (LY::RING - 1);
-        tok[q] = in ? misc->tok[e] : (int)0x80000000;
-        word[q] = in ? misc->word[e] : 0u;
-        // routed chunks in the mask words before the slice's
-        before[q] = wc > 0 && tok[q] >= 0 && (tok[q] >> dm.log_b) > c ? a.marks[marks_of(dm, grp, tok[q]) + wc - 1] : 0;
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) row_tok[k] = end ? 0 : misc->tok[((j << log_t) + (lane + 32 * k) / g_q) & (LY::RING - 1)] & 0x7fffffff;
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(bar(TOK_FREE + sl));
-      if (j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
-      if (!ok) break;
       if (!end) {
+        const int per_run = 8 >> log_rps;                  // times sixteen rows
+#pragma unroll 1
+        for (int run = 0; run < 1 << log_rps; ++run) {
+          if ((whole >> run) & 1u) continue;
+          uint32_t at = st * LY::STAGE + run * per_run * 16 * 128;
+          const int* t = misc->tok + (sl << log_t) + (run << log_run);
+#pragma unroll 1
+          for (int it = 0; it < per_run; ++it, at += 16 * 128, t += 16 / g_q) {
+            uint32_t i[NR];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          copy_async8(ptx::smem_u32(&misc->stats[st][lane + 32 * k]), a.stats.at(b, r, row_tok[k], (lane + 32 * k) % g_q));
+            for (int k = 0; k < NR; ++k) i[k] = (uint32_t)t[tok0[k]] & 0x7fffffffu;
 #pragma unroll
-        for (int q = 0; q < TPL; ++q) {
-          const int t = lane + 32 * q, i = tok[q] & 0x7fffffff, own = i >> dm.log_b;
-          if (t < TQ) {
-            misc->irow[st][t] = i;
-#pragma unroll
-            for (int s = 0; s < CPS; ++s) {
-              const bool routed = tok[q] >= 0 && c + s < own && ((word[q] >> (bit + s)) & 1u);
-              if (routed)
-                copy_async4(ptx::smem_u32(&misc->bias[st][s][t]),
-                            a.blk_bias + list0 + list_row_offset(dm, i) + before[q] + __popc(word[q] & ((1u << (bit + s)) - 1u)));
-              else
-                misc->bias[st][s][t] = tok[q] >= 0 && c + s == own ? 0.f : -INFINITY;
+            for (int k = 0; k < NR; ++k) {
+              copy_async16(dst0[k] + at + LY::AT_Q, q0[k] + (unsigned long long)i[k] * q_tok);
+              copy_async16(dst0[k] + at + LY::AT_G, g0[k] + (unsigned long long)i[k] * g_tok);
             }
           }
         }
       }
       arrive_after_copies(bar(QD_FULL + st));
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + st));
+      if (lane == 0) ptx::mbar_arrive(bar(TOK_FREE + sl));
       if (end) break;
+      n_done = j + 1;
     }
+    // a wait that ran out: the copies already issued land before the block retires
     asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok && w == 0 && lane == 0) {
+      for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(KV_FULL), 0); ++k) {}
+      for (int j = max(n_done - NST, 0); j < n_done; ++j)
+        for (int k = 0; k < 200000 && !ptx::mbar_try_wait(bar(QD_FULL + j % NST), (uint32_t)(j / NST) & 1u); ++k) {}
+    }
+  } else if (warp == W_META) {
+    // =========================== biases and statistics of every step ===========================
+    // A bias is behind two loads in a row: the count of the row's routed chunks before the slice's mask word, and the list entry.  Each
+    // has a step's time: while step j is stored, the counts of step j + 1 are under way (if its tokens are listed by then), and
+    // its biases and statistics are asked for once step j has been handed on.  (One step after the other this warp was the pace of the
+    // kernel, 3300 clk a step at 8192 tokens, 32/8 heads, chunks of 64, all of them routed, 5700-6300 with 128 tokens a step; loads,
+    // because an asynchronous copy to 32 places holds the warp up for some 200 clk.)
+    const long long list0 = (long long)grp * dm.list_rows;
+    int tok[TPL], before[TPL];           // tokens of the next step, routed chunks before the slice's mask word
+    uint32_t word[TPL];
+    long long at[TPL];                   // start of the token's list
+    int i_now[TPL];                      // tokens, biases and statistics of this step
+    float bias[CPS][TPL];
+    float2 stat[4];
+    int n_tok = 0;                       // steps whose tokens have been read
+    bool end = false;                    // the last of them is the end marker
+    // this lane's rows: lane + 32 k
+    const char* stat0 = reinterpret_cast<const char*>(a.stats.at(b, r, 0, 0));
+    uint32_t stat_at[4], stat_tok[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      stat_tok[k] = (lane + 32 * k) / g_q;
+      stat_at[k] = (uint32_t)(((lane + 32 * k) & (g_q - 1)) * a.stats.sh);
+    }
+    auto read_tokens = [&]() {
+      const int sl = n_tok++ & (n_slots - 1);
+      end = *reinterpret_cast<volatile int*>(&misc->last[sl]) != 0;
+      if (end) return;
+#pragma unroll
+      for (int q = 0; q < TPL; ++q) {
+        if (32 * q >= TQ) break;
+        const bool in = lane + 32 * q < TQ;
+        const int e = (sl << log_t) + lane + 32 * q;
+        tok[q] = in ? misc->tok[e] : (int)0x80000000;
+        word[q] = in ? misc->word[e] : 0u;
+        at[q] = list0 + list_row_offset(dm, tok[q] & 0x7fffffff);
+        before[q] = wc > 0 && tok[q] >= 0 && (tok[q] >> dm.log_b) > c ? a.marks[at[q] + wc - 1] : 0;
+      }
+    };
+    bool ok = true;
+    for (int j = 0; ok; ++j) {
+      const int st = j % NST, sl = j & (n_slots - 1);
+      if (n_tok == j) {
+        ok = wait_all(bar(TOK_FULL + sl), (uint32_t)(j >> log_slots) & 1u);
+        if (!ok) break;
+        read_tokens();
+      }
+      const bool last = end;
+      if (!last) {
+#pragma unroll
+        for (int q = 0; q < TPL; ++q) {
+          if (32 * q >= TQ) break;
+          const int own = (tok[q] & 0x7fffffff) >> dm.log_b;
+          const float* entry = a.blk_bias + at[q] + before[q];
+          i_now[q] = tok[q] & 0x7fffffff;
+#pragma unroll
+          for (int s = 0; s < CPS; ++s) {
+            bias[s][q] = tok[q] >= 0 && c + s == own ? 0.f : -INFINITY;
+            if (tok[q] >= 0 && c + s < own && ((word[q] >> (bit + s)) & 1u)) bias[s][q] = __ldg(entry + __popc(word[q] & ((1u << (bit + s)) - 1u)));
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          stat[k] = *reinterpret_cast<const float2*>(stat0 + (long long)(misc->tok[(sl << log_t) + stat_tok[k]] & 0x7fffffff) * a.stats.si + stat_at[k]);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar(TOK_FREE + sl));
+        if (__all_sync(0xffffffffu, ptx::mbar_test_wait(bar(TOK_FULL + ((j + 1) & (n_slots - 1))), (uint32_t)((j + 1) >> log_slots) & 1u))) read_tokens();
+      }
+      if (j >= NST) ok = wait_all(bar(ACC_DONE + st), (uint32_t)(j / NST - 1) & 1u);
+      if (!ok) break;
+      if (!last) {
+#pragma unroll
+        for (int q = 0; q < TPL; ++q) {
+          const int t = lane + 32 * q;
+          if (t < TQ) {
+            misc->irow[st][t] = i_now[q];
+#pragma unroll
+            for (int s = 0; s < CPS; ++s) misc->bias[st][s][t] = bias[s][q];
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) misc->stats[st][lane + 32 * k] = stat[k];
+      }
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(bar(QD_FULL + st));
+      if (last) break;
+    }
   } else if (warp == W_SD || warp == W_DP) {
     // =========================== issuers of the score products: S = Q K^T (W_SD), dP = dO V^T (W_DP) ===========================
     if (lane == 0) {
@@ -765,8 +869,9 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       for (int j = 0; ok; ++j) {
         const int buf = j & 1, st = j % NST;
         ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
-        ptx::fence_proxy_async_smem();
+        const int live = ok ? *reinterpret_cast<volatile int*>(&misc->live[st]) : -1;
+        if (live < 0) break;
+        if (live > 0) ptx::fence_proxy_async_smem();
         // the P / dS warps have read S / dP of step j-2
         if (j >= 2) ok = wait_on(bar(PDS_FULL + buf), (uint32_t)((j >> 1) - 1) & 1u);
         if (!ok) break;
@@ -793,8 +898,9 @@ attend_bwd_dkv_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       for (int j = 0; ok; ++j) {
         const int buf = j & 1, st = j % NST;
         ok = wait_on(bar(QD_FULL + st), (uint32_t)(j / NST) & 1u);
-        if (!ok || *reinterpret_cast<volatile int*>(&misc->live[st]) < 0) break;
-        ptx::fence_proxy_async_smem();
+        const int live = ok ? *reinterpret_cast<volatile int*>(&misc->live[st]) : -1;
+        if (live < 0) break;
+        if (live > 0) ptx::fence_proxy_async_smem();
         ok = wait_on(bar((SEQ && !is_v ? DS_FULL : PDS_FULL) + buf), (uint32_t)(j >> 1) & 1u);
         if (!ok) break;
         ptx::tc_fence_after();
@@ -984,7 +1090,7 @@ cudaError_t launch_kernels(const BwdArgs& a, const BwdMaps& m, cudaStream_t st) 
     constexpr uint32_t smem = dkv::Layout<HD, CPS, 32 * TPL, P2>::SMEM;
     static std::atomic<unsigned long long> configured{0};
     if ((e = allow_dynamic_smem(kern, smem, configured)) != cudaSuccess) return e;
-    e = launch_chained(kern, dim3((unsigned)(a.n_slices * groups), a.n_split), dim3(dkv::threads(P2)), smem, st, m.k, m.v, a);
+    e = launch_chained(kern, dim3((unsigned)(a.n_slices * groups), a.n_split), dim3(dkv::threads(P2)), smem, st, m.qr, m.gr, m.k, m.v, a);
     count_launch();
     if (e != cudaSuccess) return e;
   }
@@ -1041,6 +1147,9 @@ cudaError_t launch_attend_prefill_bwd_sm100(const Dims& dm, bool two_term, int n
   const int box_kv = dm.B < NKV ? dm.B : NKV;
   if (!make_map(&m.q, Q, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
   if (!make_map(&m.g, dO, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.os, dm.g_q, a.TQ)) return cudaErrorInvalidValue;
+  // (a run of the dK / dV kernel has at most 32 tokens)
+  if (!make_map(&m.qr, Q, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.qs, dm.g_q, std::min(a.TQ, 32))) return cudaErrorInvalidValue;
+  if (!make_map(&m.gr, dO, dm.d, dm.seq_q, dm.h_q, dm.batch, dm.os, dm.g_q, std::min(a.TQ, 32))) return cudaErrorInvalidValue;
   if (!make_map(&m.k, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, NKV)) return cudaErrorInvalidValue;
   if (!make_map(&m.v, V, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.vs, 1, NKV)) return cudaErrorInvalidValue;
   if (!make_map(&m.kc, K, dm.d, dm.seq_kv, dm.h_kv, dm.batch, dm.ks, 1, box_kv)) return cudaErrorInvalidValue;

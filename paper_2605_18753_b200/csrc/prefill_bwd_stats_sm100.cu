@@ -75,7 +75,7 @@ attend_bwd_stats_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       ptx::mbar_init(bar(SD_FULL + s), 1);
       ptx::mbar_init(bar(SD_FREE + s), 128);
       ptx::mbar_init(bar(KV_FULL + s), 1);
-      ptx::mbar_init(bar(REC_FULL + s), 1 + 32);
+      ptx::mbar_init(bar(REC_FULL + s), 1);
     }
     ptx::fence_barrier_init();
   }
